@@ -110,7 +110,8 @@ struct ddh_ctx {
     bool refine_active = false;                    // refinement used by the current solves
     const int* kc_ptr = nullptr;                   // assembled K (CSR, elimination order)
     const int* kc_col = nullptr;
-    const double2* kc_val = nullptr;
+    const void* kc_val = nullptr;                  // fixed point, row exponents kc_ex
+    int* kc_ex = nullptr;
     // gauss rule for loads
     double* gx = nullptr;
     double* gw = nullptr;
@@ -217,6 +218,7 @@ static void free_model(ddh_ctx* ctx) {
     ctx->nd_chains.clear();
     ctx->kc_ptr = ctx->kc_col = nullptr;
     ctx->kc_val = nullptr;
+    ctx->kc_ex = nullptr;
     ctx->gx = ctx->gw = nullptr;
     ctx->tr_off = nullptr; ctx->tr_nq = nullptr; ctx->tr_xoff = nullptr; ctx->tr_x = nullptr; ctx->tr_Q = nullptr;
 }
@@ -849,7 +851,13 @@ static ddh_status upload_model(ddh_ctx* ctx) {
     if (ctx->refine_coarse || want32) {
         if ((st = upload(ctx, m.kc_ptr, &ctx->kc_ptr))) return st;
         if ((st = upload(ctx, m.kc_col, &ctx->kc_col))) return st;
-        if ((st = upload(ctx, conv(m.kc_val), &ctx->kc_val))) return st;
+        const double2* kv;
+        const int* ke;
+        if ((st = upload(ctx, conv(m.kc_val), &kv))) return st;
+        if ((st = upload(ctx, std::vector<int>(nc, 0), &ke))) return st;
+        launch_fix_csr(ctx->kc_ptr, (double2*)kv, (int*)ke, nc, ctx->stream);
+        ctx->kc_val = kv;
+        ctx->kc_ex = (int*)ke;
     }
     // Gauss rule for the boundary loads
     {
@@ -1247,7 +1255,7 @@ static void coarse_solve(ddh_ctx* ctx, const double2* t, double2* x2, double2* t
     double2* r = tmp + (size_t)2 * R * nc;
     double2* dx = tmp + (size_t)3 * R * nc;
     coarse_solve_once(ctx, t, x2, tmp, R, done);
-    launch_csr_residual(ctx->kc_ptr, ctx->kc_col, ctx->kc_val, nc, x2, t, r, R, done, s);
+    launch_csr_residual(ctx->kc_ptr, ctx->kc_col, ctx->kc_val, ctx->kc_ex, nc, x2, t, r, R, done, s);
     coarse_solve_once(ctx, r, dx, tmp, R, done);
     launch_axpby(x2, 1.0, dx, 1.0, x2, (int64_t)R * nc, s);
     ctx->launches += 2;

@@ -1,6 +1,7 @@
 // Coarse solve K x2 = t (Sec. 2.3.3, eq. block_matrix_inversion): dense K^-1 GEMV forms for
 // small coarse systems, the nested-dissection multifrontal solve, and the CSR residual of
 // the refinement step.
+#include "ddh_fixed.cuh"
 #include "ddh_kcommon.cuh"
 #include <utility>
 
@@ -542,47 +543,80 @@ __global__ void __launch_bounds__(128) k_nd_persistent(NDDev d, NDSched sc, cons
     }
 }
 
-// r = t - K x with K in CSR (one warp per row, lanes across the row's entries, up to 8
-// right-hand sides per pass so each matrix entry is loaded once per 8)
-__global__ void k_csr_residual(const int* __restrict__ ptr, const int* __restrict__ col,
-                               const double2* __restrict__ val, int n, const double2* __restrict__ x,
-                               const double2* __restrict__ t, double2* __restrict__ r, int R,
-                               const int* __restrict__ done) {
+// r = t - K x with K in CSR, one warp per row, lanes across the row's entries, RB right-hand sides per
+// pass.  The residual cancels about eight digits of t, so its rounding is what the refined solve, and
+// through it a whole FP64 solve, comes out with; here the sum is exact (ddh_fixed.cuh with the al xl
+// products kept: K scaled by row once, x by the largest entry that the row meets), and t - K x is
+// rounded once.  FP64 bound it before (16 x 16 to 64 x 64 meshes have 30 to 57 entries per row): 32 x 32
+// elements, l = 5, 8 right-hand sides 76 us -> 58 us; the noise of an objective evaluated on the solution
+// (48 x 48 elements, central differences at step 1e-6) fell from 4e-6 to 1.1e-7.
+template <int RB>
+__global__ void __launch_bounds__(128) k_csr_residual(const int* __restrict__ ptr, const int* __restrict__ col,
+                                                      const int4* __restrict__ val, const int* __restrict__ vex, int n,
+                                                      const double2* __restrict__ x, const double2* __restrict__ t,
+                                                      double2* __restrict__ r, int R, const int* __restrict__ done) {
     if (done && *done) return;
     const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, r0 = blockIdx.y * RB, nr = min(RB, R - r0);
     if (row >= n) return;
     const int a0 = ptr[row], a1 = ptr[row + 1];
-    for (int r0 = 0; r0 < R; r0 += 8) {
-        double sx[8], sy[8];
+    const double2* xr = x + (int64_t)r0 * n;
+    unsigned m[RB];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) { sx[q] = 0; sy[q] = 0; }
+    for (int q = 0; q < RB; ++q) m[q] = 0;
+    for (int a = a0 + lane; a < a1; a += 32) {
+        const int c = col[a];
+#pragma unroll
+        for (int q = 0; q < RB; ++q)
+            if (q < nr) m[q] = max(m[q], fx_mag(xr[(int64_t)q * n + c]));
+    }
+#pragma unroll
+    for (int q = 0; q < RB; ++q) m[q] = __reduce_max_sync(0xffffffffu, m[q]) >> 20;
+    const int ea = vex[row];
+#pragma unroll
+    for (int q = 0; q < RB; ++q) {
+        if (q >= nr) break;
+        FxAcc re = {0, 0}, im = {0, 0};
+        long long lre = 0, lim = 0;
         for (int a = a0 + lane; a < a1; a += 32) {
-            const double2 av = val[a];
-            const int c = col[a];
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (r0 + q < R) {
-                    const double2 xv = x[(int64_t)(r0 + q) * n + c];
-                    sx[q] = fma(av.x, xv.x, fma(-av.y, xv.y, sx[q]));
-                    sy[q] = fma(av.x, xv.y, fma(av.y, xv.x, sy[q]));
-                }
+            const double2 xv = xr[(int64_t)q * n + col[a]];
+            const int4 v = val[a], w = fx_cpx(xv.x, xv.y, (int)m[q]);
+            fx_cmac(re, im, v, -v.z, -v.w, w);
+            lre += (long long)v.y * w.y - (long long)v.w * w.w;
+            lim += (long long)v.y * w.w + (long long)v.w * w.y;
         }
+        // carried lane sums: 2^56 (a row's few hundred entries over 32 lanes: at most 2^62 in all)
+        long long v[8] = {re.h, re.l, lre, 0, im.h, im.l, lim, 0};
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            for (int o = 16; o > 0; o >>= 1) {
-                sx[q] += __shfl_xor_sync(0xffffffffu, sx[q], o);
-                sy[q] += __shfl_xor_sync(0xffffffffu, sy[q], o);
-            }
-        if (lane < 8 && r0 + lane < R) {
-            double ox = 0, oy = 0;
+        for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (q == lane) { ox = sx[q]; oy = sy[q]; }
-            const double2 tv = t[(int64_t)(r0 + lane) * n + row];
-            r[(int64_t)(r0 + lane) * n + row] = make_double2(tv.x - ox, tv.y - oy);
+            for (int k = 0; k < 7; ++k)
+                if (k != 3) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+        if (lane < 2) {
+            const FxAcc s = {lane ? v[4] : v[0], lane ? v[5] : v[1]};
+            double hi, lo;
+            fx_exact(s, lane ? v[6] : v[2], hi, lo);
+            const int e = fx_exact_exp(ea, (int)m[q]);
+            const int64_t at = (int64_t)(r0 + q) * n + row;
+            const double tv = lane ? t[at].y : t[at].x;
+            const double v = m[q] == 0x7ff || ea == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
+                                                           : (tv - fx_scale(hi, e)) - fx_scale(lo, e);
+            reinterpret_cast<double*>(r + at)[lane] = v;
         }
     }
+}
+// rows of K in fixed point, in place; one warp per row
+__global__ void k_fix_csr(const int* __restrict__ ptr, double2* __restrict__ val, int* __restrict__ ex, int n) {
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (row >= n) return;
+    unsigned m = 0;
+    for (int a = ptr[row] + lane; a < ptr[row + 1]; a += 32) m = max(m, fx_mag(val[a]));
+    m = __reduce_max_sync(0xffffffffu, m);
+    for (int a = ptr[row] + lane; a < ptr[row + 1]; a += 32) {
+        const double2 v = val[a];
+        reinterpret_cast<int4*>(val)[a] = fx_cpx(v.x, v.y, (int)(m >> 20));
+    }
+    if (lane == 0) ex[row] = (int)(m >> 20);
 }
 
 // ------------------------------------------------------------------ launch wrappers
@@ -719,9 +753,16 @@ void launch_nd_persistent(const NDDev& d, const NDSched& s, bool f32, const doub
     }
 #undef ND_P
 }
-void launch_csr_residual(const int* ptr, const int* col, const double2* val, int n, const double2* x,
+void launch_fix_csr(const int* ptr, double2* val, int* ex, int n, cudaStream_t st) {
+    k_fix_csr<<<(n + 3) / 4, 128, 0, st>>>(ptr, val, ex, n);
+}
+void launch_csr_residual(const int* ptr, const int* col, const void* val, const int* vex, int n, const double2* x,
                          const double2* t, double2* r, int R, const int* done, cudaStream_t st) {
-    k_csr_residual<<<(n + 3) / 4, 128, 0, st>>>(ptr, col, val, n, x, t, r, R, done);
+    const int g = (n + 3) / 4;
+    const int4* v = (const int4*)val;
+    if (R >= 3) k_csr_residual<4><<<dim3(g, (R + 3) / 4), 128, 0, st>>>(ptr, col, v, vex, n, x, t, r, R, done);
+    else if (R == 2) k_csr_residual<2><<<dim3(g, 1), 128, 0, st>>>(ptr, col, v, vex, n, x, t, r, R, done);
+    else k_csr_residual<1><<<dim3(g, 1), 128, 0, st>>>(ptr, col, v, vex, n, x, t, r, R, done);
 }
 void launch_gemv(const void* A, bool f32, int n_out, int n_in, const double2* x, double2* y, const double2* c, int mode,
                  int64_t xs, int64_t ys, int R, const int* done, cudaStream_t st, int form) {

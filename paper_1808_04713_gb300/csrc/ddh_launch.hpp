@@ -149,8 +149,10 @@ void launch_nd_persistent(const NDDev& d, const NDSched& s, bool f32, const doub
 // ints of NDSched::state needed for R right-hand sides
 size_t nd_state_ints(const NDSched& s, int R);
 void nd_set_smem_limits();   // once per device before the first (captured) launch
-// r = t - K x, K in CSR (R right-hand sides, [R][n])
-void launch_csr_residual(const int* ptr, const int* col, const double2* val, int n, const double2* x,
+// r = t - K x, K in CSR with its values in fixed point (launch_fix_csr makes them from complex128 in
+// place; vex: row exponents), R right-hand sides ([R][n])
+void launch_fix_csr(const int* ptr, double2* val, int* ex, int n, cudaStream_t st);
+void launch_csr_residual(const int* ptr, const int* col, const void* val, const int* vex, int n, const double2* x,
                          const double2* t, double2* r, int R, const int* done, cudaStream_t st);
 void launch_dinv(const DevModel& dm, const double2* x, double2* y, int R, const int* done, cudaStream_t st);
 // y = A x (mode 0), y -= A x (1), y = c - A x (2).  For one right-hand side `form` picks the
