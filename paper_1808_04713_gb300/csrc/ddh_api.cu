@@ -112,10 +112,7 @@ struct ddh_ctx {
     const int* kc_col = nullptr;
     const void* kc_val = nullptr;                  // fixed point, row exponents kc_ex
     int* kc_ex = nullptr;
-    // gauss rule for loads
-    double* gx = nullptr;
-    double* gw = nullptr;
-    int nq = 0;
+    PlaneLoad pload;                               // tables of the plane-wave loads
     // work buffers (grow on demand)
     std::map<std::string, Buf> work;
     // Krylov solvers: dual interface problem (plain solve / inner preconditioner) and the
@@ -219,7 +216,7 @@ static void free_model(ddh_ctx* ctx) {
     ctx->kc_ptr = ctx->kc_col = nullptr;
     ctx->kc_val = nullptr;
     ctx->kc_ex = nullptr;
-    ctx->gx = ctx->gw = nullptr;
+    ctx->pload = PlaneLoad();
     ctx->tr_off = nullptr; ctx->tr_nq = nullptr; ctx->tr_xoff = nullptr; ctx->tr_x = nullptr; ctx->tr_Q = nullptr;
 }
 
@@ -859,16 +856,40 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         ctx->kc_val = kv;
         ctx->kc_ex = (int*)ke;
     }
-    // Gauss rule for the boundary loads
+    // plane-wave loads: boundary elements, and per degree w_q N~_m(t_q) on a Gauss-Legendre rule
     {
-        std::vector<double> x, w;
-        ctx->nq = 64;
-        gauss_legendre(ctx->nq, x, w);
-        const double* a;
-        if ((st = upload(ctx, x, &a))) return st;
-        ctx->gx = (double*)a;
-        if ((st = upload(ctx, w, &a))) return st;
-        ctx->gw = (double*)a;
+        std::vector<double> x, w, Wq, P(pmax + 1);
+        gauss_legendre(kLoadNodes, x, w);
+        std::vector<int64_t> wo;
+        for (const auto& T : m.tabs) {
+            wo.push_back((int64_t)Wq.size());
+            Wq.resize(Wq.size() + (size_t)(T.p + 1) * kLoadNodes);
+            double* W = Wq.data() + wo.back();
+            for (int q = 0; q < kLoadNodes; ++q) {
+                // orthonormal Legendre p_j at the node; N_j = g_j p_j - g_{j-1} p_{j-2}, j >= 2
+                const double t = x[q];
+                P[0] = 1.0 / std::sqrt(2.0);
+                if (T.p >= 1) P[1] = std::sqrt(1.5) * t;
+                for (int j = 2; j <= T.p; ++j)
+                    P[j] = std::sqrt((2.0 * j + 1) * (2.0 * j - 1)) / j * t * P[j - 1] -
+                           (j - 1.0) / j * std::sqrt((2.0 * j + 1) / (2.0 * j - 3)) * P[j - 2];
+                W[q] = 0.5 * (1 + t) * w[q];
+                W[kLoadNodes + q] = 0.5 * (1 - t) * w[q];
+                for (int j = 2; j <= T.p; ++j) {
+                    const double gj = 1.0 / std::sqrt((2.0 * j + 1) * (2.0 * j - 1));
+                    const double gj1 = 1.0 / std::sqrt((2.0 * j - 1) * (2.0 * j - 3));
+                    W[(size_t)j * kLoadNodes + q] = (gj * P[j] - gj1 * P[j - 2]) * w[q];
+                }
+            }
+        }
+        std::vector<int> be;
+        for (int e = 0; e < E; ++e)
+            if (bmask[e]) be.push_back(e);
+        ctx->pload.n_elems = (int)be.size();
+        if ((st = upload(ctx, be, &ctx->pload.elems))) return st;
+        if ((st = upload(ctx, x, &ctx->pload.gx))) return st;
+        if ((st = upload(ctx, Wq, &ctx->pload.Wq))) return st;
+        if ((st = upload(ctx, wo, &ctx->pload.w_off))) return st;
     }
     // Dirichlet trace tables per degree: nq = p + 40 Gauss-Legendre nodes and the weights
     // Q[m-2][i] = (S^-T (p(t_i) w_i))_m, m = 2..p, with orthonormal Legendre p_j (p_j(t) =
@@ -2344,15 +2365,13 @@ ddh_status ddh_rhs_planewave(ddh_ctx* ctx, const double* theta, int32_t R, void*
     if (!ctx->factored) return fail(ctx, DDH_ERR_NOT_READY, "factor first");
     if (!theta || R <= 0 || !b_dev) return fail(ctx, DDH_ERR_INVALID_ARG, "bad arguments");
     if (ctx->m.dirichlet) return fail(ctx, DDH_ERR_INVALID_ARG, "impedance data: not available with a Dirichlet boundary");
+    cudaSetDevice(ctx->device);
     void* th;
-    void* bt;
     ddh_status st;
     if ((st = get_work(ctx, "theta", sizeof(double) * R, &th))) return st;
-    if ((st = get_work(ctx, "bt", sizeof(double2) * (size_t)R * ctx->dm.n_local, &bt))) return st;
     CK(cudaMemcpyAsync(th, theta, sizeof(double) * R, cudaMemcpyHostToDevice, ctx->stream));
-    launch_rhs_planewave(ctx->dm, (const double*)th, ctx->m.k, ctx->gx, ctx->gw, ctx->nq, (double2*)bt, R, ctx->stream);
-    launch_basis(ctx->dm, (const double2*)bt, (double2*)b_dev, 0, R, ctx->stream);
-    ctx->launches += 2;
+    launch_rhs_planewave(ctx->dm, ctx->pload, (const double*)th, ctx->m.k, (double2*)b_dev, R, ctx->stream, 0, 1);
+    ctx->launches += 1;
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(ctx->stream));
     return DDH_OK;
@@ -2456,7 +2475,7 @@ ddh_status ddh_grad_k(ddh_ctx* ctx, const void* u_dev, const void* lam_dev, cons
     // - sum_e Re(lam^T dA_e/dk u)
     launch_grad_elem(d, (const double2*)ut, (const double2*)lt, R, ctx->m.k, 1, (double*)pe, ctx->stream);
     // + Re(lam^T db/dk): db/dk on the interpolatory basis, then its bilinear form with lam
-    launch_rhs_planewave(d, (const double*)th, ctx->m.k, ctx->gx, ctx->gw, ctx->nq, (double2*)db, R, ctx->stream, 1);
+    launch_rhs_planewave(d, ctx->pload, (const double*)th, ctx->m.k, (double2*)db, R, ctx->stream, 1, 0);
     ctx->launches += 4;
     std::vector<double> per(d.E);
     std::vector<double2> dbh((size_t)R * d.n_local), lh((size_t)R * d.n_local);

@@ -167,8 +167,19 @@ constexpr int kTraceMaxNodes = 96;
 void launch_dirichlet_trace(const DevModel& dm, const double* src, double k, const int64_t* tr_off, const int* tr_nq,
                             const int64_t* tr_xoff, const double* tr_x, const double* tr_Q, double2* out, int R,
                             cudaStream_t st);
-void launch_rhs_planewave(const DevModel& dm, const double* theta, double k, const double* gx, const double* gw,
-                          int nq, double2* bt, int R, cudaStream_t st, int dk = 0);
+// Plane-wave loads (clears `out` first): boundary elements, Gauss-Legendre nodes and, per degree table
+// t, the weights Wq[w_off[t] + m kLoadNodes + q] = w_q N~_m(t_q); dk: their derivative in k; nbasis: on
+// the N basis instead of the interpolatory one
+constexpr int kLoadNodes = 64;
+struct PlaneLoad {
+    const int* elems = nullptr;
+    int n_elems = 0;
+    const double* gx = nullptr;
+    const double* Wq = nullptr;
+    const int64_t* w_off = nullptr;
+};
+void launch_rhs_planewave(const DevModel& dm, const PlaneLoad& pl, const double* theta, double k, double2* out, int R,
+                          cudaStream_t st, int dk, int nbasis);
 void launch_grad_elem(const DevModel& dm, const double2* ut, const double2* lt, int R, double k, int mode, double* out,
                       cudaStream_t st);
 void launch_points(const DevModel& dm, const int* pe, const double* pu, int P, int R, const double2* in, double2* out,
