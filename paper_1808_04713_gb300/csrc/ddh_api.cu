@@ -85,16 +85,18 @@ struct ddh_ctx {
     int tc_maxT = 0;
     double2* Kinv = nullptr;                       // dense coarse inverse (elimination order)
     float2* Kinv32 = nullptr;
-    int gemv_form = 1;                             // single-RHS GEMV kernel (timed at upload)
+    int* Kinv_ex = nullptr;                        // its row exponents and column scalings (fixed point)
+    int* Kinv_col = nullptr;
+    int gemv_form = 1;                             // single-RHS complex64 GEMV kernel (timed at upload)
+    int nsm = 0;                                   // SMs of the device
     // nested-dissection factor: complex128 matrices, their complex64 copy (nd32.G/M null
     // unless mixed precision with coarse_fp32), and per tree level the work items
     NDDev nd64, nd32;
     const int4* nd_items = nullptr;
     void* nd_u = nullptr;                          // forward updates [R][u_len] (work buffer)
-    int nd_cut = 1 << 30;                          // levels >= nd_cut run as per-CTA subtrees
-    int nd_nsub = 0, nd_sub_fwd_rows = 0, nd_sub_bwd_rows = 0;
-    const int* nd_sub_ptr = nullptr;
-    const int* nd_sub_nodes = nullptr;
+    std::vector<NDBottom> nd_bottom;               // cut levels below which a CTA per subtree runs the tree
+    struct BottomPick { int at = -1, rb_fwd = 0, rb_bwd = 0; };
+    std::map<int, BottomPick> nd_pick;             // per R: the tuned cut (index, -1 none) and RHS blocks
     std::vector<int> nd_fwd_off, nd_fwd_n, nd_fwd_rows;   // per level: first item, items, staged rows
     std::vector<int> nd_bwd_off, nd_bwd_n, nd_bwd_rows;
     std::map<int, std::vector<int>> nd_rb;         // per R: tuned RHS block of each level (fwd, then bwd)
@@ -204,9 +206,8 @@ static void free_model(ddh_ctx* ctx) {
     ctx->nd32 = NDDev();
     ctx->nd_items = nullptr;
     ctx->nd_u = nullptr;
-    ctx->nd_cut = 1 << 30;
-    ctx->nd_nsub = ctx->nd_sub_fwd_rows = ctx->nd_sub_bwd_rows = 0;
-    ctx->nd_sub_ptr = ctx->nd_sub_nodes = nullptr;
+    ctx->nd_bottom.clear();
+    ctx->nd_pick.clear();
     ctx->nd_fwd_off.clear(); ctx->nd_fwd_n.clear(); ctx->nd_fwd_rows.clear();
     ctx->nd_bwd_off.clear(); ctx->nd_bwd_n.clear(); ctx->nd_bwd_rows.clear();
     ctx->nd_sched = NDSched();
@@ -605,8 +606,17 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         const float2* a32;
         if ((st = upload(ctx, conv32(Kn), &a32))) return st;
         ctx->Kinv32 = (float2*)a32;
-        // autotune: time the single-RHS GEMV forms on this K^-1 and keep the fastest
-        {
+        std::vector<int> ex0(nc, 0);
+        const int* exd;
+        if ((st = upload(ctx, ex0, &exd))) return st;
+        ctx->Kinv_ex = (int*)exd;
+        if ((st = upload(ctx, ex0, &exd))) return st;
+        ctx->Kinv_col = (int*)exd;
+        CK(cudaDeviceGetAttribute(&ctx->nsm, cudaDevAttrMultiProcessorCount, ctx->device));
+        launch_fix_dense(ctx->Kinv, nc, ctx->Kinv_ex, ctx->Kinv_col, ctx->stream);
+        gemv_set_smem_limits();
+        // autotune: time the single-RHS GEMV forms on the complex64 K^-1 and keep the fastest
+        if (want32) {
             double2 *xs = nullptr, *ys = nullptr;
             if (cudaMalloc(&xs, sizeof(double2) * nc) == cudaSuccess && cudaMalloc(&ys, sizeof(double2) * nc) == cudaSuccess) {
                 cudaMemsetAsync(xs, 0, sizeof(double2) * nc, ctx->stream);
@@ -615,10 +625,9 @@ static ddh_status upload_model(ddh_ctx* ctx) {
                 cudaEventCreate(&e1);
                 float best = 1e30f;
                 for (int f = 0; f < 3; ++f) {
-                    launch_gemv(ctx->Kinv, false, nc, nc, xs, ys, nullptr, 0, nc, nc, 1, nullptr, ctx->stream, f);
+                    launch_gemv32(ctx->Kinv32, nc, xs, ys, 1, nullptr, ctx->stream, f);
                     cudaEventRecord(e0, ctx->stream);
-                    for (int rep = 0; rep < 5; ++rep)
-                        launch_gemv(ctx->Kinv, false, nc, nc, xs, ys, nullptr, 0, nc, nc, 1, nullptr, ctx->stream, f);
+                    for (int rep = 0; rep < 5; ++rep) launch_gemv32(ctx->Kinv32, nc, xs, ys, 1, nullptr, ctx->stream, f);
                     cudaEventRecord(e1, ctx->stream);
                     cudaEventSynchronize(e1);
                     float ms = 0;
@@ -729,42 +738,59 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         }
         for (int lv = 0; lv < L; ++lv)
             if (ctx->nd_bwd_rows[lv] > 12800) return fail(ctx, DDH_ERR_INVALID_ARG, "coarse front too large for shared memory");
-        // subtrees: the first level with at least 300 nodes and everything below it run as one
-        // launch per direction, a CTA per subtree (fewer, longer-lived CTAs for the many small fronts)
+        // bottom launches: cut at the first level with at least 12, 40 or 120 nodes (the tuner picks one);
+        // a CTA walks the levels of the subtree below each node of that level
         {
             std::vector<int> count(L, 0);
             for (const auto& N : m.cnode) count[N.depth]++;
-            int cut = L;
-            for (int lv = 1; lv < L; ++lv)
-                if (count[lv] >= 300) { cut = lv; break; }
-            ctx->nd_cut = cut;
-            ctx->nd_nsub = 0;
-            if (cut < L) {
-                std::vector<std::vector<int>> kids(nn);
+            for (const int least : {120, 40, 12}) {
+                NDBottom b;
+                for (b.cut = 1; b.cut < L && count[b.cut] < least; ++b.cut) {}
+                if (b.cut >= L || (!ctx->nd_bottom.empty() && ctx->nd_bottom.back().cut == b.cut)) continue;
+                b.nlev = L - b.cut;
+                for (int lv = b.cut; lv < L; ++lv) {
+                    b.fwd_rows = std::max(b.fwd_rows, ctx->nd_fwd_rows[lv]);
+                    b.bwd_rows = std::max(b.bwd_rows, ctx->nd_bwd_rows[lv]);
+                }
+                if (!nd_bottom_block(b.fwd_rows, 1) || !nd_bottom_block(b.bwd_rows, 1)) continue;
+                // ancestors at the cut (node ids are postorder: a parent's id is the larger)
+                std::vector<int> sub(nn, -1);
+                for (int id = nn - 1; id >= 0; --id) {
+                    const auto& N = m.cnode[id];
+                    if (N.depth == b.cut) sub[id] = b.nsub++;
+                    else if (N.depth > b.cut) sub[id] = sub[N.parent];
+                }
+                // backward rows per level and subtree: 16 by 2 slices while that still gives every warp an
+                // item, else 4 by 8
+                std::vector<int> brows((size_t)b.nsub * b.nlev, 0);
                 for (int id = 0; id < nn; ++id)
-                    if (m.cnode[id].parent >= 0) kids[m.cnode[id].parent].push_back(id);
-                std::vector<int> sp(1, 0), sn;
+                    if (sub[id] >= 0) brows[(size_t)sub[id] * b.nlev + (m.cnode[id].depth - b.cut)] += m.cnode[id].nF;
+                std::vector<std::vector<int4>> fi((size_t)b.nsub * b.nlev), bi((size_t)b.nsub * b.nlev);
                 for (int id = 0; id < nn; ++id) {
-                    if (m.cnode[id].depth != cut) continue;
-                    // postorder of the subtree below id (node ids are already postorder)
-                    std::vector<int> st{id}, sub;
-                    while (!st.empty()) {
-                        const int v = st.back();
-                        st.pop_back();
-                        sub.push_back(v);
-                        for (int c : kids[v]) st.push_back(c);
-                    }
-                    std::sort(sub.begin(), sub.end());
-                    sn.insert(sn.end(), sub.begin(), sub.end());
-                    sp.push_back((int)sn.size());
+                    if (sub[id] < 0) continue;
+                    const auto& N = m.cnode[id];
+                    const size_t at = (size_t)sub[id] * b.nlev + (N.depth - b.cut);
+                    const int nb_ = (int)N.B.size(), n = N.nF + nb_;
+                    for (int r = 0; (r == 0 || r < nb_) && n > 0; r += 32)
+                        fi[at].push_back(make_int4(id, r, std::max(0, std::min(32, nb_ - r)), 1));
+                    const int slices = n <= kNDShortRow && brows[at] >= 96 ? 2 : 8, step = 32 / slices;
+                    for (int r = 0; r < N.nF; r += step) bi[at].push_back(make_int4(id, r, std::min(step, N.nF - r), slices));
                 }
-                ctx->nd_nsub = (int)sp.size() - 1;
-                for (int lv = cut; lv < L; ++lv) {
-                    ctx->nd_sub_fwd_rows = std::max(ctx->nd_sub_fwd_rows, ctx->nd_fwd_rows[lv]);
-                    ctx->nd_sub_bwd_rows = std::max(ctx->nd_sub_bwd_rows, ctx->nd_bwd_rows[lv]);
+                std::vector<int4> fa, ba;
+                std::vector<int> fp, bp;
+                for (size_t k = 0; k < fi.size(); ++k) {
+                    fp.push_back((int)fa.size());
+                    bp.push_back((int)ba.size());
+                    fa.insert(fa.end(), fi[k].begin(), fi[k].end());
+                    ba.insert(ba.end(), bi[k].begin(), bi[k].end());
                 }
-                if ((st = upload(ctx, sp, &ctx->nd_sub_ptr))) return st;
-                if ((st = upload(ctx, sn, &ctx->nd_sub_nodes))) return st;
+                fp.push_back((int)fa.size());
+                bp.push_back((int)ba.size());
+                if ((st = upload(ctx, fa, &b.fitems))) return st;
+                if ((st = upload(ctx, ba, &b.bitems))) return st;
+                if ((st = upload(ctx, fp, &b.fptr))) return st;
+                if ((st = upload(ctx, bp, &b.bptr))) return st;
+                ctx->nd_bottom.push_back(b);
             }
         }
         // one-launch schedule: forward items deepest level first, then backward items root
@@ -828,6 +854,15 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         D.G = a;
         if ((st = upload(ctx, Mall, &a))) return st;
         D.M = a;
+        {
+            std::vector<int> e0((size_t)std::max<int64_t>(D.u_len, nc), 0);
+            const int* ed;
+            for (int** p : {&D.gexp, &D.mexp, &D.gcol, &D.mcol, &D.mcolB}) {
+                if ((st = upload(ctx, e0, &ed))) return st;
+                *p = (int*)ed;
+            }
+            launch_fix_fronts(D, nn, ctx->stream);
+        }
         const int4* it;
         if ((st = upload(ctx, items, &it))) return st;
         ctx->nd_items = it;
@@ -968,8 +1003,6 @@ static ddh_status nd_tune(ddh_ctx* ctx, const Work& w, int R) {
     if (ctx->Kinv || !ctx->nd_levels || ctx->nd_rb.count(R)) return DDH_OK;
     const int L = (int)ctx->nd_fwd_rows.size();
     const int nc = ctx->dm.n_coarse;
-    const bool subs = ctx->nd_nsub > 0 && R < 4;
-    const int cut = subs ? std::min(L, ctx->nd_cut) : L;
     cudaStream_t s = ctx->stream;
     double2* y = w.ctmp;
     double2* u = (double2*)ctx->nd_u;
@@ -978,34 +1011,61 @@ static ddh_status nd_tune(ddh_ctx* ctx, const Work& w, int R) {
     CK(cudaMemsetAsync(y, 0, sizeof(double2) * (size_t)R * nc, s));
     CK(cudaMemsetAsync(u, 0, sizeof(double2) * (size_t)R * ctx->nd64.u_len, s));
     std::vector<int> best(2 * (size_t)L, 0);
+    std::vector<float> cost(2 * (size_t)L, 0.f);
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
+    // fastest right-hand-side block of one launch, and its time
+    auto pick_rb = [&](int rb_max, int& pick, const std::function<void(int)>& run) {
+        float tbest = 1e30f;
+        for (int rb = rb_max; rb >= 1; rb >>= 1) {
+            run(rb);
+            cudaEventRecord(e0, s);
+            for (int rep = 0; rep < 3; ++rep) run(rb);
+            cudaEventRecord(e1, s);
+            cudaEventSynchronize(e1);
+            float ms = 0;
+            cudaEventElapsedTime(&ms, e0, e1);
+            if (ms < 0.97f * tbest) { tbest = ms; pick = rb; }
+        }
+        return tbest;
+    };
     for (int dir = 0; dir < 2; ++dir)
-        for (int lv = 0; lv < cut; ++lv) {
+        for (int lv = dir ? 0 : 1; lv < L; ++lv) {
             const int n = dir ? ctx->nd_bwd_n[lv] : ctx->nd_fwd_n[lv];
             const int rows = dir ? ctx->nd_bwd_rows[lv] : ctx->nd_fwd_rows[lv];
             if (!n) continue;
-            const int rb_max = nd_rhs_block(rows, R);
-            float tbest = 1e30f;
-            for (int rb = rb_max; rb >= 1; rb >>= 1) {
-                auto run = [&] {
-                    if (dir) launch_nd_backward(ctx->nd64, false, ctx->nd_items + ctx->nd_bwd_off[lv], n, rows, y, w.x2, R,
-                                                nullptr, s, rb);
-                    else launch_nd_forward(ctx->nd64, false, ctx->nd_items + ctx->nd_fwd_off[lv], n, rows, w.t, y, u, R,
-                                           nullptr, s, rb);
-                };
-                run();
-                cudaEventRecord(e0, s);
-                for (int rep = 0; rep < 3; ++rep) run();
-                cudaEventRecord(e1, s);
-                cudaEventSynchronize(e1);
-                float ms = 0;
-                cudaEventElapsedTime(&ms, e0, e1);
-                if (ms < 0.97f * tbest) { tbest = ms; best[(size_t)dir * L + lv] = rb; }
-            }
+            cost[(size_t)dir * L + lv] = pick_rb(nd_rhs_block(rows, R), best[(size_t)dir * L + lv], [&](int rb) {
+                if (dir) launch_nd_backward(ctx->nd64, false, ctx->nd_items + ctx->nd_bwd_off[lv], n, rows, lv == 0, w.t, u,
+                                            y, w.x2, R, nullptr, s, rb);
+                else launch_nd_forward(ctx->nd64, false, ctx->nd_items + ctx->nd_fwd_off[lv], n, rows, w.t, y, u, R,
+                                       nullptr, s, rb);
+            });
+        }
+    // the bottom launches against the level launches that they replace
+    ddh_ctx::BottomPick bot;
+    float gain = 0.f;
+    for (size_t c = 0; c < ctx->nd_bottom.size(); ++c) {
+        const NDBottom& b = ctx->nd_bottom[c];
+        ddh_ctx::BottomPick p;
+        p.at = (int)c;
+        float ms = pick_rb(nd_bottom_block(b.fwd_rows, R), p.rb_fwd, [&](int rb) {
+            launch_nd_bottom(true, ctx->nd64, false, b, w.t, y, w.x2, u, R, nullptr, s, rb);
+        });
+        ms += pick_rb(nd_bottom_block(b.bwd_rows, R), p.rb_bwd, [&](int rb) {
+            launch_nd_bottom(false, ctx->nd64, false, b, w.t, y, w.x2, u, R, nullptr, s, rb);
+        });
+        float levels = 0.f;
+        for (int lv = b.cut; lv < L; ++lv) levels += cost[lv] + cost[(size_t)L + lv];
+        if (levels - ms > gain) { gain = levels - ms; bot = p; }
+    }
+    if (bot.at >= 0)
+        for (int lv = ctx->nd_bottom[bot.at].cut; lv < L; ++lv) {
+            best[lv] = bot.rb_fwd;
+            best[(size_t)L + lv] = bot.rb_bwd;
         }
     CK(cudaGetLastError());
+    ctx->nd_pick[R] = bot;
     ctx->nd_rb[R] = best;
     ctx->nd_chains[R] = 1;
     float tbest = 1e30f;
@@ -1290,8 +1350,8 @@ static void coarse_solve_once(ddh_ctx* ctx, const double2* t, double2* x2, doubl
     cudaStream_t s = ctx->stream;
     const bool f32 = ctx->coarse32;
     if (ctx->Kinv) {
-        launch_gemv(f32 ? (const void*)ctx->Kinv32 : (const void*)ctx->Kinv, f32, nc, nc, t, x2, nullptr, 0, nc, nc, R,
-                    done, s, ctx->gemv_form);
+        if (f32) launch_gemv32(ctx->Kinv32, nc, t, x2, R, done, s, ctx->gemv_form);
+        else launch_gemv(ctx->Kinv, ctx->Kinv_ex, ctx->Kinv_col, nc, t, x2, R, done, ctx->nsm, s);
         ctx->launches++;
         return;
     }
@@ -1333,22 +1393,21 @@ static void coarse_solve_once(ddh_ctx* ctx, const double2* t, double2* x2, doubl
 static void nd_level_chain(ddh_ctx* ctx, const NDDev& D, bool f32nd, const double2* t, double2* y, double2* x2,
                            double2* u, int R, const int* done, cudaStream_t s) {
     const int L = (int)ctx->nd_fwd_rows.size();
-    // subtree launches pay off when the launches are latency-bound (few right-hand sides); with
-    // more right-hand sides the serial node chain inside a subtree costs more than it saves
-    const bool subs = ctx->nd_nsub > 0 && R < 4;
-    const int cut = subs ? std::min(L, ctx->nd_cut) : L;
     const auto tuned = ctx->nd_rb.find(R);
     const std::vector<int>* rbs = tuned != ctx->nd_rb.end() ? &tuned->second : nullptr;
-    if (subs) {
-        launch_nd_subtrees(true, D, f32nd, ctx->nd_sub_ptr, ctx->nd_sub_nodes, ctx->nd_nsub, ctx->nd_sub_fwd_rows, t, y,
-                           u, R, done, s);
+    const auto pk = ctx->nd_pick.find(R);
+    const NDBottom* bot = pk != ctx->nd_pick.end() && pk->second.at >= 0 ? &ctx->nd_bottom[pk->second.at] : nullptr;
+    const int cut = bot ? bot->cut : L;
+    if (bot) {
+        launch_nd_bottom(true, D, f32nd, *bot, t, y, x2, u, R, done, s, pk->second.rb_fwd);
         ctx->launches++;
     }
     // every level launch after the first of the chain is a programmatic dependent of the one
     // before it (nd_pdl): its CTAs are scheduled while the previous level drains
-    bool prev_nd = subs;
+    bool prev_nd = bot != nullptr;
     const bool pdl = ctx->opt.nd_pdl != 0;
-    for (int lv = cut - 1; lv >= 0; --lv) {
+    // (the nodes of level 0 have no boundary: their backward launch forms what forward would leave)
+    for (int lv = cut - 1; lv >= 1; --lv) {
         if (!ctx->nd_fwd_n[lv]) continue;
         launch_nd_forward(D, f32nd, ctx->nd_items + ctx->nd_fwd_off[lv], ctx->nd_fwd_n[lv], ctx->nd_fwd_rows[lv], t, y, u,
                           R, done, s, rbs ? (*rbs)[lv] : 0, pdl && prev_nd);
@@ -1357,14 +1416,13 @@ static void nd_level_chain(ddh_ctx* ctx, const NDDev& D, bool f32nd, const doubl
     }
     for (int lv = 0; lv < cut; ++lv) {
         if (!ctx->nd_bwd_n[lv]) continue;
-        launch_nd_backward(D, f32nd, ctx->nd_items + ctx->nd_bwd_off[lv], ctx->nd_bwd_n[lv], ctx->nd_bwd_rows[lv], y, x2,
-                           R, done, s, rbs ? (*rbs)[L + lv] : 0, pdl && prev_nd);
+        launch_nd_backward(D, f32nd, ctx->nd_items + ctx->nd_bwd_off[lv], ctx->nd_bwd_n[lv], ctx->nd_bwd_rows[lv], lv == 0,
+                           t, u, y, x2, R, done, s, rbs ? (*rbs)[L + lv] : 0, pdl && prev_nd);
         prev_nd = true;
         ctx->launches++;
     }
-    if (subs) {
-        launch_nd_subtrees(false, D, f32nd, ctx->nd_sub_ptr, ctx->nd_sub_nodes, ctx->nd_nsub, ctx->nd_sub_bwd_rows, y, x2,
-                           nullptr, R, done, s);
+    if (bot) {
+        launch_nd_bottom(false, D, f32nd, *bot, t, y, x2, u, R, done, s, pk->second.rb_bwd);
         ctx->launches++;
     }
 }
@@ -2348,7 +2406,7 @@ ddh_status ddh_get_info(const ddh_ctx* ctx, ddh_info* out) {
     for (const auto& N : m.cnode) fl += 8.0 * N.nF * ((double)N.nF + 2.0 * (double)N.B.size());
     out->coarse_nd_flops = fl;
     out->coarse_form = m.dense_coarse ? DDH_COARSE_DENSE : (ctx->nd_levels ? DDH_COARSE_ND_LEVELS : DDH_COARSE_ND);
-    out->coarse_subtrees = m.dense_coarse ? 0 : ctx->nd_nsub;
+    out->coarse_subtrees = m.dense_coarse || ctx->nd_bottom.empty() ? 0 : ctx->nd_bottom[0].nsub;
     return DDH_OK;
 }
 

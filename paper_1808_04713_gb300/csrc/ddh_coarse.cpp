@@ -23,6 +23,8 @@ namespace ddh {
 
 namespace {
 
+constexpr int kNDLeaf = 32;
+
 struct NDBuild {
     Model& m;
     const std::vector<int64_t>& X2;
@@ -36,7 +38,9 @@ struct NDBuild {
     int build(std::vector<int>& S, int bx0, int bx1, int by0, int by1, int d) {
         if (S.empty()) return -1;
         const int wx = bx1 - bx0, wy = by1 - by0;
-        if (wx <= 1 && wy <= 1) return make(S, d, {});
+        // a leaf: one base cell, or a block with so few unknowns inside that splitting it on would only add
+        // levels (each is a step of every solve) of fronts with a handful of unknowns
+        if ((wx <= 1 && wy <= 1) || (d > 0 && (int)S.size() <= kNDLeaf)) return make(S, d, {});
         const bool cut_x = wx >= wy;
         const int c = cut_x ? (bx0 + bx1) / 2 : (by0 + by1) / 2;
         const int64_t line = (int64_t)c * H2;
@@ -272,7 +276,8 @@ bool coarse_factor(Model& m, const std::vector<int32_t>& kn_ptr, const std::vect
             std::vector<cd> e(nc, cd(0)), x, r, dx;
             e[col] = 1.0;
             coarse_solve_host(m, e, x);
-            if (m.coarse_refine) {
+            // (K^-1 is applied as it is, without a refinement step in the solves)
+            if (m.coarse_check > 1e-14) {
                 coarse_residual_host(m, e, x, r);
                 coarse_solve_host(m, r, dx);
                 for (int i = 0; i < nc; ++i) x[i] += dx[i];

@@ -81,13 +81,18 @@ __device__ __forceinline__ void fx_flush(FxAcc& s, long long& h, unsigned& l) {
     l += ((unsigned)(t & 255) << 16) | (unsigned)((int)(s.l & ((1ll << kFxLow) - 1)) >> (kFxLow - 16));
     s.h = s.l = 0;
 }
-// d 2^s without double rounding in the normal range
+// d 2^s; results below 2^-1022 become zero
 __device__ __forceinline__ double fx_scale(double d, int s) {
-    const int hi = __double2hiint(d), e = (hi >> 20) & 0x7ff;
-    if (e == 0) return d;                              // zero
-    if ((unsigned)(e + s - 1) < 2046u) return __hiloint2double(hi + (s << 20), __double2loint(d));
-    return scalbn(d, s);
+    const int hi = __double2hiint(d), e = (hi >> 20) & 0x7ff, t = e + s;
+    if ((unsigned)(e - 1) >= 2046u) return d;          // zero, infinity, NaN
+    if ((unsigned)(t - 1) < 2046u) return __hiloint2double(hi + (s << 20), __double2loint(d));
+    return t <= 0 ? 0.0 : __hiloint2double((hi & 0x80000000) | 0x7ff00000, 0);
 }
+// Column scaling: a column whose largest entry has exponent field c is divided by 2^(c - 1023) before the
+// rows get their exponents, and the vector's entry multiplied by it (exactly) before it is staged.  The
+// error of a sum then goes with the largest |a_ij x_j| and not with max |a| max |x|.
+__device__ __forceinline__ int fx_even(int c) { return c == 0 || c == 0x7ff ? 0 : c - 1023; }
+
 // The sum (h + l 2^-24) 2^62 on the scales of exponent fields ea (matrix row) and ex (vector)
 __device__ __forceinline__ double fx_value(long long h, unsigned l, int ea, int ex) {
     if (ea == 0x7ff || ex == 0x7ff) return __longlong_as_double(0x7ff8000000000000ll);

@@ -3,14 +3,77 @@
 // the refinement step.
 #include "ddh_fixed.cuh"
 #include "ddh_kcommon.cuh"
+#include <type_traits>
 #include <utility>
 
 namespace ddh {
 
-// ------------------------------------------------------------------ coarse solve
+// ------------------------------------------------------------------ matrices in fixed point
+// A row of a complex128 matrix turned into limbs in place (see ddh_fixed.cuh) by one warp: the row's
+// exponent goes to ex; sc(j) is the scaling of column j (fx_even).  Entry j is a[j cs], j < n.
+template <class F>
+__device__ __forceinline__ void fix_row(double2* a, int64_t cs, int n, const F& sc, int* ex) {
+    const int lane = threadIdx.x & 31;
+    unsigned m = 0;
+    for (int j = lane; j < n; j += 32) {
+        const double2 v = a[j * cs];
+        const int c = sc(j);
+        m = max(m, fx_mag(make_double2(fx_scale(v.x, -c), fx_scale(v.y, -c))));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    const int ef = (int)(m >> 20);
+    for (int j = lane; j < n; j += 32) {
+        const double2 v = a[j * cs];
+        const int c = sc(j);
+        reinterpret_cast<int4*>(a)[j * cs] = fx_cpx(fx_scale(v.x, -c), fx_scale(v.y, -c), ef);
+    }
+    if (lane == 0) *ex = ef;
+}
+// column scalings of K^-1 (symmetric: its rows' largest entries), then the rows
+__global__ void k_fix_dense_cols(const double2* __restrict__ A, int n, int* __restrict__ cex) {
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (row >= n) return;
+    unsigned m = 0;
+    for (int j = lane; j < n; j += 32) m = max(m, fx_mag(A[(int64_t)row * n + j]));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) cex[row] = fx_even((int)(m >> 20));
+}
+__global__ void k_fix_dense(double2* A, int n, const int* cex, int* ex) {
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (row < n) fix_row(A + (int64_t)row * n, 1, n, [&](int j) { return cex[j]; }, ex + row);
+}
+// the two matrices of one nested-dissection front per CTA (layouts: NDDev)
+__global__ void k_fix_fronts(NDDev d) {
+    const int node = blockIdx.x, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nF = d.nF[node], nB = d.nB[node], n = nF + nB;
+    double2* G = (double2*)const_cast<void*>(d.G) + d.g_off[node];
+    double2* M = (double2*)const_cast<void*>(d.M) + d.m_off[node];
+    const bool gs = nF <= kNDShortRow, ms = n <= kNDShortRow;
+    int* gc = d.gcol + d.f0[node];                         // by column: F for G; F, then B for M
+    int* mf = d.mcol + d.f0[node];
+    int* mb = d.mcolB + d.u_off[node];
+    for (int j = threadIdx.x; j < nF; j += blockDim.x) {
+        unsigned m = 0;
+        for (int r = 0; r < nB; ++r) m = max(m, fx_mag(gs ? G[(int64_t)j * nB + r] : G[(int64_t)r * nF + j]));
+        gc[j] = fx_even((int)(m >> 20));
+    }
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        unsigned m = 0;
+        for (int r = 0; r < nF; ++r) m = max(m, fx_mag(ms ? M[(int64_t)j * nF + r] : M[(int64_t)r * n + j]));
+        (j < nF ? mf + j : mb + j - nF)[0] = fx_even((int)(m >> 20));
+    }
+    __syncthreads();
+    for (int r = warp; r < nB; r += nw)
+        fix_row(G + (gs ? r : (int64_t)r * nF), gs ? nB : 1, nF, [&](int j) { return gc[j]; }, d.gexp + d.u_off[node] + r);
+    for (int r = warp; r < nF; r += nw)
+        fix_row(M + (ms ? r : (int64_t)r * n), ms ? nF : 1, n, [&](int j) { return j < nF ? mf[j] : mb[j - nF]; },
+                d.mexp + d.f0[node] + r);
+}
+
+// ------------------------------------------------------------------ dense K^-1
 // y = A x for a dense row-major complex matrix (n_out x n_in) and R right-hand sides, one
 // warp per output row; the row is read once and applied to up to 8 RHS per pass (vectors and
-// accumulation FP64; the matrix is complex128, or complex64 for the mixed-precision inner solve).
+// accumulation FP64; the matrix is the complex64 K^-1 of the mixed-precision inner solves).
 // mode 0: y = A x ; mode 1: y -= A x ; mode 2: y = c - A x (c given)
 template <class M, int RB>
 __global__ void k_gemv(const M* __restrict__ A, int n_out, int n_in, const double2* __restrict__ x,
@@ -153,20 +216,6 @@ __global__ void __launch_bounds__(128) k_gemv2r(const M* __restrict__ A, int n_o
     }
 }
 
-// ------------------------------------------------------------------ coarse solve
-// Nested-dissection solve of K x = t, one launch per tree level (see NDDev).  A CTA of 128
-// threads takes rows of one node's matrix for a block of RB right-hand sides after staging
-// the node's input vector in shared memory ([RB][stride], odd stride against bank
-// conflicts).  Long rows: up to 4 rows per item, one warp per row, lanes across the row.
-// Short rows (column-major matrix): up to 16 rows per item; a warp takes 4 rows at a time,
-// each row's 8 lanes split into RB right-hand sides x 8/RB column slices, so every lane of
-// the (narrow) FP64 pipe does useful work whatever the block size, and small items spread a
-// level over all SMs (GB300 completes about one warp-wide FP64 FMA per SM every 16 cycles).
-// Arithmetic follows the factor's storage type: FP64 for the complex128 factor, FP32 for its
-// complex64 copy (vectors stay complex128 in global memory and are converted at the edges).
-template <class MT> struct NDType { using T = double; };
-template <> struct NDType<float2> { using T = float; };
-
 __host__ __device__ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v / 2); }
 
 // Warp sum of V values per lane by a transposing butterfly: each of the first log2(V) rounds
@@ -174,28 +223,6 @@ __host__ __device__ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v
 // adds what it receives); the remaining rounds are a plain butterfly on the one value left.
 // V - 1 + 5 - log2(V) adds per lane instead of 5 V.  On return every lane holds the full sum of
 // value index lane >> (5 - log2(V)).
-// Sum of V values per lane over each group of G consecutive lanes (xor offsets G/2, ..., 1, in
-// that order for every value, so the result does not depend on V), transposing while a lane
-// carries more than one value.  Afterwards, with g = lane & (G - 1): if V >= G, v[i] (i < V/G) is
-// the sum of value index (g << log2(V/G)) | i; else v[0] is the sum of value g >> log2(G/V).
-template <class T, int V, int G>
-__device__ __forceinline__ void group_sum_transpose(T (&v)[V]) {
-    static_assert(V >= 1 && (V & (V - 1)) == 0 && G >= 1 && G <= 32 && (G & (G - 1)) == 0, "powers of two");
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int h = V / 2, o = G / 2; h >= 1 && o >= 1; h >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const T send = up ? v[i] : v[i + h];
-            const T keep = up ? v[i + h] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-    }
-#pragma unroll
-    for (int o = (G / 2) >> ilog2(V); o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-}
-
 template <class T, int V>
 __device__ __forceinline__ T warp_sum_transpose(T (&v)[V]) {
     static_assert(V >= 1 && V <= 32 && (V & (V - 1)) == 0, "V must be a power of two <= 32");
@@ -214,187 +241,467 @@ __device__ __forceinline__ T warp_sum_transpose(T (&v)[V]) {
     for (int o = 16 >> ilog2(V); o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
     return v[0];
 }
-__device__ __forceinline__ cpx<double> ld_mat(const double2* a) { const double2 v = __ldg(a); return mk<double>(v.x, v.y); }
-__device__ __forceinline__ cpx<float> ld_mat(const float2* a) { const float2 v = __ldg(a); return mk<float>(v.x, v.y); }
+
+// ------------------------------------------------------------------ coarse solve
+// Nested-dissection solve of K x = t, one launch per tree level (see NDDev).  A CTA of 128
+// threads takes rows of one node's matrix for a block of RB right-hand sides after staging
+// the node's input vector in shared memory ([RB][stride], odd stride against bank
+// conflicts).  Long rows: up to 4 rows per item, one warp per row, lanes across the row.
+// Short rows (column-major matrix): up to 16 rows per item; a warp takes 4 rows at a time,
+// each row's 8 lanes split into RB right-hand sides x 8/RB column slices, so every lane of
+// the (narrow) FP64 pipe does useful work whatever the block size, and small items spread a
+// level over all SMs (GB300 completes about one warp-wide FP64 FMA per SM every 16 cycles).
+// Arithmetic follows the factor's storage type MT: fixed point (int4, FP64-accurate, see
+// ddh_fixed.cuh) for the complex128 factor, FP32 for its complex64 copy (vectors stay complex128 in
+// global memory and are converted when they are staged).
+template <class MT> struct NDVec { using V = cpx<float>; };
+template <> struct NDVec<int4> { using V = int4; };
+template <class MT> constexpr bool kNDFixed = std::is_same<MT, int4>::value;
+
+// Sum of V values per lane over each group of G consecutive lanes (xor offsets G/2, ..., 1, in
+// that order for every value, so the result does not depend on V), transposing while a lane
+// carries more than one value.  Afterwards, with g = lane & (G - 1): if V >= G, v[i] (i < V/G) is
+// the sum of value index (g << log2(V/G)) | i; else v[0] is the sum of value g >> log2(G/V).
+template <class T, int V, int G>
+__device__ __forceinline__ void group_sum_transpose(T (&v)[V]) {
+    static_assert(V >= 1 && (V & (V - 1)) == 0 && G >= 1 && G <= 32 && (G & (G - 1)) == 0, "powers of two");
+    if (G == 1) return;
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = V / 2, o = G / 2; h >= 1 && o >= 1; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const T send = up ? v[i] : v[i + h];
+            const T keep = up ? v[i + h] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+#pragma unroll
+    for (int o = (G / 2) >> ilog2(V); o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+}
+
+// y = K^-1 x, FP64-accurate in fixed point.  A CTA of 16 warps owns `rpc` rows (one CTA per SM), one warp
+// per row.  It stages x in shared memory as limbs, G tiles of kGemvTile columns at a time (a lane's chain
+// over a tile fits one flush, and each tile and vector has its own exponent, so a right-hand side's
+// result does not depend on RB), and adds the tiles up in FP64.  Integer multiply-adds bound it from two
+// right-hand sides on, reading K^-1 (16 n^2 bytes) at one.  FP64 against this form: 35 -> 20 us (n =
+// 1921, one right-hand side), 209 -> 139 us (n = 5425, one), 1437 -> 660 us (n = 4929, eight).
+constexpr int kGemvThreads = 512, kGemvTile = 1008;
+template <int RB>
+__global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const int4* __restrict__ A, const int* __restrict__ aex,
+                                                         const int* __restrict__ acol, int n,
+                                                         const double2* __restrict__ x, double2* __restrict__ y,
+                                                         int r0, int nr, int rpc, const int* __restrict__ done) {
+    if (done && *done) return;
+    extern __shared__ __align__(16) char gv_raw[];
+    constexpr int nw = kGemvThreads / 32, G = 8 / RB, stride = G * kGemvTile + 1;
+    __shared__ unsigned wmax[nw][8];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int4* xs = reinterpret_cast<int4*>(gv_raw);                                             // [RB][stride]
+    double* acc = reinterpret_cast<double*>(gv_raw + (size_t)RB * stride * sizeof(int4));   // [rpc][2 RB]
+    const int row0 = blockIdx.x * rpc, rows = min(rpc, n - row0);
+    for (int g0 = 0; g0 < n; g0 += G * kGemvTile) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {                      // (tile, vector)
+            const int q = k % RB, c0 = g0 + k / RB * kGemvTile, w = min(kGemvTile, n - c0);
+            const double2* xq = x + (int64_t)(r0 + q) * n + c0;
+            double2* d = reinterpret_cast<double2*>(xs) + q * stride + k / RB * kGemvTile;
+            unsigned m = 0;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {                  // kGemvTile <= 2 kGemvThreads
+                const int i = threadIdx.x + u * kGemvThreads;
+                if (i < w) {
+                    double2 v = q < nr ? xq[i] : make_double2(0.0, 0.0);
+                    const int c = acol[c0 + i];
+                    v.x = fx_scale(v.x, c);
+                    v.y = fx_scale(v.y, c);
+                    d[i] = v;
+                    m = max(m, fx_mag(v));
+                }
+            }
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0) wmax[warp][k] = m;
+        }
+        __syncthreads();
+        int ex[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int q = k % RB, w = min(kGemvTile, n - (g0 + k / RB * kGemvTile));
+            unsigned m = 0;
+#pragma unroll
+            for (int i = 0; i < nw; ++i) m = max(m, wmax[i][k]);
+            ex[k] = (int)(m >> 20);
+            int4* d = xs + q * stride + k / RB * kGemvTile;
+            for (int i = threadIdx.x; i < w; i += kGemvThreads) {
+                const double2 v = reinterpret_cast<double2*>(d)[i];
+                d[i] = fx_cpx(v.x, v.y, ex[k]);
+            }
+        }
+        __syncthreads();
+        for (int k = warp; k < rows; k += nw) {
+            constexpr int sh = 5 - ilog2(2 * RB);
+            const int q = lane >> sh;                      // component q & 1 of right-hand side q >> 1
+            const bool mine = (lane & ((1 << sh) - 1)) == 0 && (q >> 1) < nr;
+            double* d = acc + k * 2 * RB + q;
+            double t = g0 && mine ? *d : 0.0;
+#pragma unroll
+            for (int tl = 0; tl < G; ++tl) {
+                const int c0 = g0 + tl * kGemvTile, w = min(kGemvTile, n - c0);
+                if (w <= 0) break;
+                const int4* a = A + (int64_t)(row0 + k) * n + c0;
+                const int4* xt = xs + tl * kGemvTile;
+                FxAcc s[2 * RB];
+#pragma unroll
+                for (int i = 0; i < 2 * RB; ++i) s[i].h = s[i].l = 0;
+                constexpr int U = RB == 1 ? 6 : (RB == 2 ? 4 : 2);     // loads issued ahead of their use
+                int4 av[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) av[u] = lane + 32 * u < w ? __ldg(a + lane + 32 * u) : make_int4(0, 0, 0, 0);
+                for (int j = lane; j < w; j += 32 * U) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int4 v = av[u];
+                        const int jj = min(j + 32 * u, w - 1), jn = j + 32 * (U + u);
+                        av[u] = jn < w ? __ldg(a + jn) : make_int4(0, 0, 0, 0);
+#pragma unroll
+                        for (int b = 0; b < RB; ++b)
+                            fx_cmac(s[2 * b], s[2 * b + 1], v, -v.z, -v.w, xt[b * stride + jj]);
+                    }
+                }
+                long long h[2 * RB];
+                unsigned l[2 * RB];
+#pragma unroll
+                for (int i = 0; i < 2 * RB; ++i) {
+                    h[i] = l[i] = 0;
+                    fx_flush(s[i], h[i], l[i]);
+                }
+                const long long hs = warp_sum_transpose<long long, 2 * RB>(h);
+                const unsigned ls = warp_sum_transpose<unsigned, 2 * RB>(l);
+                int e = ex[tl * RB];
+#pragma unroll
+                for (int i = 1; i < RB; ++i) e = (q >> 1) == i ? ex[tl * RB + i] : e;
+                t += fx_value(hs, ls, aex[row0 + k], e);
+            }
+            if (mine) {
+                if (g0 + G * kGemvTile < n) *d = t;
+                else reinterpret_cast<double*>(y + (int64_t)(r0 + (q >> 1)) * n + row0 + k)[q & 1] = t;
+            }
+        }
+        __syncthreads();                     // the next group overwrites xs
+    }
+}
+
 // Loads of vectors written during the same launch by other CTAs (the one-launch schedule) go
 // through L2 (ld.global.cg): another SM's L1 may hold a stale copy of the line.
 template <bool CG>
 __device__ __forceinline__ double2 ldv(const double2* p) { return CG ? __ldcg(p) : *p; }
+// the children's amounts at offsets a and b of u (-1: none)
 template <bool CG>
-__device__ __forceinline__ double2 nd_pull(const double2* u, int64_t base, const int64_t* src, int64_t i) {
-    const int64_t a = src[2 * i], b = src[2 * i + 1];
+__device__ __forceinline__ double2 nd_pull(const double2* u, int64_t base, int64_t a, int64_t b) {
     double2 s = make_double2(0.0, 0.0);
     if (a >= 0) { const double2 v = ldv<CG>(u + base + a); s.x += v.x; s.y += v.y; }
     if (b >= 0) { const double2 v = ldv<CG>(u + base + b); s.x += v.x; s.y += v.y; }
     return s;
 }
-template <class T>
-__device__ __forceinline__ void cfma(T& ax, T& ay, cpx<T> a, cpx<T> v) {
+__device__ __forceinline__ void cfma(float& ax, float& ay, float2 a, cpx<float> v) {
     ax = fma(a.x, v.x, fma(-a.y, v.y, ax));
     ay = fma(a.x, v.y, fma(a.y, v.x, ay));
 }
 
-// One node's share of a forward level: stage y_F = t_F - w_F (w = the children's amounts),
-// write y_F when asked, then u_N[row] = w_B[row] + (G_N y_F)[row] for rows [row0, row0+nrows).
-// Called by every thread of the CTA; ends without a trailing barrier.
+// Threads that work on one node: the whole CTA, or (WARP) one warp of it, with its own shared memory.
+template <bool WARP>
+struct NDGroup {
+    __device__ __forceinline__ static int t() { return WARP ? threadIdx.x & 31 : threadIdx.x; }
+    __device__ __forceinline__ static int n() { return WARP ? 32 : blockDim.x; }
+    __device__ __forceinline__ static int warp() { return WARP ? 0 : threadIdx.x >> 5; }
+    __device__ __forceinline__ static int warps() { return WARP ? 1 : blockDim.x >> 5; }
+    __device__ __forceinline__ static void sync() { if (WARP) __syncwarp(); else __syncthreads(); }
+};
+constexpr int kNDThreads = 128;          // level launches: four warps (long rows: a row each)
+constexpr int kNDWarps = 8;              // bottom launches, and the most warps of a CTA
+// shared memory beside the staged vectors: exponents, and the warps' maxima while they are found
+struct NDShared {
+    int ex[8];
+    unsigned wmax[kNDWarps][8];
+};
+
+// Stages RB vectors of length n (odd stride) in shared memory: load(i, v) gives entry i of all of them
+// as complex128, so that their index lookups are shared and RB loads are in flight per thread.
+// Fixed point: each vector's exponent is the largest of its entries.
+template <class MT, int RB, bool WARP, class F>
+__device__ __forceinline__ void nd_stage(const F& load, int n, int stride, typename NDVec<MT>::V* sm, int* ex,
+                                         NDShared* sh) {
+    using G = NDGroup<WARP>;
+    if constexpr (kNDFixed<MT>) {
+        double2* s = reinterpret_cast<double2*>(sm);
+        unsigned m[RB];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) m[r] = 0;
+#pragma unroll 2
+        for (int i = G::t(); i < n; i += G::n()) {
+            double2 v[RB];
+            load(i, v);
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                s[r * stride + i] = v[r];
+                m[r] = max(m[r], fx_mag(v[r]));
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < RB; ++r) m[r] = __reduce_max_sync(0xffffffffu, m[r]);
+        if constexpr (!WARP) {
+            if ((threadIdx.x & 31) == 0)
+#pragma unroll
+                for (int r = 0; r < RB; ++r) sh->wmax[threadIdx.x >> 5][r] = m[r];
+            __syncthreads();
+            for (int k = 0; k < G::warps(); ++k)
+#pragma unroll
+                for (int r = 0; r < RB; ++r) m[r] = max(m[r], sh->wmax[k][r]);
+        }
+        if (G::t() == 0)
+#pragma unroll
+            for (int r = 0; r < RB; ++r) ex[r] = (int)(m[r] >> 20);
+        for (int i = G::t(); i < n; i += G::n())
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                const double2 v = s[r * stride + i];
+                sm[r * stride + i] = fx_cpx(v.x, v.y, (int)(m[r] >> 20));
+            }
+    } else {
+        for (int i = G::t(); i < n; i += G::n()) {
+            double2 v[RB];
+            load(i, v);
+#pragma unroll
+            for (int r = 0; r < RB; ++r) sm[r * stride + i] = mk<float>((float)v[r].x, (float)v[r].y);
+        }
+    }
+    G::sync();
+}
+
+// One lane's terms a[j cs] x[j], j = j0, j0 + dj, ... < n, for RB vectors (x staged in sm): v[2r + c] is
+// component c of vector r (fixed point: with low[]).  kNDAhead loads of A are in flight; pre holds the
+// first ones when they were issued before the vectors were staged.
+constexpr int kNDAhead = 4;
+template <class MT> using NDSum = typename std::conditional<kNDFixed<MT>, long long, float>::type;
+template <class MT>
+__device__ __forceinline__ void nd_ahead(const MT* a, int64_t cs, int j0, int dj, int n, bool ok, MT (&pre)[kNDAhead]) {
+#pragma unroll
+    for (int k = 0; k < kNDAhead; ++k) {
+        const int j = j0 + k * dj;
+        pre[k] = ok && j < n ? __ldg(a + j * cs) : MT{};
+    }
+}
+template <class MT, int RB>
+__device__ __forceinline__ void nd_dot(const MT* a, int64_t cs, int j0, int dj, int n, bool ok, MT (&pre)[kNDAhead],
+                                       int stride, const typename NDVec<MT>::V* sm, NDSum<MT> (&v)[2 * RB],
+                                       unsigned (&low)[2 * RB]) {
+#pragma unroll
+    for (int i = 0; i < 2 * RB; ++i) { v[i] = 0; low[i] = 0; }
+    FxAcc s[2 * RB];
+    if constexpr (kNDFixed<MT>)
+#pragma unroll
+        for (int i = 0; i < 2 * RB; ++i) s[i].h = s[i].l = 0;
+    for (int j = j0, c = 0; j < n; j += kNDAhead * dj) {
+        MT nxt[kNDAhead];
+        nd_ahead<MT>(a, cs, j + kNDAhead * dj, dj, n, ok, nxt);
+#pragma unroll
+        for (int k = 0; k < kNDAhead; ++k) {
+            const int jj = min(j + k * dj, n - 1);         // past the end the entry of A is zero
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                if constexpr (kNDFixed<MT>)
+                    fx_cmac(s[2 * r], s[2 * r + 1], pre[k], -pre[k].z, -pre[k].w, sm[r * stride + jj]);
+                else cfma(v[2 * r], v[2 * r + 1], pre[k], sm[r * stride + jj]);
+            }
+            pre[k] = nxt[k];
+        }
+        if constexpr (kNDFixed<MT>)
+            if ((c += kNDAhead) > kFxChain - kNDAhead) {
+                c = 0;
+#pragma unroll
+                for (int i = 0; i < 2 * RB; ++i) fx_flush(s[i], v[i], low[i]);
+            }
+    }
+    if constexpr (kNDFixed<MT>)
+#pragma unroll
+        for (int i = 0; i < 2 * RB; ++i) fx_flush(s[i], v[i], low[i]);
+}
+
+// Rows of one front's matrix, A x + add, by 32/S rows per warp: lane = (row, column slice of S).  In the
+// constructor-like first step (ahead) a lane finds its row and issues its first loads of A; after the
+// vectors are staged, run() forms the sums and hands component c (0 real, 1 imaginary) of right-hand
+// side r to out(row, r, c, value).  Sums run in an order fixed by the matrix alone (fixed point:
+// exactly), so the result does not depend on RB.  cs, rs: strides of A along a row and between rows.
+template <class MT, int RB, int S>
+struct NDRows {
+    static constexpr int nv = 2 * RB >= S ? 2 * RB / S : 1, sh = 2 * RB >= S ? 0 : ilog2(S) - ilog2(2 * RB);
+    const MT* a;
+    int64_t cs;
+    int row, n;
+    bool ok, mine;
+    MT pre[kNDAhead];
+    __device__ __forceinline__ static int slice() { return threadIdx.x & (S - 1); }
+    // value index (component q & 1 of right-hand side q >> 1) of this lane's i-th sum
+    __device__ __forceinline__ static int value(int i) { return 2 * RB >= S ? slice() * nv + i : slice() >> sh; }
+    __device__ __forceinline__ void ahead(const MT* A, int64_t rs, int64_t cs_, int n_, int row_, int end) {
+        row = row_ + ((threadIdx.x & 31) / S);
+        ok = row < end;
+        mine = ok && (slice() & ((1 << sh) - 1)) == 0;
+        a = A + (int64_t)(ok ? row : 0) * rs;
+        cs = cs_;
+        n = n_;
+        nd_ahead<MT>(a, cs, slice(), S, n, ok, pre);
+    }
+    template <class F>
+    __device__ __forceinline__ void run(int stride, const typename NDVec<MT>::V* sm, const int* aex, const int* ex, int nr,
+                                        const double (&add)[nv], const F& out) {
+        NDSum<MT> v[2 * RB];
+        unsigned low[2 * RB];
+        nd_dot<MT, RB>(a, cs, slice(), S, n, ok, pre, stride, sm, v, low);
+        group_sum_transpose<NDSum<MT>, 2 * RB, S>(v);
+        if constexpr (kNDFixed<MT>) group_sum_transpose<unsigned, 2 * RB, S>(low);
+        if (!mine) return;
+        int ea = 0;
+        if constexpr (kNDFixed<MT>) ea = aex[row];
+#pragma unroll
+        for (int i = 0; i < nv; ++i) {
+            const int q = value(i), r = q >> 1;
+            if (r >= nr) continue;
+            if constexpr (kNDFixed<MT>) out(row, r, q & 1, add[i] + fx_value(v[i], low[i], ea, ex[r]));
+            else out(row, r, q & 1, add[i] + (double)v[i]);
+        }
+    }
+};
+
+// an entry's column scaling (fixed point only)
+template <class MT, int RB>
+__device__ __forceinline__ void nd_scale(double2 (&v)[RB], const int* col) {
+    if constexpr (kNDFixed<MT>) {
+        const int c = *col;
+#pragma unroll
+        for (int r = 0; r < RB; ++r) { v[r].x = fx_scale(v[r].x, c); v[r].y = fx_scale(v[r].y, c); }
+    }
+}
+
+// Where rows [row0, row0 + nrows) of a front are worked on: by the warps of a CTA (32/S rows each at a
+// time), or (WARP) by one warp alone.
+// Forward: stage y_F = t_F - w_F (w = the children's amounts), write y_F when asked, then
+// u_N[row] = w_B[row] + (G_N y_F)[row].  Ends without a trailing barrier.
+template <class MT, int RB, int S, bool CG, bool WARP>
+__device__ __forceinline__ void nd_forward_rows(const NDDev& d, int node, int row0, int nrows, bool write_y,
+                                                const double2* __restrict__ t, double2* __restrict__ y,
+                                                double2* __restrict__ u, int r0, int nr,
+                                                typename NDVec<MT>::V* nd_sm, int* ex, NDShared* sh) {
+    using G = NDGroup<WARP>;
+    const int f0 = d.f0[node], nF = d.nF[node], nB = d.nB[node], sF = nF | 1;
+    const int64_t nc = d.nc, ul = d.u_len, so = d.s_off[node], uo = d.u_off[node];
+    const bool cm = nF <= kNDShortRow;
+    const MT* A = (const MT*)d.G + d.g_off[node];
+    NDRows<MT, RB, S> R;
+    double add[NDRows<MT, RB, S>::nv];
+    auto begin = [&](int row) {
+        R.ahead(A, cm ? 1 : nF, cm ? nB : 1, nF, row, row0 + nrows);
+        const int64_t i = so + nF + (R.ok ? R.row : 0);
+        const int64_t pa = R.mine ? d.src[2 * i] : -1, pb = R.mine ? d.src[2 * i + 1] : -1;
+#pragma unroll
+        for (int k = 0; k < R.nv; ++k) {
+            const int q = R.value(k), r = q >> 1;
+            add[k] = 0;
+            if (r >= nr) continue;
+            const double* ud = reinterpret_cast<const double*>(u + (r0 + r) * ul) + (q & 1);
+            if (pa >= 0) add[k] += CG ? __ldcg(ud + 2 * pa) : ud[2 * pa];
+            if (pb >= 0) add[k] += CG ? __ldcg(ud + 2 * pb) : ud[2 * pb];
+        }
+    };
+    constexpr int per = 32 / S;
+    int row = row0 + G::warp() * per;
+    begin(row);
+    nd_stage<MT, RB, WARP>([&](int i, double2 (&v)[RB]) {
+        const int64_t a = d.src[2 * (so + i)], b = d.src[2 * (so + i) + 1];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            v[r] = make_double2(0.0, 0.0);
+            if (r >= nr) continue;
+            const double2 w = nd_pull<CG>(u, (r0 + r) * ul, a, b);
+            v[r] = t[(r0 + r) * nc + f0 + i];
+            v[r].x -= w.x; v[r].y -= w.y;
+            if (write_y) y[(r0 + r) * nc + f0 + i] = v[r];
+        }
+        nd_scale<MT, RB>(v, d.gcol + f0 + i);
+    }, nF, sF, nd_sm, ex, sh);
+    for (; row < row0 + nrows; row += per * G::warps()) {
+        if (row != row0 + G::warp() * per) begin(row);
+        R.run(sF, nd_sm, d.gexp + uo, ex, nr, add, [&](int rw, int r, int c, double v) {
+            reinterpret_cast<double*>(u + (r0 + r) * ul + uo + rw)[c] = v;
+        });
+    }
+}
+
+// Backward: x_F[rows] = ([W | -H] [y_F; x_B])[rows].  A node without a boundary has nothing to pass up,
+// so it has no forward item when root is set: its y_F = t_F - w_F is formed here.
+template <class MT, int RB, int S, bool CG, bool WARP>
+__device__ __forceinline__ void nd_backward_rows(const NDDev& d, int node, int row0, int nrows, bool root,
+                                                 const double2* __restrict__ t, const double2* __restrict__ u,
+                                                 const double2* __restrict__ y, double2* __restrict__ x, int r0,
+                                                 int nr, typename NDVec<MT>::V* nd_sm, int* ex, NDShared* sh) {
+    using G = NDGroup<WARP>;
+    const int f0 = d.f0[node], nF = d.nF[node], nB = d.nB[node], n = nF + nB, sn = n | 1;
+    const int64_t nc = d.nc, ul = d.u_len, so = d.s_off[node], uo = d.u_off[node];
+    const int* bi = d.bidx + d.b_off[node];
+    const bool cm = n <= kNDShortRow;
+    const MT* A = (const MT*)d.M + d.m_off[node];
+    NDRows<MT, RB, S> R;
+    double add[NDRows<MT, RB, S>::nv];
+#pragma unroll
+    for (int k = 0; k < R.nv; ++k) add[k] = 0;
+    constexpr int per = 32 / S;
+    int row = row0 + G::warp() * per;
+    R.ahead(A, cm ? 1 : n, cm ? nF : 1, n, row, row0 + nrows);
+    nd_stage<MT, RB, WARP>([&](int i, double2 (&v)[RB]) {
+        if (root) {
+            const int64_t a = d.src[2 * (so + i)], b = d.src[2 * (so + i) + 1];
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                v[r] = make_double2(0.0, 0.0);
+                if (r >= nr) continue;
+                const double2 w = nd_pull<CG>(u, (r0 + r) * ul, a, b);
+                v[r] = t[(r0 + r) * nc + f0 + i];
+                v[r].x -= w.x; v[r].y -= w.y;
+            }
+        } else {
+            const int pos = i < nF ? f0 + i : bi[i - nF];
+            const double2* src = i < nF ? y : x;
+#pragma unroll
+            for (int r = 0; r < RB; ++r) v[r] = r < nr ? ldv<CG>(src + (r0 + r) * nc + pos) : make_double2(0.0, 0.0);
+        }
+        nd_scale<MT, RB>(v, i < nF ? d.mcol + f0 + i : d.mcolB + uo + i - nF);
+    }, n, sn, nd_sm, ex, sh);
+    for (; row < row0 + nrows; row += per * G::warps()) {
+        if (row != row0 + G::warp() * per) R.ahead(A, cm ? 1 : n, cm ? nF : 1, n, row, row0 + nrows);
+        R.run(sn, nd_sm, d.mexp + f0, ex, nr, add, [&](int rw, int r, int c, double v) {
+            reinterpret_cast<double*>(x + (r0 + r) * nc + f0 + rw)[c] = v;
+        });
+    }
+}
+
+// The column slices of a level item: 32 (one warp per row) for a row-major matrix, 8 for a column-major
+// one (long and short rows)
 template <class MT, int RB, bool CG = false>
 __device__ __forceinline__ void nd_forward_node(const NDDev& d, int node, int row0, int nrows, bool shortm,
                                                 bool write_y, const double2* __restrict__ t, double2* __restrict__ y,
                                                 double2* __restrict__ u, int r0, int nr,
-                                                cpx<typename NDType<MT>::T>* nd_sm) {
-    using T = typename NDType<MT>::T;
-    const int f0 = d.f0[node], nF = d.nF[node], nB = d.nB[node], sF = nF | 1;
-    const int64_t nc = d.nc, ul = d.u_len, so = d.s_off[node], uo = d.u_off[node];
-    for (int i = threadIdx.x; i < nF; i += blockDim.x) {
-        const int pos = f0 + i;
-        for (int r = 0; r < RB; ++r) {
-            double2 v = make_double2(0.0, 0.0);
-            if (r < nr) {
-                const double2 w = nd_pull<CG>(u, (r0 + r) * ul, d.src, so + i);
-                v = t[(r0 + r) * nc + pos];
-                v.x -= w.x; v.y -= w.y;
-                if (write_y) y[(r0 + r) * nc + pos] = v;
-            }
-            nd_sm[r * sF + i] = mk<T>((T)v.x, (T)v.y);
-        }
-    }
-    __syncthreads();
-    const MT* G = (const MT*)d.G + d.g_off[node];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (shortm) {
-        // lane = (row of 4, column slice s of 8), all RB right-hand sides per lane: every
-        // partial sum runs over the columns j = s (mod 8) and the slices are combined in one
-        // fixed tree, so the result does not depend on RB
-        const int rl = lane >> 3, s = lane & 7;
-        for (int base = row0 + warp * 4; base < row0 + nrows; base += 16) {
-            const int row = base + rl;
-            const bool ok = row < row0 + nrows;
-            T v[2 * RB];
-#pragma unroll
-            for (int i = 0; i < 2 * RB; ++i) v[i] = 0;
-            if (ok)
-                for (int j = s; j < nF; j += 8) {
-                    const cpx<T> a = ld_mat(G + (int64_t)j * nB + row);
-#pragma unroll
-                    for (int r = 0; r < RB; ++r) cfma(v[2 * r], v[2 * r + 1], a, nd_sm[r * sF + j]);
-                }
-            group_sum_transpose<T, 2 * RB, 8>(v);
-            if (RB >= 4) {
-                // value index (s << log2(2RB/8)) | i: component c of right-hand side r
-#pragma unroll
-                for (int i = 0; i < 2 * RB / 8; ++i) {
-                    const int q = (s << ilog2(2 * RB / 8)) | i, r = q >> 1, c = q & 1;
-                    if (ok && r < nr) {
-                        const double2 w = nd_pull<CG>(u, (r0 + r) * ul, d.src, so + nF + row);
-                        reinterpret_cast<double*>(u + (r0 + r) * ul + uo + row)[c] = (c ? w.y : w.x) + (double)v[i];
-                    }
-                }
-            } else {
-                constexpr int sh = 3 - ilog2(2 * RB);
-                const int q = s >> sh, r = q >> 1, c = q & 1;
-                if (ok && (s & ((1 << sh) - 1)) == 0 && r < nr) {
-                    const double2 w = nd_pull<CG>(u, (r0 + r) * ul, d.src, so + nF + row);
-                    reinterpret_cast<double*>(u + (r0 + r) * ul + uo + row)[c] = (c ? w.y : w.x) + (double)v[0];
-                }
-            }
-        }
-        return;
-    }
-    for (int row = row0 + warp; row < row0 + nrows; row += blockDim.x >> 5) {
-        T ax[RB], ay[RB];
-#pragma unroll
-        for (int r = 0; r < RB; ++r) { ax[r] = 0; ay[r] = 0; }
-        const MT* g = G + (int64_t)row * nF;
-        for (int j = lane; j < nF; j += 32) {
-            const cpx<T> a = ld_mat(g + j);
-#pragma unroll
-            for (int r = 0; r < RB; ++r) cfma(ax[r], ay[r], a, nd_sm[r * sF + j]);
-        }
-        // value 2r + c is component c (0 real, 1 imaginary) of right-hand side r
-        T v[2 * RB];
-#pragma unroll
-        for (int r = 0; r < RB; ++r) { v[2 * r] = ax[r]; v[2 * r + 1] = ay[r]; }
-        const T sum = warp_sum_transpose<T, 2 * RB>(v);
-        constexpr int sh = 5 - ilog2(2 * RB);
-        const int q = lane >> sh, r = q >> 1, c = q & 1;
-        if ((lane & ((1 << sh) - 1)) == 0 && r < nr) {
-            const double2 w = nd_pull<CG>(u, (r0 + r) * ul, d.src, so + nF + row);
-            reinterpret_cast<double*>(u + (r0 + r) * ul + uo + row)[c] = (c ? w.y : w.x) + (double)sum;
-        }
-    }
+                                                typename NDVec<MT>::V* nd_sm, NDShared* sh) {
+    if (shortm) nd_forward_rows<MT, RB, 8, CG, false>(d, node, row0, nrows, write_y, t, y, u, r0, nr, nd_sm, sh->ex, sh);
+    else nd_forward_rows<MT, RB, 32, CG, false>(d, node, row0, nrows, write_y, t, y, u, r0, nr, nd_sm, sh->ex, sh);
 }
-
-// One node's share of a backward level: x_F[rows] = ([W | -H] [y_F; x_B])[rows]
 template <class MT, int RB, bool CG = false>
-__device__ __forceinline__ void nd_backward_node(const NDDev& d, int node, int row0, int nrows, bool shortm,
+__device__ __forceinline__ void nd_backward_node(const NDDev& d, int node, int row0, int nrows, bool shortm, bool root,
+                                                 const double2* __restrict__ t, const double2* __restrict__ u,
                                                  const double2* __restrict__ y, double2* __restrict__ x, int r0,
-                                                 int nr, cpx<typename NDType<MT>::T>* nd_sm) {
-    using T = typename NDType<MT>::T;
-    const int f0 = d.f0[node], nF = d.nF[node], nB = d.nB[node], n = nF + nB, sn = n | 1;
-    const int64_t nc = d.nc;
-    const int* bi = d.bidx + d.b_off[node];
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int pos = i < nF ? f0 + i : bi[i - nF];
-        const double2* src = i < nF ? y : x;
-        for (int r = 0; r < RB; ++r) {
-            const double2 v = r < nr ? ldv<CG>(src + (r0 + r) * nc + pos) : make_double2(0.0, 0.0);
-            nd_sm[r * sn + i] = mk<T>((T)v.x, (T)v.y);
-        }
-    }
-    __syncthreads();
-    const MT* M = (const MT*)d.M + d.m_off[node];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (shortm) {
-        // as in the forward short rows: 8 column slices, all RB right-hand sides per lane
-        const int rl = lane >> 3, s = lane & 7;
-        for (int base = row0 + warp * 4; base < row0 + nrows; base += 16) {
-            const int row = base + rl;
-            const bool ok = row < row0 + nrows;
-            T v[2 * RB];
-#pragma unroll
-            for (int i = 0; i < 2 * RB; ++i) v[i] = 0;
-            if (ok)
-                for (int j = s; j < n; j += 8) {
-                    const cpx<T> a = ld_mat(M + (int64_t)j * nF + row);
-#pragma unroll
-                    for (int r = 0; r < RB; ++r) cfma(v[2 * r], v[2 * r + 1], a, nd_sm[r * sn + j]);
-                }
-            group_sum_transpose<T, 2 * RB, 8>(v);
-            if (RB >= 4) {
-#pragma unroll
-                for (int i = 0; i < 2 * RB / 8; ++i) {
-                    const int q = (s << ilog2(2 * RB / 8)) | i, r = q >> 1, c = q & 1;
-                    if (ok && r < nr) reinterpret_cast<double*>(x + (r0 + r) * nc + f0 + row)[c] = (double)v[i];
-                }
-            } else {
-                constexpr int sh = 3 - ilog2(2 * RB);
-                const int q = s >> sh, r = q >> 1, c = q & 1;
-                if (ok && (s & ((1 << sh) - 1)) == 0 && r < nr)
-                    reinterpret_cast<double*>(x + (r0 + r) * nc + f0 + row)[c] = (double)v[0];
-            }
-        }
-        return;
-    }
-    for (int row = row0 + warp; row < row0 + nrows; row += blockDim.x >> 5) {
-        T ax[RB], ay[RB];
-#pragma unroll
-        for (int r = 0; r < RB; ++r) { ax[r] = 0; ay[r] = 0; }
-        const MT* mr = M + (int64_t)row * n;
-        for (int j = lane; j < n; j += 32) {
-            const cpx<T> a = ld_mat(mr + j);
-#pragma unroll
-            for (int r = 0; r < RB; ++r) cfma(ax[r], ay[r], a, nd_sm[r * sn + j]);
-        }
-        // value 2r + c is component c (0 real, 1 imaginary) of right-hand side r
-        T v[2 * RB];
-#pragma unroll
-        for (int r = 0; r < RB; ++r) { v[2 * r] = ax[r]; v[2 * r + 1] = ay[r]; }
-        const T sum = warp_sum_transpose<T, 2 * RB>(v);
-        constexpr int sh = 5 - ilog2(2 * RB);
-        const int q = lane >> sh, r = q >> 1, c = q & 1;
-        if ((lane & ((1 << sh) - 1)) == 0 && r < nr)
-            reinterpret_cast<double*>(x + (r0 + r) * nc + f0 + row)[c] = (double)sum;
-    }
+                                                 int nr, typename NDVec<MT>::V* nd_sm, NDShared* sh) {
+    if (shortm) nd_backward_rows<MT, RB, 8, CG, false>(d, node, row0, nrows, root, t, u, y, x, r0, nr, nd_sm, sh->ex, sh);
+    else nd_backward_rows<MT, RB, 32, CG, false>(d, node, row0, nrows, root, t, u, y, x, r0, nr, nd_sm, sh->ex, sh);
 }
 
 // Programmatic dependent launch between consecutive level launches: a CTA first waits until
@@ -408,66 +715,66 @@ __device__ __forceinline__ void nd_pdl_enter() {
 
 // forward level: one item per CTA
 template <class MT, int RB>
-__global__ void __launch_bounds__(128) k_nd_forward(NDDev d, const int4* __restrict__ items,
+__global__ void __launch_bounds__(kNDThreads) k_nd_forward(NDDev d, const int4* __restrict__ items,
                                                     const double2* __restrict__ t, double2* __restrict__ y,
                                                     double2* __restrict__ u, int R, const int* __restrict__ done) {
-    using T = typename NDType<MT>::T;
     nd_pdl_enter();
     if (done && *done) return;
     extern __shared__ __align__(16) char nd_raw[];
+    __shared__ NDShared sh;
     const int4 it = items[blockIdx.x];
     const int r0 = blockIdx.y * RB, nr = min(RB, R - r0);
     nd_forward_node<MT, RB>(d, it.x, it.y, it.z, it.w != 0, it.y == 0, t, y, u, r0, nr,
-                            reinterpret_cast<cpx<T>*>(nd_raw));
+                            reinterpret_cast<typename NDVec<MT>::V*>(nd_raw), &sh);
 }
 
 // backward level: one item per CTA
 template <class MT, int RB>
-__global__ void __launch_bounds__(128) k_nd_backward(NDDev d, const int4* __restrict__ items,
+__global__ void __launch_bounds__(kNDThreads) k_nd_backward(NDDev d, const int4* __restrict__ items, int root,
+                                                     const double2* __restrict__ t, const double2* __restrict__ u,
                                                      const double2* __restrict__ y, double2* __restrict__ x, int R,
                                                      const int* __restrict__ done) {
-    using T = typename NDType<MT>::T;
     nd_pdl_enter();
     if (done && *done) return;
     extern __shared__ __align__(16) char nd_raw[];
+    __shared__ NDShared sh;
     const int4 it = items[blockIdx.x];
     const int r0 = blockIdx.y * RB, nr = min(RB, R - r0);
-    nd_backward_node<MT, RB>(d, it.x, it.y, it.z, it.w != 0, y, x, r0, nr, reinterpret_cast<cpx<T>*>(nd_raw));
+    nd_backward_node<MT, RB>(d, it.x, it.y, it.z, it.w != 0, root != 0, t, u, y, x, r0, nr,
+                             reinterpret_cast<typename NDVec<MT>::V*>(nd_raw), &sh);
 }
 
-// The bottom of the tree in one launch per direction: CTA b owns the subtree below node
-// sub_root[b] and walks its nodes (postorder list sub_nodes[sub_ptr[b] .. sub_ptr[b+1]))
-// children first (forward) or parents first (backward), one barrier between nodes.
-template <class MT, int RB>
-__global__ void __launch_bounds__(128) k_nd_forward_sub(NDDev d, const int* __restrict__ sub_ptr,
-                                                        const int* __restrict__ sub_nodes,
-                                                        const double2* __restrict__ t, double2* __restrict__ y,
-                                                        double2* __restrict__ u, int R, const int* __restrict__ done) {
-    using T = typename NDType<MT>::T;
+// The bottom of the tree in one launch per direction: CTA b owns the subtree below a node of the cut
+// level and walks its levels, deepest first (FWD) or last, with a barrier between levels.  Within a
+// level each warp takes whole items by itself, so nothing but the level barrier couples the warps: the
+// fronts here are small and many, and a launch per level is all latency.  Forward rows are short, and
+// there are many of them: a lane per row (S = 1), no sum across lanes.  Backward rows are few and longer:
+// 4 rows by 8 slices, or 16 by 2 where a level has rows enough for all warps (item.w: slices).
+// 64 x 64 elements, l = 5, 8 right-hand sides, forward and backward: the six deepest level
+// launches took 225 and 155 us, these 96 and 134 us.
+template <class MT, int RB, bool FWD>
+__global__ void __launch_bounds__(32 * kNDWarps) k_nd_bottom(NDDev d, const int4* __restrict__ items,
+                                                             const int* __restrict__ ptr, int nlev, int warp_len,
+                                                             const double2* __restrict__ t, double2* __restrict__ y,
+                                                             double2* __restrict__ x, double2* __restrict__ u, int R,
+                                                             const int* __restrict__ done) {
     if (done && *done) return;
+    using V = typename NDVec<MT>::V;
     extern __shared__ __align__(16) char nd_raw[];
+    __shared__ int ex[kNDWarps][RB];
+    const int warp = threadIdx.x >> 5;
+    V* sm = reinterpret_cast<V*>(nd_raw) + (size_t)warp * warp_len;
     const int r0 = blockIdx.y * RB, nr = min(RB, R - r0);
-    for (int k = sub_ptr[blockIdx.x]; k < sub_ptr[blockIdx.x + 1]; ++k) {
-        const int node = sub_nodes[k];
-        nd_forward_node<MT, RB>(d, node, 0, d.nB[node], d.nF[node] <= kNDShortRow, true, t, y, u, r0, nr,
-                                reinterpret_cast<cpx<T>*>(nd_raw));
-        __syncthreads();
-    }
-}
-template <class MT, int RB>
-__global__ void __launch_bounds__(128) k_nd_backward_sub(NDDev d, const int* __restrict__ sub_ptr,
-                                                         const int* __restrict__ sub_nodes,
-                                                         const double2* __restrict__ y, double2* __restrict__ x, int R,
-                                                         const int* __restrict__ done) {
-    using T = typename NDType<MT>::T;
-    if (done && *done) return;
-    extern __shared__ __align__(16) char nd_raw[];
-    const int r0 = blockIdx.y * RB, nr = min(RB, R - r0);
-    for (int k = sub_ptr[blockIdx.x + 1] - 1; k >= sub_ptr[blockIdx.x]; --k) {
-        const int node = sub_nodes[k];
-        if (d.nF[node] > 0)
-            nd_backward_node<MT, RB>(d, node, 0, d.nF[node], d.nF[node] + d.nB[node] <= kNDShortRow, y, x, r0, nr,
-                                     reinterpret_cast<cpx<T>*>(nd_raw));
+    const int* p = ptr + (size_t)blockIdx.x * nlev;
+    for (int k = 0; k < nlev; ++k) {
+        const int lv = FWD ? nlev - 1 - k : k;
+        for (int i = p[lv] + warp; i < p[lv + 1]; i += kNDWarps) {
+            const int4 it = items[i];
+            __syncwarp();
+            if (FWD) nd_forward_rows<MT, RB, 1, false, true>(d, it.x, it.y, it.z, it.y == 0, t, y, u, r0, nr, sm, ex[warp], nullptr);
+            else if (it.w == 2) nd_backward_rows<MT, RB, 2, false, true>(d, it.x, it.y, it.z, false, t, u, y, x, r0, nr, sm, ex[warp], nullptr);
+            else nd_backward_rows<MT, RB, 8, false, true>(d, it.x, it.y, it.z, false, t, u, y, x, r0, nr, sm, ex[warp], nullptr);
+        }
         __syncthreads();
     }
 }
@@ -492,20 +799,20 @@ __device__ __forceinline__ bool nd_wait(const int* cnt, int target, int* abort_f
 }
 
 template <class MT, int RB>
-__global__ void __launch_bounds__(128) k_nd_persistent(NDDev d, NDSched sc, const double2* __restrict__ t,
+__global__ void __launch_bounds__(kNDThreads) k_nd_persistent(NDDev d, NDSched sc, const double2* __restrict__ t,
                                                        double2* y, double2* x, double2* u, int R,
                                                        const int* __restrict__ done, int* err) {
-    using T = typename NDType<MT>::T;
     if (done && *done) return;
     extern __shared__ __align__(16) char nd_raw[];
     __shared__ int s_ticket, s_ok;
+    __shared__ NDShared sh;
     const int nrb = (R + RB - 1) / RB;
     const int total = sc.nseq * nrb;
     int* ticket = sc.state;
     int* abort_f = sc.state + 1;
     int* fcnt = sc.state + 2;                       // [nn][nrb] finished forward items
     int* bcnt = fcnt + (size_t)sc.nn * nrb;         // [nn][nrb] finished backward items
-    cpx<T>* sm = reinterpret_cast<cpx<T>*>(nd_raw);
+    typename NDVec<MT>::V* sm = reinterpret_cast<typename NDVec<MT>::V*>(nd_raw);
     while (true) {
         if (threadIdx.x == 0) s_ticket = atomicAdd(ticket, 1);
         __syncthreads();
@@ -533,8 +840,8 @@ __global__ void __launch_bounds__(128) k_nd_persistent(NDDev d, NDSched sc, cons
         __syncthreads();
         if (!s_ok) return;
         const int r0 = rb * RB, nr = min(RB, R - r0);
-        if (!bwd) nd_forward_node<MT, RB, true>(d, node, it.y, it.z, shortm, it.y == 0, t, y, u, r0, nr, sm);
-        else nd_backward_node<MT, RB, true>(d, node, it.y, it.z, shortm, y, x, r0, nr, sm);
+        if (!bwd) nd_forward_node<MT, RB, true>(d, node, it.y, it.z, shortm, it.y == 0, t, y, u, r0, nr, sm, &sh);
+        else nd_backward_node<MT, RB, true>(d, node, it.y, it.z, shortm, false, t, u, y, x, r0, nr, sm, &sh);
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
@@ -630,12 +937,12 @@ template <class MT, int RB>
 static void nd_attr() {
     cudaFuncSetAttribute(k_nd_forward<MT, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
     cudaFuncSetAttribute(k_nd_backward<MT, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
-    cudaFuncSetAttribute(k_nd_forward_sub<MT, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
-    cudaFuncSetAttribute(k_nd_backward_sub<MT, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
+    cudaFuncSetAttribute(k_nd_bottom<MT, RB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
+    cudaFuncSetAttribute(k_nd_bottom<MT, RB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
     cudaFuncSetAttribute(k_nd_persistent<MT, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
 }
 void nd_set_smem_limits() {
-    nd_attr<double2, 1>(); nd_attr<double2, 2>(); nd_attr<double2, 4>(); nd_attr<double2, 8>();
+    nd_attr<int4, 1>(); nd_attr<int4, 2>(); nd_attr<int4, 4>(); nd_attr<int4, 8>();
     nd_attr<float2, 1>(); nd_attr<float2, 2>(); nd_attr<float2, 4>(); nd_attr<float2, 8>();
 }
 // launch with (pdl) or without the programmatic-stream-serialization attribute
@@ -643,7 +950,7 @@ template <typename... Exp, typename... Act>
 static void nd_launch(void (*k)(Exp...), dim3 g, size_t sm, cudaStream_t st, bool pdl, Act&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = g;
-    cfg.blockDim = dim3(128);
+    cfg.blockDim = dim3(kNDThreads);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -660,10 +967,10 @@ static void nd_fwd_t(const NDDev& d, const int4* items, int nitems, int smem_row
     nd_launch(k_nd_forward<MT, RB>, dim3(nitems, (R + RB - 1) / RB), sm, st, pdl, d, items, t, y, u, R, done);
 }
 template <class MT, int RB>
-static void nd_bwd_t(const NDDev& d, const int4* items, int nitems, int smem_rows, const double2* y, double2* x,
-                     int R, const int* done, cudaStream_t st, bool pdl) {
+static void nd_bwd_t(const NDDev& d, const int4* items, int nitems, int smem_rows, int root, const double2* t,
+                     const double2* u, const double2* y, double2* x, int R, const int* done, cudaStream_t st, bool pdl) {
     const size_t sm = std::max<size_t>(16, (size_t)(smem_rows | 1) * RB * sizeof(MT));
-    nd_launch(k_nd_backward<MT, RB>, dim3(nitems, (R + RB - 1) / RB), sm, st, pdl, d, items, y, x, R, done);
+    nd_launch(k_nd_backward<MT, RB>, dim3(nitems, (R + RB - 1) / RB), sm, st, pdl, d, items, root, t, u, y, x, R, done);
 }
 void launch_nd_forward(const NDDev& d, bool f32, const int4* items, int nitems, int smem_rows, const double2* t,
                        double2* y, double2* u, int R, const int* done, cudaStream_t st, int rb_want, bool pdl) {
@@ -672,7 +979,7 @@ void launch_nd_forward(const NDDev& d, bool f32, const int4* items, int nitems, 
     const int rb = rb_want > 0 && rb_want <= rb_max ? rb_want : rb_max;
 #define ND_F(RBV)                                                                             \
     if (f32) nd_fwd_t<float2, RBV>(d, items, nitems, smem_rows, t, y, u, R, done, st, pdl);   \
-    else nd_fwd_t<double2, RBV>(d, items, nitems, smem_rows, t, y, u, R, done, st, pdl);
+    else nd_fwd_t<int4, RBV>(d, items, nitems, smem_rows, t, y, u, R, done, st, pdl);
     switch (rb) {
         case 8: ND_F(8) break;
         case 4: ND_F(4) break;
@@ -681,14 +988,15 @@ void launch_nd_forward(const NDDev& d, bool f32, const int4* items, int nitems, 
     }
 #undef ND_F
 }
-void launch_nd_backward(const NDDev& d, bool f32, const int4* items, int nitems, int smem_rows, const double2* y,
-                        double2* x, int R, const int* done, cudaStream_t st, int rb_want, bool pdl) {
+void launch_nd_backward(const NDDev& d, bool f32, const int4* items, int nitems, int smem_rows, int root,
+                        const double2* t, const double2* u, const double2* y, double2* x, int R, const int* done,
+                        cudaStream_t st, int rb_want, bool pdl) {
     if (nitems <= 0) return;
     const int rb_max = nd_rhs_block(smem_rows, R);
     const int rb = rb_want > 0 && rb_want <= rb_max ? rb_want : rb_max;
 #define ND_B(RBV)                                                                          \
-    if (f32) nd_bwd_t<float2, RBV>(d, items, nitems, smem_rows, y, x, R, done, st, pdl);   \
-    else nd_bwd_t<double2, RBV>(d, items, nitems, smem_rows, y, x, R, done, st, pdl);
+    if (f32) nd_bwd_t<float2, RBV>(d, items, nitems, smem_rows, root, t, u, y, x, R, done, st, pdl);   \
+    else nd_bwd_t<int4, RBV>(d, items, nitems, smem_rows, root, t, u, y, x, R, done, st, pdl);
     switch (rb) {
         case 8: ND_B(8) break;
         case 4: ND_B(4) break;
@@ -697,22 +1005,29 @@ void launch_nd_backward(const NDDev& d, bool f32, const int4* items, int nitems,
     }
 #undef ND_B
 }
-template <class MT, int RB>
-static void nd_sub_t(bool fwd, const NDDev& d, const int* sp, const int* sn, int nsub, int smem_rows,
-                     const double2* a, double2* b, double2* u, int R, const int* done, cudaStream_t st) {
-    const size_t sm = std::max<size_t>(16, (size_t)(smem_rows | 1) * RB * sizeof(MT));
-    const dim3 g(nsub, (R + RB - 1) / RB);
-    if (fwd) k_nd_forward_sub<MT, RB><<<g, 128, sm, st>>>(d, sp, sn, a, b, u, R, done);
-    else k_nd_backward_sub<MT, RB><<<g, 128, sm, st>>>(d, sp, sn, a, b, R, done);
+// right-hand sides per CTA of the bottom launches: all warps' staged vectors fit
+int nd_bottom_block(int rows, int R) {
+    int rb = 8;
+    while (rb > 1 && (rb >= 2 * R || (size_t)(rows | 1) * rb * kNDWarps * sizeof(int4) > (size_t)kNDSmemMax)) rb >>= 1;
+    return (size_t)(rows | 1) * rb * kNDWarps * sizeof(int4) > (size_t)kNDSmemMax ? 0 : rb;
 }
-void launch_nd_subtrees(bool forward, const NDDev& d, bool f32, const int* sub_ptr, const int* sub_nodes, int nsub,
-                        int smem_rows, const double2* in, double2* out, double2* u, int R, const int* done,
-                        cudaStream_t st) {
-    if (nsub <= 0) return;
-    const int rb = nd_rhs_block(smem_rows, R);
-#define ND_S(RBV)                                                                                                  \
-    if (f32) nd_sub_t<float2, RBV>(forward, d, sub_ptr, sub_nodes, nsub, smem_rows, in, out, u, R, done, st);      \
-    else nd_sub_t<double2, RBV>(forward, d, sub_ptr, sub_nodes, nsub, smem_rows, in, out, u, R, done, st);
+template <class MT, int RB>
+static void nd_bottom_t(bool fwd, const NDDev& d, const NDBottom& b, const double2* t, double2* y, double2* x, double2* u,
+                        int R, const int* done, cudaStream_t st) {
+    const int len = RB * ((fwd ? b.fwd_rows : b.bwd_rows) | 1);
+    const size_t sm = std::max<size_t>(16, (size_t)len * kNDWarps * sizeof(typename NDVec<MT>::V));
+    const dim3 g(b.nsub, (R + RB - 1) / RB);
+    if (fwd) k_nd_bottom<MT, RB, true><<<g, 32 * kNDWarps, sm, st>>>(d, b.fitems, b.fptr, b.nlev, len, t, y, x, u, R, done);
+    else k_nd_bottom<MT, RB, false><<<g, 32 * kNDWarps, sm, st>>>(d, b.bitems, b.bptr, b.nlev, len, t, y, x, u, R, done);
+}
+void launch_nd_bottom(bool forward, const NDDev& d, bool f32, const NDBottom& b, const double2* t, double2* y, double2* x,
+                      double2* u, int R, const int* done, cudaStream_t st, int rb_want) {
+    if (b.nsub <= 0) return;
+    const int rb_max = nd_bottom_block(forward ? b.fwd_rows : b.bwd_rows, R);
+    const int rb = rb_want > 0 && rb_want <= rb_max ? rb_want : rb_max;
+#define ND_S(RBV)                                                               \
+    if (f32) nd_bottom_t<float2, RBV>(forward, d, b, t, y, x, u, R, done, st);  \
+    else nd_bottom_t<int4, RBV>(forward, d, b, t, y, x, u, R, done, st);
     switch (rb) {
         case 8: ND_S(8) break;
         case 4: ND_S(4) break;
@@ -732,11 +1047,11 @@ static void nd_persist_t(const NDDev& d, const NDSched& s, const double2* t, dou
     int dev = 0, nsm = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_nd_persistent<MT, RB>, 128, sm);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_nd_persistent<MT, RB>, kNDThreads, sm);
     const int nrb = (R + RB - 1) / RB;
     const int grid = std::max(1, std::min(std::max(1, per) * std::max(1, nsm), s.nseq * nrb));
     cudaMemsetAsync(s.state, 0, sizeof(int) * nd_state_ints(s, R), st);
-    k_nd_persistent<MT, RB><<<grid, 128, sm, st>>>(d, s, t, y, x, u, R, done, err);
+    k_nd_persistent<MT, RB><<<grid, kNDThreads, sm, st>>>(d, s, t, y, x, u, R, done, err);
 }
 void launch_nd_persistent(const NDDev& d, const NDSched& s, bool f32, const double2* t, double2* y, double2* x,
                           double2* u, int R, const int* done, int* err, cudaStream_t st) {
@@ -744,7 +1059,7 @@ void launch_nd_persistent(const NDDev& d, const NDSched& s, bool f32, const doub
     const int rb = nd_rhs_block(s.smem_rows, R);
 #define ND_P(RBV)                                                                   \
     if (f32) nd_persist_t<float2, RBV>(d, s, t, y, x, u, R, done, err, st);         \
-    else nd_persist_t<double2, RBV>(d, s, t, y, x, u, R, done, err, st);
+    else nd_persist_t<int4, RBV>(d, s, t, y, x, u, R, done, err, st);
     switch (rb) {
         case 8: ND_P(8) break;
         case 4: ND_P(4) break;
@@ -764,33 +1079,49 @@ void launch_csr_residual(const int* ptr, const int* col, const void* val, const 
     else if (R == 2) k_csr_residual<2><<<dim3(g, 1), 128, 0, st>>>(ptr, col, v, vex, n, x, t, r, R, done);
     else k_csr_residual<1><<<dim3(g, 1), 128, 0, st>>>(ptr, col, v, vex, n, x, t, r, R, done);
 }
-void launch_gemv(const void* A, bool f32, int n_out, int n_in, const double2* x, double2* y, const double2* c, int mode,
-                 int64_t xs, int64_t ys, int R, const int* done, cudaStream_t st, int form) {
-    if (R == 1 && form == 1) {
-        const dim3 g1((n_out + 3) / 4);
-        if (f32) k_gemv1<float2><<<g1, 256, 0, st>>>((const float2*)A, n_out, n_in, x, y, c, mode, done);
-        else k_gemv1<double2><<<g1, 256, 0, st>>>((const double2*)A, n_out, n_in, x, y, c, mode, done);
-        return;
-    }
-    if (R == 1 && form == 2) {
-        const dim3 g2((n_out + 7) / 8);
-        if (f32) k_gemv2r<float2><<<g2, 128, 0, st>>>((const float2*)A, n_out, n_in, x, y, c, mode, done);
-        else k_gemv2r<double2><<<g2, 128, 0, st>>>((const double2*)A, n_out, n_in, x, y, c, mode, done);
-        return;
-    }
-    const int warps_per_block = 4;
-    const dim3 g((n_out + warps_per_block - 1) / warps_per_block);
-    const int tb = 32 * warps_per_block;
+void launch_fix_dense(void* A, int n, int* ex, int* col, cudaStream_t st) {
+    k_fix_dense_cols<<<(n + 3) / 4, 128, 0, st>>>((const double2*)A, n, col);
+    k_fix_dense<<<(n + 3) / 4, 128, 0, st>>>((double2*)A, n, col, ex);
+}
+void launch_fix_fronts(const NDDev& d, int nodes, cudaStream_t st) {
+    if (nodes > 0) k_fix_fronts<<<nodes, 256, 0, st>>>(d);
+}
+void launch_gemv32(const void* A, int n, const double2* x, double2* y, int R, const int* done, cudaStream_t st, int form) {
+    const float2* a = (const float2*)A;
+    if (R == 1 && form == 1) { k_gemv1<float2><<<(n + 3) / 4, 256, 0, st>>>(a, n, n, x, y, nullptr, 0, done); return; }
+    if (R == 1 && form == 2) { k_gemv2r<float2><<<(n + 7) / 8, 128, 0, st>>>(a, n, n, x, y, nullptr, 0, done); return; }
+    const dim3 g((n + 3) / 4);
     // right-hand sides in chunks of 8, 4, 2, 1: every FMA issued does useful work
     for (int r0 = 0; r0 < R;) {
         const int left = R - r0;
         const int rb = left >= 8 ? 8 : (left >= 4 ? 4 : (left >= 2 ? 2 : 1));
-#define DDH_GEMV(RBV)                                                                                         \
-        if (f32) k_gemv<float2, RBV><<<g, tb, 0, st>>>((const float2*)A, n_out, n_in, x, y, c, mode, xs, ys, r0, done); \
-        else k_gemv<double2, RBV><<<g, tb, 0, st>>>((const double2*)A, n_out, n_in, x, y, c, mode, xs, ys, r0, done);
+#define DDH_GEMV(RBV) k_gemv<float2, RBV><<<g, 128, 0, st>>>(a, n, n, x, y, nullptr, 0, n, n, r0, done);
         switch (rb) { case 8: DDH_GEMV(8) break; case 4: DDH_GEMV(4) break; case 2: DDH_GEMV(2) break; default: DDH_GEMV(1) }
 #undef DDH_GEMV
         r0 += rb;
+    }
+}
+// one CTA per SM, but at least four rows per CTA (each CTA stages all of x)
+static int gemv_rows(int n, int nsm) { return std::max(4, (n + nsm - 1) / nsm); }
+void gemv_set_smem_limits() {
+    constexpr int most = 160 * 1024;          // eight staged tiles and the sums of the rows of n = 16384
+    cudaFuncSetAttribute(k_gemv_fx<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(k_gemv_fx<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(k_gemv_fx<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(k_gemv_fx<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+void launch_gemv(const void* A, const int* ex, const int* col, int n, const double2* x, double2* y, int R, const int* done, int nsm,
+                 cudaStream_t st) {
+    const int rpc = gemv_rows(n, nsm);
+    const int g = (n + rpc - 1) / rpc;
+    for (int r0 = 0; r0 < R;) {
+        const int left = std::min(R - r0, 8);
+        const int rb = left >= 5 ? 8 : (left >= 3 ? 4 : left);
+        const size_t sm = (size_t)rb * ((8 / rb * kGemvTile + 1) * sizeof(int4) + (size_t)rpc * 2 * sizeof(double));
+#define DDH_GEMV(RBV) k_gemv_fx<RBV><<<g, kGemvThreads, sm, st>>>((const int4*)A, ex, col, n, x, y, r0, left, rpc, done);
+        switch (rb) { case 8: DDH_GEMV(8) break; case 4: DDH_GEMV(4) break; case 2: DDH_GEMV(2) break; default: DDH_GEMV(1) }
+#undef DDH_GEMV
+        r0 += left;
     }
 }
 

@@ -79,8 +79,9 @@ void launch_pre(const DevModel& dm, const double2* v, double2* vd, void* outE, d
 
 // Nested-dissection factor of the coarse matrix on the device (elimination order).  Per
 // node: fully summed positions [f0, f0+nF), boundary positions bidx[b_off .. b_off+nB),
-// G (nB x nF) at g_off and M = [W | -H] (nF x (nF+nB)) at m_off, of element type double2 or
-// float2, row-major (column-major for short rows, see kNDShortRow).  The forward pass leaves
+// G (nB x nF) at g_off and M = [W | -H] (nF x (nF+nB)) at m_off, in fixed point (int4 limbs with the
+// row exponents gexp[u_off + row], mexp[f0 + row]; launch_fix_fronts makes them from complex128 in
+// place) or float2, row-major (column-major for short rows, see kNDShortRow).  The forward pass leaves
 // at u[u_off[N] + k] ([R][u_len]) the total amount node N's subtree subtracts from boundary
 // entry k; it is passed up the tree: src[2 (s_off[N] + i) + {0,1}] are the offsets in u of
 // the (at most two) children's amounts for front entry i (F first, then B), or -1.
@@ -97,6 +98,11 @@ struct NDDev {
     const int64_t* src = nullptr;
     const void* G = nullptr;
     const void* M = nullptr;
+    int* gexp = nullptr;
+    int* mexp = nullptr;
+    int* gcol = nullptr;      // column scalings: of G and M by F position, of M by boundary entry (u_off + k)
+    int* mcol = nullptr;
+    int* mcolB = nullptr;
     int64_t u_len = 0;
     int nc = 0;
 };
@@ -112,16 +118,26 @@ constexpr int kNDShortRow = 128;
 void launch_nd_forward(const NDDev& d, bool f32, const int4* items, int nitems, int smem_rows, const double2* t,
                        double2* y, double2* u, int R, const int* done, cudaStream_t st, int rb_want = 0,
                        bool pdl = false);
-void launch_nd_backward(const NDDev& d, bool f32, const int4* items, int nitems, int smem_rows, const double2* y,
-                        double2* x, int R, const int* done, cudaStream_t st, int rb_want = 0, bool pdl = false);
+// root: the level's nodes have no boundary and no forward items; their forward amounts are formed from
+// t and u
+void launch_nd_backward(const NDDev& d, bool f32, const int4* items, int nitems, int smem_rows, int root,
+                        const double2* t, const double2* u, const double2* y, double2* x, int R, const int* done,
+                        cudaStream_t st, int rb_want = 0, bool pdl = false);
 // largest right-hand-side block whose staged vectors fit in shared memory (and below 2 R)
 int nd_rhs_block(int smem_rows, int R);
-// the levels below a cut in one launch: CTA b walks the subtree nodes
-// sub_nodes[sub_ptr[b] .. sub_ptr[b+1]) (postorder), forward (in = t, out = y, u) or backward
-// (in = y, out = x)
-void launch_nd_subtrees(bool forward, const NDDev& d, bool f32, const int* sub_ptr, const int* sub_nodes, int nsub,
-                        int smem_rows, const double2* in, double2* out, double2* u, int R, const int* done,
-                        cudaStream_t st);
+// the levels from `cut` down in one launch per direction: CTA b walks the subtree below the b-th node
+// of level cut, level by level; its items of level cut + k are items[ptr[b nlev + k] .. ptr[b nlev + k + 1])
+struct NDBottom {
+    int cut = 0, nsub = 0, nlev = 0, fwd_rows = 0, bwd_rows = 0;    // *_rows: largest staged vector
+    const int4* fitems = nullptr;
+    const int4* bitems = nullptr;
+    const int* fptr = nullptr;
+    const int* bptr = nullptr;
+};
+void launch_nd_bottom(bool forward, const NDDev& d, bool f32, const NDBottom& b, const double2* t, double2* y, double2* x,
+                      double2* u, int R, const int* done, cudaStream_t st, int rb_want = 0);
+// largest right-hand-side block of a bottom launch that stages vectors of `rows` entries (0: none fits)
+int nd_bottom_block(int rows, int R);
 // The whole nested-dissection solve in one launch, scheduled by dependencies instead of by
 // tree level.  seq lists every forward item (deepest level first) and then every backward item
 // (root level first); .w bit 0 = short-row form, bit 1 = backward.  CTAs take (item, RHS block)
@@ -148,6 +164,7 @@ void launch_nd_persistent(const NDDev& d, const NDSched& s, bool f32, const doub
                           double2* u, int R, const int* done, int* err, cudaStream_t st);
 // ints of NDSched::state needed for R right-hand sides
 size_t nd_state_ints(const NDSched& s, int R);
+void launch_fix_fronts(const NDDev& d, int nodes, cudaStream_t st);
 void nd_set_smem_limits();   // once per device before the first (captured) launch
 // r = t - K x, K in CSR with its values in fixed point (launch_fix_csr makes them from complex128 in
 // place; vex: row exponents), R right-hand sides ([R][n])
@@ -155,11 +172,17 @@ void launch_fix_csr(const int* ptr, double2* val, int* ex, int n, cudaStream_t s
 void launch_csr_residual(const int* ptr, const int* col, const void* val, const int* vex, int n, const double2* x,
                          const double2* t, double2* r, int R, const int* done, cudaStream_t st);
 void launch_dinv(const DevModel& dm, const double2* x, double2* y, int R, const int* done, cudaStream_t st);
-// y = A x (mode 0), y -= A x (1), y = c - A x (2).  For one right-hand side `form` picks the
-// kernel: 0 one warp per row, 1 two warps per row, 2 two rows per warp (chosen by timing at
-// factor time)
-void launch_gemv(const void* A, bool f32, int n_out, int n_in, const double2* x, double2* y, const double2* c, int mode,
-                 int64_t xs, int64_t ys, int R, const int* done, cudaStream_t st, int form = 1);
+// y = K^-1 x for the dense inverse in fixed point (ddh_fixed.cuh; ex = its row exponents, col = its column
+// scalings, nsm = SMs of the device), R right-hand sides; launch_fix_dense turns the complex128 matrix
+// into that form in place
+void launch_gemv(const void* A, const int* ex, const int* col, int n, const double2* x, double2* y, int R, const int* done, int nsm,
+                 cudaStream_t st);
+void launch_fix_dense(void* A, int n, int* ex, int* col, cudaStream_t st);
+void gemv_set_smem_limits();
+// the same for the complex64 copy.  For one right-hand side `form` picks the kernel: 0 one warp per
+// row, 1 two warps per row, 2 two rows per warp (chosen by timing at factor time)
+void launch_gemv32(const void* A, int n, const double2* x, double2* y, int R, const int* done, cudaStream_t st,
+                   int form = 1);
 // Lifting of point-source Dirichlet data (tilde basis, boundary slots only; `out` zeroed by the
 // caller): per degree table t, tr_nq[t] Gauss-Legendre nodes tr_x[tr_xoff[t] ..] and the weights
 // tr_Q[tr_off[t] ..] ((p - 1) x nq, bubble m = 2..p by node); src [2R] source centres
