@@ -112,7 +112,7 @@ typedef struct {
                               1e-5; 0 = always inner_iters iterations).  The complex64 inner
                               solves cannot gain much more than 5-6 digits per application */
     int32_t coarse_form;   /* coarse solve K x2 = t (ddh_coarse_form): DDH_COARSE_AUTO (default) applies
-                              a dense K^-1 built from the factor when n_coarse <= 6144 and the
+                              a dense K^-1 built from the factor when n_coarse <= 2048 and the
                               per-level nested-dissection solve otherwise; DDH_COARSE_DENSE forces
                               the dense K^-1 (n_coarse <= 16384, else DDH_ERR_INVALID_ARG);
                               DDH_COARSE_ND and DDH_COARSE_ND_LEVELS force the nested-dissection

@@ -268,7 +268,11 @@ bool coarse_factor(Model& m, const std::vector<int32_t>& kn_ptr, const std::vect
     }
     m.coarse_refine = m.coarse_check > 1e-12;
     // ---- dense inverse for small coarse problems (elimination order), refined like the solves
-    m.dense_coarse = m.coarse_form == 1 || (m.coarse_form == 0 && nc <= 6144);   // 2, 3: nested dissection
+    // automatic form: K^-1 up to 2048 unknowns.  One application, one / eight right-hand sides: n_c = 1921
+    // dense 22 / 113 us, nested dissection 74 / 84 us; n_c = 2961 55 / 244 against 88 / 95 us, n_c = 5313
+    // 140 / 697 against 100 / 111 us; and the columns of K^-1 take
+    // n_c solves on the host (n_c = 5425: 0.70 of 0.75 s of a factorisation)
+    m.dense_coarse = m.coarse_form == 1 || (m.coarse_form == 0 && nc <= 2048);   // 2, 3: nested dissection
     m.Kinv.clear();
     if (m.dense_coarse) {
         m.Kinv.assign((size_t)nc * nc, cd(0));
