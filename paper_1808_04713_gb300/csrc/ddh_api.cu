@@ -71,6 +71,8 @@ struct ddh_ctx {
     void* sinv32 = nullptr;
     void* pq64 = nullptr;                          // Y = [A11^-1 A_1T]_E per element
     void* pq32 = nullptr;
+    void* sfx = nullptr;                           // S_E^-1 and Y in fixed point (FP64 edge passes)
+    void* yfx = nullptr;
     bool edge_form = false;                        // Krylov-loop passes with Y (no FDM)
     const int* edge_items = nullptr;               // elements by degree, descending (persistent edge pass)
     std::vector<int> deg_begin, deg_count, deg_p;  // contiguous runs of equal degree in edge_items
@@ -165,6 +167,12 @@ static ddh_status fail(ddh_ctx* ctx, ddh_status s, const std::string& msg) {
     return s;
 }
 
+static ddh_status model_alloc(ddh_ctx* ctx, size_t bytes, void** out) {
+    if (cudaMalloc(out, std::max<size_t>(16, bytes)) != cudaSuccess) { ctx->err = "cudaMalloc failed (model)"; return DDH_ERR_OOM; }
+    ctx->model_allocs.push_back(*out);
+    return DDH_OK;
+}
+
 template <class V>
 static ddh_status upload(ddh_ctx* ctx, const std::vector<V>& v, const V** out) {
     void* p = nullptr;
@@ -186,6 +194,7 @@ static void free_model(ddh_ctx* ctx) {
     ctx->work.clear();
     ctx->sinv64 = ctx->sinv32 = nullptr;
     ctx->pq64 = ctx->pq32 = nullptr;
+    ctx->sfx = ctx->yfx = nullptr;
     ctx->edge_form = false;
     ctx->edge_items = nullptr;
     ctx->deg_begin.clear(); ctx->deg_count.clear(); ctx->deg_p.clear();
@@ -344,24 +353,41 @@ static ddh_status upload_model(ddh_ctx* ctx) {
     // S^Lap restricted to each element's type-1 edge slots (symmetric n_E x n_E), one copy per
     // distinct (degree, slot pattern): on conforming meshes one per degree
     {
-        std::map<std::pair<int, std::vector<int32_t>>, int64_t> seen;
+        std::map<std::pair<int, std::vector<int32_t>>, int64_t> seen;      // pattern number
         std::vector<double> pre;
-        std::vector<int64_t> poff(E);
+        std::vector<int64_t> poff(E), peoff(E), koff, keoff;
+        std::vector<int> klen;
+        int64_t rows = 0;
         for (int e = 0; e < E; ++e) {
             const Elem& El = m.el[e];
             std::vector<int32_t> pat(m.e1_eall.begin() + El.e1_off, m.e1_eall.begin() + El.e1_off + El.nE1);
             auto key = std::make_pair(El.ptab, pat);
             auto it = seen.find(key);
-            if (it != seen.end()) { poff[e] = it->second; continue; }
+            if (it != seen.end()) { poff[e] = koff[it->second]; peoff[e] = keoff[it->second]; continue; }
             const PTable& T = m.tabs[El.ptab];
             const int ne = 4 * (El.p - 1), nE = El.nE1;
             poff[e] = (int64_t)pre.size();
+            peoff[e] = rows;
             for (int i = 0; i < nE; ++i)
                 for (int j = 0; j < nE; ++j) pre.push_back(T.Slap[(size_t)pat[i] * ne + pat[j]]);
-            seen.emplace(std::move(key), poff[e]);
+            seen.emplace(std::move(key), (int64_t)koff.size());
+            koff.push_back(poff[e]);
+            keoff.push_back(rows);
+            klen.push_back(nE);
+            rows += nE;
         }
         if ((st = upload(ctx, pre, &d.pre_all))) return st;
         if ((st = upload(ctx, poff, &d.pre_off))) return st;
+        if ((st = upload(ctx, peoff, &d.pre_ex_off))) return st;
+        // the same in fixed point for the FP64 preconditioner
+        const int64_t *ko, *ke;
+        const int* kl;
+        void *fx, *ex;
+        if ((st = upload(ctx, koff, &ko)) || (st = upload(ctx, keoff, &ke)) || (st = upload(ctx, klen, &kl))) return st;
+        if ((st = model_alloc(ctx, sizeof(int2) * pre.size(), &fx)) || (st = model_alloc(ctx, sizeof(int) * rows, &ex))) return st;
+        launch_fix_pre(d.pre_all, (int)klen.size(), ko, kl, ke, (int2*)fx, (int*)ex, ctx->stream);
+        d.pre_fx = (const int2*)fx;
+        d.pre_ex = (const int*)ex;
     }
     // slots
     if ((st = upload(ctx, m.e1_slot, &d.e1_slot))) return st;
@@ -1116,8 +1142,8 @@ static ddh_status edge_tune(ddh_ctx* ctx, const Work& w, int R, bool fp64) {
     const DevModel& d = ctx->dm;
     cudaStream_t s = ctx->stream;
     CK(cudaMemsetAsync(w.vd, 0, sizeof(double2) * (size_t)R * std::max(1, d.n_dual), s));
-    const void* sinv = fp64 ? ctx->sinv64 : ctx->sinv32;
-    const void* Y = fp64 ? ctx->pq64 : ctx->pq32;
+    const void* sinv = fp64 ? ctx->sfx : ctx->sinv32;
+    const void* Y = fp64 ? ctx->yfx : ctx->pq32;
     EdgeSched es;
     es.items = ctx->edge_items;
     std::vector<signed char> tbl(33, 0);
@@ -1290,6 +1316,26 @@ static EdgeSched edge_sched(const ddh_ctx* ctx, bool fp64, int R) {
     return es;
 }
 
+// fixed-point copies of S_E^-1 and Y for the FP64 edge passes (made on first use: a mixed context
+// only needs them for ddh_apply_dual_operator in FP64)
+static ddh_status fix_edge(ddh_ctx* ctx) {
+    if (!ctx->edge_form || ctx->sfx) return DDH_OK;
+    DevModel& d = ctx->dm;
+    void *s, *y, *se, *ye;
+    ddh_status st;
+    if ((st = model_alloc(ctx, sizeof(double2) * ctx->m.sinv.size(), &s))) return st;
+    if ((st = model_alloc(ctx, sizeof(double2) * ctx->m.pq.size(), &y))) return st;
+    if ((st = model_alloc(ctx, sizeof(int) * (size_t)d.nE1_tot, &se))) return st;
+    if ((st = model_alloc(ctx, sizeof(int) * (size_t)d.nT_tot, &ye))) return st;
+    launch_fix_edge(d, ctx->sinv64, ctx->pq64, s, (int*)se, y, (int*)ye, ctx->stream);
+    CK(cudaGetLastError());
+    d.sinv_ex = (const int*)se;
+    d.y_ex = (const int*)ye;
+    ctx->sfx = s;
+    ctx->yfx = y;
+    return DDH_OK;
+}
+
 static ddh_status get_op_work(ddh_ctx* ctx, int R, bool fp64, Work& w) {
     const DevModel& d = ctx->dm;
     const size_t es = fp64 ? sizeof(double2) : sizeof(float2);
@@ -1316,6 +1362,7 @@ static ddh_status get_op_work(ddh_ctx* ctx, int R, bool fp64, Work& w) {
     w.vd = (double2*)p;
     if ((st = get_work(ctx, "mvec", sizeof(double2) * (size_t)R * std::max(1, d.n_dual), &p))) return st;
     w.mvec = (double2*)p;
+    if (fp64 && (st = fix_edge(ctx))) return st;
     if ((st = edge_tune(ctx, w, R, fp64))) return st;
     if ((st = fdm_tune(ctx, w, R, fp64))) return st;
     return nd_tune(ctx, w, R);
@@ -1435,6 +1482,8 @@ static void apply_op(ddh_ctx* ctx, const Work& w, const double2* z, double zsign
     cudaStream_t s = ctx->stream;
     const void* sinv = std::is_same<T, double>::value ? ctx->sinv64 : ctx->sinv32;
     const void* Y = std::is_same<T, double>::value ? ctx->pq64 : ctx->pq32;
+    const void* eS = std::is_same<T, double>::value ? ctx->sfx : ctx->sinv32;     // of the edge passes
+    const void* eY = std::is_same<T, double>::value ? ctx->yfx : ctx->pq32;
     // With split_pass1, inside the Krylov loop (one-CTA edge form) pass 1 is split: the t_T rows,
     // which the coarse assembly needs, on the context stream; the x_E rows, needed only by pass 2,
     // on a forked stream beside the coarse solve.  Each output row is computed the same way
@@ -1448,12 +1497,12 @@ static void apply_op(ddh_ctx* ctx, const Work& w, const double2* z, double zsign
         if (split) {
             cudaEventRecord(ctx->ev_p1_fork, s);
             cudaStreamWaitEvent(ctx->side_p1, ctx->ev_p1_fork, 0);
-            launch_pass1_edge<T>(d, sinv, Y, z, zsign, bt, w.xE, w.tT, R, done, ctx->side_p1, &es, 0, -1, 0, 1);
+            launch_pass1_edge<T>(d, eS, eY, z, zsign, bt, w.xE, w.tT, R, done, ctx->side_p1, &es, 0, -1, 0, 1);
             cudaEventRecord(ctx->ev_p1_join, ctx->side_p1);
-            launch_pass1_edge<T>(d, sinv, Y, z, zsign, bt, w.xE, w.tT, R, done, s, &es, 0, -1, 0, 2);
+            launch_pass1_edge<T>(d, eS, eY, z, zsign, bt, w.xE, w.tT, R, done, s, &es, 0, -1, 0, 2);
             ctx->launches++;
         } else {
-            launch_pass1_edge<T>(d, sinv, Y, z, zsign, bt, w.xE, w.tT, R, done, s, &es);
+            launch_pass1_edge<T>(d, eS, eY, z, zsign, bt, w.xE, w.tT, R, done, s, &es);
         }
     }
     else launch_pass1<T>(d, sinv, ctx->edge_form ? Y : nullptr, z, zsign, bt, has_bI, w.xE, w.tT, R, done, s,
@@ -1462,7 +1511,7 @@ static void apply_op(ddh_ctx* ctx, const Work& w, const double2* z, double zsign
     ctx->launches += 2;
     coarse_solve(ctx, w.t, w.x2, w.ctmp, R, done);
     if (split) cudaStreamWaitEvent(s, ctx->ev_p1_join, 0);
-    if (ctx->edge_form && !phi_out) launch_pass2_edge<T>(d, Y, w.x2, w.xE, w.xE2, R, done, s);
+    if (ctx->edge_form && !phi_out) launch_pass2_edge<T>(d, eY, w.x2, w.xE, w.xE2, R, done, s);
     else launch_pass2<T>(d, sinv, ctx->edge_form ? Y : nullptr, w.x2, w.xE, w.xE2, phi_out ? 1 : 0, bt, has_bI, phi_out, R, done, s,
                          fdm_cfg(ctx, std::is_same<T, double>::value, R, 2));
     ctx->launches++;
@@ -2690,12 +2739,12 @@ ddh_status ddh_profile_op(ddh_ctx* ctx, int32_t R, int32_t precision, int32_t re
     if (fp64) {
         ms_out[0] = timeit([&] {
             const EdgeSched es = edge_sched(ctx, true, R);
-            if (ef) launch_pass1_edge<double>(d, sinv, Y, z, 1.0, nullptr, w.xE, w.tT, R, nullptr, s, &es);
+            if (ef) launch_pass1_edge<double>(d, ctx->sfx, ctx->yfx, z, 1.0, nullptr, w.xE, w.tT, R, nullptr, s, &es);
             else launch_pass1<double>(d, sinv, nullptr, z, 1.0, nullptr, 0, w.xE, w.tT, R, nullptr, s);
         });
         ms_out[1] = timeit([&] { launch_coarse_assemble<double>(d, w.tT, nullptr, z, 1.0, w.t, R, nullptr, s); });
         ms_out[3] = timeit([&] {
-            if (ef) launch_pass2_edge<double>(d, Y, w.x2, w.xE, w.xE2, R, nullptr, s);
+            if (ef) launch_pass2_edge<double>(d, ctx->yfx, w.x2, w.xE, w.xE2, R, nullptr, s);
             else launch_pass2<double>(d, sinv, nullptr, w.x2, w.xE, w.xE2, 0, nullptr, 0, nullptr, R, nullptr, s);
         });
         ms_out[4] = timeit([&] { launch_jump_gather<double>(d, w.xE2, w.x2, K.w, R, nullptr, s); });

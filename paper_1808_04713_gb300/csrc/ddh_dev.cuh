@@ -68,6 +68,14 @@ struct DevModel {
     const double* slap_all = nullptr;
     const double* pre_all = nullptr;    // restricted S^Lap per (degree, slot pattern), n_E^2
     const int64_t* pre_off = nullptr;   // per element: offset into pre_all
+    // fixed-point forms for the FP64 passes (ddh_fixed.cuh): pre_all's entries and row exponents (per
+    // element: offset into pre_ex), the row exponents of S_E^-1 (by type-1 slot) and the column
+    // exponents of Y (by type-2 slot)
+    const int2* pre_fx = nullptr;
+    const int* pre_ex = nullptr;
+    const int64_t* pre_ex_off = nullptr;
+    const int* sinv_ex = nullptr;
+    const int* y_ex = nullptr;
     // E1 slots
     const int* e1_slot = nullptr;
     const int* e1_row = nullptr;

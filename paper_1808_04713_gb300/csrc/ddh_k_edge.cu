@@ -1,7 +1,9 @@
 // Krylov-loop element passes with the explicit edge operators, the coarse assembly, the
 // jump gather C^ x and the Dirichlet preconditioner (Sec. 2.3.3, eqs. complicated_schur_system,
 // general_preconditioner, weight_matrix).
+#include "ddh_fixed.cuh"
 #include "ddh_kcommon.cuh"
+#include <type_traits>
 
 namespace ddh {
 
@@ -14,6 +16,64 @@ namespace ddh {
 // -- two small dense products per element and right-hand side block instead of the FDM
 // chain.  Y is formed at factor time.  The interior never enters the iteration; it is
 // rebuilt by the FDM kernels in the recovery.
+//
+// The FP64 passes hold S_E^-1 and Y in fixed point (ddh_fixed.cuh): EdgeOp<double> is four limbs per
+// entry.  S_E^-1 has an exponent per row (DevModel::sinv_ex, by type-1 slot), Y one per column (y_ex, by
+// type-2 slot), i.e. per output row of pass 1; pass 2, which sums over the columns, puts them on u_T
+// before it is staged.
+template <class T> struct EdgeOpT { using type = cpx<float>; };
+template <> struct EdgeOpT<double> { using type = int4; };
+template <class T> using EdgeOp = typename EdgeOpT<T>::type;
+
+// Fixed-point copies of S_E^-1 and Y: one CTA per element, one warp per row of S_E^-1 / column of Y
+__global__ void __launch_bounds__(256) k_fix_edge(DevModel dm, const double2* __restrict__ sinv,
+                                                  const double2* __restrict__ Y, int4* __restrict__ sfx,
+                                                  int* __restrict__ sex, int4* __restrict__ yfx, int* __restrict__ yex) {
+    const int e = blockIdx.x, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+    const int nE = dm.nE1[e], nT = dm.nT[e];
+    for (int o = warp; o < nE + nT; o += nw) {
+        const bool isS = o < nE;
+        const int ld = isS ? nE : nT;
+        const int64_t at = isS ? dm.sinv_off[e] + o : dm.pq_off[e] + (o - nE);
+        const double2* a = isS ? sinv : Y;
+        int4* f = isS ? sfx : yfx;
+        unsigned m = 0;
+        for (int j = lane; j < nE; j += 32) m = max(m, fx_mag(a[at + (int64_t)j * ld]));
+        const int ef = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
+        for (int j = lane; j < nE; j += 32) {
+            const double2 v = a[at + (int64_t)j * ld];
+            f[at + (int64_t)j * ld] = fx_cpx(v.x, v.y, ef);
+        }
+        if (lane == 0) *(isS ? sex + dm.e1_off[e] + o : yex + dm.t_off[e] + o - nE) = ef;
+    }
+}
+
+// Stages cnt vectors of length n (stride vs): load(q, i) gives entry i of vector q.  In fixed point one
+// warp per vector (n <= 128: four entries per lane), whose exponent goes to ex[q].
+template <class T, class F>
+__device__ __forceinline__ void edge_stage(const F& load, int n, int vs, int cnt, EdgeOp<T>* sm, int* ex) {
+    if constexpr (std::is_same<T, double>::value) {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        for (int q = warp; q < cnt; q += nw) {
+            cpx<double> v[4];
+            unsigned m = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = lane + 32 * k;
+                v[k] = i < n ? load(q, i) : mk<double>(0, 0);
+                m = max(m, fx_mag(make_double2(v[k].x, v[k].y)));
+            }
+            const int ef = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (lane + 32 * k < n) sm[q * vs + lane + 32 * k] = fx_cpx(v[k].x, v[k].y, ef);
+            if (lane == 0) ex[q] = ef;
+        }
+    } else {
+        for (int idx = threadIdx.x; idx < cnt * n; idx += blockDim.x) sm[idx / n * vs + idx % n] = load(idx / n, idx % n);
+    }
+}
+
 // [x_E; t_T] = [S_E^-1; Y^T] r_E for one element and RB right-hand sides: output row o < nE reads
 // S_E^-1 (column-major), o >= nE reads Y (row-major nE x nT, i.e. Y^T column-major); tpr (2 or 4)
 // threads per output row.  Every output is the same fixed tree (p0 + p2) + (p1 + p3) of the four
@@ -22,7 +82,7 @@ namespace ddh {
 // the autotuner picks do not change the result.
 // Output rows [o_lo, o_hi) only (x_E rows are o < nE, t_T rows o >= nE).
 template <class T, int RB>
-__device__ __forceinline__ void edge_rows(const DevModel& dm, const cpx<T>* S, const cpx<T>* Ye, int nE, int nT,
+__device__ __forceinline__ void edge_rows_f(const DevModel& dm, const cpx<T>* S, const cpx<T>* Ye, int nE, int nT,
                                           const cpx<T>* rE, int vs, int cnt, int tpr, int r0, int e1o, int to,
                                           cpx<T>* __restrict__ xE_out, cpx<T>* __restrict__ tT_out, int o_lo,
                                           int o_hi) {
@@ -75,9 +135,67 @@ __device__ __forceinline__ void edge_rows(const DevModel& dm, const cpx<T>* S, c
     }
 }
 
+// The same in fixed point.  Sums are exact, so the order of the columns and tpr do not matter.  Per term
+// twelve IMAD.WIDE (64 per SM and clock) stand for four FP64 FMA (two): 64 x 64 elements, p = 20, 8
+// right-hand sides went from 1.09 ms (92 % of the FP64 rate) to 0.42 ms.
+template <int RB>
+__device__ __forceinline__ void edge_rows_fx(const DevModel& dm, const int4* S, const int4* Ye, int nE, int nT,
+                                             const int4* rE, const int* ex, int vs, int cnt, int tpr, int r0, int e1o,
+                                             int to, cpx<double>* __restrict__ xE_out, cpx<double>* __restrict__ tT_out,
+                                             int o_lo, int o_hi) {
+    for (int base = 0; base < (o_hi - o_lo) * tpr; base += blockDim.x) {
+        const int slot = base + threadIdx.x;
+        const int o = o_lo + slot / tpr, part = slot % tpr;
+        FxAcc s[2 * RB];
+#pragma unroll
+        for (int i = 0; i < 2 * RB; ++i) s[i].h = s[i].l = 0;
+        if (o < o_hi) {
+            const int4* col0 = o < nE ? S + o : Ye + (o - nE);
+            const int ld = o < nE ? nE : nT;
+            // nE <= 124 and tpr >= 2: at most 62 terms, one chain
+#pragma unroll(RB <= 2 ? 8 : 2)
+            for (int j = part; j < nE; j += tpr) {
+                const int4 a = col0[(int64_t)j * ld];
+#pragma unroll
+                for (int q = 0; q < RB; ++q)
+                    if (q < cnt) fx_cmac(s[2 * q], s[2 * q + 1], a, -a.z, -a.w, rE[q * vs + j]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2 * RB; ++i) {
+            long long h = 0;
+            unsigned l = 0;
+            fx_flush(s[i], h, l);
+            if (tpr == 4) {
+                h += __shfl_xor_sync(0xffffffffu, h, 2);
+                l += __shfl_xor_sync(0xffffffffu, l, 2);
+            }
+            h += __shfl_xor_sync(0xffffffffu, h, 1);
+            l += __shfl_xor_sync(0xffffffffu, l, 1);
+            // the lanes of a row share the conversions: component i goes to lane part = i (mod tpr)
+            const int q = i >> 1;
+            if (part == i % tpr && o < o_hi && q < cnt) {
+                const int ea = o < nE ? dm.sinv_ex[e1o + o] : dm.y_ex[to + o - nE];
+                cpx<double>* d = o < nE ? xE_out + (int64_t)(r0 + q) * dm.nE1_tot + e1o + o
+                                        : tT_out + (int64_t)(r0 + q) * dm.nT_tot + to + (o - nE);
+                reinterpret_cast<double*>(d)[i & 1] = fx_value(h, l, ea, ex[q]);
+            }
+        }
+    }
+}
 template <class T, int RB>
-__global__ void __launch_bounds__(256) k_pass1_edge(DevModel dm, const cpx<T>* __restrict__ sinv,
-                                                    const cpx<T>* __restrict__ Y, const double2* __restrict__ z,
+__device__ __forceinline__ void edge_rows(const DevModel& dm, const EdgeOp<T>* S, const EdgeOp<T>* Ye, int nE, int nT,
+                                          const EdgeOp<T>* rE, const int* ex, int vs, int cnt, int tpr, int r0, int e1o,
+                                          int to, cpx<T>* __restrict__ xE_out, cpx<T>* __restrict__ tT_out, int o_lo,
+                                          int o_hi) {
+    if constexpr (std::is_same<T, double>::value)
+        edge_rows_fx<RB>(dm, S, Ye, nE, nT, rE, ex, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
+    else edge_rows_f<T, RB>(dm, S, Ye, nE, nT, rE, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
+}
+
+template <class T, int RB>
+__global__ void __launch_bounds__(256) k_pass1_edge(DevModel dm, const EdgeOp<T>* __restrict__ sinv,
+                                                    const EdgeOp<T>* __restrict__ Y, const double2* __restrict__ z,
                                                     double zsign, const double2* __restrict__ bt, int R,
                                                     cpx<T>* __restrict__ xE_out, cpx<T>* __restrict__ tT_out,
                                                     const int* __restrict__ done, int ntask, int stage_off, int vs,
@@ -90,21 +208,22 @@ __global__ void __launch_bounds__(256) k_pass1_edge(DevModel dm, const cpx<T>* _
     const int e = task % dm.E, r0 = (task / dm.E) * RB;
     const int cnt = min(RB, R - r0);
     const int nE = dm.nE1[e], e1o = dm.e1_off[e], nT = dm.nT[e], to = dm.t_off[e];
-    const cpx<T>* S = sinv + dm.sinv_off[e];
+    const EdgeOp<T>* S = sinv + dm.sinv_off[e];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + stage_off);
-    cpx<T>* S_s = reinterpret_cast<cpx<T>*>(smem + stage_off + 128);
+    EdgeOp<T>* S_s = reinterpret_cast<EdgeOp<T>*>(smem + stage_off + 128);
     if (stage_off > 0 && nE > 0 && threadIdx.x == 0)
-        bulk_load_start(bar, S_s, S, (uint32_t)(((size_t)nE * nE * sizeof(cpx<T>) + 15) & ~(size_t)15));
-    cpx<T>* rE = reinterpret_cast<cpx<T>*>(smem);     // [RB][vs]
+        bulk_load_start(bar, S_s, S, (uint32_t)(((size_t)nE * nE * sizeof(EdgeOp<T>) + 15) & ~(size_t)15));
+    EdgeOp<T>* rE = reinterpret_cast<EdgeOp<T>*>(smem);     // [RB][vs]
+    __shared__ int ex[RB];
     const int64_t off = dm.off[e];
-    for (int idx = g.t(); idx < cnt * nE; idx += g.n()) {
-        const int q = idx / nE, i = idx % nE, r = r0 + q;
+    edge_stage<T>([&](int q, int i) {
+        const int r = r0 + q;
         cpx<T> v = mk<T>(0, 0);
         const int row = dm.e1_row[e1o + i];
         if (z && row >= 0) v = (T)(zsign * dm.e1_sign[e1o + i]) * ld<T>(z, (int64_t)r * dm.n_dual + row);
         if (bt) v += ld<T>(bt, (int64_t)r * dm.n_local + off + dm.e1_slot[e1o + i]);
-        rE[q * vs + i] = v;
-    }
+        return v;
+    }, nE, vs, cnt, rE, ex);
     g.sync();
     if (stage_off > 0 && nE > 0) {
         if (!bulk_wait_all(bar, dm.err)) return;
@@ -115,7 +234,7 @@ __global__ void __launch_bounds__(256) k_pass1_edge(DevModel dm, const cpx<T>* _
     const int tpr = (nE + nT) * 4 <= (int)blockDim.x ? 4 : 2;
     // rows: 0 all output rows, 1 the x_E rows only, 2 the t_T rows only (no S_E^-1 read)
     const int o_lo = rows == 2 ? nE : 0, o_hi = rows == 1 ? nE : nE + nT;
-    edge_rows<T, RB>(dm, S, Y + dm.pq_off[e], nE, nT, rE, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
+    edge_rows<T, RB>(dm, S, Y + dm.pq_off[e], nE, nT, rE, ex, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
 }
 
 // The same pass as one persistent launch over a degree-sorted work list.  Task t is (element
@@ -126,8 +245,8 @@ __global__ void __launch_bounds__(256) k_pass1_edge(DevModel dm, const cpx<T>* _
 // mbarrier per buffer).  tpr_p[p] (2 or 4 threads per output row) is chosen per degree by the
 // autotuner; 0 = the default (4 up to 64 output rows, else 2); tpr_force (2 or 4) overrides it.
 template <class T, int RB>
-__global__ void __launch_bounds__(256) k_pass1_edge_p(DevModel dm, const cpx<T>* __restrict__ sinv,
-                                                      const cpx<T>* __restrict__ Y, const double2* __restrict__ z,
+__global__ void __launch_bounds__(256) k_pass1_edge_p(DevModel dm, const EdgeOp<T>* __restrict__ sinv,
+                                                      const EdgeOp<T>* __restrict__ Y, const double2* __restrict__ z,
                                                       double zsign, const double2* __restrict__ bt, int R,
                                                       cpx<T>* __restrict__ xE_out, cpx<T>* __restrict__ tT_out,
                                                       const int* __restrict__ done, const int* __restrict__ items,
@@ -136,17 +255,18 @@ __global__ void __launch_bounds__(256) k_pass1_edge_p(DevModel dm, const cpx<T>*
     if (done && *done) return;
     extern __shared__ __align__(128) char smem[];
     const int nrb = (R + RB - 1) / RB, ntask = nitems * nrb;
-    cpx<T>* rE = reinterpret_cast<cpx<T>*>(smem);     // [RB][vs]
+    EdgeOp<T>* rE = reinterpret_cast<EdgeOp<T>*>(smem);     // [RB][vs]
+    __shared__ int ex[RB];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + stage_off);        // 2 barriers
     __shared__ int s_fail;
     const bool staged = stage_off > 0;
-    auto buf = [&](int b) { return reinterpret_cast<cpx<T>*>(smem + stage_off + 128 + (size_t)b * buf_bytes); };
+    auto buf = [&](int b) { return reinterpret_cast<EdgeOp<T>*>(smem + stage_off + 128 + (size_t)b * buf_bytes); };
     auto task_elem = [&](int t) { return items[item0 + t / nrb]; };
     // copy of task t's S_E^-1 into buffer b (thread 0); false when there is nothing to copy
     auto issue = [&](int t, int b) {
         const int e = task_elem(t), nE = dm.nE1[e];
         if (nE == 0) return false;
-        const uint32_t bytes = (uint32_t)(((size_t)nE * nE * sizeof(cpx<T>) + 15) & ~(size_t)15);
+        const uint32_t bytes = (uint32_t)(((size_t)nE * nE * sizeof(EdgeOp<T>) + 15) & ~(size_t)15);
         const uint32_t bb = smem_u32(bar + b);
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bb), "r"(bytes) : "memory");
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -174,15 +294,15 @@ __global__ void __launch_bounds__(256) k_pass1_edge_p(DevModel dm, const cpx<T>*
         const int nE = dm.nE1[e], e1o = dm.e1_off[e], nT = dm.nT[e], to = dm.t_off[e];
         if (staged && threadIdx.x == 0 && t + (int)gridDim.x < ntask) pend[b ^ 1] = issue(t + gridDim.x, b ^ 1);
         const int64_t off = dm.off[e];
-        for (int idx = threadIdx.x; idx < cnt * nE; idx += blockDim.x) {
-            const int q = idx / nE, i = idx % nE, r = r0 + q;
+        edge_stage<T>([&](int q, int i) {
+            const int r = r0 + q;
             cpx<T> v = mk<T>(0, 0);
             const int row = dm.e1_row[e1o + i];
             if (z && row >= 0) v = (T)(zsign * dm.e1_sign[e1o + i]) * ld<T>(z, (int64_t)r * dm.n_dual + row);
             if (bt) v += ld<T>(bt, (int64_t)r * dm.n_local + off + dm.e1_slot[e1o + i]);
-            rE[q * vs + i] = v;
-        }
-        const cpx<T>* S = sinv + dm.sinv_off[e];
+            return v;
+        }, nE, vs, cnt, rE, ex);
+        const EdgeOp<T>* S = sinv + dm.sinv_off[e];
         if (staged && nE > 0) {
             if (threadIdx.x == 0) {
                 bool ok = !pend[b];
@@ -196,7 +316,7 @@ __global__ void __launch_bounds__(256) k_pass1_edge_p(DevModel dm, const cpx<T>*
         if (s_fail) break;
         int tpr = tpr_force > 0 ? tpr_force : (tpr_p ? (int)tpr_p[dm.p[e]] : 0);
         if (tpr != 2 && tpr != 4) tpr = nE + nT <= 64 ? 4 : 2;
-        edge_rows<T, RB>(dm, S, Y + dm.pq_off[e], nE, nT, rE, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, 0,
+        edge_rows<T, RB>(dm, S, Y + dm.pq_off[e], nE, nT, rE, ex, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, 0,
                          nE + nT);
         __syncthreads();
     }
@@ -210,20 +330,21 @@ __global__ void __launch_bounds__(256) k_pass1_edge_p(DevModel dm, const cpx<T>*
 }
 
 template <class T, int RB>
-__global__ void __launch_bounds__(128) k_pass2_edge(DevModel dm, const cpx<T>* __restrict__ Y,
+__global__ void __launch_bounds__(128) k_pass2_edge(DevModel dm, const EdgeOp<T>* __restrict__ Y,
                                                     const double2* __restrict__ x2, const cpx<T>* __restrict__ xE_in,
                                                     cpx<T>* __restrict__ xE_out, int R, const int* __restrict__ done,
                                                     int ntask) {
     if (done && *done) return;
-    __shared__ cpx<T> uT[RB][128];
+    __shared__ EdgeOp<T> uT[RB * 128];
+    __shared__ int ex[RB];
     const CtaGroup g;
     const int task = blockIdx.x;
     if (task >= ntask) return;
     const int e = task % dm.E, r0 = (task / dm.E) * RB;
     const int cnt = min(RB, R - r0);
     const int nE = dm.nE1[e], e1o = dm.e1_off[e], nT = dm.nT[e], to = dm.t_off[e];
-    for (int idx = g.t(); idx < cnt * nT; idx += g.n()) {
-        const int q = idx / nT, i = idx % nT, r = r0 + q;
+    edge_stage<T>([&](int q, int i) {
+        const int r = r0 + q;
         cpx<T> u = mk<T>(0, 0);
         for (int a = dm.t_ptr[to + i]; a < dm.t_ptr[to + i + 1]; ++a) {
             const double2 xv = x2[(int64_t)r * dm.n_coarse + dm.t_col[a]];
@@ -231,21 +352,50 @@ __global__ void __launch_bounds__(128) k_pass2_edge(DevModel dm, const cpx<T>* _
             u.x += w * (T)xv.x;
             u.y += w * (T)xv.y;
         }
-        uT[q][i] = u;
-    }
+        if constexpr (std::is_same<T, double>::value) {
+            // the column's exponent: Y_t u_t = (Y_t 2^(1023 - y_ex)) (u_t 2^(y_ex - 1023))
+            const int c = dm.y_ex[to + i] - 1023;
+            u.x = fx_scale(u.x, c);
+            u.y = fx_scale(u.y, c);
+        }
+        return u;
+    }, nT, 128, cnt, uT, ex);
     g.sync();
     // one thread per row i of Y, all RB right-hand sides at once: each Y entry is read once
-    const cpx<T>* Ye = Y + dm.pq_off[e];
+    const EdgeOp<T>* Ye = Y + dm.pq_off[e];
     for (int i = g.t(); i < nE; i += g.n()) {
-        const cpx<T>* yr = Ye + (int64_t)i * nT;
+        const EdgeOp<T>* yr = Ye + (int64_t)i * nT;
         cpx<T> a[RB];
+        if constexpr (std::is_same<T, double>::value) {
+            FxAcc s[2 * RB];
+            long long h[2 * RB];
+            unsigned l[2 * RB];
 #pragma unroll
-        for (int q = 0; q < RB; ++q) a[q] = mk<T>(0, 0);
-        for (int t = 0; t < nT; ++t) {
-            const cpx<T> y = yr[t];
+            for (int k = 0; k < 2 * RB; ++k) { s[k].h = s[k].l = 0; h[k] = 0; l[k] = 0; }
+            for (int t = 0; t < nT;) {
+                const int end = min(nT, t + kFxChain);
+#pragma unroll(RB <= 2 ? 8 : 2)
+                for (; t < end; ++t) {
+                    const int4 y = yr[t];
+#pragma unroll
+                    for (int q = 0; q < RB; ++q)
+                        if (q < cnt) fx_cmac(s[2 * q], s[2 * q + 1], y, -y.z, -y.w, uT[q * 128 + t]);
+                }
+#pragma unroll
+                for (int k = 0; k < 2 * RB; ++k) fx_flush(s[k], h[k], l[k]);
+            }
 #pragma unroll
             for (int q = 0; q < RB; ++q)
-                if (q < cnt) fma_c(a[q], y, uT[q][t]);
+                if (q < cnt) a[q] = mk<T>(fx_value(h[2 * q], l[2 * q], 1023, ex[q]), fx_value(h[2 * q + 1], l[2 * q + 1], 1023, ex[q]));
+        } else {
+#pragma unroll
+            for (int q = 0; q < RB; ++q) a[q] = mk<T>(0, 0);
+            for (int t = 0; t < nT; ++t) {
+                const cpx<T> y = yr[t];
+#pragma unroll
+                for (int q = 0; q < RB; ++q)
+                    if (q < cnt) fma_c(a[q], y, uT[q * 128 + t]);
+            }
         }
 #pragma unroll
         for (int q = 0; q < RB; ++q)
@@ -350,36 +500,89 @@ __global__ void k_dinv(DevModel dm, const double2* __restrict__ x, double2* __re
 // one CTA per (element, block of RB RHS), each S^Lap entry read once per CTA.
 // out_E = S x for the restricted stiffness Schur complement S (n_E x n_E, symmetric, read from
 // global memory column by column: coalesced across output rows, shared by the elements of a
-// degree pattern and L1/L2-resident); tpr adjacent threads share an output row
+// degree pattern and L1/L2-resident); tpr adjacent threads share an output row.  FP64: S and x in fixed
+// point (two limbs per real entry, DevModel::pre_fx, exponents pre_ex by row; four per complex entry)
 template <class T, int RB>
-__device__ __forceinline__ void pre_apply(const double* __restrict__ S, int nE, int cnt, const cpx<T>* in,
+__device__ __forceinline__ void pre_apply(const DevModel& dm, int e, int nE, int cnt, const EdgeOp<T>* in, const int* ex,
                                           cpx<T>* __restrict__ out, int64_t ostride,
                                           const double* __restrict__ wout = nullptr) {
     const int tpr = nE <= 32 ? 4 : (nE <= 64 ? 2 : 1);
     const int chunk = (nE + tpr - 1) / tpr;
+    const double* S = dm.pre_all + dm.pre_off[e];
+    const int2* F = dm.pre_fx + dm.pre_off[e];
     for (int base = 0; base < nE * tpr; base += blockDim.x) {
         const int slot = base + threadIdx.x;
         const int i = slot / tpr, part = slot % tpr;
-        cpx<T> acc[RB];
+        const int j1 = i < nE ? min(nE, (part + 1) * chunk) : 0;
+        if constexpr (std::is_same<T, double>::value) {
+            // real times complex: one product per component and term, so nE <= 124 terms are one chain
+            FxAcc s[2 * RB];
 #pragma unroll
-        for (int q = 0; q < RB; ++q) acc[q] = mk<T>(0, 0);
-        if (i < nE) {
-            const int j1 = min(nE, (part + 1) * chunk);
+            for (int k = 0; k < 2 * RB; ++k) s[k].h = s[k].l = 0;
+#pragma unroll(RB <= 2 ? 8 : 2)
+            for (int j = part * chunk; j < j1; ++j) {
+                const int2 a = __ldg(F + (int64_t)j * nE + i);
+#pragma unroll
+                for (int q = 0; q < RB; ++q)
+                    if (q < cnt) {
+                        const int4 x = in[q * nE + j];
+                        fx_mac(s[2 * q], a.x, a.y, x.x, x.y);
+                        fx_mac(s[2 * q + 1], a.x, a.y, x.z, x.w);
+                    }
+            }
+#pragma unroll
+            for (int q = 0; q < RB; ++q) {
+                long long h[2] = {0, 0};
+                unsigned l[2] = {0, 0};
+                fx_flush(s[2 * q], h[0], l[0]);
+                fx_flush(s[2 * q + 1], h[1], l[1]);
+                for (int o = 1; o < tpr; o <<= 1)
+                    for (int c = 0; c < 2; ++c) {
+                        h[c] += __shfl_xor_sync(0xffffffffu, h[c], o);
+                        l[c] += __shfl_xor_sync(0xffffffffu, l[c], o);
+                    }
+                if (part == 0 && i < nE && q < cnt) {
+                    const int ea = dm.pre_ex[dm.pre_ex_off[e] + i];
+                    const cpx<double> v = mk<double>(fx_value(h[0], l[0], ea, ex[q]), fx_value(h[1], l[1], ea, ex[q]));
+                    out[(int64_t)q * ostride + i] = wout ? wout[i] * v : v;
+                }
+            }
+        } else {
+            cpx<T> acc[RB];
+#pragma unroll
+            for (int q = 0; q < RB; ++q) acc[q] = mk<T>(0, 0);
             for (int j = part * chunk; j < j1; ++j) {
                 const T sv = (T)__ldg(S + (int64_t)j * nE + i);
 #pragma unroll
                 for (int q = 0; q < RB; ++q)
                     if (q < cnt) fma_r(acc[q], sv, in[q * nE + j]);
             }
-        }
 #pragma unroll
-        for (int q = 0; q < RB; ++q) {
-            for (int o = 1; o < tpr; o <<= 1) {
-                acc[q].x += __shfl_xor_sync(0xffffffffu, acc[q].x, o);
-                acc[q].y += __shfl_xor_sync(0xffffffffu, acc[q].y, o);
+            for (int q = 0; q < RB; ++q) {
+                for (int o = 1; o < tpr; o <<= 1) {
+                    acc[q].x += __shfl_xor_sync(0xffffffffu, acc[q].x, o);
+                    acc[q].y += __shfl_xor_sync(0xffffffffu, acc[q].y, o);
+                }
+                if (part == 0 && i < nE && q < cnt) out[(int64_t)q * ostride + i] = wout ? (T)wout[i] * acc[q] : acc[q];
             }
-            if (part == 0 && i < nE && q < cnt) out[(int64_t)q * ostride + i] = wout ? (T)wout[i] * acc[q] : acc[q];
         }
+    }
+}
+// fixed-point copies of the restricted S^Lap, one warp per row (grid: pattern, 8 warps per CTA)
+__global__ void k_fix_pre(const double* __restrict__ S, const int64_t* __restrict__ off, const int* __restrict__ len,
+                          const int64_t* __restrict__ eoff, int2* __restrict__ fx, int* __restrict__ ex) {
+    const int k = blockIdx.x, nE = len[k], warp = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+    for (int i = warp; i < nE; i += nw) {
+        const double* a = S + off[k] + i;                  // row i = column i (symmetric)
+        unsigned m = 0;
+        for (int j = lane; j < nE; j += 32) m = max(m, (unsigned)__double2hiint(a[(int64_t)j * nE]) & 0x7fffffffu);
+        const int ef = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
+        for (int j = lane; j < nE; j += 32) {
+            int2 f;
+            fx_split(fx_int(a[(int64_t)j * nE], ef), f.x, f.y);
+            fx[off[k] + i + (int64_t)j * nE] = f;
+        }
+        if (lane == 0) ex[eoff[k] + i] = ef;
     }
 }
 
@@ -388,23 +591,23 @@ __global__ void __launch_bounds__(128) k_pre_elem(DevModel dm, const double2* __
                                                   int R, const int* __restrict__ done) {
     if (done && *done) return;
     extern __shared__ __align__(128) char smem[];
+    __shared__ int ex[RB];
     const int e = blockIdx.x, r0 = blockIdx.y * RB;
     const int cnt = min(RB, R - r0);
     const int nE = dm.nE1[e], e1o = dm.e1_off[e];
-    cpx<T>* in = reinterpret_cast<cpx<T>*>(smem);                 // [RB][nE]
-    for (int idx = threadIdx.x; idx < cnt * nE; idx += blockDim.x) {
-        const int q = idx / nE, i = idx % nE;
+    EdgeOp<T>* in = reinterpret_cast<EdgeOp<T>*>(smem);                 // [RB][nE]
+    edge_stage<T>([&](int q, int i) {
         const int row = dm.e1_row[e1o + i];
         cpx<T> val = mk<T>(0, 0);
         if (row >= 0) {
             const double w = dm.e1_win ? dm.e1_sign[e1o + i] * dm.e1_win[e1o + i] : dm.e1_sign[e1o + i];
             val = (T)w * ld<T>(v, (int64_t)(r0 + q) * dm.n_dual + row);
         }
-        in[q * nE + i] = val;
-    }
+        return val;
+    }, nE, nE, cnt, in, ex);
     __syncthreads();
     // Poisson mode: out = (rho_e w) .* (S^Lap (w .* C1^T v)), the diagonally scaled W^T A W
-    pre_apply<T, RB>(dm.pre_all + dm.pre_off[e], nE, cnt, in, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot,
+    pre_apply<T, RB>(dm, e, nE, cnt, in, ex, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot,
                      dm.e1_wout ? dm.e1_wout + e1o : nullptr);
 }
 
@@ -415,12 +618,12 @@ __global__ void __launch_bounds__(128) k_pre_elem_kry(DevModel dm, KrylovDev K, 
     if (K.ctl[1]) return;
     const int jj = K.ctl[0];
     extern __shared__ __align__(128) char smem[];
+    __shared__ int ex[RB];
     const int e = blockIdx.x, r0 = blockIdx.y * RB;
     const int cnt = min(RB, R - r0);
     const int nE = dm.nE1[e], e1o = dm.e1_off[e];
-    cpx<T>* in = reinterpret_cast<cpx<T>*>(smem);
-    for (int idx = threadIdx.x; idx < cnt * nE; idx += blockDim.x) {
-        const int q = idx / nE, i = idx % nE;
+    EdgeOp<T>* in = reinterpret_cast<EdgeOp<T>*>(smem);
+    edge_stage<T>([&](int q, int i) {
         const int row = dm.e1_row[e1o + i];
         cpx<T> val = mk<T>(0, 0);
         if (row >= 0) {
@@ -432,10 +635,10 @@ __global__ void __launch_bounds__(128) k_pre_elem_kry(DevModel dm, KrylovDev K, 
                 val = (T)(0.5 * dm.e1_sign[e1o + i]) * ld<T>(K.V, at);
             }
         }
-        in[q * nE + i] = val;
-    }
+        return val;
+    }, nE, nE, cnt, in, ex);
     __syncthreads();
-    pre_apply<T, RB>(dm.pre_all + dm.pre_off[e], nE, cnt, in, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot);
+    pre_apply<T, RB>(dm, e, nE, cnt, in, ex, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot);
 }
 
 // z = D^-1 (outE[c] - outE[f]) with D = 2 I, written to zw and to the Krylov store Zb[r][j]
@@ -489,7 +692,7 @@ static int edge_p_layout(int rb, int maxE1, int* buf_bytes, size_t* total) {
     return fit ? (int)base : 0;
 }
 template <class T, int RB>
-static void edge_p_t(const DevModel& dm, const cpx<T>* S, const cpx<T>* Yp, const double2* z, double zsign,
+static void edge_p_t(const DevModel& dm, const EdgeOp<T>* S, const EdgeOp<T>* Yp, const double2* z, double zsign,
                      const double2* bt, void* xE, void* tT, int R, const int* done, const EdgeSched& es, int item0,
                      int nitems, int tpr_force, cudaStream_t st) {
     int buf = 0;
@@ -512,8 +715,8 @@ void launch_pass1_edge(const DevModel& dm, const void* sinv, const void* Y, cons
                        const double2* bt, void* xE, void* tT, int R, const int* done, cudaStream_t st,
                        const EdgeSched* es, int item0, int nitems, int tpr_force, int rows) {
     const int rb = rhs_block(R);
-    const cpx<T>* S = (const cpx<T>*)sinv;
-    const cpx<T>* Yp = (const cpx<T>*)Y;
+    const EdgeOp<T>* S = (const EdgeOp<T>*)sinv;
+    const EdgeOp<T>* Yp = (const EdgeOp<T>*)Y;
     if (es && es->items && rows == 0) {
         if (nitems < 0) nitems = dm.E;
         switch (rb) {
@@ -545,7 +748,7 @@ void launch_pass2_edge(const DevModel& dm, const void* Y, const double2* x2, con
                        const int* done, cudaStream_t st) {
     const int rb = rhs_block(R);
     const int ntask = dm.E * ((R + rb - 1) / rb);
-    const cpx<T>* Yp = (const cpx<T>*)Y;
+    const EdgeOp<T>* Yp = (const EdgeOp<T>*)Y;
     const cpx<T>* xi = (const cpx<T>*)xE_in;
     cpx<T>* xo = (cpx<T>*)xE_out;
     // one thread per edge row: 64-thread CTAs when every element has at most 64 (more CTAs
@@ -596,6 +799,14 @@ template void launch_jump_gather<double>(const DevModel&, const void*, const dou
 template void launch_jump_gather<float>(const DevModel&, const void*, const double2*, double2*, int, const int*, cudaStream_t);
 template void launch_pre<double>(const DevModel&, const double2*, double2*, void*, double2*, double2*, int, int, const int*, cudaStream_t);
 template void launch_pre<float>(const DevModel&, const double2*, double2*, void*, double2*, double2*, int, int, const int*, cudaStream_t);
+void launch_fix_edge(const DevModel& dm, const void* sinv, const void* Y, void* sfx, int* sex, void* yfx, int* yex,
+                     cudaStream_t st) {
+    k_fix_edge<<<dm.E, 256, 0, st>>>(dm, (const double2*)sinv, (const double2*)Y, (int4*)sfx, sex, (int4*)yfx, yex);
+}
+void launch_fix_pre(const double* S, int npat, const int64_t* off, const int* len, const int64_t* eoff, int2* fx, int* ex,
+                    cudaStream_t st) {
+    if (npat > 0) k_fix_pre<<<npat, 256, 0, st>>>(S, off, len, eoff, fx, ex);
+}
 void launch_dinv(const DevModel& dm, const double2* x, double2* y, int R, const int* done, cudaStream_t st) {
     k_dinv<<<dim3((dm.n_dual + 127) / 128, R), 128, 0, st>>>(dm, x, y, 1, done);
 }

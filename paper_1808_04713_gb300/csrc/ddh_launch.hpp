@@ -54,6 +54,14 @@ void launch_pass1_edge(const DevModel& dm, const void* sinv, const void* Y, cons
                        const double2* bt, void* xE, void* tT, int R, const int* done, cudaStream_t st,
                        const EdgeSched* es = nullptr, int item0 = 0, int nitems = -1, int tpr_force = 0,
                        int rows = 0);
+// in FP64 both take the operators in fixed point: launch_fix_edge makes sfx, yfx (four ints per entry)
+// and their exponents from the complex128 S_E^-1 and Y
+void launch_fix_edge(const DevModel& dm, const void* sinv, const void* Y, void* sfx, int* sex, void* yfx, int* yex,
+                     cudaStream_t st);
+// the same for npat restricted S^Lap (real, two ints per entry): pattern k is len[k]^2 entries at off[k],
+// its exponents at eoff[k]
+void launch_fix_pre(const double* S, int npat, const int64_t* off, const int* len, const int64_t* eoff, int2* fx, int* ex,
+                    cudaStream_t st);
 // default CTA size of the one-CTA-per-task edge pass for elements of at most maxNo output rows
 int edge_cta_threads(int maxNo);
 template <class T>
