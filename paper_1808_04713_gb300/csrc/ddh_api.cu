@@ -124,6 +124,9 @@ struct ddh_ctx {
     KState kin, kout;
     // Poisson mode: extreme Ritz values of P^-1 F from the PCG coefficients of the last solve
     std::vector<double> pcg_lmin, pcg_lmax;
+    // captured PCG iterations per R (with their kernel counts), and the iterations of the last solve
+    std::map<int, std::pair<cudaGraphExec_t, int64_t>> pcg_graphs;
+    int pcg_hint = 0;
     // per-degree tables of the Dirichlet trace lifting (ddh_dirichlet_point_source)
     const int64_t* tr_off = nullptr;
     const int* tr_nq = nullptr;
@@ -184,8 +187,15 @@ static ddh_status upload(ddh_ctx* ctx, const std::vector<V>& v, const V** out) {
     return DDH_OK;
 }
 
+static void drop_pcg_graphs(ddh_ctx* ctx) {
+    for (auto& kv : ctx->pcg_graphs) cudaGraphExecDestroy(kv.second.first);
+    ctx->pcg_graphs.clear();
+}
+
 static void free_model(ddh_ctx* ctx) {
     cudaStreamSynchronize(ctx->stream);
+    drop_pcg_graphs(ctx);
+    ctx->pcg_hint = 0;
     for (void* p : ctx->model_allocs) cudaFree(p);
     ctx->model_allocs.clear();
     ctx->kin.release();
@@ -239,6 +249,7 @@ static ddh_status get_work(ddh_ctx* ctx, const std::string& name, size_t bytes, 
             for (auto& kv : ks->graphs) cudaGraphExecDestroy(kv.second);
             ks->graphs.clear();
         }
+        drop_pcg_graphs(ctx);
         if (cudaMalloc(&b.p, bytes) != cudaSuccess) { b.bytes = 0; ctx->err = "cudaMalloc failed (" + name + ")"; return DDH_ERR_OOM; }
         b.bytes = bytes;
     }
@@ -2055,7 +2066,7 @@ static ddh_status solve_pcg(ddh_ctx* ctx, const double2* b_dev, double2* u_dev, 
     const int maxit = std::max(1, ctx->opt.maxit);
     const int64_t nd = d.n_dual;
     const size_t vb = sizeof(double2) * (size_t)R * std::max<int64_t>(1, nd);
-    void *g, *nu, *rv, *z, *dv, *Fd, *part, *sc, *ah, *bh;
+    void *g, *nu, *rv, *z, *dv, *Fd, *part, *sc, *cnt, *ah, *bh;
     if ((sts = get_work(ctx, "pcg_g", vb, &g))) return sts;
     if ((sts = get_work(ctx, "pcg_nu", vb, &nu))) return sts;
     if ((sts = get_work(ctx, "pcg_r", vb, &rv))) return sts;
@@ -2063,65 +2074,88 @@ static ddh_status solve_pcg(ddh_ctx* ctx, const double2* b_dev, double2* u_dev, 
     if ((sts = get_work(ctx, "pcg_d", vb, &dv))) return sts;
     if ((sts = get_work(ctx, "pcg_Fd", vb, &Fd))) return sts;
     if ((sts = get_work(ctx, "pcg_part", sizeof(double) * (size_t)R * kPcgBlocks, &part))) return sts;
-    if ((sts = get_work(ctx, "pcg_sc", sizeof(double) * 8 * (size_t)R, &sc))) return sts;
+    if ((sts = get_work(ctx, "pcg_sc", sizeof(double) * kPcgScalars * (size_t)R, &sc))) return sts;
+    if ((sts = get_work(ctx, "pcg_cnt", sizeof(int) * (size_t)R, &cnt))) return sts;
     if ((sts = get_work(ctx, "pcg_ah", sizeof(double) * (size_t)R * maxit, &ah))) return sts;
     if ((sts = get_work(ctx, "pcg_bh", sizeof(double) * (size_t)R * maxit, &bh))) return sts;
     double2 *G = (double2*)g, *NU = (double2*)nu, *RV = (double2*)rv, *Z = (double2*)z, *D = (double2*)dv,
             *FD = (double2*)Fd;
-    double *PART = (double*)part, *SC = (double*)sc, *AH = (double*)ah, *BH = (double*)bh;
+    const PcgBufs B{(double*)sc, (double*)part, (int*)cnt, (double*)ah, (double*)bh, maxit};
+    double* SC = B.sc;
     const double tol2 = tol * tol;
     std::vector<int> its(R, 0);
     std::vector<double> res(R, 0.0), pr;
-    std::vector<double> hsc(8 * (size_t)R, 0.0);
+    std::vector<double> hsc(kPcgScalars * (size_t)R, 0.0);
     // g = C^ A^-1 b^ (interior loads included)
     apply_op<double>(ctx, w, nullptr, 0.0, (const double2*)bt, 1, G, nullptr, R, nullptr);
-    CK(cudaMemsetAsync(SC, 0, sizeof(double) * 8 * (size_t)R, st));
-    CK(cudaMemsetAsync(AH, 0, sizeof(double) * (size_t)R * maxit, st));
-    CK(cudaMemsetAsync(BH, 0, sizeof(double) * (size_t)R * maxit, st));
+    CK(cudaMemsetAsync(SC, 0, sizeof(double) * kPcgScalars * (size_t)R, st));
+    CK(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)R, st));
+    CK(cudaMemsetAsync(ah, 0, sizeof(double) * (size_t)R * maxit, st));
+    CK(cudaMemsetAsync(bh, 0, sizeof(double) * (size_t)R * maxit, st));
     int done_all = 0;
     if (nd > 0) {
         CK(cudaMemsetAsync(NU, 0, vb, st));
         CK(cudaMemcpyAsync(RV, G, vb, cudaMemcpyDeviceToDevice, st));
-        launch_dual_dot(RV, RV, nd, PART, R, st);
-        launch_pcg_scalar(PART, SC, 0, 0, tol2, AH, BH, maxit, R, st);
+        launch_pcg_dot(RV, RV, nd, B, 0, tol2, R, st);
         apply_prec<double>(ctx, w, RV, Z, R, nullptr);
-        launch_dual_dot(RV, Z, nd, PART, R, st);
-        launch_pcg_scalar(PART, SC, 1, 0, tol2, AH, BH, maxit, R, st);
+        launch_pcg_dot(RV, Z, nd, B, 1, 0.0, R, st);
         CK(cudaMemcpyAsync(D, Z, vb, cudaMemcpyDeviceToDevice, st));
-        ctx->launches += 4;
-        int it = 0;
-        for (; it < maxit; ++it) {
+        ctx->launches += 2;
+        auto body = [&] {
             apply_op<double>(ctx, w, D, 1.0, nullptr, 0, FD, nullptr, R, nullptr);   // F d
-            launch_dual_dot(D, FD, nd, PART, R, st);
-            launch_pcg_scalar(PART, SC, 2, it, tol2, AH, BH, maxit, R, st);
-            launch_pcg_xr(NU, RV, D, FD, SC, nd, PART, R, st);
-            launch_pcg_scalar(PART, SC, 3, it, tol2, AH, BH, maxit, R, st);
+            launch_pcg_dot(D, FD, nd, B, 2, 0.0, R, st);
+            launch_pcg_xr(NU, RV, D, FD, nd, B, R, st);
+            apply_prec<double>(ctx, w, RV, Z, R, nullptr);
+            launch_pcg_dot(RV, Z, nd, B, 4, 0.0, R, st);
+            launch_pcg_d(D, Z, SC, nd, R, st);
             ctx->launches += 4;
-            CK(cudaMemcpyAsync(hsc.data(), SC, sizeof(double) * 8 * (size_t)R, cudaMemcpyDeviceToHost, st));
+        };
+        cudaGraphExec_t ge = nullptr;
+        int64_t per = 0;
+        if (ctx->opt.use_graph) {
+            auto it = ctx->pcg_graphs.find(R);
+            if (it == ctx->pcg_graphs.end()) {
+                const int64_t before = ctx->launches;
+                cudaGraph_t gr;
+                CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+                body();
+                const cudaError_t ce = cudaStreamEndCapture(st, &gr);
+                if (ce != cudaSuccess) return fail(ctx, DDH_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(ce));
+                CK(cudaGraphInstantiate(&ge, gr, 0));
+                cudaGraphDestroy(gr);
+                it = ctx->pcg_graphs.emplace(R, std::make_pair(ge, ctx->launches - before)).first;
+                ctx->launches = before;
+            }
+            ge = it->second.first;
+            per = it->second.second;
+        }
+        // the flags are read after as many iterations as the previous solve took, then after each one
+        for (int it = 0; it < maxit && !done_all;) {
+            const int batch = std::min(it == 0 ? std::max(1, ctx->pcg_hint) : 1, maxit - it);
+            for (int k = 0; k < batch; ++k) {
+                if (ge) { CK(cudaGraphLaunch(ge, st)); ctx->launches += per; }
+                else body();
+            }
+            it += batch;
+            CK(cudaMemcpyAsync(hsc.data(), SC, sizeof(double) * hsc.size(), cudaMemcpyDeviceToHost, st));
             CK(cudaStreamSynchronize(st));
             done_all = 1;
-            for (int r = 0; r < R; ++r) done_all &= hsc[8 * r + 4] != 0.0;
-            if (done_all) break;
-            apply_prec<double>(ctx, w, RV, Z, R, nullptr);
-            launch_dual_dot(RV, Z, nd, PART, R, st);
-            launch_pcg_scalar(PART, SC, 4, it, tol2, AH, BH, maxit, R, st);
-            launch_pcg_d(D, Z, SC, nd, R, st);
-            ctx->launches += 3;
+            for (int r = 0; r < R; ++r) done_all &= hsc[kPcgScalars * r + 4] != 0.0;
         }
-        CK(cudaMemcpyAsync(hsc.data(), SC, sizeof(double) * 8 * (size_t)R, cudaMemcpyDeviceToHost, st));
         std::vector<double> ha((size_t)R * maxit), hb((size_t)R * maxit);
-        CK(cudaMemcpyAsync(ha.data(), AH, sizeof(double) * ha.size(), cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(hb.data(), BH, sizeof(double) * hb.size(), cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(ha.data(), ah, sizeof(double) * ha.size(), cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(hb.data(), bh, sizeof(double) * hb.size(), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
         ctx->pcg_lmin.assign(R, 0.0);
         ctx->pcg_lmax.assign(R, 0.0);
         for (int r = 0; r < R; ++r) {
-            const bool dn = hsc[8 * r + 4] != 0.0;
-            its[r] = dn ? (int)hsc[8 * r + 5] : maxit;
-            res[r] = hsc[8 * r + 3] > 0 ? std::sqrt(hsc[8 * r + 6] / hsc[8 * r + 3]) : 0.0;
+            const bool dn = hsc[kPcgScalars * r + 4] != 0.0;
+            its[r] = dn ? (int)hsc[kPcgScalars * r + 5] : maxit;
+            res[r] = hsc[kPcgScalars * r + 3] > 0 ? std::sqrt(hsc[kPcgScalars * r + 6] / hsc[kPcgScalars * r + 3]) : 0.0;
             lanczos_extremes(ha.data() + (size_t)r * maxit, hb.data() + (size_t)r * maxit, its[r], ctx->pcg_lmin[r],
                              ctx->pcg_lmax[r]);
         }
+        ctx->pcg_hint = *std::max_element(its.begin(), its.end());
         // recovery: A^ phi = b^ - C^T nu
         apply_op<double>(ctx, w, NU, -1.0, (const double2*)bt, 1, nullptr, (double2*)phit, R, nullptr);
     } else {
