@@ -81,12 +81,19 @@ __device__ __forceinline__ void fx_flush(FxAcc& s, long long& h, unsigned& l) {
     l += ((unsigned)(t & 255) << 16) | (unsigned)((int)(s.l & ((1ll << kFxLow) - 1)) >> (kFxLow - 16));
     s.h = s.l = 0;
 }
-// d 2^s; results below 2^-1022 become zero
+// 2^s, -1022 <= s <= 1023
+__device__ __forceinline__ double fx_pow2(int s) { return __longlong_as_double((long long)(1023 + s) << 52); }
+// d 2^s; results below 2^-1022 become zero.  On the 64-bit pattern: written on its two 32-bit halves
+// (__double2hiint, __hiloint2double) the build lost the low half of one of two sums in k_gemv_fx, an
+// error of 2^-21.
 __device__ __forceinline__ double fx_scale(double d, int s) {
-    const int hi = __double2hiint(d), e = (hi >> 20) & 0x7ff, t = e + s;
-    if ((unsigned)(e - 1) >= 2046u) return d;          // zero, infinity, NaN
-    if ((unsigned)(t - 1) < 2046u) return __hiloint2double(hi + (s << 20), __double2loint(d));
-    return t <= 0 ? 0.0 : __hiloint2double((hi & 0x80000000) | 0x7ff00000, 0);
+    const long long b = __double_as_longlong(d);
+    const int e = (int)(b >> 52) & 0x7ff, t = e + s;
+    long long r = b + ((long long)s << 52);
+    if (t <= 0) r = 0;
+    if (t >= 0x7ff) r = (b & (1ll << 63)) | (0x7ffll << 52);
+    if (e == 0 || e == 0x7ff) r = b;                   // zero, infinity, NaN
+    return __longlong_as_double(r);
 }
 // Column scaling: a column whose largest entry has exponent field c is divided by 2^(c - 1023) before the
 // rows get their exponents, and the vector's entry multiplied by it (exactly) before it is staged.  The
@@ -101,7 +108,9 @@ __device__ __forceinline__ double fx_value(long long h, unsigned l, int ea, int 
     int k = __clzll(h ^ (h >> 63)) - 1;                // headroom of h
     k = k < 24 ? k : 24;
     const long long v = (h << k) + (l >> (24 - k));
-    return fx_scale(__ll2double_rn(v), 2 * kFxLow + 8 - k + ea + ex - 2044 - 2 * kFxBits);
+    const int s = 2 * kFxLow + 8 - k + ea + ex - 2044 - 2 * kFxBits, a = max(min(s, 1000), -1000);
+    const double d = __dmul_rn(__ll2double_rn(v), fx_pow2(a));
+    return s == a ? d : __dmul_rn(d, fx_pow2(max(s - a, -1000)));
 }
 
 // A sum with its al xl products kept, s + ll, split in two FP64 numbers that hold it to 2^-96 of the
