@@ -95,93 +95,85 @@ __global__ void k_basis(DevModel dm, const double2* __restrict__ x, double2* __r
 }
 
 // (A phi) per element in FP64 (interpolatory basis), out = b - A phi (b may be null).  The
-// operator is applied one direction at a time with the sparse 1-D tables: along x2,
-//   T1 = Phi Mt^T,  T2 = Phi Kt^T   (T[c][b] = sum_d X[b][d] Phi[c][d]),
-// then along x1, (A Phi)[a][b] = sum_c Kt[a][c] T1[c][b] + Mt[a][c] (T2 + c_e T1)[c][b], plus
-// the Robin terms (T1 on the sides a = 0, 1; Mt along x1 on the sides b = 0, 1).  Every row
-// of Mt and Kt has at most six entries (cand_list), so this is O(p^2) per element.
+// operator is applied one direction at a time with the sparse 1-D tables: along x1,
+//   P = Mt Phi,  Q = Kt Phi + c_e P,
+// then along x2, A Phi = Q Mt^T + P Kt^T, plus the Robin terms (P on the sides b = 0, 1; Mt along x2 of
+// Phi on the sides a = 0, 1).  A row of Mt couples i to i - 2, i, i + 2 (rows 0 to 3: to the first two
+// also), one of Kt from 2 on only to itself, so about 18 FP64 operations per value are left, two per SM
+// and clock; in both directions a warp's threads share a row (or two) of Mt, so that hardly any tap is
+// issued for nothing.  64 x 64 elements, p = 20, 8 right-hand sides: 1.40 ms with index lists of up to
+// six columns per row, 1.05 ms now (a thread per line, neighbours in registers: 1.07 ms, and three times
+// slower on 16 x 16 elements: too few threads).
+struct MtTaps {
+    double w[4][33];                     // row i: columns i - 2, i, i + 2 (i >= 4); 0, 1, 2, 3 (i < 2); 0, 1, i, i + 2
+    __device__ __forceinline__ void load(const double* __restrict__ Mt, int i, int p) {
+        const double* m = Mt + i * (p + 1);
+        w[0][i] = m[i < 4 ? 0 : i - 2];
+        w[1][i] = m[i < 4 ? 1 : i];
+        w[2][i] = i < 2 ? m[2] : (i < 4 ? m[i] : (i + 2 <= p ? m[i + 2] : 0.0));
+        w[3][i] = i < 2 ? m[3] : (i < 4 && i + 2 <= p ? m[i + 2] : 0.0);
+    }
+    // (Mt f)_i, f at stride st
+    __device__ __forceinline__ cpx<double> row(const cpx<double>* f, int st, int i, int p) const {
+        const int c0 = i < 4 ? 0 : i - 2, c1 = i < 4 ? 1 : i, c2 = i < 2 ? 2 : (i < 4 ? i : min(i + 2, p));
+        cpx<double> s = w[0][i] * f[c0 * st];
+        fma_r(s, w[1][i], f[c1 * st]);
+        fma_r(s, w[2][i], f[c2 * st]);
+        if (i < 4) fma_r(s, w[3][i], f[(i < 2 ? 3 : min(i + 2, p)) * st]);
+        return s;
+    }
+};
 __global__ void __launch_bounds__(128) k_elem_matvec(DevModel dm, const double2* __restrict__ phi,
                                                      const double2* __restrict__ b, double2* __restrict__ out) {
     extern __shared__ __align__(128) char smem[];
+    __shared__ MtTaps M;
     const int e = blockIdx.x, r = blockIdx.y;
-    const int p = dm.p[e], N = p + 1;
-    const int NP = dm.pmax + 1;
-    // only what the matvec reads: the tile, two products, the side sums and the 1-D mass table
-    struct {
-        cpx<double>* tile;
-        double* Mt;
-    } s;
-    s.tile = reinterpret_cast<cpx<double>*>(smem);   // [N][N], index c + N b
-    cpx<double>* T1 = s.tile + NP * NP;
-    cpx<double>* T2 = T1 + NP * NP;
-    cpx<double>* S1 = T2 + NP * NP;                  // [2][N]: sum_c Mt[a][c] Phi[c][b'] for b' = 0, 1
-    s.Mt = reinterpret_cast<double*>(S1 + 2 * NP);
-    {
-        const double* Mt = dm.Mt_all + dm.tab_Mt[dm.ptab[e]];
-        for (int i = threadIdx.x; i < N * N; i += blockDim.x) s.Mt[i] = Mt[i];
-    }
+    const int p = dm.p[e], N = p + 1, ld = N | 1;           // odd: lines along x2 start in different banks
+    cpx<double>* X = reinterpret_cast<cpx<double>*>(smem);  // [a + ld b]
+    cpx<double>* P = X + (size_t)N * ld;
+    cpx<double>* Q = P + (size_t)N * ld;
     const int64_t base = (int64_t)r * dm.n_local + dm.off[e];
-    for (int i = threadIdx.x; i < N * N; i += blockDim.x) { const double2 v = phi[base + i]; s.tile[i] = mk<double>(v.x, v.y); }
-    __syncthreads();
+    const double ce = dm.c[e], ks = dm.ks[e];
+    const double* pml = dm.pml ? dm.pml + 6 * (int64_t)e : nullptr;
+    if (threadIdx.x < N) M.load(dm.Mt_all + dm.tab_Mt[dm.ptab[e]], threadIdx.x, p);
+    for (int i = threadIdx.x; i < N * N; i += blockDim.x) {
+        const double2 v = phi[base + i];
+        X[i % N + ld * (i / N)] = mk<double>(v.x, v.y);
+    }
     double gam[4];
     elem_gam<double>(dm, e, gam);
-    const double ce = dm.c[e], ks = dm.ks[e];
-    for (int idx = threadIdx.x; idx < N * N; idx += blockDim.x) {
-        const int c = idx % N, bb = idx / N;
-        int cd[6];
-        const int nd = cand_list(bb, p, cd);
-        cpx<double> t1 = mk<double>(0, 0), t2 = mk<double>(0, 0);
-        for (int q = 0; q < nd; ++q) {
-            const int d = cd[q];
-            const cpx<double> v = s.tile[c + N * d];
-            fma_r(t1, s.Mt[bb * N + d], v);
-            const double kv = kt<double>(bb, d);
-            if (kv != 0.0) fma_r(t2, kv, v);
-        }
-        T1[idx] = t1;
-        if (dm.pml) {
-            // PML: pb M(x1) K(x2) + pc M (x) M on this side of the product
-            const double* q = dm.pml + 6 * (int64_t)e;
-            T2[idx] = mk<double>(q[2], q[3]) * t2 + mk<double>(q[4], q[5]) * t1;
-        } else {
-            T2[idx] = t2 + ce * t1;
-        }
-    }
-    for (int idx = threadIdx.x; idx < 2 * N; idx += blockDim.x) {
-        const int a = idx % N, bp = idx / N;
-        int ca[6];
-        const int na = cand_list(a, p, ca);
-        cpx<double> v = mk<double>(0, 0);
-        for (int q = 0; q < na; ++q) fma_r(v, s.Mt[a * N + ca[q]], s.tile[ca[q] + N * bp]);
-        S1[idx] = v;
+    __syncthreads();
+    for (int i = threadIdx.x; i < N * N; i += blockDim.x) {
+        const int bb = i % N, a = i / N;
+        const cpx<double>* x = X + ld * bb;
+        const cpx<double> mx = M.row(x, 1, a, p);
+        const cpx<double> kx = a >= 2 ? x[a] : 0.5 * (x[a] - x[1 - a]);
+        P[a + ld * bb] = mx;
+        // PML: pa K(x1) M(x2) + pb M(x1) K(x2) + pc M (x) M
+        Q[a + ld * bb] = pml ? mk<double>(pml[0], pml[1]) * kx + mk<double>(pml[4], pml[5]) * mx : kx + ce * mx;
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < N * N; idx += blockDim.x) {
-        const int a = idx % N, bb = idx / N;
-        int ca[6];
-        const int na = cand_list(a, p, ca);
-        cpx<double> v = mk<double>(0, 0);
-        for (int q = 0; q < na; ++q) {
-            const int c = ca[q];
-            fma_r(v, s.Mt[a * N + c], T2[c + N * bb]);
-            const double kv = kt<double>(a, c);
-            if (kv != 0.0) {
-                if (dm.pml) fma_c(v, mk<double>(kv * dm.pml[6 * (int64_t)e], kv * dm.pml[6 * (int64_t)e + 1]), T1[c + N * bb]);
-                else fma_r(v, kv, T1[c + N * bb]);
-            }
-        }
+    for (int i = threadIdx.x; i < N * N; i += blockDim.x) {
+        const int a = i % N, bb = i / N;
+        const cpx<double> pv = P[a + ld * bb];
+        const cpx<double> kp = bb >= 2 ? pv : 0.5 * (pv - P[a + ld * (1 - bb)]);
+        cpx<double> v = M.row(Q + a, ld, bb, p);
+        v += pml ? mk<double>(pml[2], pml[3]) * kp : kp;
         // Robin: i g (...) with g the imaginary part of gamma_eff on the side
-        cpx<double> rob = mk<double>(0, 0);
-        if (a == 1 && gam[0] != 0.0) rob += gam[0] * T1[1 + N * bb];
-        if (a == 0 && gam[1] != 0.0) rob += gam[1] * T1[0 + N * bb];
-        if (bb == 1 && gam[2] != 0.0) rob += gam[2] * S1[a + N * 1];
-        if (bb == 0 && gam[3] != 0.0) rob += gam[3] * S1[a + N * 0];
-        v.x -= rob.y;
-        v.y += rob.x;
-        v = ks * v;                      // element coefficient (1 for Helmholtz: exact)
+        const double ga = a == 1 ? gam[0] : (a == 0 ? gam[1] : 0.0), gb = bb == 1 ? gam[2] : (bb == 0 ? gam[3] : 0.0);
+        if (ga != 0.0) {
+            const cpx<double> q = M.row(X + a, ld, bb, p);
+            v.x = fma(-ga, q.y, v.x);
+            v.y = fma(ga, q.x, v.y);
+        }
+        if (gb != 0.0) {
+            v.x = fma(-gb, pv.y, v.x);
+            v.y = fma(gb, pv.x, v.y);
+        }
+        if (ks != 1.0) v = ks * v;                 // element coefficient (1 for Helmholtz)
         double2 o = make_double2(-v.x, -v.y);
-        if (b) { const double2 bv = b[base + idx]; o.x += bv.x; o.y += bv.y; }
-        out[base + idx] = o;
+        if (b) { const double2 bv = b[base + i]; o.x += bv.x; o.y += bv.y; }
+        out[base + i] = o;
     }
 }
 
@@ -437,13 +429,9 @@ void launch_interior_nz(const DevModel& dm, const double2* bt, int* flag, int R,
 void launch_basis(const DevModel& dm, const double2* x, double2* y, int conj_in, int R, cudaStream_t st) {
     k_basis<<<dim3(dm.E, R), 128, 0, st>>>(dm, x, y, conj_in);
 }
-static size_t elem_matvec_smem(int pmax) {
-    const size_t NP = pmax + 1;
-    return sizeof(cpx<double>) * (3 * NP * NP + 2 * NP) + sizeof(double) * NP * NP;
-}
+static size_t elem_matvec_smem(int pmax) { return sizeof(cpx<double>) * 3 * (size_t)(pmax + 1) * ((pmax + 1) | 1); }
 void launch_elem_matvec(const DevModel& dm, const double2* phi, const double2* b, double2* out, int R, cudaStream_t st) {
-    const size_t sm = elem_matvec_smem(dm.pmax);
-    k_elem_matvec<<<dim3(dm.E, R), 128, sm, st>>>(dm, phi, b, out);
+    k_elem_matvec<<<dim3(dm.E, R), 128, elem_matvec_smem(dm.pmax), st>>>(dm, phi, b, out);
 }
 void launch_conf_gather(const DevModel& dm, const double2* x, double* norm2, int R, cudaStream_t st) {
     k_conf_gather<<<dim3((dm.n_conf + 255) / 256, R), 256, 0, st>>>(dm, x, norm2);
@@ -463,7 +451,8 @@ void launch_readback(const DevModel& dm, const double2* phi, double2* z, int R, 
 
 
 void set_misc_limits(int pmax) {
-    cudaFuncSetAttribute(k_elem_matvec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)elem_matvec_smem(pmax));
+    // for the largest degree: another context may need more than this one
+    cudaFuncSetAttribute(k_elem_matvec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)elem_matvec_smem(32));
     cudaFuncSetAttribute(k_grad_elem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)elem_smem_bytes<double>(pmax, 0));
 }
 
