@@ -73,6 +73,7 @@ struct ddh_ctx {
     void* pq32 = nullptr;
     void* sfx = nullptr;                           // S_E^-1 and Y in fixed point (FP64 edge passes)
     void* yfx = nullptr;
+    void* y2fx = nullptr;                          // Y again, column-major, for pass 2
     bool edge_form = false;                        // Krylov-loop passes with Y (no FDM)
     const int* edge_items = nullptr;               // elements by degree, descending (persistent edge pass)
     std::vector<int> deg_begin, deg_count, deg_p;  // contiguous runs of equal degree in edge_items
@@ -204,7 +205,7 @@ static void free_model(ddh_ctx* ctx) {
     ctx->work.clear();
     ctx->sinv64 = ctx->sinv32 = nullptr;
     ctx->pq64 = ctx->pq32 = nullptr;
-    ctx->sfx = ctx->yfx = nullptr;
+    ctx->sfx = ctx->yfx = ctx->y2fx = nullptr;
     ctx->edge_form = false;
     ctx->edge_items = nullptr;
     ctx->deg_begin.clear(); ctx->deg_count.clear(); ctx->deg_p.clear();
@@ -289,6 +290,7 @@ static ddh_status upload_model(ddh_ctx* ctx) {
     for (int e = 0; e < E; ++e) {
         d.maxE1 = std::max(d.maxE1, m.el[e].nE1);
         d.maxNo = std::max(d.maxNo, m.el[e].nE1 + m.el[e].nT);
+        d.maxY = std::max(d.maxY, m.el[e].nE1 * m.el[e].nT);
     }
     if ((st = upload(ctx, p, &d.p))) return st;
     if ((st = upload(ctx, off, &d.off))) return st;
@@ -483,6 +485,7 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         if ((st = upload(ctx, rows, &d.c2t_row))) return st;
         if ((st = upload(ctx, w, &d.c2t_w))) return st;
     }
+    d.n_hb = (int)m.hblk_row0.size();
     if ((st = upload(ctx, m.hblk_row0, &d.hb_row0))) return st;
     if ((st = upload(ctx, m.hblk_n, &d.hb_n))) return st;
     if ((st = upload(ctx, m.hblk_off, &d.hb_off))) return st;
@@ -1332,18 +1335,22 @@ static EdgeSched edge_sched(const ddh_ctx* ctx, bool fp64, int R) {
 static ddh_status fix_edge(ddh_ctx* ctx) {
     if (!ctx->edge_form || ctx->sfx) return DDH_OK;
     DevModel& d = ctx->dm;
-    void *s, *y, *se, *ye;
     ddh_status st;
-    if ((st = model_alloc(ctx, sizeof(double2) * ctx->m.sinv.size(), &s))) return st;
-    if ((st = model_alloc(ctx, sizeof(double2) * ctx->m.pq.size(), &y))) return st;
-    if ((st = model_alloc(ctx, sizeof(int) * (size_t)d.nE1_tot, &se))) return st;
-    if ((st = model_alloc(ctx, sizeof(int) * (size_t)d.nT_tot, &ye))) return st;
-    launch_fix_edge(d, ctx->sinv64, ctx->pq64, s, (int*)se, y, (int*)ye, ctx->stream);
+    EdgeFix f;
+    const size_t ys = sizeof(int4) * ctx->m.pq.size();
+    if ((st = model_alloc(ctx, sizeof(int4) * ctx->m.sinv.size(), (void**)&f.s))) return st;
+    if ((st = model_alloc(ctx, ys, (void**)&f.y)) || (st = model_alloc(ctx, ys, (void**)&f.y2))) return st;
+    if ((st = model_alloc(ctx, sizeof(int) * (size_t)d.nE1_tot, (void**)&f.sex))) return st;
+    if ((st = model_alloc(ctx, sizeof(int) * (size_t)d.nT_tot, (void**)&f.yex))) return st;
+    if ((st = model_alloc(ctx, sizeof(int) * (size_t)d.nE1_tot, (void**)&f.y2ex))) return st;
+    launch_fix_edge(d, ctx->sinv64, ctx->pq64, f, ctx->stream);
     CK(cudaGetLastError());
-    d.sinv_ex = (const int*)se;
-    d.y_ex = (const int*)ye;
-    ctx->sfx = s;
-    ctx->yfx = y;
+    d.sinv_ex = f.sex;
+    d.y_ex = f.yex;
+    d.y2_ex = f.y2ex;
+    ctx->sfx = f.s;
+    ctx->yfx = f.y;
+    ctx->y2fx = f.y2;
     return DDH_OK;
 }
 
@@ -1522,7 +1529,7 @@ static void apply_op(ddh_ctx* ctx, const Work& w, const double2* z, double zsign
     ctx->launches += 2;
     coarse_solve(ctx, w.t, w.x2, w.ctmp, R, done);
     if (split) cudaStreamWaitEvent(s, ctx->ev_p1_join, 0);
-    if (ctx->edge_form && !phi_out) launch_pass2_edge<T>(d, eY, w.x2, w.xE, w.xE2, R, done, s);
+    if (ctx->edge_form && !phi_out) launch_pass2_edge<T>(d, std::is_same<T, double>::value ? ctx->y2fx : eY, w.x2, w.xE, w.xE2, R, done, s);
     else launch_pass2<T>(d, sinv, ctx->edge_form ? Y : nullptr, w.x2, w.xE, w.xE2, phi_out ? 1 : 0, bt, has_bI, phi_out, R, done, s,
                          fdm_cfg(ctx, std::is_same<T, double>::value, R, 2));
     ctx->launches++;
@@ -1549,8 +1556,7 @@ static void apply_prec(ddh_ctx* ctx, const Work& w, const double2* v, double2* z
         ctx->launches += 1;
         return;
     }
-    launch_pre<T>(d, v, w.vd, w.outE, w.mvec, z, 0, R, done, ctx->stream);
-    ctx->launches += 4;
+    ctx->launches += launch_pre<T>(d, v, w.vd, w.outE, w.mvec, z, R, done, ctx->stream);
 }
 
 // ---------------------------------------------------------------- Krylov state
@@ -2778,11 +2784,11 @@ ddh_status ddh_profile_op(ddh_ctx* ctx, int32_t R, int32_t precision, int32_t re
         });
         ms_out[1] = timeit([&] { launch_coarse_assemble<double>(d, w.tT, nullptr, z, 1.0, w.t, R, nullptr, s); });
         ms_out[3] = timeit([&] {
-            if (ef) launch_pass2_edge<double>(d, ctx->yfx, w.x2, w.xE, w.xE2, R, nullptr, s);
+            if (ef) launch_pass2_edge<double>(d, ctx->y2fx, w.x2, w.xE, w.xE2, R, nullptr, s);
             else launch_pass2<double>(d, sinv, nullptr, w.x2, w.xE, w.xE2, 0, nullptr, 0, nullptr, R, nullptr, s);
         });
         ms_out[4] = timeit([&] { launch_jump_gather<double>(d, w.xE2, w.x2, K.w, R, nullptr, s); });
-        ms_out[5] = timeit([&] { launch_pre<double>(d, K.vin, w.vd, w.outE, w.mvec, K.zw, 0, R, nullptr, s); });
+        ms_out[5] = timeit([&] { launch_pre<double>(d, K.vin, w.vd, w.outE, w.mvec, K.zw, R, nullptr, s); });
     } else {
         ms_out[0] = timeit([&] {
             if (ef && ctx->tc_W) launch_pass1_tc(d, ctx->tc_W, ctx->tc_off, ctx->tc_items, d.E, z, 1.0, w.xE, w.tT, R, nullptr, s,
@@ -2799,7 +2805,7 @@ ddh_status ddh_profile_op(ddh_ctx* ctx, int32_t R, int32_t precision, int32_t re
             else launch_pass2<float>(d, sinv, nullptr, w.x2, w.xE, w.xE2, 0, nullptr, 0, nullptr, R, nullptr, s);
         });
         ms_out[4] = timeit([&] { launch_jump_gather<float>(d, w.xE2, w.x2, K.w, R, nullptr, s); });
-        ms_out[5] = timeit([&] { launch_pre<float>(d, K.vin, w.vd, w.outE, w.mvec, K.zw, 0, R, nullptr, s); });
+        ms_out[5] = timeit([&] { launch_pre<float>(d, K.vin, w.vd, w.outE, w.mvec, K.zw, R, nullptr, s); });
     }
     // the coarse solve as the solves run it: the complex64 copy (refined) for mixed precision
     // with coarse_fp32, else FP64

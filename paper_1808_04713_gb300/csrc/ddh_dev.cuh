@@ -29,6 +29,7 @@ template <class T> __device__ __forceinline__ void fma_r(cpx<T>& a, T s, cpx<T> 
 struct DevModel {
     int E = 0, l = 0, pmax = 0;
     int maxE1 = 0;                      // largest number of type-1 edge slots of an element
+    int maxY = 0;                       // largest nE1 nT of an element
     int maxNo = 0;                      // largest nE1 + nT of an element (edge-pass output rows)
     int* err = nullptr;                 // device error word (0 = ok), read by the host after solves
     int64_t n_local = 0;
@@ -76,6 +77,7 @@ struct DevModel {
     const int64_t* pre_ex_off = nullptr;
     const int* sinv_ex = nullptr;
     const int* y_ex = nullptr;
+    const int* y2_ex = nullptr;         // row exponents of the column-major copy of Y (by type-1 slot)
     // E1 slots
     const int* e1_slot = nullptr;
     const int* e1_row = nullptr;
@@ -106,6 +108,7 @@ struct DevModel {
     const int* c2t_ptr = nullptr;       // C2^T: CSR by coarse dof over (row, weight)
     const int* c2t_row = nullptr;
     const double* c2t_w = nullptr;
+    int n_hb = 0;                       // hanging row blocks (0: conforming mesh, D diagonal)
     const int* hb_row0 = nullptr;
     const int* hb_n = nullptr;
     const int64_t* hb_off = nullptr;

@@ -19,32 +19,57 @@ namespace ddh {
 //
 // The FP64 passes hold S_E^-1 and Y in fixed point (ddh_fixed.cuh): EdgeOp<double> is four limbs per
 // entry.  S_E^-1 has an exponent per row (DevModel::sinv_ex, by type-1 slot), Y one per column (y_ex, by
-// type-2 slot), i.e. per output row of pass 1; pass 2, which sums over the columns, puts them on u_T
-// before it is staged.
+// type-2 slot), i.e. per output row of pass 1.  Pass 2, which sums over the columns, reads a copy of Y
+// that is column-major, so that a warp's load is contiguous over the rows, with the columns' scalings
+// taken out (they go on u_T) and an exponent per row (y2_ex, by type-1 slot): 64 x 64 elements, p = 20, 8
+// right-hand sides 174 us for pass 2, from 184 us with rows of Y read as they lie.
 template <class T> struct EdgeOpT { using type = cpx<float>; };
 template <> struct EdgeOpT<double> { using type = int4; };
 template <class T> using EdgeOp = typename EdgeOpT<T>::type;
 
-// Fixed-point copies of S_E^-1 and Y: one CTA per element, one warp per row of S_E^-1 / column of Y
+// Fixed-point copies of S_E^-1 and Y: one CTA per element, one warp per row of S_E^-1 / column of Y, then
+// one per row of Y for the copy that pass 2 reads
 __global__ void __launch_bounds__(256) k_fix_edge(DevModel dm, const double2* __restrict__ sinv,
-                                                  const double2* __restrict__ Y, int4* __restrict__ sfx,
-                                                  int* __restrict__ sex, int4* __restrict__ yfx, int* __restrict__ yex) {
+                                                  const double2* __restrict__ Y, EdgeFix f) {
     const int e = blockIdx.x, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31;
     const int nE = dm.nE1[e], nT = dm.nT[e];
+    __shared__ int cy[128];
     for (int o = warp; o < nE + nT; o += nw) {
         const bool isS = o < nE;
         const int ld = isS ? nE : nT;
         const int64_t at = isS ? dm.sinv_off[e] + o : dm.pq_off[e] + (o - nE);
         const double2* a = isS ? sinv : Y;
-        int4* f = isS ? sfx : yfx;
+        int4* d = isS ? f.s : f.y;
         unsigned m = 0;
         for (int j = lane; j < nE; j += 32) m = max(m, fx_mag(a[at + (int64_t)j * ld]));
         const int ef = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
         for (int j = lane; j < nE; j += 32) {
             const double2 v = a[at + (int64_t)j * ld];
-            f[at + (int64_t)j * ld] = fx_cpx(v.x, v.y, ef);
+            d[at + (int64_t)j * ld] = fx_cpx(v.x, v.y, ef);
         }
-        if (lane == 0) *(isS ? sex + dm.e1_off[e] + o : yex + dm.t_off[e] + o - nE) = ef;
+        if (lane == 0) {
+            *(isS ? f.sex + dm.e1_off[e] + o : f.yex + dm.t_off[e] + o - nE) = ef;
+            if (!isS) cy[o - nE] = fx_even(ef);
+        }
+    }
+    __syncthreads();
+    const double2* a = Y + dm.pq_off[e];
+    for (int i = warp; i < nE; i += nw) {
+        double2 v[4];
+        unsigned m = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {                      // nT <= 128
+            const int t = lane + 32 * k;
+            v[k] = t < nT ? a[(int64_t)i * nT + t] : make_double2(0.0, 0.0);
+            const int c = t < nT ? cy[t] : 0;
+            v[k] = make_double2(fx_scale(v[k].x, -c), fx_scale(v[k].y, -c));
+            m = max(m, fx_mag(v[k]));
+        }
+        const int ef = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (lane + 32 * k < nT) f.y2[dm.pq_off[e] + (int64_t)(lane + 32 * k) * nE + i] = fx_cpx(v[k].x, v[k].y, ef);
+        if (lane == 0) f.y2ex[dm.e1_off[e] + i] = ef;
     }
 }
 
@@ -136,7 +161,7 @@ __device__ __forceinline__ void edge_rows_f(const DevModel& dm, const cpx<T>* S,
 }
 
 // The same in fixed point.  Sums are exact, so the order of the columns and tpr do not matter.  Per term
-// twelve IMAD.WIDE (64 per SM and clock) stand for four FP64 FMA (two): 64 x 64 elements, p = 20, 8
+// twelve IMAD.WIDE (26 per SM and clock) stand for four FP64 FMA (two): 64 x 64 elements, p = 20, 8
 // right-hand sides went from 1.09 ms (92 % of the FP64 rate) to 0.42 ms.
 template <int RB>
 __device__ __forceinline__ void edge_rows_fx(const DevModel& dm, const int4* S, const int4* Ye, int nE, int nT,
@@ -333,16 +358,22 @@ template <class T, int RB>
 __global__ void __launch_bounds__(128) k_pass2_edge(DevModel dm, const EdgeOp<T>* __restrict__ Y,
                                                     const double2* __restrict__ x2, const cpx<T>* __restrict__ xE_in,
                                                     cpx<T>* __restrict__ xE_out, int R, const int* __restrict__ done,
-                                                    int ntask) {
+                                                    int ntask, int y_bytes) {
     if (done && *done) return;
     __shared__ EdgeOp<T> uT[RB * 128];
     __shared__ int ex[RB];
+    extern __shared__ __align__(128) char smem[];
     const CtaGroup g;
     const int task = blockIdx.x;
     if (task >= ntask) return;
     const int e = task % dm.E, r0 = (task / dm.E) * RB;
     const int cnt = min(RB, R - r0);
     const int nE = dm.nE1[e], e1o = dm.e1_off[e], nT = dm.nT[e], to = dm.t_off[e];
+    // FP64: Y comes into shared memory (one bulk copy, in flight while u_T is gathered)
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
+    int4* Y_s = reinterpret_cast<int4*>(smem + 128);
+    const bool staged = y_bytes > 0 && nE > 0 && nT > 0;
+    if (staged && threadIdx.x == 0) bulk_load_start(bar, Y_s, Y + dm.pq_off[e], (uint32_t)(nE * nT * sizeof(int4)));
     edge_stage<T>([&](int q, int i) {
         const int r = r0 + q;
         cpx<T> u = mk<T>(0, 0);
@@ -353,18 +384,23 @@ __global__ void __launch_bounds__(128) k_pass2_edge(DevModel dm, const EdgeOp<T>
             u.y += w * (T)xv.y;
         }
         if constexpr (std::is_same<T, double>::value) {
-            // the column's exponent: Y_t u_t = (Y_t 2^(1023 - y_ex)) (u_t 2^(y_ex - 1023))
-            const int c = dm.y_ex[to + i] - 1023;
+            // the column's scaling: Y_t u_t = (Y_t 2^-c) (u_t 2^c)
+            const int c = fx_even(dm.y_ex[to + i]);
             u.x = fx_scale(u.x, c);
             u.y = fx_scale(u.y, c);
         }
         return u;
     }, nT, 128, cnt, uT, ex);
     g.sync();
+    if (staged && !bulk_wait_all(bar, dm.err)) return;
     // one thread per row i of Y, all RB right-hand sides at once: each Y entry is read once
     const EdgeOp<T>* Ye = Y + dm.pq_off[e];
+    if constexpr (std::is_same<T, double>::value)
+        if (staged) Ye = Y_s;
     for (int i = g.t(); i < nE; i += g.n()) {
-        const EdgeOp<T>* yr = Ye + (int64_t)i * nT;
+        // FP64: the column-major copy
+        constexpr bool fx = std::is_same<T, double>::value;
+        const EdgeOp<T>* yr = fx ? Ye + i : Ye + (int64_t)i * nT;
         cpx<T> a[RB];
         if constexpr (std::is_same<T, double>::value) {
             FxAcc s[2 * RB];
@@ -376,7 +412,7 @@ __global__ void __launch_bounds__(128) k_pass2_edge(DevModel dm, const EdgeOp<T>
                 const int end = min(nT, t + kFxChain);
 #pragma unroll(RB <= 2 ? 8 : 2)
                 for (; t < end; ++t) {
-                    const int4 y = yr[t];
+                    const int4 y = yr[t * nE];
 #pragma unroll
                     for (int q = 0; q < RB; ++q)
                         if (q < cnt) fx_cmac(s[2 * q], s[2 * q + 1], y, -y.z, -y.w, uT[q * 128 + t]);
@@ -386,7 +422,10 @@ __global__ void __launch_bounds__(128) k_pass2_edge(DevModel dm, const EdgeOp<T>
             }
 #pragma unroll
             for (int q = 0; q < RB; ++q)
-                if (q < cnt) a[q] = mk<T>(fx_value(h[2 * q], l[2 * q], 1023, ex[q]), fx_value(h[2 * q + 1], l[2 * q + 1], 1023, ex[q]));
+                if (q < cnt) {
+                    const int ea = dm.y2_ex[e1o + i];
+                    a[q] = mk<T>(fx_value(h[2 * q], l[2 * q], ea, ex[q]), fx_value(h[2 * q + 1], l[2 * q + 1], ea, ex[q]));
+                }
         } else {
 #pragma unroll
             for (int q = 0; q < RB; ++q) a[q] = mk<T>(0, 0);
@@ -588,7 +627,7 @@ __global__ void k_fix_pre(const double* __restrict__ S, const int64_t* __restric
 
 template <class T, int RB>
 __global__ void __launch_bounds__(128) k_pre_elem(DevModel dm, const double2* __restrict__ v, cpx<T>* __restrict__ outE,
-                                                  int R, const int* __restrict__ done) {
+                                                  int R, const int* __restrict__ done, int with_d) {
     if (done && *done) return;
     extern __shared__ __align__(128) char smem[];
     __shared__ int ex[RB];
@@ -601,7 +640,12 @@ __global__ void __launch_bounds__(128) k_pre_elem(DevModel dm, const double2* __
         cpx<T> val = mk<T>(0, 0);
         if (row >= 0) {
             const double w = dm.e1_win ? dm.e1_sign[e1o + i] * dm.e1_win[e1o + i] : dm.e1_sign[e1o + i];
-            val = (T)w * ld<T>(v, (int64_t)(r0 + q) * dm.n_dual + row);
+            double2 x = v[(int64_t)(r0 + q) * dm.n_dual + row];
+            if (with_d) {
+                const double dd = dm.row_dinv ? dm.row_dinv[row] : 0.5;
+                x = make_double2(dd * x.x, dd * x.y);
+            }
+            val = (T)w * mk<T>((T)x.x, (T)x.y);
         }
         return val;
     }, nE, nE, cnt, in, ex);
@@ -661,7 +705,7 @@ __global__ void k_pre_rows_kry(DevModel dm, KrylovDev K, const cpx<T>* __restric
 // m[row] = outE[c] - outE[f] + (C2 K^Lap C2^T v)[row]
 template <class T>
 __global__ void k_pre_rows(DevModel dm, const cpx<T>* __restrict__ outE, const double2* __restrict__ v,
-                           double2* __restrict__ m, int lumped, const int* __restrict__ done) {
+                           double2* __restrict__ m, int with_d, const int* __restrict__ done) {
     if (done && *done) return;
     const int row = blockIdx.x * blockDim.x + threadIdx.x;
     const int r = blockIdx.y;
@@ -670,7 +714,11 @@ __global__ void k_pre_rows(DevModel dm, const cpx<T>* __restrict__ outE, const d
     const int c = dm.row_c[row], f = dm.row_f[row];
     if (c >= 0) { const cpx<T> a = outE[(int64_t)r * dm.nE1_tot + c]; sx += (double)a.x; sy += (double)a.y; }
     if (f >= 0) { const cpx<T> a = outE[(int64_t)r * dm.nE1_tot + f]; sx -= (double)a.x; sy -= (double)a.y; }
-    if (!lumped)
+    if (with_d) {
+        const double dd = dm.row_dinv ? dm.row_dinv[row] : 0.5;
+        sx *= dd;
+        sy *= dd;
+    } else
         for (int a = dm.mh_ptr[row]; a < dm.mh_ptr[row + 1]; ++a) {
             const double2 vv = v[(int64_t)r * dm.n_dual + dm.mh_col[a]];
             sx += dm.mh_val[a] * vv.x;
@@ -754,11 +802,13 @@ void launch_pass2_edge(const DevModel& dm, const void* Y, const double2* x2, con
     // one thread per edge row: 64-thread CTAs when every element has at most 64 (more CTAs
     // resident per SM to hide the gather latency)
     const int nt = dm.maxE1 <= 64 ? 64 : 128;
+    // FP64: room for the largest Y (nE + nT <= 124 at p = 32, so at most 62 x 62 entries)
+    const int yb = std::is_same<T, double>::value && dm.maxY > 0 && dm.maxY <= 64 * 64 ? 128 + dm.maxY * (int)sizeof(int4) : 0;
     switch (rb) {
-        case 8: k_pass2_edge<T, 8><<<ntask, nt, 0, st>>>(dm, Yp, x2, xi, xo, R, done, ntask); break;
-        case 4: k_pass2_edge<T, 4><<<ntask, nt, 0, st>>>(dm, Yp, x2, xi, xo, R, done, ntask); break;
-        case 2: k_pass2_edge<T, 2><<<ntask, nt, 0, st>>>(dm, Yp, x2, xi, xo, R, done, ntask); break;
-        default: k_pass2_edge<T, 1><<<ntask, nt, 0, st>>>(dm, Yp, x2, xi, xo, R, done, ntask);
+        case 8: k_pass2_edge<T, 8><<<ntask, nt, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb); break;
+        case 4: k_pass2_edge<T, 4><<<ntask, nt, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb); break;
+        case 2: k_pass2_edge<T, 2><<<ntask, nt, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb); break;
+        default: k_pass2_edge<T, 1><<<ntask, nt, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb);
     }
 }
 template void launch_pass1_edge<double>(const DevModel&, const void*, const void*, const double2*, double, const double2*, void*, void*, int, const int*, cudaStream_t, const EdgeSched*, int, int, int, int);
@@ -776,32 +826,36 @@ void launch_jump_gather(const DevModel& dm, const void* xE, const double2* x2, d
     k_jump_gather<T><<<dim3((dm.n_dual + 127) / 128, R), 128, 0, st>>>(dm, (const cpx<T>*)xE, x2, w, done);
 }
 template <class T>
-void launch_pre(const DevModel& dm, const double2* v, double2* vd, void* outE, double2* m, double2* z, int lumped,
-                int R, const int* done, cudaStream_t st) {
+int launch_pre(const DevModel& dm, const double2* v, double2* vd, void* outE, double2* m, double2* z,
+               int R, const int* done, cudaStream_t st) {
     const dim3 gr((dm.n_dual + 127) / 128, R);
-    k_dinv<<<gr, 128, 0, st>>>(dm, v, vd, lumped, done);
+    // without hanging rows D is diagonal and there is no C2 K C2^T: D^-1 goes into the two kernels (64 x 64
+    // elements, p = 20, 8 right-hand sides: 261 -> 249 us for an application)
+    const int with_d = dm.n_hb == 0;
+    if (!with_d) k_dinv<<<gr, 128, 0, st>>>(dm, v, vd, 0, done);
+    const double2* in = with_d ? v : vd;
     const int rb = rhs_block(R);
     const dim3 g(dm.E, (R + rb - 1) / rb);
     const size_t sm = sizeof(cpx<T>) * (size_t)rb * dm.maxE1 + 16;
     switch (rb) {
-        case 8: k_pre_elem<T, 8><<<g, 128, sm, st>>>(dm, vd, (cpx<T>*)outE, R, done); break;
-        case 4: k_pre_elem<T, 4><<<g, 128, sm, st>>>(dm, vd, (cpx<T>*)outE, R, done); break;
-        case 2: k_pre_elem<T, 2><<<g, 128, sm, st>>>(dm, vd, (cpx<T>*)outE, R, done); break;
-        default: k_pre_elem<T, 1><<<g, 128, sm, st>>>(dm, vd, (cpx<T>*)outE, R, done);
+        case 8: k_pre_elem<T, 8><<<g, 128, sm, st>>>(dm, in, (cpx<T>*)outE, R, done, with_d); break;
+        case 4: k_pre_elem<T, 4><<<g, 128, sm, st>>>(dm, in, (cpx<T>*)outE, R, done, with_d); break;
+        case 2: k_pre_elem<T, 2><<<g, 128, sm, st>>>(dm, in, (cpx<T>*)outE, R, done, with_d); break;
+        default: k_pre_elem<T, 1><<<g, 128, sm, st>>>(dm, in, (cpx<T>*)outE, R, done, with_d);
     }
-    k_pre_rows<T><<<gr, 128, 0, st>>>(dm, (const cpx<T>*)outE, vd, m, lumped, done);
-    k_dinv<<<gr, 128, 0, st>>>(dm, m, z, lumped, done);
+    k_pre_rows<T><<<gr, 128, 0, st>>>(dm, (const cpx<T>*)outE, in, with_d ? z : m, with_d, done);
+    if (!with_d) k_dinv<<<gr, 128, 0, st>>>(dm, m, z, 0, done);
+    return with_d ? 2 : 4;
 }
 
 template void launch_coarse_assemble<double>(const DevModel&, const void*, const double2*, const double2*, double, double2*, int, const int*, cudaStream_t);
 template void launch_coarse_assemble<float>(const DevModel&, const void*, const double2*, const double2*, double, double2*, int, const int*, cudaStream_t);
 template void launch_jump_gather<double>(const DevModel&, const void*, const double2*, double2*, int, const int*, cudaStream_t);
 template void launch_jump_gather<float>(const DevModel&, const void*, const double2*, double2*, int, const int*, cudaStream_t);
-template void launch_pre<double>(const DevModel&, const double2*, double2*, void*, double2*, double2*, int, int, const int*, cudaStream_t);
-template void launch_pre<float>(const DevModel&, const double2*, double2*, void*, double2*, double2*, int, int, const int*, cudaStream_t);
-void launch_fix_edge(const DevModel& dm, const void* sinv, const void* Y, void* sfx, int* sex, void* yfx, int* yex,
-                     cudaStream_t st) {
-    k_fix_edge<<<dm.E, 256, 0, st>>>(dm, (const double2*)sinv, (const double2*)Y, (int4*)sfx, sex, (int4*)yfx, yex);
+template int launch_pre<double>(const DevModel&, const double2*, double2*, void*, double2*, double2*, int, const int*, cudaStream_t);
+template int launch_pre<float>(const DevModel&, const double2*, double2*, void*, double2*, double2*, int, const int*, cudaStream_t);
+void launch_fix_edge(const DevModel& dm, const void* sinv, const void* Y, const EdgeFix& f, cudaStream_t st) {
+    k_fix_edge<<<dm.E, 256, 0, st>>>(dm, (const double2*)sinv, (const double2*)Y, f);
 }
 void launch_fix_pre(const double* S, int npat, const int64_t* off, const int* len, const int64_t* eoff, int2* fx, int* ex,
                     cudaStream_t st) {
@@ -834,6 +888,8 @@ static void set_edge_pass_limits(int maxE1) {
     // the whole unified L1/shared array as shared memory: the staged S_E^-1 limits residency
     cudaFuncSetAttribute(k_pass1_edge<T, RB>, cudaFuncAttributePreferredSharedMemoryCarveout,
                          (int)cudaSharedmemCarveoutMaxShared);
+    if (std::is_same<T, double>::value)
+        cudaFuncSetAttribute(k_pass2_edge<T, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 + 64 * 64 * (int)sizeof(int4));
     int buf = 0;
     size_t tot = 0;
     edge_p_layout<T>(RB, maxE1, &buf, &tot);

@@ -54,10 +54,17 @@ void launch_pass1_edge(const DevModel& dm, const void* sinv, const void* Y, cons
                        const double2* bt, void* xE, void* tT, int R, const int* done, cudaStream_t st,
                        const EdgeSched* es = nullptr, int item0 = 0, int nitems = -1, int tpr_force = 0,
                        int rows = 0);
-// in FP64 both take the operators in fixed point: launch_fix_edge makes sfx, yfx (four ints per entry)
-// and their exponents from the complex128 S_E^-1 and Y
-void launch_fix_edge(const DevModel& dm, const void* sinv, const void* Y, void* sfx, int* sex, void* yfx, int* yex,
-                     cudaStream_t st);
+// in FP64 both take the operators in fixed point (pass 1: s, y; pass 2: y2), which launch_fix_edge makes
+// from the complex128 S_E^-1 and Y: four ints per entry, exponents by type-1 / type-2 slot
+struct EdgeFix {
+    int4* s = nullptr;
+    int* sex = nullptr;
+    int4* y = nullptr;
+    int* yex = nullptr;
+    int4* y2 = nullptr;
+    int* y2ex = nullptr;
+};
+void launch_fix_edge(const DevModel& dm, const void* sinv, const void* Y, const EdgeFix& f, cudaStream_t st);
 // the same for npat restricted S^Lap (real, two ints per entry): pattern k is len[k]^2 entries at off[k],
 // its exponents at eoff[k]
 void launch_fix_pre(const double* S, int npat, const int64_t* off, const int* len, const int64_t* eoff, int2* fx, int* ex,
@@ -81,9 +88,10 @@ int fdm_qb_max(int pmax, int rb, bool fp64);
 template <class T>
 void launch_jump_gather(const DevModel& dm, const void* xE, const double2* x2, double2* w, int R, const int* done,
                         cudaStream_t st);
+// z = P^-1 v; returns the number of launches
 template <class T>
-void launch_pre(const DevModel& dm, const double2* v, double2* vd, void* outE, double2* m, double2* z, int lumped,
-                int R, const int* done, cudaStream_t st);
+int launch_pre(const DevModel& dm, const double2* v, double2* vd, void* outE, double2* m, double2* z,
+               int R, const int* done, cudaStream_t st);
 
 // Nested-dissection factor of the coarse matrix on the device (elimination order).  Per
 // node: fully summed positions [f0, f0+nF), boundary positions bidx[b_off .. b_off+nB),
