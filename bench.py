@@ -44,12 +44,14 @@ UNIT = "solves/s"
 WORKLOAD = "random_eps_64"
 TOL = 1e-10
 CPU_SAMPLE_BLOCK = 16           # the oracle times the 16 x 16-element corner of the workload
-# FP64 peak derived from unit counts and clocks: 152 SMs x 2 FP64 FMA per SM per clock x 2 FLOP
-# x 2.07 GHz = 1.26 TFLOP/s (the nominal 1.25; cuBLAS DGEMM measured 1.10 on this GPU)
-FP64_PEAK_TFLOPS = 1.25
+# The FP64-accurate dense products run in fixed point on the integer pipe: 2.3 complex multiply-adds (twelve
+# 32 x 32 + 64 bit multiply-adds each, timed) per SM and clock x 8 FLOP x 152 SMs x 2.07 GHz.  The FP64 pipe
+# (2 FMA per SM and clock) would give 1.25 TFLOP/s.
+FIXED_PEAK_TFLOPS = 5.8
 FP32_PEAK_TFLOPS = 70.0         # FP32 SIMT FMA throughput timed on this GPU
-# DRAM bytes of one coarse solve of the headline workload (8 RHS in two chains of 4) from an ncu
-# capture of its 52 level launches (cold cache per launch; profiles/nd_coarse_random_eps_64.md)
+# DRAM bytes of one coarse solve of the headline workload (8 RHS in two chains of 4) from an ncu capture
+# with one launch per tree level (cold cache per launch; profiles/nd_coarse_random_eps_64.md); the lower
+# levels have since become one launch per direction, which reads the same factor
 ND_TRAFFIC_BYTES_2CHAINS = 290.1e6
 
 
@@ -197,14 +199,14 @@ def roofline(comp_ms, info, R: int, p: int, fp64_elements: bool, coarse_name: st
     fl = work[dom]
     t = comp_ms[dom] * 1e-3
     fp64 = dom == 2 or fp64_elements
-    peak = FP64_PEAK_TFLOPS if fp64 else FP32_PEAK_TFLOPS
+    peak = FIXED_PEAK_TFLOPS if fp64 else FP32_PEAK_TFLOPS
     names = {0: "pass 1 (k_pass1_edge: [S_E^-1; Y^T] r_E)", 2: coarse_name,
              3: "pass 2 (k_pass2_edge: x_E - Y u_T)", 5: "preconditioner (k_pre_elem_kry + k_pre_rows_kry)"}
     achieved = fl / t / 1e12
     return {"kernel": names[dom], "bound": "alu", "achieved": round(achieved, 4), "peak": peak, "unit": "TFLOP/s",
             "frac": round(achieved / peak, 4), "traffic": None, "flops_per_launch": fl,
-            "peak_source": ("FP64 1.25 TFLOP/s derived from 152 SMs x 2 FP64 FMA/clk x 2.07 GHz "
-                            "(cuBLAS DGEMM measured 1.10)") if fp64 else "FP32 SIMT 70 TFLOP/s timed on this GPU",
+            "peak_source": ("fixed point 5.8 TFLOP/s: 152 SMs x 2.3 complex multiply-adds/clk (timed) x 8 FLOP "
+                            "x 2.07 GHz; the FP64 pipe's peak is 1.25") if fp64 else "FP32 SIMT 70 TFLOP/s timed on this GPU",
             "component_ms": {k: round(float(v), 5) for k, v in zip(COMPONENTS, comp_ms)}}
 
 
@@ -543,11 +545,11 @@ def run_ours(args):
         _, s2, b2, u2, c2 = _form("plane_16x16", ddh.PREC_FP64, local, stream, flush, 3, max(3, args.steps))
         i2 = s2.info()
         comp2 = s2.profile_op(1, ddh.PREC_FP64, reps=20)
-        c2["roofline"] = roofline(comp2, i2, 1, 16, True, "coarse solve (dense K^-1 GEMV, FP64)")
+        c2["roofline"] = roofline(comp2, i2, 1, 16, True, "coarse solve (dense K^-1 GEMV, fixed point)")
         # the same coarse solve measured against the nested-dissection factor's work (the
         # method's own coarse cost): what the dense GEMV delivers per unit of necessary work
         c2["roofline"]["coarse_frac_of_nd_work"] = round(i2.coarse_nd_flops / (comp2[2] * 1e-3) / 1e12
-                                                          / FP64_PEAK_TFLOPS, 4)
+                                                          / FIXED_PEAK_TFLOPS, 4)
         c2["roofline"]["coarse_nd_flops"] = i2.coarse_nd_flops
         s2.close()
         del b2, u2
