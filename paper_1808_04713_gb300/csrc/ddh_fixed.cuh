@@ -125,18 +125,7 @@ __device__ __forceinline__ void fx_exact(const FxAcc& s, long long ll, double& h
 }
 __device__ __forceinline__ int fx_exact_exp(int ea, int ex) { return 2 * kFxLow + ea + ex - 2044 - 2 * kFxBits; }
 
-// Stage one complex vector of length n per call of a warp, in place: lane's entries s[i] (i = lane,
-// lane + 32, ...) were written by this lane as FP64 and m is the largest |hi word| it saw; turns them
-// into limbs and returns the shared exponent field.
-__device__ __forceinline__ int fx_stage_warp(double2* s, int n, unsigned m) {
-    m = __reduce_max_sync(0xffffffffu, m);
-    const int ef = (int)(m >> 20);
-    for (int i = threadIdx.x & 31; i < n; i += 32) {
-        const double2 v = s[i];
-        reinterpret_cast<int4*>(s)[i] = fx_cpx(v.x, v.y, ef);
-    }
-    return ef;
-}
+// the larger |hi word| of a complex number: its exponent field above bit 20
 __device__ __forceinline__ unsigned fx_mag(const double2& v) {
     const unsigned a = (unsigned)__double2hiint(v.x) & 0x7fffffffu, b = (unsigned)__double2hiint(v.y) & 0x7fffffffu;
     return a > b ? a : b;

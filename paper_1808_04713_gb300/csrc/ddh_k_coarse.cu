@@ -247,10 +247,9 @@ __device__ __forceinline__ T warp_sum_transpose(T (&v)[V]) {
 // threads takes rows of one node's matrix for a block of RB right-hand sides after staging
 // the node's input vector in shared memory ([RB][stride], odd stride against bank
 // conflicts).  Long rows: up to 4 rows per item, one warp per row, lanes across the row.
-// Short rows (column-major matrix): up to 16 rows per item; a warp takes 4 rows at a time,
-// each row's 8 lanes split into RB right-hand sides x 8/RB column slices, so every lane of
-// the (narrow) FP64 pipe does useful work whatever the block size, and small items spread a
-// level over all SMs (GB300 completes about one warp-wide FP64 FMA per SM every 16 cycles).
+// Short rows (column-major matrix): up to 16 rows per item, 32/S rows per warp at a time with S lanes
+// (column slices) each, and all right-hand sides of the block in a lane, so that an entry of the matrix
+// is loaded once; small items spread a level over all SMs.
 // Arithmetic follows the factor's storage type MT: fixed point (int4, FP64-accurate, see
 // ddh_fixed.cuh) for the complex128 factor, FP32 for its complex64 copy (vectors stay complex128 in
 // global memory and are converted when they are staged).
