@@ -100,7 +100,6 @@ cd elem_entry(const Model& m, const Elem& E, int a, int b, int c, int d, bool st
     const PTable& T = m.tabs[E.ptab];
     const int N = E.p + 1;
     const double Mac = T.Mt[(size_t)a * N + c], Mbd = T.Mt[(size_t)b * N + d];
-    if ((Mac == 0.0 && Kt(a, c) == 0.0) || (Mbd == 0.0 && Kt(b, d) == 0.0)) return 0.0;   // every term below
     cd v = Kt(a, c) * Mbd + Mac * Kt(b, d);
     if (stiff_only) return v;
     if (E.pml) v = E.pa * (Kt(a, c) * Mbd) + E.pb * (Mac * Kt(b, d)) + E.pc * (Mac * Mbd);
@@ -112,55 +111,40 @@ cd elem_entry(const Model& m, const Elem& E, int a, int b, int c, int d, bool st
     return E.rho * v;
 }
 
-// c += a b and c -= a b over rows of complex numbers, in real arithmetic: std::complex products test every
-// result for NaN, which keeps the compiler from vectorising the loops that the factorisation spends its
-// time in (24 x 24 elements, p = 16, one thread: the element factors 530 ms, with the in-place inverse and
-// the skipped zeros below 217 ms).
-static inline void row_axpy(cd* __restrict__ c_, cd a, const cd* __restrict__ b_, int n) {
-    double* __restrict__ c = reinterpret_cast<double*>(c_);
-    const double* __restrict__ b = reinterpret_cast<const double*>(b_);
-    const double ar = a.real(), ai = a.imag();
-    for (int j = 0; j < n; ++j) {
-        const double br = b[2 * j], bi = b[2 * j + 1];
-        c[2 * j] += ar * br - ai * bi;
-        c[2 * j + 1] += ar * bi + ai * br;
-    }
-}
-
-// Complex Gauss-Jordan inverse with partial pivoting (row-major), in place: column c of the inverse takes
-// the place of column c of A as that is eliminated.  For n >= 128 the row eliminations of each pivot step
-// run on the pool.
+// Complex Gauss-Jordan inverse with partial pivoting on the augmented system [A | I]
+// (row-major).  For n >= 128 the row eliminations of each pivot step run on the pool.
 static bool invert(int n, std::vector<cd> A, std::vector<cd>& inv, double& minpiv, int nthreads = 1) {
+    inv.assign((size_t)n * n, cd(0));
+    for (int i = 0; i < n; ++i) inv[(size_t)i * n + i] = 1.0;
     double scale = 0;
     for (auto& v : A) scale = std::max(scale, std::abs(v));
     minpiv = 1e300;
     const bool par = nthreads > 1 && n >= 128;
-    std::vector<int> from(n);                // column of the inverse held in column c
-    for (int c = 0; c < n; ++c) from[c] = c;
     for (int c = 0; c < n; ++c) {
         int piv = c;
-        double pv = std::abs(A[(size_t)c * n + c]);
-        for (int r = c + 1; r < n; ++r) {
-            const double v = std::abs(A[(size_t)r * n + c]);
-            if (v > pv) { piv = r; pv = v; }
-        }
+        for (int r = c + 1; r < n; ++r)
+            if (std::abs(A[(size_t)r * n + c]) > std::abs(A[(size_t)piv * n + c])) piv = r;
+        const double pv = std::abs(A[(size_t)piv * n + c]);
         minpiv = std::min(minpiv, pv / (scale > 0 ? scale : 1.0));
         if (pv == 0.0 || !std::isfinite(pv)) return false;
-        if (piv != c) {
-            std::swap_ranges(A.begin() + (size_t)c * n, A.begin() + (size_t)(c + 1) * n, A.begin() + (size_t)piv * n);
-            std::swap(from[c], from[piv]);
-        }
-        cd* ac = &A[(size_t)c * n];
-        const cd d = 1.0 / ac[c];
-        ac[c] = 1.0;
-        for (int j = 0; j < n; ++j) ac[j] *= d;
+        if (piv != c)
+            for (int j = 0; j < n; ++j) {
+                std::swap(A[(size_t)c * n + j], A[(size_t)piv * n + j]);
+                std::swap(inv[(size_t)c * n + j], inv[(size_t)piv * n + j]);
+            }
+        const cd d = 1.0 / A[(size_t)c * n + c];
+        for (int j = c; j < n; ++j) A[(size_t)c * n + j] *= d;
+        for (int j = 0; j < n; ++j) inv[(size_t)c * n + j] *= d;
         auto elim = [&](int r) {
             if (r == c) return;
-            cd* ar = &A[(size_t)r * n];
-            const cd f = ar[c];
+            const cd f = A[(size_t)r * n + c];
             if (f == cd(0)) return;
-            ar[c] = 0;
-            row_axpy(ar, -f, ac, n);
+            cd* ar = &A[(size_t)r * n];
+            const cd* ac = &A[(size_t)c * n];
+            cd* ir = &inv[(size_t)r * n];
+            const cd* ic = &inv[(size_t)c * n];
+            for (int j = c; j < n; ++j) ar[j] -= f * ac[j];
+            for (int j = 0; j < n; ++j) ir[j] -= f * ic[j];
         };
         if (par) {
             const int chunk = 16, nchunks = (n + chunk - 1) / chunk;
@@ -171,37 +155,11 @@ static bool invert(int n, std::vector<cd> A, std::vector<cd>& inv, double& minpi
             for (int r = 0; r < n; ++r) elim(r);
         }
     }
-    inv.resize((size_t)n * n);
-    for (int i = 0; i < n; ++i)
-        for (int c = 0; c < n; ++c) inv[(size_t)i * n + from[c]] = A[(size_t)i * n + c];
     return true;
 }
 
-// C (m x n) = A (m x k) * B (k x n), row-major, optionally C = C0 - A*B.  Zeros of A are skipped, and those
-// of B where at most a quarter of it is filled (the couplings between edges and cross).
+// C (m x n) = A (m x k) * B (k x n), row-major, optionally C = C0 - A*B
 static void gemm(int M, int K, int N, const cd* A, const cd* B, cd* C, bool subtract, int nthreads) {
-    if (nthreads == 1 && M >= 8) {
-        std::vector<int> at(K + 1), col;
-        const size_t most = (size_t)K * N / 4;
-        for (int kk = 0; kk < K && col.size() <= most; ++kk) {
-            for (int j = 0; j < N; ++j)
-                if (B[(size_t)kk * N + j] != cd(0)) col.push_back(j);
-            at[kk + 1] = (int)col.size();
-        }
-        if (col.size() <= most) {
-            for (int i = 0; i < M; ++i) {
-                cd* c = C + (size_t)i * N;
-                if (!subtract) std::fill(c, c + N, cd(0));
-                for (int kk = 0; kk < K; ++kk) {
-                    const cd av = subtract ? -A[(size_t)i * K + kk] : A[(size_t)i * K + kk];
-                    if (av == cd(0)) continue;
-                    for (int q = at[kk]; q < at[kk + 1]; ++q)
-                        row_axpy(c + col[q], av, B + (size_t)kk * N + col[q], 1);
-                }
-            }
-            return;
-        }
-    }
     parallel_for(M, nthreads, [&](int i) {
         cd* c = C + (size_t)i * N;
         if (!subtract) for (int j = 0; j < N; ++j) c[j] = 0;
@@ -209,7 +167,8 @@ static void gemm(int M, int K, int N, const cd* A, const cd* B, cd* C, bool subt
         for (int kk = 0; kk < K; ++kk) {
             const cd av = subtract ? -a[kk] : a[kk];
             if (av == cd(0)) continue;
-            row_axpy(c, av, B + (size_t)kk * N, N);
+            const cd* b = B + (size_t)kk * N;
+            for (int j = 0; j < N; ++j) c[j] += av * b[j];
         }
     });
 }
@@ -462,10 +421,10 @@ bool factor(Model& m, int nthreads, std::string& err) {
             yo += s2 + (s2 & 1);
         }
         m.pq.assign((size_t)yo + 2, cd(0));
-        parallel_for(E, nthreads, [&](int e) {
+        for (int e = 0; e < E; ++e) {
             std::copy(ef[e].Y.begin(), ef[e].Y.end(), m.pq.begin() + m.el[e].pq_off);
             std::vector<cd>().swap(ef[e].Y);
-        });
+        }
     }
     m.min_gap = 1e300;
     if (m.check_factor) {
@@ -498,29 +457,19 @@ bool factor(Model& m, int nthreads, std::string& err) {
             ef[e].Se.clear();
             ef[e].Se.shrink_to_fit();
         }
-        const int chunk = 64;
-        parallel_for((nc + chunk - 1) / chunk, nthreads, [&](int q) {
-            for (int g = q * chunk; g < std::min(nc, (q + 1) * chunk); ++g) {
-                auto& r = rows[g];
-                std::sort(r.begin(), r.end(), [](const auto& x, const auto& y) { return x.first < y.first; });
-                size_t n = 0;
-                for (size_t i = 0; i < r.size();) {
-                    cd v = 0;
-                    size_t j = i;
-                    for (; j < r.size() && r[j].first == r[i].first; ++j) v += r[j].second;
-                    r[n++] = {r[i].first, v};
-                    i = j;
-                }
-                r.resize(n);
-            }
-        });
-        for (int g = 0; g < nc; ++g) kn_ptr[g + 1] = kn_ptr[g] + (int32_t)rows[g].size();
-        kn_col.resize(kn_ptr[nc]);
-        kn_val.resize(kn_ptr[nc]);
         for (int g = 0; g < nc; ++g) {
-            int32_t at = kn_ptr[g];
-            for (const auto& e : rows[g]) { kn_col[at] = e.first; kn_val[at++] = e.second; }
-            std::vector<std::pair<int, cd>>().swap(rows[g]);
+            auto& r = rows[g];
+            std::sort(r.begin(), r.end(), [](const auto& x, const auto& y) { return x.first < y.first; });
+            for (size_t i = 0; i < r.size();) {
+                cd v = 0;
+                size_t j = i;
+                for (; j < r.size() && r[j].first == r[i].first; ++j) v += r[j].second;
+                kn_col.push_back(r[i].first);
+                kn_val.push_back(v);
+                i = j;
+            }
+            kn_ptr[g + 1] = (int32_t)kn_col.size();
+            std::vector<std::pair<int, cd>>().swap(r);
         }
     }
     if (!coarse_factor(m, kn_ptr, kn_col, kn_val, nthreads, err)) return false;
