@@ -2737,6 +2737,10 @@ ddh_status ddh_apply_dual_operator(ddh_ctx* ctx, int32_t which, const void* v_de
     if ((st = get_op_work(ctx, R, fp64, w))) return st;
     const double2* v = (const double2*)v_dev;
     double2* out = (double2*)out_dev;
+    // FP64: F as the solves apply it, with the refined coarse solve where the factor's self-check asks for
+    // one (products in fixed point lose more than FP64 sums on fronts close to singular)
+    ctx->refine_active = fp64;
+    struct Off { ddh_ctx* c; ~Off() { c->refine_active = false; } } off_guard{ctx};
     if (which == 0) {
         if (fp64) apply_op<double>(ctx, w, v, 1.0, nullptr, 0, out, nullptr, R, nullptr);
         else apply_op<float>(ctx, w, v, 1.0, nullptr, 0, out, nullptr, R, nullptr);
