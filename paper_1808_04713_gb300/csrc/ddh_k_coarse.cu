@@ -934,11 +934,11 @@ int nd_rhs_block(int smem_rows, int R) {
 }
 template <class MT, int RB>
 static void nd_attr() {
-    cudaFuncSetAttribute(k_nd_forward<MT, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
-    cudaFuncSetAttribute(k_nd_backward<MT, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
-    cudaFuncSetAttribute(k_nd_bottom<MT, RB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
-    cudaFuncSetAttribute(k_nd_bottom<MT, RB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
-    cudaFuncSetAttribute(k_nd_persistent<MT, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNDSmemMax);
+    raise_smem_limit(k_nd_forward<MT, RB>, kNDSmemMax);
+    raise_smem_limit(k_nd_backward<MT, RB>, kNDSmemMax);
+    raise_smem_limit(k_nd_bottom<MT, RB, true>, kNDSmemMax);
+    raise_smem_limit(k_nd_bottom<MT, RB, false>, kNDSmemMax);
+    raise_smem_limit(k_nd_persistent<MT, RB>, kNDSmemMax);
 }
 void nd_set_smem_limits() {
     nd_attr<int4, 1>(); nd_attr<int4, 2>(); nd_attr<int4, 4>(); nd_attr<int4, 8>();
@@ -1104,10 +1104,10 @@ void launch_gemv32(const void* A, int n, const double2* x, double2* y, int R, co
 static int gemv_rows(int n, int nsm) { return std::max(4, (n + nsm - 1) / nsm); }
 void gemv_set_smem_limits() {
     constexpr int most = 160 * 1024;          // eight staged tiles and the sums of the rows of n = 16384
-    cudaFuncSetAttribute(k_gemv_fx<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    cudaFuncSetAttribute(k_gemv_fx<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    cudaFuncSetAttribute(k_gemv_fx<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    cudaFuncSetAttribute(k_gemv_fx<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    raise_smem_limit(k_gemv_fx<1>, most);
+    raise_smem_limit(k_gemv_fx<2>, most);
+    raise_smem_limit(k_gemv_fx<4>, most);
+    raise_smem_limit(k_gemv_fx<8>, most);
 }
 void launch_gemv(const void* A, const int* ex, const int* col, int n, const double2* x, double2* y, int R, const int* done, int nsm,
                  cudaStream_t st) {

@@ -883,17 +883,16 @@ template void launch_pre_krylov<float>(const DevModel&, const KrylovDev&, void*,
 
 template <class T, int RB>
 static void set_edge_pass_limits(int maxE1) {
-    cudaFuncSetAttribute(k_pass1_edge<T, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)edge_smem_total<T>(RB, maxE1));
+    raise_smem_limit(k_pass1_edge<T, RB>, (int)edge_smem_total<T>(RB, maxE1));
     // the whole unified L1/shared array as shared memory: the staged S_E^-1 limits residency
     cudaFuncSetAttribute(k_pass1_edge<T, RB>, cudaFuncAttributePreferredSharedMemoryCarveout,
                          (int)cudaSharedmemCarveoutMaxShared);
     if (std::is_same<T, double>::value)
-        cudaFuncSetAttribute(k_pass2_edge<T, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 + 64 * 64 * (int)sizeof(int4));
+        raise_smem_limit(k_pass2_edge<T, RB>, 128 + 64 * 64 * (int)sizeof(int4));
     int buf = 0;
     size_t tot = 0;
     edge_p_layout<T>(RB, maxE1, &buf, &tot);
-    cudaFuncSetAttribute(k_pass1_edge_p<T, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tot);
+    raise_smem_limit(k_pass1_edge_p<T, RB>, (int)tot);
 }
 void set_edge_limits(int pmax, int maxE1) {
     (void)pmax;
@@ -903,22 +902,22 @@ void set_edge_limits(int pmax, int maxE1) {
     set_edge_pass_limits<float, 4>(maxE1); set_edge_pass_limits<float, 8>(maxE1);
     const int pre64 = (int)(sizeof(cpx<double>) * 8 * (size_t)maxE1 + sizeof(double) * (size_t)maxE1 * maxE1 + 16);
     const int pre32 = (int)(sizeof(cpx<float>) * 8 * (size_t)maxE1 + sizeof(float) * (size_t)maxE1 * maxE1 + 16);
-    cudaFuncSetAttribute(k_pre_elem<double, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre64);
-    cudaFuncSetAttribute(k_pre_elem<double, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre64);
-    cudaFuncSetAttribute(k_pre_elem<double, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre64);
-    cudaFuncSetAttribute(k_pre_elem<double, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre64);
-    cudaFuncSetAttribute(k_pre_elem<float, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre32);
-    cudaFuncSetAttribute(k_pre_elem<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre32);
-    cudaFuncSetAttribute(k_pre_elem<float, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre32);
-    cudaFuncSetAttribute(k_pre_elem<float, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre32);
-    cudaFuncSetAttribute(k_pre_elem_kry<double, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre64);
-    cudaFuncSetAttribute(k_pre_elem_kry<double, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre64);
-    cudaFuncSetAttribute(k_pre_elem_kry<double, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre64);
-    cudaFuncSetAttribute(k_pre_elem_kry<double, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre64);
-    cudaFuncSetAttribute(k_pre_elem_kry<float, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre32);
-    cudaFuncSetAttribute(k_pre_elem_kry<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre32);
-    cudaFuncSetAttribute(k_pre_elem_kry<float, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre32);
-    cudaFuncSetAttribute(k_pre_elem_kry<float, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, pre32);
+    raise_smem_limit(k_pre_elem<double, 1>, pre64);
+    raise_smem_limit(k_pre_elem<double, 2>, pre64);
+    raise_smem_limit(k_pre_elem<double, 4>, pre64);
+    raise_smem_limit(k_pre_elem<double, 8>, pre64);
+    raise_smem_limit(k_pre_elem<float, 1>, pre32);
+    raise_smem_limit(k_pre_elem<float, 2>, pre32);
+    raise_smem_limit(k_pre_elem<float, 4>, pre32);
+    raise_smem_limit(k_pre_elem<float, 8>, pre32);
+    raise_smem_limit(k_pre_elem_kry<double, 1>, pre64);
+    raise_smem_limit(k_pre_elem_kry<double, 2>, pre64);
+    raise_smem_limit(k_pre_elem_kry<double, 4>, pre64);
+    raise_smem_limit(k_pre_elem_kry<double, 8>, pre64);
+    raise_smem_limit(k_pre_elem_kry<float, 1>, pre32);
+    raise_smem_limit(k_pre_elem_kry<float, 2>, pre32);
+    raise_smem_limit(k_pre_elem_kry<float, 4>, pre32);
+    raise_smem_limit(k_pre_elem_kry<float, 8>, pre32);
 }
 
 }  // namespace ddh

@@ -514,19 +514,19 @@ template <class T>
 void set_pass1_limits(int pmax, int maxE1) {
     const int b1 = (int)pass_smem_max<T>(pmax, 1, maxE1), b2 = (int)pass_smem_max<T>(pmax, 2, maxE1);
     const int b4 = (int)pass_smem_max<T>(pmax, 4, maxE1), b8 = (int)pass_smem_max<T>(pmax, 8, maxE1);
-    cudaFuncSetAttribute(k_pass1<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b1);
-    cudaFuncSetAttribute(k_pass1<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, b2);
-    cudaFuncSetAttribute(k_pass1<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, b4);
-    cudaFuncSetAttribute(k_pass1<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, b8);
+    raise_smem_limit(k_pass1<T, 1>, b1);
+    raise_smem_limit(k_pass1<T, 2>, b2);
+    raise_smem_limit(k_pass1<T, 4>, b4);
+    raise_smem_limit(k_pass1<T, 8>, b8);
 }
 template <class T>
 void set_pass2_limits(int pmax, int maxE1) {
     const int b1 = (int)pass_smem_max<T>(pmax, 1, maxE1), b2 = (int)pass_smem_max<T>(pmax, 2, maxE1);
     const int b4 = (int)pass_smem_max<T>(pmax, 4, maxE1), b8 = (int)pass_smem_max<T>(pmax, 8, maxE1);
-    cudaFuncSetAttribute(k_pass2<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b1);
-    cudaFuncSetAttribute(k_pass2<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, b2);
-    cudaFuncSetAttribute(k_pass2<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, b4);
-    cudaFuncSetAttribute(k_pass2<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, b8);
+    raise_smem_limit(k_pass2<T, 1>, b1);
+    raise_smem_limit(k_pass2<T, 2>, b2);
+    raise_smem_limit(k_pass2<T, 4>, b4);
+    raise_smem_limit(k_pass2<T, 8>, b8);
 }
 
 }  // namespace ddh

@@ -565,10 +565,10 @@ void launch_pcg_d(double2* d, const double2* z, const double* sc, int64_t n, int
 }
 
 void set_krylov_limits() {
-    cudaFuncSetAttribute(k_cgs_first<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4096 * (int)sizeof(double2));
-    cudaFuncSetAttribute(k_cgs_second<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4096 * (int)sizeof(double2));
-    cudaFuncSetAttribute(k_cgs_first<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4096 * (int)sizeof(float2));
-    cudaFuncSetAttribute(k_cgs_second<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4096 * (int)sizeof(float2));
+    raise_smem_limit(k_cgs_first<double2>, 4096 * (int)sizeof(double2));
+    raise_smem_limit(k_cgs_second<double2>, 4096 * (int)sizeof(double2));
+    raise_smem_limit(k_cgs_first<float2>, 4096 * (int)sizeof(float2));
+    raise_smem_limit(k_cgs_second<float2>, 4096 * (int)sizeof(float2));
 }
 
 }  // namespace ddh

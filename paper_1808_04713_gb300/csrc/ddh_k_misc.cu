@@ -451,9 +451,8 @@ void launch_readback(const DevModel& dm, const double2* phi, double2* z, int R, 
 
 
 void set_misc_limits(int pmax) {
-    // for the largest degree: another context may need more than this one
-    cudaFuncSetAttribute(k_elem_matvec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)elem_matvec_smem(32));
-    cudaFuncSetAttribute(k_grad_elem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)elem_smem_bytes<double>(pmax, 0));
+    raise_smem_limit(k_elem_matvec, (int)elem_matvec_smem(pmax));
+    raise_smem_limit(k_grad_elem, (int)elem_smem_bytes<double>(pmax, 0));
 }
 
 size_t pass_smem(int pmax, bool fp64) {

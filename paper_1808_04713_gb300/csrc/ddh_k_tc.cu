@@ -274,9 +274,9 @@ void launch_pass1_tc(const DevModel& dm, const float* W, const int64_t* w_off, c
 void set_tc_limits(int maxE1, int maxT) {
     for (int R : {16, 32, 64}) {
         const int b = (int)tc_smem_bytes(maxE1, maxT, R, nullptr);
-        if (R == 16) cudaFuncSetAttribute(k_pass1_tc<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (R == 32) cudaFuncSetAttribute(k_pass1_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (R == 64) cudaFuncSetAttribute(k_pass1_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+        if (R == 16) raise_smem_limit(k_pass1_tc<16>, b);
+        if (R == 32) raise_smem_limit(k_pass1_tc<32>, b);
+        if (R == 64) raise_smem_limit(k_pass1_tc<64>, b);
     }
 }
 

@@ -4,6 +4,7 @@
 #include "ddh_kernels.cuh"
 #include "ddh_launch.hpp"
 #include <algorithm>
+#include <mutex>
 
 namespace ddh {
 
@@ -151,7 +152,17 @@ inline size_t edge_smem_total(int rb, int maxE1) {
     return (size_t)off + 128 + (((size_t)maxE1 * maxE1 * sizeof(cpx<T>) + 127) & ~(size_t)127);
 }
 
-// dynamic shared-memory limits of each unit's kernels (set once per device)
+// Lets launches of kernel k ask for `bytes` of dynamic shared memory.  The limit belongs to the kernel and the
+// device, not to a context, so it only ever grows: a context of low degree leaves a larger one what it needs.
+template <class K>
+inline void raise_smem_limit(K* k, int bytes) {
+    static std::mutex m;
+    std::lock_guard<std::mutex> lock(m);
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, k) == cudaSuccess && fa.maxDynamicSharedSizeBytes < bytes)
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+// dynamic shared-memory limits of each unit's kernels, raised to what a context of these sizes launches with
 template <class T> void set_pass1_limits(int pmax, int maxE1);   // ddh_k_fdm_pass1_*.cu
 template <class T> void set_pass2_limits(int pmax, int maxE1);   // ddh_k_fdm_pass2_*.cu
 void set_edge_limits(int pmax, int maxE1);
