@@ -125,9 +125,10 @@ struct ddh_ctx {
     KState kin, kout;
     // Poisson mode: extreme Ritz values of P^-1 F from the PCG coefficients of the last solve
     std::vector<double> pcg_lmin, pcg_lmax;
-    // captured PCG iterations per R (with their kernel counts), and the iterations of the last solve
+    // captured PCG iterations per R (with their kernel counts); their stop word on the host
     std::map<int, std::pair<cudaGraphExec_t, int64_t>> pcg_graphs;
-    int pcg_hint = 0;
+    int* pcg_its = nullptr;                        // pinned; written by the device (PcgBufs::host)
+    cudaEvent_t pcg_ev[2] = {nullptr, nullptr};
     // per-degree tables of the Dirichlet trace lifting (ddh_dirichlet_point_source)
     const int64_t* tr_off = nullptr;
     const int* tr_nq = nullptr;
@@ -196,7 +197,6 @@ static void drop_pcg_graphs(ddh_ctx* ctx) {
 static void free_model(ddh_ctx* ctx) {
     cudaStreamSynchronize(ctx->stream);
     drop_pcg_graphs(ctx);
-    ctx->pcg_hint = 0;
     for (void* p : ctx->model_allocs) cudaFree(p);
     ctx->model_allocs.clear();
     ctx->kin.release();
@@ -2081,12 +2081,16 @@ static ddh_status solve_pcg(ddh_ctx* ctx, const double2* b_dev, double2* u_dev, 
     if ((sts = get_work(ctx, "pcg_Fd", vb, &Fd))) return sts;
     if ((sts = get_work(ctx, "pcg_part", sizeof(double) * (size_t)R * kPcgBlocks, &part))) return sts;
     if ((sts = get_work(ctx, "pcg_sc", sizeof(double) * kPcgScalars * (size_t)R, &sc))) return sts;
-    if ((sts = get_work(ctx, "pcg_cnt", sizeof(int) * (size_t)R, &cnt))) return sts;
+    if ((sts = get_work(ctx, "pcg_cnt", sizeof(int) * (size_t)(R + 2), &cnt))) return sts;
     if ((sts = get_work(ctx, "pcg_ah", sizeof(double) * (size_t)R * maxit, &ah))) return sts;
     if ((sts = get_work(ctx, "pcg_bh", sizeof(double) * (size_t)R * maxit, &bh))) return sts;
     double2 *G = (double2*)g, *NU = (double2*)nu, *RV = (double2*)rv, *Z = (double2*)z, *D = (double2*)dv,
             *FD = (double2*)Fd;
-    const PcgBufs B{(double*)sc, (double*)part, (int*)cnt, (double*)ah, (double*)bh, maxit};
+    if (!ctx->pcg_its) {
+        CK(cudaMallocHost((void**)&ctx->pcg_its, sizeof(int)));
+        for (auto& e : ctx->pcg_ev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    }
+    const PcgBufs B{(double*)sc, (double*)part, (int*)cnt, (double*)ah, (double*)bh, ctx->pcg_its, maxit};
     double* SC = B.sc;
     const double tol2 = tol * tol;
     std::vector<int> its(R, 0);
@@ -2095,10 +2099,11 @@ static ddh_status solve_pcg(ddh_ctx* ctx, const double2* b_dev, double2* u_dev, 
     // g = C^ A^-1 b^ (interior loads included)
     apply_op<double>(ctx, w, nullptr, 0.0, (const double2*)bt, 1, G, nullptr, R, nullptr);
     CK(cudaMemsetAsync(SC, 0, sizeof(double) * kPcgScalars * (size_t)R, st));
-    CK(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)R, st));
+    CK(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)(R + 2), st));
     CK(cudaMemsetAsync(ah, 0, sizeof(double) * (size_t)R * maxit, st));
     CK(cudaMemsetAsync(bh, 0, sizeof(double) * (size_t)R * maxit, st));
-    int done_all = 0;
+    bool done_all = true;
+    *ctx->pcg_its = maxit + 1;                     // nothing of an earlier solve is in flight
     if (nd > 0) {
         CK(cudaMemsetAsync(NU, 0, vb, st));
         CK(cudaMemcpyAsync(RV, G, vb, cudaMemcpyDeviceToDevice, st));
@@ -2107,13 +2112,14 @@ static ddh_status solve_pcg(ddh_ctx* ctx, const double2* b_dev, double2* u_dev, 
         launch_pcg_dot(RV, Z, nd, B, 1, 0.0, R, st);
         CK(cudaMemcpyAsync(D, Z, vb, cudaMemcpyDeviceToDevice, st));
         ctx->launches += 2;
+        const int* stop = B.cnt + R + 1;
         auto body = [&] {
-            apply_op<double>(ctx, w, D, 1.0, nullptr, 0, FD, nullptr, R, nullptr);   // F d
+            apply_op<double>(ctx, w, D, 1.0, nullptr, 0, FD, nullptr, R, stop);   // F d
             launch_pcg_dot(D, FD, nd, B, 2, 0.0, R, st);
             launch_pcg_xr(NU, RV, D, FD, nd, B, R, st);
-            apply_prec<double>(ctx, w, RV, Z, R, nullptr);
+            apply_prec<double>(ctx, w, RV, Z, R, stop);
             launch_pcg_dot(RV, Z, nd, B, 4, 0.0, R, st);
-            launch_pcg_d(D, Z, SC, nd, R, st);
+            launch_pcg_d(D, Z, nd, B, R, st);
             ctx->launches += 4;
         };
         cudaGraphExec_t ge = nullptr;
@@ -2135,19 +2141,17 @@ static ddh_status solve_pcg(ddh_ctx* ctx, const double2* b_dev, double2* u_dev, 
             ge = it->second.first;
             per = it->second.second;
         }
-        // the flags are read after as many iterations as the previous solve took, then after each one
-        for (int it = 0; it < maxit && !done_all;) {
-            const int batch = std::min(it == 0 ? std::max(1, ctx->pcg_hint) : 1, maxit - it);
-            for (int k = 0; k < batch; ++k) {
-                if (ge) { CK(cudaGraphLaunch(ge, st)); ctx->launches += per; }
-                else body();
-            }
-            it += batch;
-            CK(cudaMemcpyAsync(hsc.data(), SC, sizeof(double) * hsc.size(), cudaMemcpyDeviceToHost, st));
-            CK(cudaStreamSynchronize(st));
-            done_all = 1;
-            for (int r = 0; r < R; ++r) done_all &= hsc[kPcgScalars * r + 4] != 0.0;
+        // an iteration's outcome is read while the next one runs: no gap between them on the device, and one
+        // iteration of kernels that return at once past convergence
+        for (int it = 0; it < maxit; ++it) {
+            if (ge) { CK(cudaGraphLaunch(ge, st)); ctx->launches += per; }
+            else body();
+            CK(cudaEventRecord(ctx->pcg_ev[it & 1], st));
+            if (it == 0) continue;
+            CK(cudaEventSynchronize(ctx->pcg_ev[(it - 1) & 1]));
+            if (*(volatile int*)ctx->pcg_its <= it) break;
         }
+        CK(cudaMemcpyAsync(hsc.data(), SC, sizeof(double) * hsc.size(), cudaMemcpyDeviceToHost, st));
         std::vector<double> ha((size_t)R * maxit), hb((size_t)R * maxit);
         CK(cudaMemcpyAsync(ha.data(), ah, sizeof(double) * ha.size(), cudaMemcpyDeviceToHost, st));
         CK(cudaMemcpyAsync(hb.data(), bh, sizeof(double) * hb.size(), cudaMemcpyDeviceToHost, st));
@@ -2156,19 +2160,18 @@ static ddh_status solve_pcg(ddh_ctx* ctx, const double2* b_dev, double2* u_dev, 
         ctx->pcg_lmax.assign(R, 0.0);
         for (int r = 0; r < R; ++r) {
             const bool dn = hsc[kPcgScalars * r + 4] != 0.0;
+            done_all = done_all && dn;
             its[r] = dn ? (int)hsc[kPcgScalars * r + 5] : maxit;
             res[r] = hsc[kPcgScalars * r + 3] > 0 ? std::sqrt(hsc[kPcgScalars * r + 6] / hsc[kPcgScalars * r + 3]) : 0.0;
             lanczos_extremes(ha.data() + (size_t)r * maxit, hb.data() + (size_t)r * maxit, its[r], ctx->pcg_lmin[r],
                              ctx->pcg_lmax[r]);
         }
-        ctx->pcg_hint = *std::max_element(its.begin(), its.end());
         // recovery: A^ phi = b^ - C^T nu
         apply_op<double>(ctx, w, NU, -1.0, (const double2*)bt, 1, nullptr, (double2*)phit, R, nullptr);
     } else {
         apply_op<double>(ctx, w, nullptr, 0.0, (const double2*)bt, 1, nullptr, (double2*)phit, R, nullptr);
         ctx->pcg_lmin.assign(R, 0.0);
         ctx->pcg_lmax.assign(R, 0.0);
-        done_all = 1;
     }
     launch_basis(d, (const double2*)phit, u_dev, 0, R, st);
     ctx->launches++;
@@ -2839,6 +2842,9 @@ void ddh_destroy(ddh_ctx* ctx) {
     cudaStreamDestroy(ctx->side_p1);
     cudaEventDestroy(ctx->ev_p1_fork);
     cudaEventDestroy(ctx->ev_p1_join);
+    for (auto& e : ctx->pcg_ev)
+        if (e) cudaEventDestroy(e);
+    if (ctx->pcg_its) cudaFreeHost(ctx->pcg_its);
     delete ctx;
 }
 

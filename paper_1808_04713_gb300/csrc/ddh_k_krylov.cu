@@ -424,7 +424,8 @@ __global__ void k_norm2_sum(const double* __restrict__ part, int nb, double* __r
 // to 64 partial sums per right-hand side; the CTA that finishes last adds them with one warp and
 // updates the scalars), so the iterates are the same on every run.  Nothing that the host would have
 // to supply changes from one iteration to the next, so an iteration is a graph that can be replayed
-// several times between two looks at the flags; iterations past convergence change nothing (alpha = 0).
+// while the host still waits for the flag of the one before; cnt[R + 1] is set when every right-hand side is
+// done and stops the kernels of a later iteration at their first line.
 
 // adds the partial sums of one dot product and updates the scalars of right-hand side r (one warp):
 //   mode 0: ||g||^2 (also ||r||^2; done when g = 0)   mode 1: rz = (r, z)
@@ -440,9 +441,17 @@ __device__ __forceinline__ void pcg_scalar(const PcgBufs& P, int r, int nb, int 
     if (lane) return;
     double* c = P.sc + kPcgScalars * r;
     const bool done = c[4] != 0.0;
-    const int it = (int)c[7];
+    const int it = (int)c[7], R = gridDim.y;
+    auto finish = [&](int its) {
+        c[4] = 1.0;
+        c[5] = its;
+        if (atomicAdd(P.cnt + R, 1) == R - 1) {
+            P.cnt[R + 1] = 1;
+            *P.host = its;               // the last right-hand side to finish took the most iterations
+        }
+    };
     switch (mode) {
-        case 0: c[3] = s; c[6] = s; c[7] = 0.0; c[8] = tol2; if (s == 0.0) { c[4] = 1.0; c[5] = 0.0; } break;
+        case 0: c[3] = s; c[6] = s; c[7] = 0.0; c[8] = tol2; if (s == 0.0) finish(0); break;
         case 1: c[0] = s; break;
         case 2:
             c[1] = (done || s == 0.0) ? 0.0 : c[0] / s;
@@ -450,7 +459,7 @@ __device__ __forceinline__ void pcg_scalar(const PcgBufs& P, int r, int nb, int 
             break;
         case 3:
             c[6] = s;
-            if (!done && s <= c[8] * c[3]) { c[4] = 1.0; c[5] = it + 1; }
+            if (!done && s <= c[8] * c[3]) finish(it + 1);
             break;
         default:
             c[2] = (done || c[0] == 0.0) ? 0.0 : s / c[0];
@@ -477,6 +486,7 @@ __device__ __forceinline__ void pcg_finish(const PcgBufs& P, double s, int mode,
 // Re(conj(a_r) . b_r), then the scalar update of `mode`
 __global__ void k_pcg_dot(const double2* __restrict__ a, const double2* __restrict__ b, int64_t n, PcgBufs P, int mode,
                           double tol2) {
+    if (mode > 1 && P.cnt[gridDim.y + 1]) return;
     const int r = blockIdx.y;
     double s = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -489,6 +499,7 @@ __global__ void k_pcg_dot(const double2* __restrict__ a, const double2* __restri
 // nu += alpha d, r -= alpha F d, ||r||^2 and its test (mode 3)
 __global__ void k_pcg_xr(double2* __restrict__ nu, double2* __restrict__ rv, const double2* __restrict__ d,
                          const double2* __restrict__ Fd, int64_t n, PcgBufs P) {
+    if (P.cnt[gridDim.y + 1]) return;
     const int r = blockIdx.y;
     const double al = P.sc[kPcgScalars * r + 1];
     double s = 0;
@@ -506,9 +517,10 @@ __global__ void k_pcg_xr(double2* __restrict__ nu, double2* __restrict__ rv, con
 }
 
 // d = z + beta d
-__global__ void k_pcg_d(double2* __restrict__ d, const double2* __restrict__ z, const double* __restrict__ sc, int64_t n) {
+__global__ void k_pcg_d(double2* __restrict__ d, const double2* __restrict__ z, int64_t n, PcgBufs P) {
+    if (P.cnt[gridDim.y + 1]) return;
     const int r = blockIdx.y;
-    const double be = sc[kPcgScalars * r + 2];
+    const double be = P.sc[kPcgScalars * r + 2];
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t q = (int64_t)r * n + i;
         const double2 zv = z[q], dv = d[q];
@@ -560,8 +572,8 @@ void launch_pcg_xr(double2* nu, double2* r, const double2* d, const double2* Fd,
                    cudaStream_t st) {
     k_pcg_xr<<<pcg_grid(n, R), 256, 0, st>>>(nu, r, d, Fd, n, B);
 }
-void launch_pcg_d(double2* d, const double2* z, const double* sc, int64_t n, int R, cudaStream_t st) {
-    k_pcg_d<<<pcg_grid(n, R), 256, 0, st>>>(d, z, sc, n);
+void launch_pcg_d(double2* d, const double2* z, int64_t n, const PcgBufs& B, int R, cudaStream_t st) {
+    k_pcg_d<<<pcg_grid(n, R), 256, 0, st>>>(d, z, n, B);
 }
 
 void set_krylov_limits() {

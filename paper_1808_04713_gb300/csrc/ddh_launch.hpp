@@ -244,8 +244,9 @@ void launch_scale_f32(const double2* x, double a, float2* out, int64_t n, cudaSt
 // out[r] = ||x_r||^2 (deterministic; part: R x 64 doubles of scratch)
 void launch_norm2(const double2* x, int64_t n, double* out, double* part, int R, cudaStream_t st);
 // PCG of the Poisson mode: dot products with their scalar update (modes of pcg_scalar; mode 0 takes
-// tol^2), nu/r update with ||r||^2 and the stopping test, and d = z + beta d.  part: R x kPcgBlocks, cnt: R
-// zeros, ah / bh: R x maxit
+// tol^2), nu/r update with ||r||^2 and the stopping test, and d = z + beta d.  part: R x kPcgBlocks, ah / bh:
+// R x maxit, cnt: R + 2 zeros (CTAs finished per right-hand side, right-hand sides done, all of them done);
+// *host, in pinned memory, becomes the number of iterations once all are done
 constexpr int kPcgBlocks = 64, kPcgScalars = 9;
 struct PcgBufs {
     double* sc;
@@ -253,13 +254,14 @@ struct PcgBufs {
     int* cnt;
     double* ah;
     double* bh;
+    int* host;
     int maxit;
 };
 void launch_pcg_dot(const double2* a, const double2* b, int64_t n, const PcgBufs& B, int mode, double tol2, int R,
                     cudaStream_t st);
 void launch_pcg_xr(double2* nu, double2* r, const double2* d, const double2* Fd, int64_t n, const PcgBufs& B, int R,
                    cudaStream_t st);
-void launch_pcg_d(double2* d, const double2* z, const double* sc, int64_t n, int R, cudaStream_t st);
+void launch_pcg_d(double2* d, const double2* z, int64_t n, const PcgBufs& B, int R, cudaStream_t st);
 void launch_conf_scatter(const DevModel& dm, const double2* x, double2* out, int R, cudaStream_t st);
 void launch_conf_gather_vec(const DevModel& dm, const double2* x, double2* out, double sign, int R, cudaStream_t st);
 void launch_inject(const DevModel& dm, const double2* rc, double2* b, int R, cudaStream_t st);
