@@ -15,6 +15,7 @@
 
 #include "../../include/ddh.h"
 #include "ddh_host.hpp"
+#include "ddh_fixed.cuh"
 #include "ddh_launch.hpp"
 
 using namespace ddh;
@@ -71,9 +72,6 @@ struct ddh_ctx {
     void* sinv32 = nullptr;
     void* pq64 = nullptr;                          // Y = [A11^-1 A_1T]_E per element
     void* pq32 = nullptr;
-    void* sfx = nullptr;                           // S_E^-1 and Y in fixed point (FP64 edge passes)
-    void* yfx = nullptr;
-    void* y2fx = nullptr;                          // Y again, column-major, for pass 2
     bool edge_form = false;                        // Krylov-loop passes with Y (no FDM)
     const int* edge_items = nullptr;               // elements by degree, descending (persistent edge pass)
     std::vector<int> deg_begin, deg_count, deg_p;  // contiguous runs of equal degree in edge_items
@@ -88,8 +86,8 @@ struct ddh_ctx {
     int tc_maxT = 0;
     double2* Kinv = nullptr;                       // dense coarse inverse (elimination order)
     float2* Kinv32 = nullptr;
-    int* Kinv_ex = nullptr;                        // its row exponents and column scalings (fixed point)
-    int* Kinv_col = nullptr;
+    FxMat Kinv_fx;                                 // the same split (ddh_fixed.cuh), with its exponents
+    int* Kinv_ex = nullptr;
     int gemv_form = 1;                             // single-RHS complex64 GEMV kernel (timed at upload)
     int nsm = 0;                                   // SMs of the device
     // nested-dissection factor: complex128 matrices, their complex64 copy (nd32.G/M null
@@ -115,7 +113,8 @@ struct ddh_ctx {
     bool refine_active = false;                    // refinement used by the current solves
     const int* kc_ptr = nullptr;                   // assembled K (CSR, elimination order)
     const int* kc_col = nullptr;
-    const void* kc_val = nullptr;                  // fixed point, row exponents kc_ex
+    const double2* kc_val = nullptr;
+    FxMat kc_fx;                                   // the same split, with its rows' exponents
     int* kc_ex = nullptr;
     PlaneLoad pload;                               // tables of the plane-wave loads
     // work buffers (grow on demand)
@@ -172,6 +171,12 @@ static ddh_status fail(ddh_ctx* ctx, ddh_status s, const std::string& msg) {
     return s;
 }
 
+static ddh_status model_alloc(ddh_ctx* ctx, size_t bytes, void** out);
+// room for n split entries (ddh_fixed.cuh; bulk copies of an odd number of fractions read one more)
+static ddh_status alloc_split(ddh_ctx* ctx, size_t n, FxMat& m) {
+    ddh_status st = model_alloc(ctx, sizeof(int4) * n, (void**)&m.i);
+    return st ? st : model_alloc(ctx, sizeof(float2) * (n + 1), (void**)&m.f);
+}
 static ddh_status model_alloc(ddh_ctx* ctx, size_t bytes, void** out) {
     if (cudaMalloc(out, std::max<size_t>(16, bytes)) != cudaSuccess) { ctx->err = "cudaMalloc failed (model)"; return DDH_ERR_OOM; }
     ctx->model_allocs.push_back(*out);
@@ -205,7 +210,6 @@ static void free_model(ddh_ctx* ctx) {
     ctx->work.clear();
     ctx->sinv64 = ctx->sinv32 = nullptr;
     ctx->pq64 = ctx->pq32 = nullptr;
-    ctx->sfx = ctx->yfx = ctx->y2fx = nullptr;
     ctx->edge_form = false;
     ctx->edge_items = nullptr;
     ctx->deg_begin.clear(); ctx->deg_count.clear(); ctx->deg_p.clear();
@@ -392,14 +396,15 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         if ((st = upload(ctx, pre, &d.pre_all))) return st;
         if ((st = upload(ctx, poff, &d.pre_off))) return st;
         if ((st = upload(ctx, peoff, &d.pre_ex_off))) return st;
-        // the same in fixed point for the FP64 preconditioner
+        // the same split for the FP64 preconditioner
         const int64_t *ko, *ke;
         const int* kl;
-        void *fx, *ex;
+        void* ex;
         if ((st = upload(ctx, koff, &ko)) || (st = upload(ctx, keoff, &ke)) || (st = upload(ctx, klen, &kl))) return st;
-        if ((st = model_alloc(ctx, sizeof(int2) * pre.size(), &fx)) || (st = model_alloc(ctx, sizeof(int) * rows, &ex))) return st;
-        launch_fix_pre(d.pre_all, (int)klen.size(), ko, kl, ke, (int2*)fx, (int*)ex, ctx->stream);
-        d.pre_fx = (const int2*)fx;
+        if ((st = model_alloc(ctx, sizeof(int) * rows, &ex))) return st;
+        if ((st = model_alloc(ctx, sizeof(int2) * pre.size(), (void**)&d.pre_fx.i))) return st;
+        if ((st = model_alloc(ctx, sizeof(float) * pre.size(), (void**)&d.pre_fx.f))) return st;
+        launch_fix_pre(d.pre_all, (int)klen.size(), ko, kl, ke, d.pre_fx, (int*)ex, ctx->stream);
         d.pre_ex = (const int*)ex;
     }
     // slots
@@ -646,14 +651,10 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         const float2* a32;
         if ((st = upload(ctx, conv32(Kn), &a32))) return st;
         ctx->Kinv32 = (float2*)a32;
-        std::vector<int> ex0(nc, 0);
-        const int* exd;
-        if ((st = upload(ctx, ex0, &exd))) return st;
-        ctx->Kinv_ex = (int*)exd;
-        if ((st = upload(ctx, ex0, &exd))) return st;
-        ctx->Kinv_col = (int*)exd;
+        if ((st = model_alloc(ctx, sizeof(int) * (size_t)nc * gemv_tiles(nc), (void**)&ctx->Kinv_ex))) return st;
+        if ((st = alloc_split(ctx, (size_t)nc * nc, ctx->Kinv_fx))) return st;
         CK(cudaDeviceGetAttribute(&ctx->nsm, cudaDevAttrMultiProcessorCount, ctx->device));
-        launch_fix_dense(ctx->Kinv, nc, ctx->Kinv_ex, ctx->Kinv_col, ctx->stream);
+        launch_fix_dense(ctx->Kinv, nc, ctx->Kinv_fx, ctx->Kinv_ex, ctx->stream);
         gemv_set_smem_limits();
         // autotune: time the single-RHS GEMV forms on the complex64 K^-1 and keep the fastest
         if (want32) {
@@ -894,15 +895,10 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         D.G = a;
         if ((st = upload(ctx, Mall, &a))) return st;
         D.M = a;
-        {
-            std::vector<int> e0((size_t)std::max<int64_t>(D.u_len, nc), 0);
-            const int* ed;
-            for (int** p : {&D.gexp, &D.mexp, &D.gcol, &D.mcol, &D.mcolB}) {
-                if ((st = upload(ctx, e0, &ed))) return st;
-                *p = (int*)ed;
-            }
-            launch_fix_fronts(D, nn, ctx->stream);
-        }
+        if ((st = model_alloc(ctx, sizeof(int) * (size_t)D.u_len, (void**)&D.gexp))) return st;
+        if ((st = model_alloc(ctx, sizeof(int) * (size_t)nc, (void**)&D.mexp))) return st;
+        if ((st = alloc_split(ctx, Gall.size(), D.gfx)) || (st = alloc_split(ctx, Mall.size(), D.mfx))) return st;
+        launch_fix_fronts(D, nn, ctx->stream);
         const int4* it;
         if ((st = upload(ctx, items, &it))) return st;
         ctx->nd_items = it;
@@ -923,13 +919,10 @@ static ddh_status upload_model(ddh_ctx* ctx) {
     if (ctx->refine_coarse || want32) {
         if ((st = upload(ctx, m.kc_ptr, &ctx->kc_ptr))) return st;
         if ((st = upload(ctx, m.kc_col, &ctx->kc_col))) return st;
-        const double2* kv;
-        const int* ke;
-        if ((st = upload(ctx, conv(m.kc_val), &kv))) return st;
-        if ((st = upload(ctx, std::vector<int>(nc, 0), &ke))) return st;
-        launch_fix_csr(ctx->kc_ptr, (double2*)kv, (int*)ke, nc, ctx->stream);
-        ctx->kc_val = kv;
-        ctx->kc_ex = (int*)ke;
+        if ((st = upload(ctx, conv(m.kc_val), &ctx->kc_val))) return st;
+        if ((st = model_alloc(ctx, sizeof(int) * (size_t)nc, (void**)&ctx->kc_ex))) return st;
+        if ((st = alloc_split(ctx, m.kc_val.size(), ctx->kc_fx))) return st;
+        launch_fix_csr(ctx->kc_ptr, ctx->kc_val, ctx->kc_fx, ctx->kc_ex, nc, ctx->stream);
     }
     // plane-wave loads: boundary elements, and per degree w_q N~_m(t_q) on a Gauss-Legendre rule
     {
@@ -1156,8 +1149,8 @@ static ddh_status edge_tune(ddh_ctx* ctx, const Work& w, int R, bool fp64) {
     const DevModel& d = ctx->dm;
     cudaStream_t s = ctx->stream;
     CK(cudaMemsetAsync(w.vd, 0, sizeof(double2) * (size_t)R * std::max(1, d.n_dual), s));
-    const void* sinv = fp64 ? ctx->sfx : ctx->sinv32;
-    const void* Y = fp64 ? ctx->yfx : ctx->pq32;
+    const void* sinv = fp64 ? ctx->sinv64 : ctx->sinv32;
+    const void* Y = fp64 ? ctx->pq64 : ctx->pq32;
     EdgeSched es;
     es.items = ctx->edge_items;
     std::vector<signed char> tbl(33, 0);
@@ -1168,12 +1161,11 @@ static ddh_status edge_tune(ddh_ctx* ctx, const Work& w, int R, bool fp64) {
     for (size_t g = 0; g < ctx->deg_p.size(); ++g) {
         float best = 1e30f;
         int pick = 0;
-        for (int tpr : {4, 2}) {
+        if (fp64) pick = 4 * ctx->deg_p[g] <= 64 ? 4 : 2;          // fixed (edge_tpr)
+        else for (int tpr : {4, 2}) {
             auto run = [&] {
-                if (fp64) launch_pass1_edge<double>(d, sinv, Y, w.vd, 1.0, nullptr, w.xE, w.tT, R, nullptr, s, &es,
-                                                    ctx->deg_begin[g], ctx->deg_count[g], tpr);
-                else launch_pass1_edge<float>(d, sinv, Y, w.vd, 1.0, nullptr, w.xE, w.tT, R, nullptr, s, &es,
-                                              ctx->deg_begin[g], ctx->deg_count[g], tpr);
+                launch_pass1_edge<float>(d, sinv, Y, w.vd, 1.0, nullptr, w.xE, w.tT, R, nullptr, s, &es,
+                                         ctx->deg_begin[g], ctx->deg_count[g], tpr);
             };
             run();
             cudaEventRecord(e0, s);
@@ -1330,27 +1322,27 @@ static EdgeSched edge_sched(const ddh_ctx* ctx, bool fp64, int R) {
     return es;
 }
 
-// fixed-point copies of S_E^-1 and Y for the FP64 edge passes (made on first use: a mixed context
-// only needs them for ddh_apply_dual_operator in FP64)
+// split S_E^-1 and Y for the FP64 edge passes (made on first use: a mixed context only needs them for
+// ddh_apply_dual_operator in FP64)
 static ddh_status fix_edge(ddh_ctx* ctx) {
-    if (!ctx->edge_form || ctx->sfx) return DDH_OK;
     DevModel& d = ctx->dm;
+    if (!ctx->edge_form || d.y2_ex) return DDH_OK;
     ddh_status st;
     EdgeFix f;
-    const size_t ys = sizeof(int4) * ctx->m.pq.size();
-    if ((st = model_alloc(ctx, sizeof(int4) * ctx->m.sinv.size(), (void**)&f.s))) return st;
-    if ((st = model_alloc(ctx, ys, (void**)&f.y)) || (st = model_alloc(ctx, ys, (void**)&f.y2))) return st;
+    if ((st = alloc_split(ctx, ctx->m.sinv.size(), f.s)) || (st = alloc_split(ctx, ctx->m.pq.size(), f.y)) ||
+        (st = alloc_split(ctx, ctx->m.pq.size(), f.y2)))
+        return st;
     if ((st = model_alloc(ctx, sizeof(int) * (size_t)d.nE1_tot, (void**)&f.sex))) return st;
     if ((st = model_alloc(ctx, sizeof(int) * (size_t)d.nT_tot, (void**)&f.yex))) return st;
     if ((st = model_alloc(ctx, sizeof(int) * (size_t)d.nE1_tot, (void**)&f.y2ex))) return st;
     launch_fix_edge(d, ctx->sinv64, ctx->pq64, f, ctx->stream);
     CK(cudaGetLastError());
+    d.sinv_fx = f.s;
+    d.y_fx = f.y;
+    d.y2_fx = f.y2;
     d.sinv_ex = f.sex;
     d.y_ex = f.yex;
     d.y2_ex = f.y2ex;
-    ctx->sfx = f.s;
-    ctx->yfx = f.y;
-    ctx->y2fx = f.y2;
     return DDH_OK;
 }
 
@@ -1401,7 +1393,7 @@ static void coarse_solve(ddh_ctx* ctx, const double2* t, double2* x2, double2* t
     double2* r = tmp + (size_t)2 * R * nc;
     double2* dx = tmp + (size_t)3 * R * nc;
     coarse_solve_once(ctx, t, x2, tmp, R, done);
-    launch_csr_residual(ctx->kc_ptr, ctx->kc_col, ctx->kc_val, ctx->kc_ex, nc, x2, t, r, R, done, s);
+    launch_csr_residual(ctx->kc_ptr, ctx->kc_col, ctx->kc_val, ctx->kc_fx, ctx->kc_ex, nc, x2, t, r, R, done, s);
     coarse_solve_once(ctx, r, dx, tmp, R, done);
     launch_axpby(x2, 1.0, dx, 1.0, x2, (int64_t)R * nc, s);
     ctx->launches += 2;
@@ -1416,7 +1408,7 @@ static void coarse_solve_once(ddh_ctx* ctx, const double2* t, double2* x2, doubl
     const bool f32 = ctx->coarse32;
     if (ctx->Kinv) {
         if (f32) launch_gemv32(ctx->Kinv32, nc, t, x2, R, done, s, ctx->gemv_form);
-        else launch_gemv(ctx->Kinv, ctx->Kinv_ex, ctx->Kinv_col, nc, t, x2, R, done, ctx->nsm, s);
+        else launch_gemv(ctx->Kinv, ctx->Kinv_fx, ctx->Kinv_ex, nc, t, x2, R, done, ctx->nsm, s);
         ctx->launches++;
         return;
     }
@@ -1500,8 +1492,6 @@ static void apply_op(ddh_ctx* ctx, const Work& w, const double2* z, double zsign
     cudaStream_t s = ctx->stream;
     const void* sinv = std::is_same<T, double>::value ? ctx->sinv64 : ctx->sinv32;
     const void* Y = std::is_same<T, double>::value ? ctx->pq64 : ctx->pq32;
-    const void* eS = std::is_same<T, double>::value ? ctx->sfx : ctx->sinv32;     // of the edge passes
-    const void* eY = std::is_same<T, double>::value ? ctx->yfx : ctx->pq32;
     // With split_pass1, inside the Krylov loop (one-CTA edge form) pass 1 is split: the t_T rows,
     // which the coarse assembly needs, on the context stream; the x_E rows, needed only by pass 2,
     // on a forked stream beside the coarse solve.  Each output row is computed the same way
@@ -1515,12 +1505,12 @@ static void apply_op(ddh_ctx* ctx, const Work& w, const double2* z, double zsign
         if (split) {
             cudaEventRecord(ctx->ev_p1_fork, s);
             cudaStreamWaitEvent(ctx->side_p1, ctx->ev_p1_fork, 0);
-            launch_pass1_edge<T>(d, eS, eY, z, zsign, bt, w.xE, w.tT, R, done, ctx->side_p1, &es, 0, -1, 0, 1);
+            launch_pass1_edge<T>(d, sinv, Y, z, zsign, bt, w.xE, w.tT, R, done, ctx->side_p1, &es, 0, -1, 0, 1);
             cudaEventRecord(ctx->ev_p1_join, ctx->side_p1);
-            launch_pass1_edge<T>(d, eS, eY, z, zsign, bt, w.xE, w.tT, R, done, s, &es, 0, -1, 0, 2);
+            launch_pass1_edge<T>(d, sinv, Y, z, zsign, bt, w.xE, w.tT, R, done, s, &es, 0, -1, 0, 2);
             ctx->launches++;
         } else {
-            launch_pass1_edge<T>(d, eS, eY, z, zsign, bt, w.xE, w.tT, R, done, s, &es);
+            launch_pass1_edge<T>(d, sinv, Y, z, zsign, bt, w.xE, w.tT, R, done, s, &es);
         }
     }
     else launch_pass1<T>(d, sinv, ctx->edge_form ? Y : nullptr, z, zsign, bt, has_bI, w.xE, w.tT, R, done, s,
@@ -1529,7 +1519,7 @@ static void apply_op(ddh_ctx* ctx, const Work& w, const double2* z, double zsign
     ctx->launches += 2;
     coarse_solve(ctx, w.t, w.x2, w.ctmp, R, done);
     if (split) cudaStreamWaitEvent(s, ctx->ev_p1_join, 0);
-    if (ctx->edge_form && !phi_out) launch_pass2_edge<T>(d, std::is_same<T, double>::value ? ctx->y2fx : eY, w.x2, w.xE, w.xE2, R, done, s);
+    if (ctx->edge_form && !phi_out) launch_pass2_edge<T>(d, Y, w.x2, w.xE, w.xE2, R, done, s);
     else launch_pass2<T>(d, sinv, ctx->edge_form ? Y : nullptr, w.x2, w.xE, w.xE2, phi_out ? 1 : 0, bt, has_bI, phi_out, R, done, s,
                          fdm_cfg(ctx, std::is_same<T, double>::value, R, 2));
     ctx->launches++;
@@ -2786,12 +2776,12 @@ ddh_status ddh_profile_op(ddh_ctx* ctx, int32_t R, int32_t precision, int32_t re
     if (fp64) {
         ms_out[0] = timeit([&] {
             const EdgeSched es = edge_sched(ctx, true, R);
-            if (ef) launch_pass1_edge<double>(d, ctx->sfx, ctx->yfx, z, 1.0, nullptr, w.xE, w.tT, R, nullptr, s, &es);
+            if (ef) launch_pass1_edge<double>(d, sinv, Y, z, 1.0, nullptr, w.xE, w.tT, R, nullptr, s, &es);
             else launch_pass1<double>(d, sinv, nullptr, z, 1.0, nullptr, 0, w.xE, w.tT, R, nullptr, s);
         });
         ms_out[1] = timeit([&] { launch_coarse_assemble<double>(d, w.tT, nullptr, z, 1.0, w.t, R, nullptr, s); });
         ms_out[3] = timeit([&] {
-            if (ef) launch_pass2_edge<double>(d, ctx->y2fx, w.x2, w.xE, w.xE2, R, nullptr, s);
+            if (ef) launch_pass2_edge<double>(d, Y, w.x2, w.xE, w.xE2, R, nullptr, s);
             else launch_pass2<double>(d, sinv, nullptr, w.x2, w.xE, w.xE2, 0, nullptr, 0, nullptr, R, nullptr, s);
         });
         ms_out[4] = timeit([&] { launch_jump_gather<double>(d, w.xE2, w.x2, K.w, R, nullptr, s); });
@@ -2904,6 +2894,53 @@ ddh_status ddh_table_gauss(int32_t m, double* x, double* w) {
     gauss_legendre(m, xx, ww);
     std::memcpy(x, xx.data(), sizeof(double) * m);
     std::memcpy(w, ww.data(), sizeof(double) * m);
+    return DDH_OK;
+}
+ddh_status ddh_fixed_dot(int32_t n, int32_t lanes, const double* a, const double* x, double* out, int32_t* fp64) {
+    if (n < 0 || lanes < 1 || !a || !x || !out || !fp64) return DDH_ERR_INVALID_ARG;
+    if ((int64_t)lanes * ((n / lanes + 1) / kFxChain + 1) > kFxFlushes) return DDH_ERR_INVALID_ARG;
+    auto at = [](const double* v, int j) { return make_double2(v[2 * j], v[2 * j + 1]); };
+    unsigned ma = 0, mx = 0;
+    for (int j = 0; j < n; ++j) {
+        ma = std::max(ma, fx_mag(at(a, j)));
+        mx = std::max(mx, fx_mag(at(x, j)));
+    }
+    const int ea = fx_exp(ma), ex = fx_exp(mx);
+    long long h[2] = {0, 0}, l[2] = {0, 0};
+    for (int lane = 0; lane < lanes; ++lane) {
+        FxSum s;
+        fx_clear(s);
+        auto flush = [&] {
+            for (int i = 0; i < 2; ++i) fx_flush(s, i, h[i], l[i]);
+            fx_clear(s);
+        };
+        int c = 0;
+        for (int j = lane; j < n; j += lanes) {
+            const FxVec v = fx_vec(at(x, j), ex);
+            int4 ai;
+            float2 af;
+            fx_put(FxMat{&ai, &af}, 0, at(a, j), ea);
+            fx_mac(s, fx_entry(ai, af), v.i, v.f);
+            if (++c == kFxChain) {
+                c = 0;
+                flush();
+            }
+        }
+        flush();
+    }
+    const bool special = ea == 0x7ff || ex == 0x7ff;
+    FxWeight w = {0.f, 0.f};
+    double sx = 0, sy = 0;
+    for (int j = 0; j < n; ++j) {
+        const double2 u = at(a, j), v = at(x, j);
+        if (!special) fx_weigh(w, fx_split(u.x, ea).h, fx_split(u.y, ea).h, fx_vec(v, ex).i);
+        sx = std::fma(u.x, v.x, std::fma(-u.y, v.y, sx));
+        sy = std::fma(u.x, v.y, std::fma(u.y, v.x, sy));
+    }
+    for (int i = 0; i < 2; ++i) {
+        fp64[i] = !fx_value(h[i], l[i], ea, ex, out[i]) && (special || !fx_heavy(i ? w.y : w.x));
+        if (fp64[i]) out[i] = i ? sy : sx;
+    }
     return DDH_OK;
 }
 

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include "ddh_fixed.cuh"
 
 namespace ddh {
 
@@ -69,15 +70,17 @@ struct DevModel {
     const double* slap_all = nullptr;
     const double* pre_all = nullptr;    // restricted S^Lap per (degree, slot pattern), n_E^2
     const int64_t* pre_off = nullptr;   // per element: offset into pre_all
-    // fixed-point forms for the FP64 passes (ddh_fixed.cuh): pre_all's entries and row exponents (per
-    // element: offset into pre_ex), the row exponents of S_E^-1 (by type-1 slot) and the column
-    // exponents of Y (by type-2 slot)
-    const int2* pre_fx = nullptr;
+    // split matrices of the FP64 passes (ddh_fixed.cuh) with their exponents: pre_all by row (per element: offset
+    // into pre_ex), S_E^-1 by row (type-1 slot), Y by column (type-2 slot), and Y again, column-major, by row
+    FxRealMat pre_fx;
     const int* pre_ex = nullptr;
     const int64_t* pre_ex_off = nullptr;
+    FxMat sinv_fx;
     const int* sinv_ex = nullptr;
+    FxMat y_fx;
     const int* y_ex = nullptr;
-    const int* y2_ex = nullptr;         // row exponents of the column-major copy of Y (by type-1 slot)
+    FxMat y2_fx;
+    const int* y2_ex = nullptr;
     // E1 slots
     const int* e1_slot = nullptr;
     const int* e1_row = nullptr;

@@ -8,66 +8,40 @@
 
 namespace ddh {
 
-// ------------------------------------------------------------------ matrices in fixed point
-// A row of a complex128 matrix turned into limbs in place (see ddh_fixed.cuh) by one warp: the row's
-// exponent goes to ex; sc(j) is the scaling of column j (fx_even).  Entry j is a[j cs], j < n.
-template <class F>
-__device__ __forceinline__ void fix_row(double2* a, int64_t cs, int n, const F& sc, int* ex) {
+// ------------------------------------------------------------------ split matrices (ddh_fixed.cuh)
+// row a[j cs], j < n, to d[j cs], its exponent to ex, by one warp
+__device__ __forceinline__ void fix_row(const double2* a, const FxMat& d, int64_t cs, int n, int* ex) {
     const int lane = threadIdx.x & 31;
     unsigned m = 0;
-    for (int j = lane; j < n; j += 32) {
-        const double2 v = a[j * cs];
-        const int c = sc(j);
-        m = max(m, fx_mag(make_double2(fx_scale(v.x, -c), fx_scale(v.y, -c))));
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
-    const int ef = (int)(m >> 20);
-    for (int j = lane; j < n; j += 32) {
-        const double2 v = a[j * cs];
-        const int c = sc(j);
-        reinterpret_cast<int4*>(a)[j * cs] = fx_cpx(fx_scale(v.x, -c), fx_scale(v.y, -c), ef);
-    }
+    for (int j = lane; j < n; j += 32) m = max(m, fx_mag(a[j * cs]));
+    const int ef = fx_exp(__reduce_max_sync(0xffffffffu, m));
+    for (int j = lane; j < n; j += 32) fx_put(d, j * cs, a[j * cs], ef);
     if (lane == 0) *ex = ef;
 }
-// column scalings of K^-1 (symmetric: its rows' largest entries), then the rows
-__global__ void k_fix_dense_cols(const double2* __restrict__ A, int n, int* __restrict__ cex) {
-    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+// K^-1: one exponent per row and tile of kGemvTile columns
+constexpr int kGemvThreads = 512, kGemvTile = 736;
+__global__ void k_fix_dense(const double2* __restrict__ A, int n, FxMat d, int* __restrict__ ex) {
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nt = (n + kGemvTile - 1) / kGemvTile;
     if (row >= n) return;
-    unsigned m = 0;
-    for (int j = lane; j < n; j += 32) m = max(m, fx_mag(A[(int64_t)row * n + j]));
-    m = __reduce_max_sync(0xffffffffu, m);
-    if (lane == 0) cex[row] = fx_even((int)(m >> 20));
-}
-__global__ void k_fix_dense(double2* A, int n, const int* cex, int* ex) {
-    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (row < n) fix_row(A + (int64_t)row * n, 1, n, [&](int j) { return cex[j]; }, ex + row);
+    for (int t = 0; t < nt; ++t) {
+        const int64_t at = (int64_t)row * n + t * kGemvTile;
+        fix_row(A + at, d.at(at), 1, min(kGemvTile, n - t * kGemvTile), ex + (int64_t)row * nt + t);
+    }
 }
 // the two matrices of one nested-dissection front per CTA (layouts: NDDev)
 __global__ void k_fix_fronts(NDDev d) {
     const int node = blockIdx.x, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int nF = d.nF[node], nB = d.nB[node], n = nF + nB;
-    double2* G = (double2*)const_cast<void*>(d.G) + d.g_off[node];
-    double2* M = (double2*)const_cast<void*>(d.M) + d.m_off[node];
+    const int64_t go = d.g_off[node], mo = d.m_off[node];
     const bool gs = nF <= kNDShortRow, ms = n <= kNDShortRow;
-    int* gc = d.gcol + d.f0[node];                         // by column: F for G; F, then B for M
-    int* mf = d.mcol + d.f0[node];
-    int* mb = d.mcolB + d.u_off[node];
-    for (int j = threadIdx.x; j < nF; j += blockDim.x) {
-        unsigned m = 0;
-        for (int r = 0; r < nB; ++r) m = max(m, fx_mag(gs ? G[(int64_t)j * nB + r] : G[(int64_t)r * nF + j]));
-        gc[j] = fx_even((int)(m >> 20));
+    for (int r = warp; r < nB; r += nw) {
+        const int64_t at = go + (gs ? r : (int64_t)r * nF);
+        fix_row((const double2*)d.G + at, d.gfx.at(at), gs ? nB : 1, nF, d.gexp + d.u_off[node] + r);
     }
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        unsigned m = 0;
-        for (int r = 0; r < nF; ++r) m = max(m, fx_mag(ms ? M[(int64_t)j * nF + r] : M[(int64_t)r * n + j]));
-        (j < nF ? mf + j : mb + j - nF)[0] = fx_even((int)(m >> 20));
+    for (int r = warp; r < nF; r += nw) {
+        const int64_t at = mo + (ms ? r : (int64_t)r * n);
+        fix_row((const double2*)d.M + at, d.mfx.at(at), ms ? nF : 1, n, d.mexp + d.f0[node] + r);
     }
-    __syncthreads();
-    for (int r = warp; r < nB; r += nw)
-        fix_row(G + (gs ? r : (int64_t)r * nF), gs ? nB : 1, nF, [&](int j) { return gc[j]; }, d.gexp + d.u_off[node] + r);
-    for (int r = warp; r < nF; r += nw)
-        fix_row(M + (ms ? r : (int64_t)r * n), ms ? nF : 1, n, [&](int j) { return j < nF ? mf[j] : mb[j - nF]; },
-                d.mexp + d.f0[node] + r);
 }
 
 // ------------------------------------------------------------------ dense K^-1
@@ -250,12 +224,25 @@ __device__ __forceinline__ T warp_sum_transpose(T (&v)[V]) {
 // Short rows (column-major matrix): up to 16 rows per item, 32/S rows per warp at a time with S lanes
 // (column slices) each, and all right-hand sides of the block in a lane, so that an entry of the matrix
 // is loaded once; small items spread a level over all SMs.
-// Arithmetic follows the factor's storage type MT: fixed point (int4, FP64-accurate, see
-// ddh_fixed.cuh) for the complex128 factor, FP32 for its complex64 copy (vectors stay complex128 in
-// global memory and are converted when they are staged).
-template <class MT> struct NDVec { using V = cpx<float>; };
-template <> struct NDVec<int4> { using V = int4; };
-template <class MT> constexpr bool kNDFixed = std::is_same<MT, int4>::value;
+// Arithmetic follows the factor's storage type MT: the FP64-accurate products of ddh_fixed.cuh for the
+// complex128 factor, FP32 for its complex64 copy (vectors stay complex128 in global memory and are
+// converted when they are staged).
+template <class MT> constexpr bool kNDFixed = std::is_same<MT, double2>::value;
+// bytes of a staged entry, and of len of them (rounded up to keep what follows aligned)
+template <class MT> constexpr int kNDEntry = kNDFixed<MT> ? 32 : 8;
+template <class MT> __host__ __device__ constexpr size_t nd_bytes(size_t len) { return (kNDEntry<MT> * len + 15) & ~(size_t)15; }
+// the longest vector that is staged in limbs; the rows of a front with a longer one are summed in FP64 from
+// global memory
+constexpr int kNDFixedRows = 6144;
+// RB staged vectors at stride: limbs and fractions, or complex64
+template <class MT, int RB>
+struct NDStaged {
+    int4* i;
+    float4* f;
+    float2* v;
+    __device__ __forceinline__ NDStaged(char* sm, int stride)
+        : i(reinterpret_cast<int4*>(sm)), f(reinterpret_cast<float4*>(i + RB * stride)), v(reinterpret_cast<float2*>(sm)) {}
+};
 
 // Sum of V values per lane over each group of G consecutive lanes (xor offsets G/2, ..., 1, in
 // that order for every value, so the result does not depend on V), transposing while a lane
@@ -280,16 +267,13 @@ __device__ __forceinline__ void group_sum_transpose(T (&v)[V]) {
     for (int o = (G / 2) >> ilog2(V); o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
 }
 
-// y = K^-1 x, FP64-accurate in fixed point.  A CTA of 16 warps owns `rpc` rows (one CTA per SM), one warp
-// per row.  It stages x in shared memory as limbs, G tiles of kGemvTile columns at a time (a lane's chain
-// over a tile fits one flush, and each tile and vector has its own exponent, so a right-hand side's
-// result does not depend on RB), and adds the tiles up in FP64.  Integer multiply-adds bound it from two
-// right-hand sides on, reading K^-1 (16 n^2 bytes) at one.  FP64 against this form: 35 -> 20 us (n =
-// 1921, one right-hand side), 209 -> 139 us (n = 5425, one), 1437 -> 660 us (n = 4929, eight).
-constexpr int kGemvThreads = 512, kGemvTile = 1008;
+// y = K^-1 x with the products of ddh_fixed.cuh.  A CTA of 16 warps owns `rpc` rows (one CTA per SM), one warp
+// per row.  It stages x in shared memory as limbs, G tiles of kGemvTile columns at a time (each tile of a
+// row and of a vector has its own exponent, so a right-hand side's result does not depend on RB), and adds
+// the tiles up in FP64.  n = 1921: 23 us for one right-hand side (35 us in FP64; reading 24 n^2 bytes bounds it),
+// 126 us for eight; n = 2961: 60 and 295 us.
 template <int RB>
-__global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const int4* __restrict__ A, const int* __restrict__ aex,
-                                                         const int* __restrict__ acol, int n,
+__global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const double2* __restrict__ A, FxMat Ax, const int* __restrict__ aex, int n,
                                                          const double2* __restrict__ x, double2* __restrict__ y,
                                                          int r0, int nr, int rpc, const int* __restrict__ done) {
     if (done && *done) return;
@@ -298,8 +282,9 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const int4* __restrict
     __shared__ unsigned wmax[nw][8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int4* xs = reinterpret_cast<int4*>(gv_raw);                                             // [RB][stride]
-    double* acc = reinterpret_cast<double*>(gv_raw + (size_t)RB * stride * sizeof(int4));   // [rpc][2 RB]
-    const int row0 = blockIdx.x * rpc, rows = min(rpc, n - row0);
+    float4* xf = reinterpret_cast<float4*>(xs + RB * stride);
+    double* acc = reinterpret_cast<double*>(xf + RB * stride);                              // [rpc][2 RB]
+    const int row0 = blockIdx.x * rpc, rows = min(rpc, n - row0), nt = (n + kGemvTile - 1) / kGemvTile;
     for (int g0 = 0; g0 < n; g0 += G * kGemvTile) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) {                      // (tile, vector)
@@ -311,10 +296,7 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const int4* __restrict
             for (int u = 0; u < 2; ++u) {                  // kGemvTile <= 2 kGemvThreads
                 const int i = threadIdx.x + u * kGemvThreads;
                 if (i < w) {
-                    double2 v = q < nr ? xq[i] : make_double2(0.0, 0.0);
-                    const int c = acol[c0 + i];
-                    v.x = fx_scale(v.x, c);
-                    v.y = fx_scale(v.y, c);
+                    const double2 v = q < nr ? xq[i] : make_double2(0.0, 0.0);
                     d[i] = v;
                     m = max(m, fx_mag(v));
                 }
@@ -326,15 +308,15 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const int4* __restrict
         int ex[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            const int q = k % RB, w = min(kGemvTile, n - (g0 + k / RB * kGemvTile));
+            const int at = k % RB * stride + k / RB * kGemvTile, w = min(kGemvTile, n - (g0 + k / RB * kGemvTile));
             unsigned m = 0;
 #pragma unroll
             for (int i = 0; i < nw; ++i) m = max(m, wmax[i][k]);
-            ex[k] = (int)(m >> 20);
-            int4* d = xs + q * stride + k / RB * kGemvTile;
+            ex[k] = fx_exp(m);
             for (int i = threadIdx.x; i < w; i += kGemvThreads) {
-                const double2 v = reinterpret_cast<double2*>(d)[i];
-                d[i] = fx_cpx(v.x, v.y, ex[k]);
+                const FxVec v = fx_vec(reinterpret_cast<double2*>(xs)[at + i], ex[k]);
+                xs[at + i] = v.i;
+                xf[at + i] = v.f;
             }
         }
         __syncthreads();
@@ -344,43 +326,65 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const int4* __restrict
             const bool mine = (lane & ((1 << sh) - 1)) == 0 && (q >> 1) < nr;
             double* d = acc + k * 2 * RB + q;
             double t = g0 && mine ? *d : 0.0;
-#pragma unroll
+#pragma unroll 1
             for (int tl = 0; tl < G; ++tl) {
                 const int c0 = g0 + tl * kGemvTile, w = min(kGemvTile, n - c0);
                 if (w <= 0) break;
-                const int4* a = A + (int64_t)(row0 + k) * n + c0;
-                const int4* xt = xs + tl * kGemvTile;
-                FxAcc s[2 * RB];
+                const double2* a = A + (int64_t)(row0 + k) * n + c0;
+                const int ea = aex[(int64_t)(row0 + k) * nt + c0 / kGemvTile], o = tl * kGemvTile;
+                FxSum s[RB];
 #pragma unroll
-                for (int i = 0; i < 2 * RB; ++i) s[i].h = s[i].l = 0;
+                for (int i = 0; i < RB; ++i) fx_clear(s[i]);
                 constexpr int U = RB == 1 ? 6 : (RB == 2 ? 4 : 2);     // loads issued ahead of their use
                 int4 av[U];
+                float2 af[U];
+                const FxMat ax = Ax.at((int64_t)(row0 + k) * n + c0);
+                auto fetch = [&](int u, int j) {
+                    av[u] = j < w ? __ldg(ax.i + j) : make_int4(0, 0, 0, 0);
+                    af[u] = j < w ? __ldg(ax.f + j) : make_float2(0.f, 0.f);
+                };
 #pragma unroll
-                for (int u = 0; u < U; ++u) av[u] = lane + 32 * u < w ? __ldg(a + lane + 32 * u) : make_int4(0, 0, 0, 0);
+                for (int u = 0; u < U; ++u) fetch(u, lane + 32 * u);
                 for (int j = lane; j < w; j += 32 * U) {
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const int4 v = av[u];
-                        const int jj = min(j + 32 * u, w - 1), jn = j + 32 * (U + u);
-                        av[u] = jn < w ? __ldg(a + jn) : make_int4(0, 0, 0, 0);
+                        const FxEntry v = fx_entry(av[u], af[u]);
+                        const int jj = o + min(j + 32 * u, w - 1);
+                        fetch(u, j + 32 * (U + u));
 #pragma unroll
-                        for (int b = 0; b < RB; ++b)
-                            fx_cmac(s[2 * b], s[2 * b + 1], v, -v.z, -v.w, xt[b * stride + jj]);
+                        for (int b = 0; b < RB; ++b) fx_mac(s[b], v, xs[b * stride + jj], xf[b * stride + jj]);
                     }
                 }
-                long long h[2 * RB];
-                unsigned l[2 * RB];
+                long long h[2 * RB], l[2 * RB];
 #pragma unroll
                 for (int i = 0; i < 2 * RB; ++i) {
                     h[i] = l[i] = 0;
-                    fx_flush(s[i], h[i], l[i]);
+                    fx_flush(s[i >> 1], i & 1, h[i], l[i]);
                 }
-                const long long hs = warp_sum_transpose<long long, 2 * RB>(h);
-                const unsigned ls = warp_sum_transpose<unsigned, 2 * RB>(l);
-                int e = ex[tl * RB];
+                const long long hs = warp_sum_transpose<long long, 2 * RB>(h), ls = warp_sum_transpose<long long, 2 * RB>(l);
+                int e = 0;
 #pragma unroll
-                for (int i = 1; i < RB; ++i) e = (q >> 1) == i ? ex[tl * RB + i] : e;
-                t += fx_value(hs, ls, aex[row0 + k], e);
+                for (int i = 0; i < 8; ++i) e = i == tl * RB + (q >> 1) ? ex[i] : e;
+                double v = 0;
+                const bool bad = (q >> 1) < nr && !fx_value(hs, ls, ea, e, v);
+                if (__any_sync(0xffffffffu, bad)) {
+#pragma unroll 1
+                    for (int b = 0; b < nr; ++b) {
+                        const bool this_b = bad && (q >> 1) == b;
+                        if (!__any_sync(0xffffffffu, this_b)) continue;
+                        const double2* xq = x + (int64_t)(r0 + b) * n + c0;
+                        int eb = 0;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) eb = i == tl * RB + b ? ex[i] : eb;
+                        double2 r;
+                        const int4 *ai = ax.i, *xi = xs + b * stride + o;
+                        const unsigned keep = fx_again(32, this_b ? 1u << (q & 1) : 0, w, ea, eb, [=](int j) { return a[j]; },
+                                                       [=](int j) { const int4 u = ai[j]; return make_int2(u.x, u.z); },
+                                                       [=](int j) { return xi[j]; }, [=](int j) { return xq[j]; }, r);
+                        if (this_b && !(keep >> (q & 1) & 1)) v = q & 1 ? r.y : r.x;
+                    }
+                }
+                t += v;
             }
             if (mine) {
                 if (g0 + G * kGemvTile < n) *d = t;
@@ -403,7 +407,7 @@ __device__ __forceinline__ double2 nd_pull(const double2* u, int64_t base, int64
     if (b >= 0) { const double2 v = ldv<CG>(u + base + b); s.x += v.x; s.y += v.y; }
     return s;
 }
-__device__ __forceinline__ void cfma(float& ax, float& ay, float2 a, cpx<float> v) {
+__device__ __forceinline__ void cfma(float& ax, float& ay, float2 a, float2 v) {
     ax = fma(a.x, v.x, fma(-a.y, v.y, ax));
     ay = fma(a.x, v.y, fma(a.y, v.x, ay));
 }
@@ -421,19 +425,21 @@ constexpr int kNDThreads = 128;          // level launches: four warps (long row
 constexpr int kNDWarps = 8;              // bottom launches, and the most warps of a CTA
 // shared memory beside the staged vectors: exponents, and the warps' maxima while they are found
 struct NDShared {
-    int ex[8];
-    unsigned wmax[kNDWarps][8];
+    int ex[4];
+    unsigned wmax[kNDWarps][4];
 };
 
 // Stages RB vectors of length n (odd stride) in shared memory: load(i, v) gives entry i of all of them
 // as complex128, so that their index lookups are shared and RB loads are in flight per thread.
-// Fixed point: each vector's exponent is the largest of its entries.
+// Fixed point: each vector's exponent is that of its largest entry (2047, i.e. FP64 for all results, where
+// it is too long to be staged).
 template <class MT, int RB, bool WARP, class F>
-__device__ __forceinline__ void nd_stage(const F& load, int n, int stride, typename NDVec<MT>::V* sm, int* ex,
-                                         NDShared* sh) {
+__device__ __forceinline__ void nd_stage(const F& load, int n, int stride, char* sm, int* ex, NDShared* sh) {
     using G = NDGroup<WARP>;
+    const NDStaged<MT, RB> st(sm, stride);
     if constexpr (kNDFixed<MT>) {
         double2* s = reinterpret_cast<double2*>(sm);
+        const bool fit = n <= kNDFixedRows;
         unsigned m[RB];
 #pragma unroll
         for (int r = 0; r < RB; ++r) m[r] = 0;
@@ -443,7 +449,7 @@ __device__ __forceinline__ void nd_stage(const F& load, int n, int stride, typen
             load(i, v);
 #pragma unroll
             for (int r = 0; r < RB; ++r) {
-                s[r * stride + i] = v[r];
+                if (fit) s[r * stride + i] = v[r];
                 m[r] = max(m[r], fx_mag(v[r]));
             }
         }
@@ -460,128 +466,179 @@ __device__ __forceinline__ void nd_stage(const F& load, int n, int stride, typen
         }
         if (G::t() == 0)
 #pragma unroll
-            for (int r = 0; r < RB; ++r) ex[r] = (int)(m[r] >> 20);
-        for (int i = G::t(); i < n; i += G::n())
+            for (int r = 0; r < RB; ++r) ex[r] = fit ? fx_exp(m[r]) : 0x7ff;
+        if (fit)
+            for (int i = G::t(); i < n; i += G::n())
 #pragma unroll
-            for (int r = 0; r < RB; ++r) {
-                const double2 v = s[r * stride + i];
-                sm[r * stride + i] = fx_cpx(v.x, v.y, (int)(m[r] >> 20));
-            }
+                for (int r = 0; r < RB; ++r) {
+                    const FxVec w = fx_vec(s[r * stride + i], fx_exp(m[r]));
+                    st.i[r * stride + i] = w.i;
+                    st.f[r * stride + i] = w.f;
+                }
     } else {
         for (int i = G::t(); i < n; i += G::n()) {
             double2 v[RB];
             load(i, v);
 #pragma unroll
-            for (int r = 0; r < RB; ++r) sm[r * stride + i] = mk<float>((float)v[r].x, (float)v[r].y);
+            for (int r = 0; r < RB; ++r) st.v[r * stride + i] = make_float2((float)v[r].x, (float)v[r].y);
         }
     }
     G::sync();
 }
 
-// One lane's terms a[j cs] x[j], j = j0, j0 + dj, ... < n, for RB vectors (x staged in sm): v[2r + c] is
-// component c of vector r (fixed point: with low[]).  kNDAhead loads of A are in flight; pre holds the
-// first ones when they were issued before the vectors were staged.
+// One lane's terms a[j cs] x[j], j = j0, j0 + dj, ... < n, for RB vectors (staged): v[2r + c] is component c of
+// vector r (fixed point: with low[]).  kNDAhead loads of A are in flight; pre holds
+// the first ones when they were issued before the vectors were staged.
 constexpr int kNDAhead = 4;
 template <class MT> using NDSum = typename std::conditional<kNDFixed<MT>, long long, float>::type;
+// the matrix that the sums read, and an entry of it in registers
+struct NDSplit {
+    int4 i;
+    float2 f;
+};
+template <class MT> using NDMat = typename std::conditional<kNDFixed<MT>, FxMat, const MT*>::type;
+template <class MT> using NDItem = typename std::conditional<kNDFixed<MT>, NDSplit, MT>::type;
 template <class MT>
-__device__ __forceinline__ void nd_ahead(const MT* a, int64_t cs, int j0, int dj, int n, bool ok, MT (&pre)[kNDAhead]) {
+__device__ __forceinline__ void nd_ahead(const NDMat<MT>& a, int64_t cs, int j0, int dj, int n, bool ok,
+                                         NDItem<MT> (&pre)[kNDAhead]) {
 #pragma unroll
     for (int k = 0; k < kNDAhead; ++k) {
         const int j = j0 + k * dj;
-        pre[k] = ok && j < n ? __ldg(a + j * cs) : MT{};
+        pre[k] = NDItem<MT>{};
+        if (ok && j < n) {
+            if constexpr (kNDFixed<MT>) pre[k] = {__ldg(a.i + j * cs), __ldg(a.f + j * cs)};
+            else pre[k] = __ldg(a + j * cs);
+        }
     }
 }
 template <class MT, int RB>
-__device__ __forceinline__ void nd_dot(const MT* a, int64_t cs, int j0, int dj, int n, bool ok, MT (&pre)[kNDAhead],
-                                       int stride, const typename NDVec<MT>::V* sm, NDSum<MT> (&v)[2 * RB],
-                                       unsigned (&low)[2 * RB]) {
+__device__ __forceinline__ void nd_dot(const NDMat<MT>& a, int64_t cs, int j0, int dj, int n, bool ok,
+                                       NDItem<MT> (&pre)[kNDAhead], int stride, const NDStaged<MT, RB>& st, NDSum<MT> (&v)[2 * RB],
+                                       long long (&low)[2 * RB]) {
 #pragma unroll
     for (int i = 0; i < 2 * RB; ++i) { v[i] = 0; low[i] = 0; }
-    FxAcc s[2 * RB];
+    FxSum s[RB];
     if constexpr (kNDFixed<MT>)
 #pragma unroll
-        for (int i = 0; i < 2 * RB; ++i) s[i].h = s[i].l = 0;
+        for (int r = 0; r < RB; ++r) fx_clear(s[r]);
+    auto flush = [&] {
+        if constexpr (kNDFixed<MT>)
+#pragma unroll
+            for (int i = 0; i < 2 * RB; ++i) fx_flush(s[i >> 1], i & 1, v[i], low[i]);
+#pragma unroll
+        for (int r = 0; r < RB; ++r) fx_clear(s[r]);
+    };
     for (int j = j0, c = 0; j < n; j += kNDAhead * dj) {
-        MT nxt[kNDAhead];
+        NDItem<MT> nxt[kNDAhead];
         nd_ahead<MT>(a, cs, j + kNDAhead * dj, dj, n, ok, nxt);
 #pragma unroll
         for (int k = 0; k < kNDAhead; ++k) {
             const int jj = min(j + k * dj, n - 1);         // past the end the entry of A is zero
+            if constexpr (kNDFixed<MT>) {
+                const FxEntry e = fx_entry(pre[k].i, pre[k].f);
 #pragma unroll
-            for (int r = 0; r < RB; ++r) {
-                if constexpr (kNDFixed<MT>)
-                    fx_cmac(s[2 * r], s[2 * r + 1], pre[k], -pre[k].z, -pre[k].w, sm[r * stride + jj]);
-                else cfma(v[2 * r], v[2 * r + 1], pre[k], sm[r * stride + jj]);
+                for (int r = 0; r < RB; ++r) fx_mac(s[r], e, st.i[r * stride + jj], st.f[r * stride + jj]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < RB; ++r) cfma(v[2 * r], v[2 * r + 1], pre[k], st.v[r * stride + jj]);
             }
             pre[k] = nxt[k];
         }
         if constexpr (kNDFixed<MT>)
             if ((c += kNDAhead) > kFxChain - kNDAhead) {
                 c = 0;
-#pragma unroll
-                for (int i = 0; i < 2 * RB; ++i) fx_flush(s[i], v[i], low[i]);
+                flush();
             }
     }
-    if constexpr (kNDFixed<MT>)
-#pragma unroll
-        for (int i = 0; i < 2 * RB; ++i) fx_flush(s[i], v[i], low[i]);
+    if constexpr (kNDFixed<MT>) flush();
 }
 
 // Rows of one front's matrix, A x + add, by 32/S rows per warp: lane = (row, column slice of S).  In the
 // constructor-like first step (ahead) a lane finds its row and issues its first loads of A; after the
 // vectors are staged, run() forms the sums and hands component c (0 real, 1 imaginary) of right-hand
-// side r to out(row, r, c, value).  Sums run in an order fixed by the matrix alone (fixed point:
-// exactly), so the result does not depend on RB.  cs, rs: strides of A along a row and between rows.
+// side r to out(row, r, c, value).  Sums run in an order fixed by the matrix and S alone, so the result
+// does not depend on RB.  cs, rs: strides of A along a row and between rows; load: the staged vectors'
+// entries, for the results that are formed again in FP64.
 template <class MT, int RB, int S>
 struct NDRows {
     static constexpr int nv = 2 * RB >= S ? 2 * RB / S : 1, sh = 2 * RB >= S ? 0 : ilog2(S) - ilog2(2 * RB);
-    const MT* a;
+    const MT* a;                         // the row
+    NDMat<MT> ax;                        // and split
     int64_t cs;
-    int row, n;
+    int row, n, ea;
     bool ok, mine;
-    MT pre[kNDAhead];
+    NDItem<MT> pre[kNDAhead];
     __device__ __forceinline__ static int slice() { return threadIdx.x & (S - 1); }
     // value index (component q & 1 of right-hand side q >> 1) of this lane's i-th sum
     __device__ __forceinline__ static int value(int i) { return 2 * RB >= S ? slice() * nv + i : slice() >> sh; }
-    __device__ __forceinline__ void ahead(const MT* A, int64_t rs, int64_t cs_, int n_, int row_, int end) {
+    __device__ __forceinline__ void ahead(const MT* A, const FxMat& Ax, int64_t rs, int64_t cs_, int n_, const int* aex, int row_,
+                                          int end) {
         row = row_ + ((threadIdx.x & 31) / S);
         ok = row < end;
         mine = ok && (slice() & ((1 << sh) - 1)) == 0;
         a = A + (int64_t)(ok ? row : 0) * rs;
         cs = cs_;
         n = n_;
-        nd_ahead<MT>(a, cs, slice(), S, n, ok, pre);
+        ea = 0;
+        if constexpr (kNDFixed<MT>) {
+            ax = Ax.at((int64_t)(ok ? row : 0) * rs);
+            if (ok) ea = aex[row];
+        } else ax = a;
+        nd_ahead<MT>(ax, cs, slice(), S, n, ok, pre);
     }
-    template <class F>
-    __device__ __forceinline__ void run(int stride, const typename NDVec<MT>::V* sm, const int* aex, const int* ex, int nr,
-                                        const double (&add)[nv], const F& out) {
+    template <class L, class F>
+    __device__ __forceinline__ void run(int stride, char* sm, const int* ex, int nr, const double (&add)[nv], const L& load,
+                                        const F& out) {
         NDSum<MT> v[2 * RB];
-        unsigned low[2 * RB];
-        nd_dot<MT, RB>(a, cs, slice(), S, n, ok, pre, stride, sm, v, low);
+        long long low[2 * RB];
+        nd_dot<MT, RB>(ax, cs, slice(), S, kNDFixed<MT> && n > kNDFixedRows ? 0 : n, ok, pre, stride,
+                       NDStaged<MT, RB>(sm, stride), v, low);
         group_sum_transpose<NDSum<MT>, 2 * RB, S>(v);
-        if constexpr (kNDFixed<MT>) group_sum_transpose<unsigned, 2 * RB, S>(low);
+        double val[nv];
+        if constexpr (kNDFixed<MT>) {
+            group_sum_transpose<long long, 2 * RB, S>(low);
+            unsigned bad = 0;                              // bit i: value i is to be formed in FP64
+#pragma unroll
+            for (int i = 0; i < nv; ++i) {
+                const int r = value(i) >> 1;
+                val[i] = 0;
+                if (mine && r < nr && !fx_value(v[i], low[i], ea, ex[r], val[i])) bad |= 1u << i;
+            }
+            if (__any_sync(0xffffffffu, bad != 0)) again(bad, nr, val, ex, NDStaged<MT, RB>(sm, stride).i, stride, load);
+        } else {
+#pragma unroll
+            for (int i = 0; i < nv; ++i) val[i] = (double)v[i];
+        }
         if (!mine) return;
-        int ea = 0;
-        if constexpr (kNDFixed<MT>) ea = aex[row];
 #pragma unroll
         for (int i = 0; i < nv; ++i) {
             const int q = value(i), r = q >> 1;
-            if (r >= nr) continue;
-            if constexpr (kNDFixed<MT>) out(row, r, q & 1, add[i] + fx_value(v[i], low[i], ea, ex[r]));
-            else out(row, r, q & 1, add[i] + (double)v[i]);
+            if (r < nr) out(row, r, q & 1, add[i] + val[i]);
+        }
+    }
+    template <class L>
+    __device__ __forceinline__ void again(unsigned bad, int nr, double (&val)[nv], const int* ex, const int4* xi, int stride,
+                                          const L& load) {
+#pragma unroll 1
+        for (int r = 0; r < nr; ++r) {
+            unsigned b = 0;
+#pragma unroll
+            for (int i = 0; i < nv; ++i)
+                if ((bad >> i & 1) && (value(i) >> 1) == r) b |= 1u << (value(i) & 1);
+            if (!__any_sync(0xffffffffu, b != 0)) continue;
+            double2 d;
+            const MT* a_ = a;
+            const int4 *ai = ax.i, *xr = xi + r * stride;
+            const int64_t cs_ = cs;
+            b &= ~fx_again(S, b, n, ea, ex[r], [=](int j) { const MT u = a_[j * cs_]; return make_double2((double)u.x, (double)u.y); },
+                           [=](int j) { const int4 u = ai[j * cs_]; return make_int2(u.x, u.z); }, [=](int j) { return xr[j]; },
+                           [=](int j) { double2 x[RB]; load(j, x); return x[r]; }, d);
+#pragma unroll
+            for (int i = 0; i < nv; ++i)
+                if ((value(i) >> 1) == r && (b >> (value(i) & 1) & 1) && (bad >> i & 1)) val[i] = value(i) & 1 ? d.y : d.x;
         }
     }
 };
-
-// an entry's column scaling (fixed point only)
-template <class MT, int RB>
-__device__ __forceinline__ void nd_scale(double2 (&v)[RB], const int* col) {
-    if constexpr (kNDFixed<MT>) {
-        const int c = *col;
-#pragma unroll
-        for (int r = 0; r < RB; ++r) { v[r].x = fx_scale(v[r].x, c); v[r].y = fx_scale(v[r].y, c); }
-    }
-}
 
 // Where rows [row0, row0 + nrows) of a front are worked on: by the warps of a CTA (32/S rows each at a
 // time), or (WARP) by one warp alone.
@@ -591,7 +648,7 @@ template <class MT, int RB, int S, bool CG, bool WARP>
 __device__ __forceinline__ void nd_forward_rows(const NDDev& d, int node, int row0, int nrows, bool write_y,
                                                 const double2* __restrict__ t, double2* __restrict__ y,
                                                 double2* __restrict__ u, int r0, int nr,
-                                                typename NDVec<MT>::V* nd_sm, int* ex, NDShared* sh) {
+                                                char* nd_sm, int* ex, NDShared* sh) {
     using G = NDGroup<WARP>;
     const int f0 = d.f0[node], nF = d.nF[node], nB = d.nB[node], sF = nF | 1;
     const int64_t nc = d.nc, ul = d.u_len, so = d.s_off[node], uo = d.u_off[node];
@@ -600,7 +657,7 @@ __device__ __forceinline__ void nd_forward_rows(const NDDev& d, int node, int ro
     NDRows<MT, RB, S> R;
     double add[NDRows<MT, RB, S>::nv];
     auto begin = [&](int row) {
-        R.ahead(A, cm ? 1 : nF, cm ? nB : 1, nF, row, row0 + nrows);
+        R.ahead(A, d.gfx.at(d.g_off[node]), cm ? 1 : nF, cm ? nB : 1, nF, d.gexp + uo, row, row0 + nrows);
         const int64_t i = so + nF + (R.ok ? R.row : 0);
         const int64_t pa = R.mine ? d.src[2 * i] : -1, pb = R.mine ? d.src[2 * i + 1] : -1;
 #pragma unroll
@@ -616,8 +673,9 @@ __device__ __forceinline__ void nd_forward_rows(const NDDev& d, int node, int ro
     constexpr int per = 32 / S;
     int row = row0 + G::warp() * per;
     begin(row);
-    nd_stage<MT, RB, WARP>([&](int i, double2 (&v)[RB]) {
-        const int64_t a = d.src[2 * (so + i)], b = d.src[2 * (so + i) + 1];
+    const int64_t* src = d.src + 2 * so;
+    const auto load = [=](int i, double2 (&v)[RB]) {
+        const int64_t a = src[2 * i], b = src[2 * i + 1];
 #pragma unroll
         for (int r = 0; r < RB; ++r) {
             v[r] = make_double2(0.0, 0.0);
@@ -627,11 +685,11 @@ __device__ __forceinline__ void nd_forward_rows(const NDDev& d, int node, int ro
             v[r].x -= w.x; v[r].y -= w.y;
             if (write_y) y[(r0 + r) * nc + f0 + i] = v[r];
         }
-        nd_scale<MT, RB>(v, d.gcol + f0 + i);
-    }, nF, sF, nd_sm, ex, sh);
+    };
+    nd_stage<MT, RB, WARP>(load, nF, sF, nd_sm, ex, sh);
     for (; row < row0 + nrows; row += per * G::warps()) {
         if (row != row0 + G::warp() * per) begin(row);
-        R.run(sF, nd_sm, d.gexp + uo, ex, nr, add, [&](int rw, int r, int c, double v) {
+        R.run(sF, nd_sm, ex, nr, add, load, [&](int rw, int r, int c, double v) {
             reinterpret_cast<double*>(u + (r0 + r) * ul + uo + rw)[c] = v;
         });
     }
@@ -643,10 +701,10 @@ template <class MT, int RB, int S, bool CG, bool WARP>
 __device__ __forceinline__ void nd_backward_rows(const NDDev& d, int node, int row0, int nrows, bool root,
                                                  const double2* __restrict__ t, const double2* __restrict__ u,
                                                  const double2* __restrict__ y, double2* __restrict__ x, int r0,
-                                                 int nr, typename NDVec<MT>::V* nd_sm, int* ex, NDShared* sh) {
+                                                 int nr, char* nd_sm, int* ex, NDShared* sh) {
     using G = NDGroup<WARP>;
     const int f0 = d.f0[node], nF = d.nF[node], nB = d.nB[node], n = nF + nB, sn = n | 1;
-    const int64_t nc = d.nc, ul = d.u_len, so = d.s_off[node], uo = d.u_off[node];
+    const int64_t nc = d.nc, ul = d.u_len, so = d.s_off[node];
     const int* bi = d.bidx + d.b_off[node];
     const bool cm = n <= kNDShortRow;
     const MT* A = (const MT*)d.M + d.m_off[node];
@@ -656,10 +714,11 @@ __device__ __forceinline__ void nd_backward_rows(const NDDev& d, int node, int r
     for (int k = 0; k < R.nv; ++k) add[k] = 0;
     constexpr int per = 32 / S;
     int row = row0 + G::warp() * per;
-    R.ahead(A, cm ? 1 : n, cm ? nF : 1, n, row, row0 + nrows);
-    nd_stage<MT, RB, WARP>([&](int i, double2 (&v)[RB]) {
+    R.ahead(A, d.mfx.at(d.m_off[node]), cm ? 1 : n, cm ? nF : 1, n, d.mexp + f0, row, row0 + nrows);
+    const int64_t* src = d.src + 2 * so;
+    const auto load = [=](int i, double2 (&v)[RB]) {
         if (root) {
-            const int64_t a = d.src[2 * (so + i)], b = d.src[2 * (so + i) + 1];
+            const int64_t a = src[2 * i], b = src[2 * i + 1];
 #pragma unroll
             for (int r = 0; r < RB; ++r) {
                 v[r] = make_double2(0.0, 0.0);
@@ -670,15 +729,15 @@ __device__ __forceinline__ void nd_backward_rows(const NDDev& d, int node, int r
             }
         } else {
             const int pos = i < nF ? f0 + i : bi[i - nF];
-            const double2* src = i < nF ? y : x;
+            const double2* from = i < nF ? y : x;
 #pragma unroll
-            for (int r = 0; r < RB; ++r) v[r] = r < nr ? ldv<CG>(src + (r0 + r) * nc + pos) : make_double2(0.0, 0.0);
+            for (int r = 0; r < RB; ++r) v[r] = r < nr ? ldv<CG>(from + (r0 + r) * nc + pos) : make_double2(0.0, 0.0);
         }
-        nd_scale<MT, RB>(v, i < nF ? d.mcol + f0 + i : d.mcolB + uo + i - nF);
-    }, n, sn, nd_sm, ex, sh);
+    };
+    nd_stage<MT, RB, WARP>(load, n, sn, nd_sm, ex, sh);
     for (; row < row0 + nrows; row += per * G::warps()) {
-        if (row != row0 + G::warp() * per) R.ahead(A, cm ? 1 : n, cm ? nF : 1, n, row, row0 + nrows);
-        R.run(sn, nd_sm, d.mexp + f0, ex, nr, add, [&](int rw, int r, int c, double v) {
+        if (row != row0 + G::warp() * per) R.ahead(A, d.mfx.at(d.m_off[node]), cm ? 1 : n, cm ? nF : 1, n, d.mexp + f0, row, row0 + nrows);
+        R.run(sn, nd_sm, ex, nr, add, load, [&](int rw, int r, int c, double v) {
             reinterpret_cast<double*>(x + (r0 + r) * nc + f0 + rw)[c] = v;
         });
     }
@@ -690,7 +749,7 @@ template <class MT, int RB, bool CG = false>
 __device__ __forceinline__ void nd_forward_node(const NDDev& d, int node, int row0, int nrows, bool shortm,
                                                 bool write_y, const double2* __restrict__ t, double2* __restrict__ y,
                                                 double2* __restrict__ u, int r0, int nr,
-                                                typename NDVec<MT>::V* nd_sm, NDShared* sh) {
+                                                char* nd_sm, NDShared* sh) {
     if (shortm) nd_forward_rows<MT, RB, 8, CG, false>(d, node, row0, nrows, write_y, t, y, u, r0, nr, nd_sm, sh->ex, sh);
     else nd_forward_rows<MT, RB, 32, CG, false>(d, node, row0, nrows, write_y, t, y, u, r0, nr, nd_sm, sh->ex, sh);
 }
@@ -698,7 +757,7 @@ template <class MT, int RB, bool CG = false>
 __device__ __forceinline__ void nd_backward_node(const NDDev& d, int node, int row0, int nrows, bool shortm, bool root,
                                                  const double2* __restrict__ t, const double2* __restrict__ u,
                                                  const double2* __restrict__ y, double2* __restrict__ x, int r0,
-                                                 int nr, typename NDVec<MT>::V* nd_sm, NDShared* sh) {
+                                                 int nr, char* nd_sm, NDShared* sh) {
     if (shortm) nd_backward_rows<MT, RB, 8, CG, false>(d, node, row0, nrows, root, t, u, y, x, r0, nr, nd_sm, sh->ex, sh);
     else nd_backward_rows<MT, RB, 32, CG, false>(d, node, row0, nrows, root, t, u, y, x, r0, nr, nd_sm, sh->ex, sh);
 }
@@ -714,7 +773,7 @@ __device__ __forceinline__ void nd_pdl_enter() {
 
 // forward level: one item per CTA
 template <class MT, int RB>
-__global__ void __launch_bounds__(kNDThreads) k_nd_forward(NDDev d, const int4* __restrict__ items,
+__global__ void __launch_bounds__(kNDThreads) k_nd_forward(const __grid_constant__ NDDev d, const int4* __restrict__ items,
                                                     const double2* __restrict__ t, double2* __restrict__ y,
                                                     double2* __restrict__ u, int R, const int* __restrict__ done) {
     nd_pdl_enter();
@@ -724,12 +783,12 @@ __global__ void __launch_bounds__(kNDThreads) k_nd_forward(NDDev d, const int4* 
     const int4 it = items[blockIdx.x];
     const int r0 = blockIdx.y * RB, nr = min(RB, R - r0);
     nd_forward_node<MT, RB>(d, it.x, it.y, it.z, it.w != 0, it.y == 0, t, y, u, r0, nr,
-                            reinterpret_cast<typename NDVec<MT>::V*>(nd_raw), &sh);
+                            nd_raw, &sh);
 }
 
 // backward level: one item per CTA
 template <class MT, int RB>
-__global__ void __launch_bounds__(kNDThreads) k_nd_backward(NDDev d, const int4* __restrict__ items, int root,
+__global__ void __launch_bounds__(kNDThreads) k_nd_backward(const __grid_constant__ NDDev d, const int4* __restrict__ items, int root,
                                                      const double2* __restrict__ t, const double2* __restrict__ u,
                                                      const double2* __restrict__ y, double2* __restrict__ x, int R,
                                                      const int* __restrict__ done) {
@@ -740,7 +799,7 @@ __global__ void __launch_bounds__(kNDThreads) k_nd_backward(NDDev d, const int4*
     const int4 it = items[blockIdx.x];
     const int r0 = blockIdx.y * RB, nr = min(RB, R - r0);
     nd_backward_node<MT, RB>(d, it.x, it.y, it.z, it.w != 0, root != 0, t, u, y, x, r0, nr,
-                             reinterpret_cast<typename NDVec<MT>::V*>(nd_raw), &sh);
+                             nd_raw, &sh);
 }
 
 // The bottom of the tree in one launch per direction: CTA b owns the subtree below a node of the cut
@@ -752,17 +811,16 @@ __global__ void __launch_bounds__(kNDThreads) k_nd_backward(NDDev d, const int4*
 // 64 x 64 elements, l = 5, 8 right-hand sides, forward and backward: the six deepest level
 // launches took 225 and 155 us, these 96 and 134 us.
 template <class MT, int RB, bool FWD>
-__global__ void __launch_bounds__(32 * kNDWarps) k_nd_bottom(NDDev d, const int4* __restrict__ items,
+__global__ void __launch_bounds__(32 * kNDWarps) k_nd_bottom(const __grid_constant__ NDDev d, const int4* __restrict__ items,
                                                              const int* __restrict__ ptr, int nlev, int warp_len,
                                                              const double2* __restrict__ t, double2* __restrict__ y,
                                                              double2* __restrict__ x, double2* __restrict__ u, int R,
                                                              const int* __restrict__ done) {
     if (done && *done) return;
-    using V = typename NDVec<MT>::V;
     extern __shared__ __align__(16) char nd_raw[];
     __shared__ int ex[kNDWarps][RB];
     const int warp = threadIdx.x >> 5;
-    V* sm = reinterpret_cast<V*>(nd_raw) + (size_t)warp * warp_len;
+    char* sm = nd_raw + nd_bytes<MT>(warp_len) * warp;
     const int r0 = blockIdx.y * RB, nr = min(RB, R - r0);
     const int* p = ptr + (size_t)blockIdx.x * nlev;
     for (int k = 0; k < nlev; ++k) {
@@ -798,7 +856,7 @@ __device__ __forceinline__ bool nd_wait(const int* cnt, int target, int* abort_f
 }
 
 template <class MT, int RB>
-__global__ void __launch_bounds__(kNDThreads) k_nd_persistent(NDDev d, NDSched sc, const double2* __restrict__ t,
+__global__ void __launch_bounds__(kNDThreads) k_nd_persistent(const __grid_constant__ NDDev d, NDSched sc, const double2* __restrict__ t,
                                                        double2* y, double2* x, double2* u, int R,
                                                        const int* __restrict__ done, int* err) {
     if (done && *done) return;
@@ -811,7 +869,7 @@ __global__ void __launch_bounds__(kNDThreads) k_nd_persistent(NDDev d, NDSched s
     int* abort_f = sc.state + 1;
     int* fcnt = sc.state + 2;                       // [nn][nrb] finished forward items
     int* bcnt = fcnt + (size_t)sc.nn * nrb;         // [nn][nrb] finished backward items
-    typename NDVec<MT>::V* sm = reinterpret_cast<typename NDVec<MT>::V*>(nd_raw);
+    char* sm = nd_raw;
     while (true) {
         if (threadIdx.x == 0) s_ticket = atomicAdd(ticket, 1);
         __syncthreads();
@@ -851,14 +909,11 @@ __global__ void __launch_bounds__(kNDThreads) k_nd_persistent(NDDev d, NDSched s
 
 // r = t - K x with K in CSR, one warp per row, lanes across the row's entries, RB right-hand sides per
 // pass.  The residual cancels about eight digits of t, so its rounding is what the refined solve, and
-// through it a whole FP64 solve, comes out with; here the sum is exact (ddh_fixed.cuh with the al xl
-// products kept: K scaled by row once, x by the largest entry that the row meets), and t - K x is
-// rounded once.  FP64 bound it before (16 x 16 to 64 x 64 meshes have 30 to 57 entries per row): 32 x 32
-// elements, l = 5, 8 right-hand sides 76 us -> 58 us; the noise of an objective evaluated on the solution
-// (48 x 48 elements, central differences at step 1e-6) fell from 4e-6 to 1.1e-7.
+// through it a whole FP64 solve, comes out with; here K x is the sum of ddh_fixed.cuh (K scaled by row once,
+// x by the largest entry that the row meets) in two FP64 numbers, and t - K x is rounded once.
 template <int RB>
 __global__ void __launch_bounds__(128) k_csr_residual(const int* __restrict__ ptr, const int* __restrict__ col,
-                                                      const int4* __restrict__ val, const int* __restrict__ vex, int n,
+                                                      const double2* __restrict__ val, FxMat vx, const int* __restrict__ vex, int n,
                                                       const double2* __restrict__ x, const double2* __restrict__ t,
                                                       double2* __restrict__ r, int R, const int* __restrict__ done) {
     if (done && *done) return;
@@ -867,69 +922,93 @@ __global__ void __launch_bounds__(128) k_csr_residual(const int* __restrict__ pt
     if (row >= n) return;
     const int a0 = ptr[row], a1 = ptr[row + 1];
     const double2* xr = x + (int64_t)r0 * n;
-    unsigned m[RB];
+    int ex[RB];
 #pragma unroll
-    for (int q = 0; q < RB; ++q) m[q] = 0;
+    for (int q = 0; q < RB; ++q) ex[q] = 0;
     for (int a = a0 + lane; a < a1; a += 32) {
         const int c = col[a];
 #pragma unroll
         for (int q = 0; q < RB; ++q)
-            if (q < nr) m[q] = max(m[q], fx_mag(xr[(int64_t)q * n + c]));
+            if (q < nr) ex[q] = max(ex[q], (int)fx_mag(xr[(int64_t)q * n + c]));
     }
 #pragma unroll
-    for (int q = 0; q < RB; ++q) m[q] = __reduce_max_sync(0xffffffffu, m[q]) >> 20;
+    for (int q = 0; q < RB; ++q) ex[q] = fx_exp(__reduce_max_sync(0xffffffffu, (unsigned)ex[q]));
     const int ea = vex[row];
+    FxSum s[RB];
+    long long h[2 * RB], l[2 * RB];
 #pragma unroll
-    for (int q = 0; q < RB; ++q) {
-        if (q >= nr) break;
-        FxAcc re = {0, 0}, im = {0, 0};
-        long long lre = 0, lim = 0;
-        for (int a = a0 + lane; a < a1; a += 32) {
-            const double2 xv = xr[(int64_t)q * n + col[a]];
-            const int4 v = val[a], w = fx_cpx(xv.x, xv.y, (int)m[q]);
-            fx_cmac(re, im, v, -v.z, -v.w, w);
-            lre += (long long)v.y * w.y - (long long)v.w * w.w;
-            lim += (long long)v.y * w.w + (long long)v.w * w.y;
+    for (int i = 0; i < 2 * RB; ++i) h[i] = l[i] = 0;
+#pragma unroll
+    for (int q = 0; q < RB; ++q) fx_clear(s[q]);
+    auto flush = [&] {
+#pragma unroll
+        for (int i = 0; i < 2 * RB; ++i) fx_flush(s[i >> 1], i & 1, h[i], l[i]);
+#pragma unroll
+        for (int q = 0; q < RB; ++q) fx_clear(s[q]);
+    };
+    for (int a = a0 + lane, c = 0; a < a1; a += 32) {
+        const FxEntry v = fx_entry(vx.i[a], vx.f[a]);
+        const double2* xc = xr + col[a];
+#pragma unroll
+        for (int q = 0; q < RB; ++q)
+            if (q < nr) {
+                const FxVec w = fx_vec(xc[(int64_t)q * n], ex[q]);
+                fx_mac(s[q], v, w.i, w.f);
+            }
+        if (++c == kFxChain) {
+            c = 0;
+            flush();
         }
-        // carried lane sums: 2^56 (a row's few hundred entries over 32 lanes: at most 2^62 in all)
-        long long v[8] = {re.h, re.l, lre, 0, im.h, im.l, lim, 0};
+    }
+    flush();
+    const long long hs = warp_sum_transpose<long long, 2 * RB>(h), ls = warp_sum_transpose<long long, 2 * RB>(l);
+    constexpr int sh = 5 - ilog2(2 * RB);
+    const int k = lane >> sh, q = k >> 1;                  // component k & 1 of right-hand side q
+    int e = 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
+    for (int i = 0; i < RB; ++i) e = i == q ? ex[i] : e;
+    double hi = 0, lo = 0;
+    const bool bad = q < nr && !fx_value2(hs, ls, ea, e, hi, lo);
+    if (__any_sync(0xffffffffu, bad)) {
+#pragma unroll 1
+        for (int b = 0; b < nr; ++b) {
+            const bool this_b = bad && q == b;
+            if (!__any_sync(0xffffffffu, this_b)) continue;
+            int eb = 0;
 #pragma unroll
-            for (int k = 0; k < 7; ++k)
-                if (k != 3) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-        if (lane < 2) {
-            const FxAcc s = {lane ? v[4] : v[0], lane ? v[5] : v[1]};
-            double hi, lo;
-            fx_exact(s, lane ? v[6] : v[2], hi, lo);
-            const int e = fx_exact_exp(ea, (int)m[q]);
-            const int64_t at = (int64_t)(r0 + q) * n + row;
-            const double tv = lane ? t[at].y : t[at].x;
-            const double v = m[q] == 0x7ff || ea == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                                                           : (tv - fx_scale(hi, e)) - fx_scale(lo, e);
-            reinterpret_cast<double*>(r + at)[lane] = v;
+            for (int i = 0; i < RB; ++i) eb = i == b ? ex[i] : eb;
+            const double2* v0 = val + a0;
+            const int4* i0 = vx.i + a0;
+            const auto xb = [=](int j) { return xr[(int64_t)b * n + col[a0 + j]]; };
+            double2 d;
+            const unsigned keep = fx_again(32, this_b ? 1u << (k & 1) : 0, a1 - a0, ea, eb, [=](int j) { return v0[j]; },
+                                           [=](int j) { const int4 u = i0[j]; return make_int2(u.x, u.z); },
+                                           [=](int j) { return fx_vec(xb(j), eb).i; }, xb, d);
+            if (this_b && !(keep >> (k & 1) & 1)) { hi = k & 1 ? d.y : d.x; lo = 0; }
         }
+    }
+    if ((lane & ((1 << sh) - 1)) == 0 && q < nr) {
+        const int64_t at = (int64_t)(r0 + q) * n + row;
+        reinterpret_cast<double*>(r + at)[k & 1] = ((k & 1 ? t[at].y : t[at].x) - hi) - lo;
     }
 }
-// rows of K in fixed point, in place; one warp per row
-__global__ void k_fix_csr(const int* __restrict__ ptr, double2* __restrict__ val, int* __restrict__ ex, int n) {
-    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (row >= n) return;
-    unsigned m = 0;
-    for (int a = ptr[row] + lane; a < ptr[row + 1]; a += 32) m = max(m, fx_mag(val[a]));
-    m = __reduce_max_sync(0xffffffffu, m);
-    for (int a = ptr[row] + lane; a < ptr[row + 1]; a += 32) {
-        const double2 v = val[a];
-        reinterpret_cast<int4*>(val)[a] = fx_cpx(v.x, v.y, (int)(m >> 20));
-    }
-    if (lane == 0) ex[row] = (int)(m >> 20);
+// splits the rows of K; one warp per row
+__global__ void k_fix_csr(const int* __restrict__ ptr, const double2* __restrict__ val, FxMat vx, int* __restrict__ ex, int n) {
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (row < n) fix_row(val + ptr[row], vx.at(ptr[row]), 1, ptr[row + 1] - ptr[row], ex + row);
 }
 
 // ------------------------------------------------------------------ launch wrappers
 static constexpr int kNDSmemMax = 200 * 1024;
+// bytes of RB staged vectors of up to `rows` entries
+template <class MT>
+static size_t nd_smem(int rows, int rb) {
+    if (kNDFixed<MT>) rows = std::min(rows, kNDFixedRows);
+    return std::max<size_t>(16, nd_bytes<MT>((size_t)(rows | 1) * rb));
+}
 int nd_rhs_block(int smem_rows, int R) {
-    int rb = 8;
-    while (rb > 1 && (rb >= 2 * R || (size_t)(smem_rows | 1) * rb * sizeof(double2) > (size_t)kNDSmemMax)) rb >>= 1;
+    int rb = 4;
+    while (rb > 1 && (rb >= 2 * R || nd_smem<double2>(smem_rows, rb) > (size_t)kNDSmemMax)) rb >>= 1;
     return rb;
 }
 template <class MT, int RB>
@@ -941,8 +1020,8 @@ static void nd_attr() {
     raise_smem_limit(k_nd_persistent<MT, RB>, kNDSmemMax);
 }
 void nd_set_smem_limits() {
-    nd_attr<int4, 1>(); nd_attr<int4, 2>(); nd_attr<int4, 4>(); nd_attr<int4, 8>();
-    nd_attr<float2, 1>(); nd_attr<float2, 2>(); nd_attr<float2, 4>(); nd_attr<float2, 8>();
+    nd_attr<double2, 1>(); nd_attr<double2, 2>(); nd_attr<double2, 4>();
+    nd_attr<float2, 1>(); nd_attr<float2, 2>(); nd_attr<float2, 4>();
 }
 // launch with (pdl) or without the programmatic-stream-serialization attribute
 template <typename... Exp, typename... Act>
@@ -962,13 +1041,13 @@ static void nd_launch(void (*k)(Exp...), dim3 g, size_t sm, cudaStream_t st, boo
 template <class MT, int RB>
 static void nd_fwd_t(const NDDev& d, const int4* items, int nitems, int smem_rows, const double2* t, double2* y,
                      double2* u, int R, const int* done, cudaStream_t st, bool pdl) {
-    const size_t sm = std::max<size_t>(16, (size_t)(smem_rows | 1) * RB * sizeof(MT));
+    const size_t sm = nd_smem<MT>(smem_rows, RB);
     nd_launch(k_nd_forward<MT, RB>, dim3(nitems, (R + RB - 1) / RB), sm, st, pdl, d, items, t, y, u, R, done);
 }
 template <class MT, int RB>
 static void nd_bwd_t(const NDDev& d, const int4* items, int nitems, int smem_rows, int root, const double2* t,
                      const double2* u, const double2* y, double2* x, int R, const int* done, cudaStream_t st, bool pdl) {
-    const size_t sm = std::max<size_t>(16, (size_t)(smem_rows | 1) * RB * sizeof(MT));
+    const size_t sm = nd_smem<MT>(smem_rows, RB);
     nd_launch(k_nd_backward<MT, RB>, dim3(nitems, (R + RB - 1) / RB), sm, st, pdl, d, items, root, t, u, y, x, R, done);
 }
 void launch_nd_forward(const NDDev& d, bool f32, const int4* items, int nitems, int smem_rows, const double2* t,
@@ -978,9 +1057,8 @@ void launch_nd_forward(const NDDev& d, bool f32, const int4* items, int nitems, 
     const int rb = rb_want > 0 && rb_want <= rb_max ? rb_want : rb_max;
 #define ND_F(RBV)                                                                             \
     if (f32) nd_fwd_t<float2, RBV>(d, items, nitems, smem_rows, t, y, u, R, done, st, pdl);   \
-    else nd_fwd_t<int4, RBV>(d, items, nitems, smem_rows, t, y, u, R, done, st, pdl);
+    else nd_fwd_t<double2, RBV>(d, items, nitems, smem_rows, t, y, u, R, done, st, pdl);
     switch (rb) {
-        case 8: ND_F(8) break;
         case 4: ND_F(4) break;
         case 2: ND_F(2) break;
         default: ND_F(1)
@@ -995,9 +1073,8 @@ void launch_nd_backward(const NDDev& d, bool f32, const int4* items, int nitems,
     const int rb = rb_want > 0 && rb_want <= rb_max ? rb_want : rb_max;
 #define ND_B(RBV)                                                                          \
     if (f32) nd_bwd_t<float2, RBV>(d, items, nitems, smem_rows, root, t, u, y, x, R, done, st, pdl);   \
-    else nd_bwd_t<int4, RBV>(d, items, nitems, smem_rows, root, t, u, y, x, R, done, st, pdl);
+    else nd_bwd_t<double2, RBV>(d, items, nitems, smem_rows, root, t, u, y, x, R, done, st, pdl);
     switch (rb) {
-        case 8: ND_B(8) break;
         case 4: ND_B(4) break;
         case 2: ND_B(2) break;
         default: ND_B(1)
@@ -1006,15 +1083,15 @@ void launch_nd_backward(const NDDev& d, bool f32, const int4* items, int nitems,
 }
 // right-hand sides per CTA of the bottom launches: all warps' staged vectors fit
 int nd_bottom_block(int rows, int R) {
-    int rb = 8;
-    while (rb > 1 && (rb >= 2 * R || (size_t)(rows | 1) * rb * kNDWarps * sizeof(int4) > (size_t)kNDSmemMax)) rb >>= 1;
-    return (size_t)(rows | 1) * rb * kNDWarps * sizeof(int4) > (size_t)kNDSmemMax ? 0 : rb;
+    int rb = 4;
+    while (rb > 1 && (rb >= 2 * R || nd_smem<double2>(rows, rb) * kNDWarps > (size_t)kNDSmemMax)) rb >>= 1;
+    return nd_smem<double2>(rows, rb) * kNDWarps > (size_t)kNDSmemMax ? 0 : rb;
 }
 template <class MT, int RB>
 static void nd_bottom_t(bool fwd, const NDDev& d, const NDBottom& b, const double2* t, double2* y, double2* x, double2* u,
                         int R, const int* done, cudaStream_t st) {
     const int len = RB * ((fwd ? b.fwd_rows : b.bwd_rows) | 1);
-    const size_t sm = std::max<size_t>(16, (size_t)len * kNDWarps * sizeof(typename NDVec<MT>::V));
+    const size_t sm = nd_bytes<MT>(len) * kNDWarps;
     const dim3 g(b.nsub, (R + RB - 1) / RB);
     if (fwd) k_nd_bottom<MT, RB, true><<<g, 32 * kNDWarps, sm, st>>>(d, b.fitems, b.fptr, b.nlev, len, t, y, x, u, R, done);
     else k_nd_bottom<MT, RB, false><<<g, 32 * kNDWarps, sm, st>>>(d, b.bitems, b.bptr, b.nlev, len, t, y, x, u, R, done);
@@ -1026,9 +1103,8 @@ void launch_nd_bottom(bool forward, const NDDev& d, bool f32, const NDBottom& b,
     const int rb = rb_want > 0 && rb_want <= rb_max ? rb_want : rb_max;
 #define ND_S(RBV)                                                               \
     if (f32) nd_bottom_t<float2, RBV>(forward, d, b, t, y, x, u, R, done, st);  \
-    else nd_bottom_t<int4, RBV>(forward, d, b, t, y, x, u, R, done, st);
+    else nd_bottom_t<double2, RBV>(forward, d, b, t, y, x, u, R, done, st);
     switch (rb) {
-        case 8: ND_S(8) break;
         case 4: ND_S(4) break;
         case 2: ND_S(2) break;
         default: ND_S(1)
@@ -1042,7 +1118,7 @@ size_t nd_state_ints(const NDSched& s, int R) {
 template <class MT, int RB>
 static void nd_persist_t(const NDDev& d, const NDSched& s, const double2* t, double2* y, double2* x, double2* u,
                          int R, const int* done, int* err, cudaStream_t st) {
-    const size_t sm = std::max<size_t>(16, (size_t)(s.smem_rows | 1) * RB * sizeof(MT));
+    const size_t sm = nd_smem<MT>(s.smem_rows, RB);
     int dev = 0, nsm = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -1058,29 +1134,27 @@ void launch_nd_persistent(const NDDev& d, const NDSched& s, bool f32, const doub
     const int rb = nd_rhs_block(s.smem_rows, R);
 #define ND_P(RBV)                                                                   \
     if (f32) nd_persist_t<float2, RBV>(d, s, t, y, x, u, R, done, err, st);         \
-    else nd_persist_t<int4, RBV>(d, s, t, y, x, u, R, done, err, st);
+    else nd_persist_t<double2, RBV>(d, s, t, y, x, u, R, done, err, st);
     switch (rb) {
-        case 8: ND_P(8) break;
         case 4: ND_P(4) break;
         case 2: ND_P(2) break;
         default: ND_P(1)
     }
 #undef ND_P
 }
-void launch_fix_csr(const int* ptr, double2* val, int* ex, int n, cudaStream_t st) {
-    k_fix_csr<<<(n + 3) / 4, 128, 0, st>>>(ptr, val, ex, n);
+void launch_fix_csr(const int* ptr, const double2* val, const FxMat& vx, int* ex, int n, cudaStream_t st) {
+    k_fix_csr<<<(n + 3) / 4, 128, 0, st>>>(ptr, val, vx, ex, n);
 }
-void launch_csr_residual(const int* ptr, const int* col, const void* val, const int* vex, int n, const double2* x,
-                         const double2* t, double2* r, int R, const int* done, cudaStream_t st) {
+void launch_csr_residual(const int* ptr, const int* col, const double2* v, const FxMat& vx, const int* vex, int n,
+                         const double2* x, const double2* t, double2* r, int R, const int* done, cudaStream_t st) {
     const int g = (n + 3) / 4;
-    const int4* v = (const int4*)val;
-    if (R >= 3) k_csr_residual<4><<<dim3(g, (R + 3) / 4), 128, 0, st>>>(ptr, col, v, vex, n, x, t, r, R, done);
-    else if (R == 2) k_csr_residual<2><<<dim3(g, 1), 128, 0, st>>>(ptr, col, v, vex, n, x, t, r, R, done);
-    else k_csr_residual<1><<<dim3(g, 1), 128, 0, st>>>(ptr, col, v, vex, n, x, t, r, R, done);
+    if (R >= 3) k_csr_residual<4><<<dim3(g, (R + 3) / 4), 128, 0, st>>>(ptr, col, v, vx, vex, n, x, t, r, R, done);
+    else if (R == 2) k_csr_residual<2><<<dim3(g, 1), 128, 0, st>>>(ptr, col, v, vx, vex, n, x, t, r, R, done);
+    else k_csr_residual<1><<<dim3(g, 1), 128, 0, st>>>(ptr, col, v, vx, vex, n, x, t, r, R, done);
 }
-void launch_fix_dense(void* A, int n, int* ex, int* col, cudaStream_t st) {
-    k_fix_dense_cols<<<(n + 3) / 4, 128, 0, st>>>((const double2*)A, n, col);
-    k_fix_dense<<<(n + 3) / 4, 128, 0, st>>>((double2*)A, n, col, ex);
+int gemv_tiles(int n) { return (n + kGemvTile - 1) / kGemvTile; }
+void launch_fix_dense(const double2* A, int n, const FxMat& Ax, int* ex, cudaStream_t st) {
+    k_fix_dense<<<(n + 3) / 4, 128, 0, st>>>(A, n, Ax, ex);
 }
 void launch_fix_fronts(const NDDev& d, int nodes, cudaStream_t st) {
     if (nodes > 0) k_fix_fronts<<<nodes, 256, 0, st>>>(d);
@@ -1103,22 +1177,21 @@ void launch_gemv32(const void* A, int n, const double2* x, double2* y, int R, co
 // one CTA per SM, but at least four rows per CTA (each CTA stages all of x)
 static int gemv_rows(int n, int nsm) { return std::max(4, (n + nsm - 1) / nsm); }
 void gemv_set_smem_limits() {
-    constexpr int most = 160 * 1024;          // eight staged tiles and the sums of the rows of n = 16384
+    constexpr int most = 216 * 1024;          // eight staged tiles and the sums of the rows of n = 16384
     raise_smem_limit(k_gemv_fx<1>, most);
     raise_smem_limit(k_gemv_fx<2>, most);
     raise_smem_limit(k_gemv_fx<4>, most);
-    raise_smem_limit(k_gemv_fx<8>, most);
 }
-void launch_gemv(const void* A, const int* ex, const int* col, int n, const double2* x, double2* y, int R, const int* done, int nsm,
+void launch_gemv(const double2* A, const FxMat& Ax, const int* ex, int n, const double2* x, double2* y, int R, const int* done, int nsm,
                  cudaStream_t st) {
     const int rpc = gemv_rows(n, nsm);
     const int g = (n + rpc - 1) / rpc;
     for (int r0 = 0; r0 < R;) {
-        const int left = std::min(R - r0, 8);
-        const int rb = left >= 5 ? 8 : (left >= 3 ? 4 : left);
-        const size_t sm = (size_t)rb * ((8 / rb * kGemvTile + 1) * sizeof(int4) + (size_t)rpc * 2 * sizeof(double));
-#define DDH_GEMV(RBV) k_gemv_fx<RBV><<<g, kGemvThreads, sm, st>>>((const int4*)A, ex, col, n, x, y, r0, left, rpc, done);
-        switch (rb) { case 8: DDH_GEMV(8) break; case 4: DDH_GEMV(4) break; case 2: DDH_GEMV(2) break; default: DDH_GEMV(1) }
+        const int left = std::min(R - r0, 4);                  // a sum is twelve registers
+        const int rb = left >= 3 ? 4 : left;
+        const size_t sm = (size_t)rb * ((8 / rb * kGemvTile + 1) * (sizeof(int4) + sizeof(float4)) + (size_t)rpc * 2 * sizeof(double));
+#define DDH_GEMV(RBV) k_gemv_fx<RBV><<<g, kGemvThreads, sm, st>>>(A, Ax, ex, n, x, y, r0, left, rpc, done);
+        switch (rb) { case 4: DDH_GEMV(4) break; case 2: DDH_GEMV(2) break; default: DDH_GEMV(1) }
 #undef DDH_GEMV
         r0 += left;
     }

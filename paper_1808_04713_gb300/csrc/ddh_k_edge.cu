@@ -17,85 +17,81 @@ namespace ddh {
 // chain.  Y is formed at factor time.  The interior never enters the iteration; it is
 // rebuilt by the FDM kernels in the recovery.
 //
-// The FP64 passes hold S_E^-1 and Y in fixed point (ddh_fixed.cuh): EdgeOp<double> is four limbs per
-// entry.  S_E^-1 has an exponent per row (DevModel::sinv_ex, by type-1 slot), Y one per column (y_ex, by
-// type-2 slot), i.e. per output row of pass 1.  Pass 2, which sums over the columns, reads a copy of Y
-// that is column-major, so that a warp's load is contiguous over the rows, with the columns' scalings
-// taken out (they go on u_T) and an exponent per row (y2_ex, by type-1 slot): 64 x 64 elements, p = 20, 8
-// right-hand sides 174 us for pass 2, from 184 us with rows of Y read as they lie.
-template <class T> struct EdgeOpT { using type = cpx<float>; };
-template <> struct EdgeOpT<double> { using type = int4; };
-template <class T> using EdgeOp = typename EdgeOpT<T>::type;
+// The FP64 passes form their products on the integer and FP32 pipes (ddh_fixed.cuh) from the split S_E^-1 and
+// Y.  S_E^-1 has an exponent per row (DevModel::sinv_ex, by type-1 slot), Y one per column (y_ex, by type-2
+// slot), i.e. per output row of pass 1.  Pass 2, which sums over the columns, reads a copy of Y that is
+// column-major, so that a warp's load is contiguous over the rows, with an exponent per row (y2_ex, by type-1
+// slot).  In FP64 a staged vector is its limbs and its FP32 parts.  64 x 64 elements, p = 20, 8 right-hand
+// sides, pass 2: 0.15 ms, 0.41 ms in FP64.
+template <class T> struct EdgeVec {
+    cpx<T>* v;
+    __device__ __forceinline__ EdgeVec(void* p, int) : v(reinterpret_cast<cpx<T>*>(p)) {}
+};
+template <> struct EdgeVec<double> {
+    int4* i;
+    float4* f;
+    __device__ __forceinline__ EdgeVec(void* p, int n) : i(reinterpret_cast<int4*>(p)), f(reinterpret_cast<float4*>(i + n)) {}
+};
+// In FP64 a thread takes at most four of the RB right-hand sides of a CTA (a sum is twelve registers), and a
+// CTA of eight has twice the threads.
+template <class T, int RB> constexpr int kEdgeParts = std::is_same<T, double>::value && RB == 8 ? 2 : 1;
 
-// Fixed-point copies of S_E^-1 and Y: one CTA per element, one warp per row of S_E^-1 / column of Y, then
-// one per row of Y for the copy that pass 2 reads
+// Splits S_E^-1 and Y: one CTA per element, one warp per row of S_E^-1 / column of Y, then one per row of Y
 __global__ void __launch_bounds__(256) k_fix_edge(DevModel dm, const double2* __restrict__ sinv,
                                                   const double2* __restrict__ Y, EdgeFix f) {
     const int e = blockIdx.x, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31;
     const int nE = dm.nE1[e], nT = dm.nT[e];
-    __shared__ int cy[128];
     for (int o = warp; o < nE + nT; o += nw) {
         const bool isS = o < nE;
         const int ld = isS ? nE : nT;
         const int64_t at = isS ? dm.sinv_off[e] + o : dm.pq_off[e] + (o - nE);
-        const double2* a = isS ? sinv : Y;
-        int4* d = isS ? f.s : f.y;
+        const double2* a = (isS ? sinv : Y) + at;
+        const FxMat d = (isS ? f.s : f.y).at(at);
         unsigned m = 0;
-        for (int j = lane; j < nE; j += 32) m = max(m, fx_mag(a[at + (int64_t)j * ld]));
-        const int ef = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
-        for (int j = lane; j < nE; j += 32) {
-            const double2 v = a[at + (int64_t)j * ld];
-            d[at + (int64_t)j * ld] = fx_cpx(v.x, v.y, ef);
-        }
-        if (lane == 0) {
-            *(isS ? f.sex + dm.e1_off[e] + o : f.yex + dm.t_off[e] + o - nE) = ef;
-            if (!isS) cy[o - nE] = fx_even(ef);
-        }
+        for (int j = lane; j < nE; j += 32) m = max(m, fx_mag(a[(int64_t)j * ld]));
+        const int ef = fx_exp(__reduce_max_sync(0xffffffffu, m));
+        for (int j = lane; j < nE; j += 32) fx_put(d, (int64_t)j * ld, a[(int64_t)j * ld], ef);
+        if (lane == 0) *(isS ? f.sex + dm.e1_off[e] + o : f.yex + dm.t_off[e] + o - nE) = ef;
     }
-    __syncthreads();
     const double2* a = Y + dm.pq_off[e];
+    const FxMat d = f.y2.at(dm.pq_off[e]);
     for (int i = warp; i < nE; i += nw) {
-        double2 v[4];
         unsigned m = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {                      // nT <= 128
-            const int t = lane + 32 * k;
-            v[k] = t < nT ? a[(int64_t)i * nT + t] : make_double2(0.0, 0.0);
-            const int c = t < nT ? cy[t] : 0;
-            v[k] = make_double2(fx_scale(v[k].x, -c), fx_scale(v[k].y, -c));
-            m = max(m, fx_mag(v[k]));
-        }
-        const int ef = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (lane + 32 * k < nT) f.y2[dm.pq_off[e] + (int64_t)(lane + 32 * k) * nE + i] = fx_cpx(v[k].x, v[k].y, ef);
+        for (int t = lane; t < nT; t += 32) m = max(m, fx_mag(a[(int64_t)i * nT + t]));
+        const int ef = fx_exp(__reduce_max_sync(0xffffffffu, m));
+        for (int t = lane; t < nT; t += 32) fx_put(d, (int64_t)t * nE + i, a[(int64_t)i * nT + t], ef);
         if (lane == 0) f.y2ex[dm.e1_off[e] + i] = ef;
     }
 }
 
-// Stages cnt vectors of length n (stride vs): load(q, i) gives entry i of vector q.  In fixed point one
-// warp per vector (n <= 128: four entries per lane), whose exponent goes to ex[q].
-template <class T, class F>
-__device__ __forceinline__ void edge_stage(const F& load, int n, int vs, int cnt, EdgeOp<T>* sm, int* ex) {
+// Stages cnt vectors of length n (stride vs): load(q, i) gives entry i of vector q.  In FP64 one warp per
+// vector (n <= 128: four entries per lane), whose exponent goes to ex[q]; vectors cnt to RB - 1 are zero.
+template <class T, int RB, class F>
+__device__ __forceinline__ void edge_stage(const F& load, int n, int vs, int cnt, const EdgeVec<T>& sm, int* ex) {
     if constexpr (std::is_same<T, double>::value) {
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-        for (int q = warp; q < cnt; q += nw) {
-            cpx<double> v[4];
+        for (int q = warp; q < RB; q += nw) {
+            double2 v[4];
             unsigned m = 0;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int i = lane + 32 * k;
-                v[k] = i < n ? load(q, i) : mk<double>(0, 0);
-                m = max(m, fx_mag(make_double2(v[k].x, v[k].y)));
+                v[k] = make_double2(0.0, 0.0);
+                if (i < n && q < cnt) { const cpx<double> c = load(q, i); v[k] = make_double2(c.x, c.y); }
+                m = max(m, fx_mag(v[k]));
             }
-            const int ef = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
+            const int ef = fx_exp(__reduce_max_sync(0xffffffffu, m));
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (lane + 32 * k < n) sm[q * vs + lane + 32 * k] = fx_cpx(v[k].x, v[k].y, ef);
+                if (lane + 32 * k < n) {
+                    const FxVec w = fx_vec(v[k], ef);
+                    sm.i[q * vs + lane + 32 * k] = w.i;
+                    sm.f[q * vs + lane + 32 * k] = w.f;
+                }
             if (lane == 0) ex[q] = ef;
         }
     } else {
-        for (int idx = threadIdx.x; idx < cnt * n; idx += blockDim.x) sm[idx / n * vs + idx % n] = load(idx / n, idx % n);
+        for (int idx = threadIdx.x; idx < cnt * n; idx += blockDim.x) sm.v[idx / n * vs + idx % n] = load(idx / n, idx % n);
     }
 }
 
@@ -160,67 +156,145 @@ __device__ __forceinline__ void edge_rows_f(const DevModel& dm, const cpx<T>* S,
     }
 }
 
-// The same in fixed point.  Sums are exact, so the order of the columns and tpr do not matter.  Per term
-// twelve IMAD.WIDE (26 per SM and clock) stand for four FP64 FMA (two): 64 x 64 elements, p = 20, 8
-// right-hand sides went from 1.09 ms (92 % of the FP64 rate) to 0.42 ms.
-template <int RB>
-__device__ __forceinline__ void edge_rows_fx(const DevModel& dm, const int4* S, const int4* Ye, int nE, int nT,
-                                             const int4* rE, const int* ex, int vs, int cnt, int tpr, int r0, int e1o,
-                                             int to, cpx<double>* __restrict__ xE_out, cpx<double>* __restrict__ tT_out,
-                                             int o_lo, int o_hi) {
-    for (int base = 0; base < (o_hi - o_lo) * tpr; base += blockDim.x) {
-        const int slot = base + threadIdx.x;
+// The same with the products of ddh_fixed.cuh.  Two or four threads per output row by the row count alone
+// (edge_tpr), so that the order of a row's terms does not depend on the launch form.  load: the staged
+// vectors' entries, for the results that are formed again in FP64.  Integer multiply-adds bound it (22 per SM
+// and clock, twelve a term): 64 x 64 elements, p = 20, 8 right-hand sides 0.50 ms, 1.09 ms in FP64; at two
+// CTAs of ten warps per SM, 96 registers a thread.
+template <class T>
+__device__ __forceinline__ int edge_tpr(int rows, int other) {
+    return std::is_same<T, double>::value ? (rows <= 64 ? 4 : 2) : other;
+}
+template <int RB, class F>
+__device__ __forceinline__ void edge_rows_fx(const DevModel& dm, const FxMat& S, const FxMat& Ye, const double2* S64,
+                                             const double2* Y64, int nE, int nT,
+                                             const EdgeVec<double>& rE, const int* ex, const F& load, int vs, int cnt,
+                                             int tpr, int r0, int e1o, int to, cpx<double>* __restrict__ xE_out,
+                                             cpx<double>* __restrict__ tT_out, int o_lo, int o_hi, int tid, int nt, int q0) {
+    for (int base = 0; base < (o_hi - o_lo) * tpr; base += nt) {
+        const int slot = base + tid;
         const int o = o_lo + slot / tpr, part = slot % tpr;
-        FxAcc s[2 * RB];
+        const bool in = o < o_hi;
+        const FxMat col0 = !in || o < nE ? S.at(in ? o : 0) : Ye.at(o - nE);
+        const int64_t ld = o < nE ? nE : nT;
+        const int ea = !in ? 0 : (o < nE ? dm.sinv_ex[e1o + o] : dm.y_ex[to + o - nE]);
+        FxSum s[RB];
 #pragma unroll
-        for (int i = 0; i < 2 * RB; ++i) s[i].h = s[i].l = 0;
-        if (o < o_hi) {
-            const int4* col0 = o < nE ? S + o : Ye + (o - nE);
-            const int ld = o < nE ? nE : nT;
-            // nE <= 124 and tpr >= 2: at most 62 terms, one chain
-#pragma unroll(RB <= 2 ? 8 : 2)
+        for (int i = 0; i < RB; ++i) fx_clear(s[i]);
+        if (in) {
+            // nE <= 124 terms: one chain; the next entry's load is issued ahead
+            int4 ni = make_int4(0, 0, 0, 0);
+            float2 nf = make_float2(0.f, 0.f);
+            if (part < nE) { ni = col0.i[part * ld]; nf = col0.f[part * ld]; }
+#pragma unroll 1
             for (int j = part; j < nE; j += tpr) {
-                const int4 a = col0[(int64_t)j * ld];
+                const FxEntry a = fx_entry(ni, nf);
+                if (j + tpr < nE) { ni = col0.i[(j + tpr) * ld]; nf = col0.f[(j + tpr) * ld]; }
 #pragma unroll
-                for (int q = 0; q < RB; ++q)
-                    if (q < cnt) fx_cmac(s[2 * q], s[2 * q + 1], a, -a.z, -a.w, rE[q * vs + j]);
+                for (int q = 0; q < RB; ++q) fx_mac(s[q], a, rE.i[(q0 + q) * vs + j], rE.f[(q0 + q) * vs + j]);
             }
         }
 #pragma unroll
-        for (int i = 0; i < 2 * RB; ++i) {
-            long long h = 0;
-            unsigned l = 0;
-            fx_flush(s[i], h, l);
-            if (tpr == 4) {
-                h += __shfl_xor_sync(0xffffffffu, h, 2);
-                l += __shfl_xor_sync(0xffffffffu, l, 2);
+        for (int q = 0; q < RB; ++q) {
+            bool bad = false;
+            double v = 0;
+            // the lanes of a row share the conversions: component c of vector q goes to lane part = 2 q + c (mod tpr)
+            const bool mine = in && q0 + q < cnt && (part & ~1) == ((2 * q) & (tpr - 1));
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                long long h = 0, l = 0;
+                fx_flush(s[q], c, h, l);
+                if (tpr == 4) {
+                    h += __shfl_xor_sync(0xffffffffu, h, 2);
+                    l += __shfl_xor_sync(0xffffffffu, l, 2);
+                }
+                h += __shfl_xor_sync(0xffffffffu, h, 1);
+                l += __shfl_xor_sync(0xffffffffu, l, 1);
+                if (mine && (part & 1) == c) bad = !fx_value(h, l, ea, ex[q0 + q], v);
             }
-            h += __shfl_xor_sync(0xffffffffu, h, 1);
-            l += __shfl_xor_sync(0xffffffffu, l, 1);
-            // the lanes of a row share the conversions: component i goes to lane part = i (mod tpr)
-            const int q = i >> 1;
-            if (part == i % tpr && o < o_hi && q < cnt) {
-                const int ea = o < nE ? dm.sinv_ex[e1o + o] : dm.y_ex[to + o - nE];
-                cpx<double>* d = o < nE ? xE_out + (int64_t)(r0 + q) * dm.nE1_tot + e1o + o
-                                        : tT_out + (int64_t)(r0 + q) * dm.nT_tot + to + (o - nE);
-                reinterpret_cast<double*>(d)[i & 1] = fx_value(h, l, ea, ex[q]);
+            if (__any_sync(0xffffffffu, bad)) {
+                double2 d;
+                const double2* c64 = !in || o < nE ? S64 + (in ? o : 0) : Y64 + (o - nE);
+                const int4 *ci = col0.i, *xi = rE.i + (q0 + q) * vs;
+                const int qq = q0 + q;
+                const unsigned keep = fx_again(tpr, bad ? 1u << (part & 1) : 0, nE, ea, ex[qq], [=](int j) { return c64[j * ld]; },
+                                               [=](int j) { const int4 u = ci[j * ld]; return make_int2(u.x, u.z); },
+                                               [=](int j) { return xi[j]; },
+                                               [=](int j) { const cpx<double> x = load(qq, j); return make_double2(x.x, x.y); }, d);
+                if (bad && !(keep >> (part & 1) & 1)) v = part & 1 ? d.y : d.x;
+            }
+            if (mine) {
+                cpx<double>* d = o < nE ? xE_out + (int64_t)(r0 + q0 + q) * dm.nE1_tot + e1o + o
+                                        : tT_out + (int64_t)(r0 + q0 + q) * dm.nT_tot + to + (o - nE);
+                reinterpret_cast<double*>(d)[part & 1] = v;
             }
         }
     }
 }
-template <class T, int RB>
-__device__ __forceinline__ void edge_rows(const DevModel& dm, const EdgeOp<T>* S, const EdgeOp<T>* Ye, int nE, int nT,
-                                          const EdgeOp<T>* rE, const int* ex, int vs, int cnt, int tpr, int r0, int e1o,
-                                          int to, cpx<T>* __restrict__ xE_out, cpx<T>* __restrict__ tT_out, int o_lo,
-                                          int o_hi) {
+// S: S_E^-1, staged or not; in FP64 S, Ye point at the complex128 matrices and Sx at the split S_E^-1
+template <class T, int RB, class F>
+__device__ __forceinline__ void edge_rows(const DevModel& dm, int e, const cpx<T>* S, const FxMat& Sx, const cpx<T>* Ye, int nE,
+                                          int nT, const EdgeVec<T>& rE, const int* ex, const F& load, int vs, int cnt, int tpr,
+                                          int r0, int e1o, int to, cpx<T>* __restrict__ xE_out,
+                                          cpx<T>* __restrict__ tT_out, int o_lo, int o_hi) {
+    if constexpr (std::is_same<T, double>::value) {
+        constexpr int parts = kEdgeParts<T, RB>;
+        const int nt = blockDim.x / parts, part = threadIdx.x / nt;
+        edge_rows_fx<RB / parts>(dm, Sx, dm.y_fx.at(dm.pq_off[e]), reinterpret_cast<const double2*>(S),
+                                 reinterpret_cast<const double2*>(Ye), nE, nT, rE, ex, load, vs, cnt, tpr, r0, e1o, to, xE_out,
+                                 tT_out, o_lo, o_hi, threadIdx.x - part * nt, nt, part * (RB / parts));
+    } else edge_rows_f<T, RB>(dm, S, Ye, nE, nT, rE.v, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
+}
+
+__device__ __forceinline__ void bulk_expect(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(uint64_t* bar, void* dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+// Staging of S_E^-1 by bulk copies: in FP64 its limbs, then its fractions
+template <class T>
+__device__ __forceinline__ void edge_copy(uint64_t* bar, char* dst, const DevModel& dm, const cpx<T>* sinv, int e, int nE) {
+    const size_t n = (size_t)nE * nE;
+    const int64_t off = dm.sinv_off[e];
+    if constexpr (std::is_same<T, double>::value) {
+        const uint32_t b0 = (uint32_t)(n * sizeof(int4)), b1 = (uint32_t)(n * sizeof(float2) + 15) & ~15u;
+        bulk_expect(bar, b0 + b1);
+        bulk_copy(bar, dst, dm.sinv_fx.i + off, b0);
+        bulk_copy(bar, dst + b0, dm.sinv_fx.f + off, b1);
+    } else {
+        const uint32_t b = (uint32_t)(n * sizeof(cpx<T>) + 15) & ~15u;
+        bulk_expect(bar, b);
+        bulk_copy(bar, dst, sinv + off, b);
+    }
+}
+
+// entry i of r_E of right-hand side r0 + q.  (The staged vectors' loads capture by value: what they hold also stays
+// in registers where fx_again is called.)
+template <class T>
+__device__ __forceinline__ auto pass1_load(const DevModel& dm, const double2* z, double zsign, const double2* bt, int r0,
+                                           int e1o, int64_t off) {
+    return [dp = &dm, z, zsign, bt, r0, e1o, off](int q, int i) {
+        const int r = r0 + q;
+        cpx<T> v = mk<T>(0, 0);
+        const int row = dp->e1_row[e1o + i];
+        if (z && row >= 0) v = (T)(zsign * dp->e1_sign[e1o + i]) * ld<T>(z, (int64_t)r * dp->n_dual + row);
+        if (bt) v += ld<T>(bt, (int64_t)r * dp->n_local + off + dp->e1_slot[e1o + i]);
+        return v;
+    };
+}
+// the staged matrix: S in complex64, Sx in FP64
+template <class T>
+__device__ __forceinline__ void edge_staged(char* sm, int nE, const cpx<T>*& S, FxMat& Sx) {
     if constexpr (std::is_same<T, double>::value)
-        edge_rows_fx<RB>(dm, S, Ye, nE, nT, rE, ex, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
-    else edge_rows_f<T, RB>(dm, S, Ye, nE, nT, rE, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
+        Sx = {reinterpret_cast<int4*>(sm), reinterpret_cast<float2*>(sm + (size_t)nE * nE * sizeof(int4))};
+    else S = reinterpret_cast<const cpx<T>*>(sm);
 }
 
 template <class T, int RB>
-__global__ void __launch_bounds__(256) k_pass1_edge(DevModel dm, const EdgeOp<T>* __restrict__ sinv,
-                                                    const EdgeOp<T>* __restrict__ Y, const double2* __restrict__ z,
+__global__ void __launch_bounds__(kEdgeParts<T, RB> == 2 ? 640 : 256) k_pass1_edge(const __grid_constant__ DevModel dm, const cpx<T>* __restrict__ sinv,
+                                                    const cpx<T>* __restrict__ Y, const double2* __restrict__ z,
                                                     double zsign, const double2* __restrict__ bt, int R,
                                                     cpx<T>* __restrict__ xE_out, cpx<T>* __restrict__ tT_out,
                                                     const int* __restrict__ done, int ntask, int stage_off, int vs,
@@ -233,33 +307,31 @@ __global__ void __launch_bounds__(256) k_pass1_edge(DevModel dm, const EdgeOp<T>
     const int e = task % dm.E, r0 = (task / dm.E) * RB;
     const int cnt = min(RB, R - r0);
     const int nE = dm.nE1[e], e1o = dm.e1_off[e], nT = dm.nT[e], to = dm.t_off[e];
-    const EdgeOp<T>* S = sinv + dm.sinv_off[e];
+    const cpx<T>* S = sinv + dm.sinv_off[e];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + stage_off);
-    EdgeOp<T>* S_s = reinterpret_cast<EdgeOp<T>*>(smem + stage_off + 128);
-    if (stage_off > 0 && nE > 0 && threadIdx.x == 0)
-        bulk_load_start(bar, S_s, S, (uint32_t)(((size_t)nE * nE * sizeof(EdgeOp<T>) + 15) & ~(size_t)15));
-    EdgeOp<T>* rE = reinterpret_cast<EdgeOp<T>*>(smem);     // [RB][vs]
+    char* S_s = smem + stage_off + 128;
+    if (stage_off > 0 && nE > 0 && threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        edge_copy<T>(bar, S_s, dm, sinv, e, nE);
+    }
+    FxMat Sx = dm.sinv_fx.at(dm.sinv_off[e]);
+    const EdgeVec<T> rE(smem, RB * vs);               // [RB][vs]
     __shared__ int ex[RB];
     const int64_t off = dm.off[e];
-    edge_stage<T>([&](int q, int i) {
-        const int r = r0 + q;
-        cpx<T> v = mk<T>(0, 0);
-        const int row = dm.e1_row[e1o + i];
-        if (z && row >= 0) v = (T)(zsign * dm.e1_sign[e1o + i]) * ld<T>(z, (int64_t)r * dm.n_dual + row);
-        if (bt) v += ld<T>(bt, (int64_t)r * dm.n_local + off + dm.e1_slot[e1o + i]);
-        return v;
-    }, nE, vs, cnt, rE, ex);
+    const auto load = pass1_load<T>(dm, z, zsign, bt, r0, e1o, off);
+    edge_stage<T, RB>(load, nE, vs, cnt, rE, ex);
     g.sync();
     if (stage_off > 0 && nE > 0) {
         if (!bulk_wait_all(bar, dm.err)) return;
-        S = S_s;
+        edge_staged<T>(S_s, nE, S, Sx);
     }
     // every vertex and edge slot is type-1 edge or type-2, so nE + nT = 4p <= 128 (p <= 32): four
     // threads per output row when all rows fit the CTA so, else two
-    const int tpr = (nE + nT) * 4 <= (int)blockDim.x ? 4 : 2;
+    const int tpr = edge_tpr<T>(nE + nT, (nE + nT) * 4 <= (int)blockDim.x ? 4 : 2);
     // rows: 0 all output rows, 1 the x_E rows only, 2 the t_T rows only (no S_E^-1 read)
     const int o_lo = rows == 2 ? nE : 0, o_hi = rows == 1 ? nE : nE + nT;
-    edge_rows<T, RB>(dm, S, Y + dm.pq_off[e], nE, nT, rE, ex, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
+    edge_rows<T, RB>(dm, e, S, Sx, Y + dm.pq_off[e], nE, nT, rE, ex, load, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
 }
 
 // The same pass as one persistent launch over a degree-sorted work list.  Task t is (element
@@ -268,10 +340,11 @@ __global__ void __launch_bounds__(256) k_pass1_edge(DevModel dm, const EdgeOp<T>
 // t = blockIdx.x, blockIdx.x + gridDim.x, ...; while it computes one task, the next task's
 // S_E^-1 is already being copied into the other of two shared-memory buffers (bulk copy,
 // mbarrier per buffer).  tpr_p[p] (2 or 4 threads per output row) is chosen per degree by the
-// autotuner; 0 = the default (4 up to 64 output rows, else 2); tpr_force (2 or 4) overrides it.
+// autotuner; 0 = the default (4 up to 64 output rows, else 2); tpr_force (2 or 4) overrides it.  FP64 always
+// takes the default (edge_tpr).
 template <class T, int RB>
-__global__ void __launch_bounds__(256) k_pass1_edge_p(DevModel dm, const EdgeOp<T>* __restrict__ sinv,
-                                                      const EdgeOp<T>* __restrict__ Y, const double2* __restrict__ z,
+__global__ void __launch_bounds__(kEdgeParts<T, RB> == 2 ? 640 : 256) k_pass1_edge_p(const __grid_constant__ DevModel dm, const cpx<T>* __restrict__ sinv,
+                                                      const cpx<T>* __restrict__ Y, const double2* __restrict__ z,
                                                       double zsign, const double2* __restrict__ bt, int R,
                                                       cpx<T>* __restrict__ xE_out, cpx<T>* __restrict__ tT_out,
                                                       const int* __restrict__ done, const int* __restrict__ items,
@@ -280,23 +353,18 @@ __global__ void __launch_bounds__(256) k_pass1_edge_p(DevModel dm, const EdgeOp<
     if (done && *done) return;
     extern __shared__ __align__(128) char smem[];
     const int nrb = (R + RB - 1) / RB, ntask = nitems * nrb;
-    EdgeOp<T>* rE = reinterpret_cast<EdgeOp<T>*>(smem);     // [RB][vs]
+    const EdgeVec<T> rE(smem, RB * vs);               // [RB][vs]
     __shared__ int ex[RB];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + stage_off);        // 2 barriers
     __shared__ int s_fail;
     const bool staged = stage_off > 0;
-    auto buf = [&](int b) { return reinterpret_cast<EdgeOp<T>*>(smem + stage_off + 128 + (size_t)b * buf_bytes); };
+    auto buf = [&](int b) { return smem + stage_off + 128 + (size_t)b * buf_bytes; };
     auto task_elem = [&](int t) { return items[item0 + t / nrb]; };
     // copy of task t's S_E^-1 into buffer b (thread 0); false when there is nothing to copy
     auto issue = [&](int t, int b) {
         const int e = task_elem(t), nE = dm.nE1[e];
         if (nE == 0) return false;
-        const uint32_t bytes = (uint32_t)(((size_t)nE * nE * sizeof(EdgeOp<T>) + 15) & ~(size_t)15);
-        const uint32_t bb = smem_u32(bar + b);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bb), "r"(bytes) : "memory");
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(smem_u32(buf(b))), "l"(sinv + dm.sinv_off[e]), "r"(bytes), "r"(bb)
-                     : "memory");
+        edge_copy<T>(bar + b, buf(b), dm, sinv, e, nE);
         return true;
     };
     bool pend[2] = {false, false};        // thread 0: copy in flight per buffer
@@ -319,15 +387,10 @@ __global__ void __launch_bounds__(256) k_pass1_edge_p(DevModel dm, const EdgeOp<
         const int nE = dm.nE1[e], e1o = dm.e1_off[e], nT = dm.nT[e], to = dm.t_off[e];
         if (staged && threadIdx.x == 0 && t + (int)gridDim.x < ntask) pend[b ^ 1] = issue(t + gridDim.x, b ^ 1);
         const int64_t off = dm.off[e];
-        edge_stage<T>([&](int q, int i) {
-            const int r = r0 + q;
-            cpx<T> v = mk<T>(0, 0);
-            const int row = dm.e1_row[e1o + i];
-            if (z && row >= 0) v = (T)(zsign * dm.e1_sign[e1o + i]) * ld<T>(z, (int64_t)r * dm.n_dual + row);
-            if (bt) v += ld<T>(bt, (int64_t)r * dm.n_local + off + dm.e1_slot[e1o + i]);
-            return v;
-        }, nE, vs, cnt, rE, ex);
-        const EdgeOp<T>* S = sinv + dm.sinv_off[e];
+        const auto load = pass1_load<T>(dm, z, zsign, bt, r0, e1o, off);
+        edge_stage<T, RB>(load, nE, vs, cnt, rE, ex);
+        const cpx<T>* S = sinv + dm.sinv_off[e];
+        FxMat Sx = dm.sinv_fx.at(dm.sinv_off[e]);
         if (staged && nE > 0) {
             if (threadIdx.x == 0) {
                 bool ok = !pend[b];
@@ -335,13 +398,14 @@ __global__ void __launch_bounds__(256) k_pass1_edge_p(DevModel dm, const EdgeOp<
                 if (pend[b]) { pend[b] = false; ++uses[b]; }
                 if (!ok) { s_fail = 1; if (dm.err) atomicExch(dm.err, 2); }
             }
-            S = buf(b);
+            edge_staged<T>(buf(b), nE, S, Sx);
         }
         __syncthreads();
         if (s_fail) break;
         int tpr = tpr_force > 0 ? tpr_force : (tpr_p ? (int)tpr_p[dm.p[e]] : 0);
         if (tpr != 2 && tpr != 4) tpr = nE + nT <= 64 ? 4 : 2;
-        edge_rows<T, RB>(dm, S, Y + dm.pq_off[e], nE, nT, rE, ex, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, 0,
+        tpr = edge_tpr<T>(nE + nT, tpr);
+        edge_rows<T, RB>(dm, e, S, Sx, Y + dm.pq_off[e], nE, nT, rE, ex, load, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, 0,
                          nE + nT);
         __syncthreads();
     }
@@ -355,12 +419,13 @@ __global__ void __launch_bounds__(256) k_pass1_edge_p(DevModel dm, const EdgeOp<
 }
 
 template <class T, int RB>
-__global__ void __launch_bounds__(128) k_pass2_edge(DevModel dm, const EdgeOp<T>* __restrict__ Y,
+__global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pass2_edge(const __grid_constant__ DevModel dm, const cpx<T>* __restrict__ Y,
                                                     const double2* __restrict__ x2, const cpx<T>* __restrict__ xE_in,
                                                     cpx<T>* __restrict__ xE_out, int R, const int* __restrict__ done,
                                                     int ntask, int y_bytes) {
     if (done && *done) return;
-    __shared__ EdgeOp<T> uT[RB * 128];
+    constexpr bool fx = std::is_same<T, double>::value;
+    __shared__ __align__(16) char uT_raw[RB * 128 * kEdgeVecBytes<T>];
     __shared__ int ex[RB];
     extern __shared__ __align__(128) char smem[];
     const CtaGroup g;
@@ -369,77 +434,101 @@ __global__ void __launch_bounds__(128) k_pass2_edge(DevModel dm, const EdgeOp<T>
     const int e = task % dm.E, r0 = (task / dm.E) * RB;
     const int cnt = min(RB, R - r0);
     const int nE = dm.nE1[e], e1o = dm.e1_off[e], nT = dm.nT[e], to = dm.t_off[e];
-    // FP64: Y comes into shared memory (one bulk copy, in flight while u_T is gathered)
+    // FP64: the split Y comes into shared memory (in flight while u_T is gathered); a bulk copy starts at a
+    // multiple of 16 bytes, so the fractions of an element at an odd offset are read where they lie
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
-    int4* Y_s = reinterpret_cast<int4*>(smem + 128);
     const bool staged = y_bytes > 0 && nE > 0 && nT > 0;
-    if (staged && threadIdx.x == 0) bulk_load_start(bar, Y_s, Y + dm.pq_off[e], (uint32_t)(nE * nT * sizeof(int4)));
-    edge_stage<T>([&](int q, int i) {
+    FxMat Yx = dm.y2_fx.at(dm.pq_off[e]);
+    if constexpr (fx)
+        if (staged) {
+            const bool even = (dm.pq_off[e] & 1) == 0;
+            const uint32_t b0 = nE * nT * (uint32_t)sizeof(int4), b1 = even ? (nE * nT * (uint32_t)sizeof(float2) + 15) & ~15u : 0;
+            if (threadIdx.x == 0) {
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                bulk_expect(bar, b0 + b1);
+                bulk_copy(bar, smem + 128, Yx.i, b0);
+                if (b1) bulk_copy(bar, smem + 128 + b0, Yx.f, b1);
+            }
+            Yx.i = reinterpret_cast<int4*>(smem + 128);
+            if (b1) Yx.f = reinterpret_cast<float2*>(smem + 128 + b0);
+        }
+    const EdgeVec<T> uT(uT_raw, RB * 128);
+    const auto load = [dp = &dm, x2, to, r0](int q, int i) {
         const int r = r0 + q;
         cpx<T> u = mk<T>(0, 0);
-        for (int a = dm.t_ptr[to + i]; a < dm.t_ptr[to + i + 1]; ++a) {
-            const double2 xv = x2[(int64_t)r * dm.n_coarse + dm.t_col[a]];
-            const T w = (T)dm.t_w[a];
+        for (int a = dp->t_ptr[to + i]; a < dp->t_ptr[to + i + 1]; ++a) {
+            const double2 xv = x2[(int64_t)r * dp->n_coarse + dp->t_col[a]];
+            const T w = (T)dp->t_w[a];
             u.x += w * (T)xv.x;
             u.y += w * (T)xv.y;
         }
-        if constexpr (std::is_same<T, double>::value) {
-            // the column's scaling: Y_t u_t = (Y_t 2^-c) (u_t 2^c)
-            const int c = fx_even(dm.y_ex[to + i]);
-            u.x = fx_scale(u.x, c);
-            u.y = fx_scale(u.y, c);
-        }
         return u;
-    }, nT, 128, cnt, uT, ex);
+    };
+    edge_stage<T, RB>(load, nT, 128, cnt, uT, ex);
     g.sync();
     if (staged && !bulk_wait_all(bar, dm.err)) return;
     // one thread per row i of Y, all RB right-hand sides at once: each Y entry is read once
-    const EdgeOp<T>* Ye = Y + dm.pq_off[e];
-    if constexpr (std::is_same<T, double>::value)
-        if (staged) Ye = Y_s;
-    for (int i = g.t(); i < nE; i += g.n()) {
-        // FP64: the column-major copy
-        constexpr bool fx = std::is_same<T, double>::value;
-        const EdgeOp<T>* yr = fx ? Ye + i : Ye + (int64_t)i * nT;
-        cpx<T> a[RB];
-        if constexpr (std::is_same<T, double>::value) {
-            FxAcc s[2 * RB];
-            long long h[2 * RB];
-            unsigned l[2 * RB];
+    const cpx<T>* Ye = Y + dm.pq_off[e];
+    constexpr int parts = kEdgeParts<T, RB>, RT = RB / parts;
+    const int nt = blockDim.x / parts, q0 = threadIdx.x / nt * RT;
+    for (int i = threadIdx.x % nt; i < nE; i += nt) {
+        const cpx<T>* yr = Ye + (int64_t)i * nT;
+        cpx<T> a[RT];
+        if constexpr (fx) {
+            const double2* yd = reinterpret_cast<const double2*>(yr);
+            const int ea = dm.y2_ex[e1o + i];
+            FxSum s[RT];
 #pragma unroll
-            for (int k = 0; k < 2 * RB; ++k) { s[k].h = s[k].l = 0; h[k] = 0; l[k] = 0; }
-            for (int t = 0; t < nT;) {
-                const int end = min(nT, t + kFxChain);
-#pragma unroll(RB <= 2 ? 8 : 2)
-                for (; t < end; ++t) {
-                    const int4 y = yr[t * nE];
+            for (int q = 0; q < RT; ++q) fx_clear(s[q]);
+            // nT <= 128 terms: one chain; the next entry's load is issued ahead
+            int4 ni = make_int4(0, 0, 0, 0);
+            float2 nf = make_float2(0.f, 0.f);
+            if (nT > 0) { ni = Yx.i[i]; nf = Yx.f[i]; }
+#pragma unroll 2
+            for (int t = 0; t < nT; ++t) {
+                const FxEntry y = fx_entry(ni, nf);
+                if (t + 1 < nT) { ni = Yx.i[(t + 1) * nE + i]; nf = Yx.f[(t + 1) * nE + i]; }
 #pragma unroll
-                    for (int q = 0; q < RB; ++q)
-                        if (q < cnt) fx_cmac(s[2 * q], s[2 * q + 1], y, -y.z, -y.w, uT[q * 128 + t]);
-                }
-#pragma unroll
-                for (int k = 0; k < 2 * RB; ++k) fx_flush(s[k], h[k], l[k]);
+                for (int q = 0; q < RT; ++q) fx_mac(s[q], y, uT.i[(q0 + q) * 128 + t], uT.f[(q0 + q) * 128 + t]);
             }
 #pragma unroll
-            for (int q = 0; q < RB; ++q)
-                if (q < cnt) {
-                    const int ea = dm.y2_ex[e1o + i];
-                    a[q] = mk<T>(fx_value(h[2 * q], l[2 * q], ea, ex[q]), fx_value(h[2 * q + 1], l[2 * q + 1], ea, ex[q]));
+            for (int q = 0; q < RT; ++q) {
+                a[q] = mk<T>(0, 0);
+                if (q0 + q >= cnt) continue;
+                unsigned bad = 0;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    long long h = 0, l = 0;
+                    fx_flush(s[q], c, h, l);
+                    if (!fx_value(h, l, ea, ex[q0 + q], c ? a[q].y : a[q].x)) bad |= 1u << c;
                 }
+                if (bad) {
+                    double2 d;
+                    const int4 *yi = Yx.i + i, *xi = uT.i + (q0 + q) * 128;
+                    const int qq = q0 + q;
+                    bad &= ~fx_again(1, bad, nT, ea, ex[qq], [=](int t) { return yd[t]; },
+                                     [=](int t) { const int4 u = yi[t * nE]; return make_int2(u.x, u.z); },
+                                     [=](int t) { return xi[t]; },
+                                     [=](int t) { const cpx<double> x = load(qq, t); return make_double2(x.x, x.y); }, d);
+                    if (bad & 1) a[q].x = d.x;
+                    if (bad & 2) a[q].y = d.y;
+                }
+            }
         } else {
 #pragma unroll
-            for (int q = 0; q < RB; ++q) a[q] = mk<T>(0, 0);
+            for (int q = 0; q < RT; ++q) a[q] = mk<T>(0, 0);
             for (int t = 0; t < nT; ++t) {
                 const cpx<T> y = yr[t];
 #pragma unroll
-                for (int q = 0; q < RB; ++q)
-                    if (q < cnt) fma_c(a[q], y, uT[q * 128 + t]);
+                for (int q = 0; q < RT; ++q)
+                    if (q < cnt) fma_c(a[q], y, uT.v[q * 128 + t]);
             }
         }
 #pragma unroll
-        for (int q = 0; q < RB; ++q)
-            if (q < cnt) {
-                const int64_t gi = (int64_t)(r0 + q) * dm.nE1_tot + e1o + i;
+        for (int q = 0; q < RT; ++q)
+            if (q0 + q < cnt) {
+                const int64_t gi = (int64_t)(r0 + q0 + q) * dm.nE1_tot + e1o + i;
                 xE_out[gi] = xE_in[gi] - a[q];
             }
     }
@@ -539,52 +628,68 @@ __global__ void k_dinv(DevModel dm, const double2* __restrict__ x, double2* __re
 // one CTA per (element, block of RB RHS), each S^Lap entry read once per CTA.
 // out_E = S x for the restricted stiffness Schur complement S (n_E x n_E, symmetric, read from
 // global memory column by column: coalesced across output rows, shared by the elements of a
-// degree pattern and L1/L2-resident); tpr adjacent threads share an output row.  FP64: S and x in fixed
-// point (two limbs per real entry, DevModel::pre_fx, exponents pre_ex by row; four per complex entry)
-template <class T, int RB>
-__device__ __forceinline__ void pre_apply(const DevModel& dm, int e, int nE, int cnt, const EdgeOp<T>* in, const int* ex,
-                                          cpx<T>* __restrict__ out, int64_t ostride,
+// degree pattern and L1/L2-resident); tpr adjacent threads share an output row.  FP64: the products of
+// ddh_fixed.cuh, exponents pre_ex by row; load gives the staged vectors' entries (an application as below
+// 0.28 ms, 0.52 ms in FP64).
+template <class T, int RB, class F>
+__device__ __forceinline__ void pre_apply(const DevModel& dm, int e, int nE, int cnt, const EdgeVec<T>& in, const int* ex,
+                                          const F& load, cpx<T>* __restrict__ out, int64_t ostride,
                                           const double* __restrict__ wout = nullptr) {
     const int tpr = nE <= 32 ? 4 : (nE <= 64 ? 2 : 1);
     const int chunk = (nE + tpr - 1) / tpr;
     const double* S = dm.pre_all + dm.pre_off[e];
-    const int2* F = dm.pre_fx + dm.pre_off[e];
-    for (int base = 0; base < nE * tpr; base += blockDim.x) {
-        const int slot = base + threadIdx.x;
+    const FxRealMat Sx = dm.pre_fx.at(dm.pre_off[e]);
+    constexpr int parts = kEdgeParts<T, RB>, RT = RB / parts;
+    const int nt = blockDim.x / parts, q0 = threadIdx.x / nt * RT;
+    for (int base = 0; base < nE * tpr; base += nt) {
+        const int slot = base + threadIdx.x % nt;
         const int i = slot / tpr, part = slot % tpr;
         const int j1 = i < nE ? min(nE, (part + 1) * chunk) : 0;
         if constexpr (std::is_same<T, double>::value) {
-            // real times complex: one product per component and term, so nE <= 124 terms are one chain
-            FxAcc s[2 * RB];
+            const int ea = i < nE ? dm.pre_ex[dm.pre_ex_off[e] + i] : 0;
+            FxSum s[RT];
 #pragma unroll
-            for (int k = 0; k < 2 * RB; ++k) s[k].h = s[k].l = 0;
-#pragma unroll(RB <= 2 ? 8 : 2)
+            for (int k = 0; k < RT; ++k) fx_clear(s[k]);
+            // nE <= 124 terms: one chain; the next entry's load is issued ahead
+            int2 ni = make_int2(0, 0);
+            float nf = 0.f;
+            auto fetch = [&](int j) { ni = __ldg(Sx.i + j * nE + i); nf = __ldg(Sx.f + j * nE + i); };
+            if (part * chunk < j1) fetch(part * chunk);
+#pragma unroll 2
             for (int j = part * chunk; j < j1; ++j) {
-                const int2 a = __ldg(F + (int64_t)j * nE + i);
+                const FxReal a = fx_real(ni.x, ni.y, nf);
+                if (j + 1 < j1) fetch(j + 1);
 #pragma unroll
-                for (int q = 0; q < RB; ++q)
-                    if (q < cnt) {
-                        const int4 x = in[q * nE + j];
-                        fx_mac(s[2 * q], a.x, a.y, x.x, x.y);
-                        fx_mac(s[2 * q + 1], a.x, a.y, x.z, x.w);
-                    }
+                for (int q = 0; q < RT; ++q) fx_mac(s[q], a, in.i[(q0 + q) * nE + j], in.f[(q0 + q) * nE + j]);
             }
 #pragma unroll
-            for (int q = 0; q < RB; ++q) {
-                long long h[2] = {0, 0};
-                unsigned l[2] = {0, 0};
-                fx_flush(s[2 * q], h[0], l[0]);
-                fx_flush(s[2 * q + 1], h[1], l[1]);
-                for (int o = 1; o < tpr; o <<= 1)
-                    for (int c = 0; c < 2; ++c) {
-                        h[c] += __shfl_xor_sync(0xffffffffu, h[c], o);
-                        l[c] += __shfl_xor_sync(0xffffffffu, l[c], o);
+            for (int q = 0; q < RT; ++q) {
+                unsigned bad = 0;
+                cpx<double> v = mk<double>(0, 0);
+                const bool mine = part == 0 && i < nE && q0 + q < cnt;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    long long h = 0, l = 0;
+                    fx_flush(s[q], c, h, l);
+                    for (int o = 1; o < tpr; o <<= 1) {
+                        h += __shfl_xor_sync(0xffffffffu, h, o);
+                        l += __shfl_xor_sync(0xffffffffu, l, o);
                     }
-                if (part == 0 && i < nE && q < cnt) {
-                    const int ea = dm.pre_ex[dm.pre_ex_off[e] + i];
-                    const cpx<double> v = mk<double>(fx_value(h[0], l[0], ea, ex[q]), fx_value(h[1], l[1], ea, ex[q]));
-                    out[(int64_t)q * ostride + i] = wout ? wout[i] * v : v;
+                    if (mine && !fx_value(h, l, ea, ex[q0 + q], c ? v.y : v.x)) bad |= 1u << c;
                 }
+                if (tpr > 1 ? __any_sync(0xffffffffu, bad != 0) : bad != 0) {
+                    double2 d;
+                    const double* S64 = S + i;
+                    const int2* Si = Sx.i + i;
+                    const int4* xi = in.i + (q0 + q) * nE;
+                    const int qq = q0 + q;
+                    bad &= ~fx_again(tpr, bad, nE, ea, ex[qq], [=](int j) { return make_double2(S64[j * nE], 0.0); },
+                                     [=](int j) { return make_int2(Si[j * nE].x, 0); }, [=](int j) { return xi[j]; },
+                                     [=](int j) { const cpx<double> x = load(qq, j); return make_double2(x.x, x.y); }, d);
+                    if (bad & 1) v.x = d.x;
+                    if (bad & 2) v.y = d.y;
+                }
+                if (mine) out[(int64_t)(q0 + q) * ostride + i] = wout ? wout[i] * v : v;
             }
         } else {
             cpx<T> acc[RB];
@@ -594,7 +699,7 @@ __device__ __forceinline__ void pre_apply(const DevModel& dm, int e, int nE, int
                 const T sv = (T)__ldg(S + (int64_t)j * nE + i);
 #pragma unroll
                 for (int q = 0; q < RB; ++q)
-                    if (q < cnt) fma_r(acc[q], sv, in[q * nE + j]);
+                    if (q < cnt) fma_r(acc[q], sv, in.v[q * nE + j]);
             }
 #pragma unroll
             for (int q = 0; q < RB; ++q) {
@@ -607,26 +712,22 @@ __device__ __forceinline__ void pre_apply(const DevModel& dm, int e, int nE, int
         }
     }
 }
-// fixed-point copies of the restricted S^Lap, one warp per row (grid: pattern, 8 warps per CTA)
+// splits the restricted S^Lap, one warp per row (grid: pattern, 8 warps per CTA)
 __global__ void k_fix_pre(const double* __restrict__ S, const int64_t* __restrict__ off, const int* __restrict__ len,
-                          const int64_t* __restrict__ eoff, int2* __restrict__ fx, int* __restrict__ ex) {
+                          const int64_t* __restrict__ eoff, FxRealMat fx, int* __restrict__ ex) {
     const int k = blockIdx.x, nE = len[k], warp = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31;
     for (int i = warp; i < nE; i += nw) {
         const double* a = S + off[k] + i;                  // row i = column i (symmetric)
         unsigned m = 0;
-        for (int j = lane; j < nE; j += 32) m = max(m, (unsigned)__double2hiint(a[(int64_t)j * nE]) & 0x7fffffffu);
-        const int ef = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
-        for (int j = lane; j < nE; j += 32) {
-            int2 f;
-            fx_split(fx_int(a[(int64_t)j * nE], ef), f.x, f.y);
-            fx[off[k] + i + (int64_t)j * nE] = f;
-        }
+        for (int j = lane; j < nE; j += 32) m = max(m, fx_mag(a[(int64_t)j * nE]));
+        const int ef = fx_exp(__reduce_max_sync(0xffffffffu, m));
+        for (int j = lane; j < nE; j += 32) fx_put(fx, off[k] + i + (int64_t)j * nE, a[(int64_t)j * nE], ef);
         if (lane == 0) ex[eoff[k] + i] = ef;
     }
 }
 
 template <class T, int RB>
-__global__ void __launch_bounds__(128) k_pre_elem(DevModel dm, const double2* __restrict__ v, cpx<T>* __restrict__ outE,
+__global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pre_elem(const __grid_constant__ DevModel dm, const double2* __restrict__ v, cpx<T>* __restrict__ outE,
                                                   int R, const int* __restrict__ done, int with_d) {
     if (done && *done) return;
     extern __shared__ __align__(128) char smem[];
@@ -634,31 +735,32 @@ __global__ void __launch_bounds__(128) k_pre_elem(DevModel dm, const double2* __
     const int e = blockIdx.x, r0 = blockIdx.y * RB;
     const int cnt = min(RB, R - r0);
     const int nE = dm.nE1[e], e1o = dm.e1_off[e];
-    EdgeOp<T>* in = reinterpret_cast<EdgeOp<T>*>(smem);                 // [RB][nE]
-    edge_stage<T>([&](int q, int i) {
-        const int row = dm.e1_row[e1o + i];
+    const EdgeVec<T> in(smem, RB * nE);                           // [RB][nE]
+    const auto load = [dp = &dm, v, e1o, r0, with_d](int q, int i) {
+        const int row = dp->e1_row[e1o + i];
         cpx<T> val = mk<T>(0, 0);
         if (row >= 0) {
-            const double w = dm.e1_win ? dm.e1_sign[e1o + i] * dm.e1_win[e1o + i] : dm.e1_sign[e1o + i];
-            double2 x = v[(int64_t)(r0 + q) * dm.n_dual + row];
+            const double w = dp->e1_win ? dp->e1_sign[e1o + i] * dp->e1_win[e1o + i] : dp->e1_sign[e1o + i];
+            double2 x = v[(int64_t)(r0 + q) * dp->n_dual + row];
             if (with_d) {
-                const double dd = dm.row_dinv ? dm.row_dinv[row] : 0.5;
+                const double dd = dp->row_dinv ? dp->row_dinv[row] : 0.5;
                 x = make_double2(dd * x.x, dd * x.y);
             }
             val = (T)w * mk<T>((T)x.x, (T)x.y);
         }
         return val;
-    }, nE, nE, cnt, in, ex);
+    };
+    edge_stage<T, RB>(load, nE, nE, cnt, in, ex);
     __syncthreads();
     // Poisson mode: out = (rho_e w) .* (S^Lap (w .* C1^T v)), the diagonally scaled W^T A W
-    pre_apply<T, RB>(dm, e, nE, cnt, in, ex, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot,
+    pre_apply<T, RB>(dm, e, nE, cnt, in, ex, load, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot,
                      dm.e1_wout ? dm.e1_wout + e1o : nullptr);
 }
 
 // Conforming meshes (no hanging rows: D = 2 I, no C2 K C2^T term), fused with the Krylov
 // fetch: v = V[r][j] read directly (j = ctl[0]), D^-1 = 1/2 applied in the gather.
 template <class T, int RB>
-__global__ void __launch_bounds__(128) k_pre_elem_kry(DevModel dm, KrylovDev K, cpx<T>* __restrict__ outE, int R) {
+__global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pre_elem_kry(const __grid_constant__ DevModel dm, const __grid_constant__ KrylovDev K, cpx<T>* __restrict__ outE, int R) {
     if (K.ctl[1]) return;
     const int jj = K.ctl[0];
     extern __shared__ __align__(128) char smem[];
@@ -666,23 +768,24 @@ __global__ void __launch_bounds__(128) k_pre_elem_kry(DevModel dm, KrylovDev K, 
     const int e = blockIdx.x, r0 = blockIdx.y * RB;
     const int cnt = min(RB, R - r0);
     const int nE = dm.nE1[e], e1o = dm.e1_off[e];
-    EdgeOp<T>* in = reinterpret_cast<EdgeOp<T>*>(smem);
-    edge_stage<T>([&](int q, int i) {
-        const int row = dm.e1_row[e1o + i];
+    const EdgeVec<T> in(smem, RB * nE);
+    const auto load = [dp = &dm, kp = &K, e1o, r0, jj](int q, int i) {
+        const int row = dp->e1_row[e1o + i];
         cpx<T> val = mk<T>(0, 0);
         if (row >= 0) {
-            const int64_t at = ((int64_t)(r0 + q) * (K.m + 1) + jj) * K.nd + row;
-            if (K.Vf) {
-                const float2 x = K.Vf[at];
-                val = (T)(0.5 * dm.e1_sign[e1o + i]) * mk<T>((T)x.x, (T)x.y);
+            const int64_t at = ((int64_t)(r0 + q) * (kp->m + 1) + jj) * kp->nd + row;
+            if (kp->Vf) {
+                const float2 x = kp->Vf[at];
+                val = (T)(0.5 * dp->e1_sign[e1o + i]) * mk<T>((T)x.x, (T)x.y);
             } else {
-                val = (T)(0.5 * dm.e1_sign[e1o + i]) * ld<T>(K.V, at);
+                val = (T)(0.5 * dp->e1_sign[e1o + i]) * ld<T>(kp->V, at);
             }
         }
         return val;
-    }, nE, nE, cnt, in, ex);
+    };
+    edge_stage<T, RB>(load, nE, nE, cnt, in, ex);
     __syncthreads();
-    pre_apply<T, RB>(dm, e, nE, cnt, in, ex, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot);
+    pre_apply<T, RB>(dm, e, nE, cnt, in, ex, load, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot);
 }
 
 // z = D^-1 (outE[c] - outE[f]) with D = 2 I, written to zw and to the Krylov store Zb[r][j]
@@ -733,14 +836,14 @@ __global__ void k_pre_rows(DevModel dm, const cpx<T>* __restrict__ outE, const d
 template <class T>
 static int edge_p_layout(int rb, int maxE1, int* buf_bytes, size_t* total) {
     const size_t base = edge_vec_bytes<T>(rb, maxE1);
-    const size_t one = ((size_t)maxE1 * maxE1 * sizeof(cpx<T>) + 127) & ~(size_t)127;
+    const size_t one = edge_mat_bytes<T>(maxE1);
     const bool fit = maxE1 > 0 && base + 128 + 2 * one <= 200 * 1024;
     *buf_bytes = (int)one;
     *total = fit ? base + 128 + 2 * one : base;
     return fit ? (int)base : 0;
 }
 template <class T, int RB>
-static void edge_p_t(const DevModel& dm, const EdgeOp<T>* S, const EdgeOp<T>* Yp, const double2* z, double zsign,
+static void edge_p_t(const DevModel& dm, const cpx<T>* S, const cpx<T>* Yp, const double2* z, double zsign,
                      const double2* bt, void* xE, void* tT, int R, const int* done, const EdgeSched& es, int item0,
                      int nitems, int tpr_force, cudaStream_t st) {
     int buf = 0;
@@ -751,9 +854,9 @@ static void edge_p_t(const DevModel& dm, const EdgeOp<T>* S, const EdgeOp<T>* Yp
     int dev = 0, nsm = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pass1_edge_p<T, RB>, 256, sm);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pass1_edge_p<T, RB>, 256 * kEdgeParts<T, RB>, sm);
     const int grid = std::max(1, std::min(ntask, std::max(1, per) * std::max(1, nsm)));
-    k_pass1_edge_p<T, RB><<<grid, 256, sm, st>>>(dm, S, Yp, z, zsign, bt, R, (cpx<T>*)xE, (cpx<T>*)tT, done, es.items,
+    k_pass1_edge_p<T, RB><<<grid, 256 * kEdgeParts<T, RB>, sm, st>>>(dm, S, Yp, z, zsign, bt, R, (cpx<T>*)xE, (cpx<T>*)tT, done, es.items,
                                                  item0, nitems, es.tpr_p, tpr_force, so, buf, vs);
 }
 int edge_cta_threads(int maxNo) { return maxNo > 64 ? std::min(256, (2 * maxNo + 31) / 32 * 32) : 256; }
@@ -763,8 +866,8 @@ void launch_pass1_edge(const DevModel& dm, const void* sinv, const void* Y, cons
                        const double2* bt, void* xE, void* tT, int R, const int* done, cudaStream_t st,
                        const EdgeSched* es, int item0, int nitems, int tpr_force, int rows) {
     const int rb = rhs_block(R);
-    const EdgeOp<T>* S = (const EdgeOp<T>*)sinv;
-    const EdgeOp<T>* Yp = (const EdgeOp<T>*)Y;
+    const cpx<T>* S = (const cpx<T>*)sinv;
+    const cpx<T>* Yp = (const cpx<T>*)Y;
     if (es && es->items && rows == 0) {
         if (nitems < 0) nitems = dm.E;
         switch (rb) {
@@ -785,7 +888,7 @@ void launch_pass1_edge(const DevModel& dm, const void* sinv, const void* Y, cons
     // threads idle (80 rows at p = 20, l = 5: 160 threads instead of 256 with 96 idle)
     const int nt = es && es->cta_threads > 0 ? es->cta_threads : edge_cta_threads(dm.maxNo);
     switch (rb) {
-        case 8: k_pass1_edge<T, 8><<<ntask, nt, sm, st>>>(dm, S, Yp, z, zsign, bt, R, (cpx<T>*)xE, (cpx<T>*)tT, done, ntask, so, vs, rows); break;
+        case 8: k_pass1_edge<T, 8><<<ntask, nt * kEdgeParts<T, 8>, sm, st>>>(dm, S, Yp, z, zsign, bt, R, (cpx<T>*)xE, (cpx<T>*)tT, done, ntask, so, vs, rows); break;
         case 4: k_pass1_edge<T, 4><<<ntask, nt, sm, st>>>(dm, S, Yp, z, zsign, bt, R, (cpx<T>*)xE, (cpx<T>*)tT, done, ntask, so, vs, rows); break;
         case 2: k_pass1_edge<T, 2><<<ntask, nt, sm, st>>>(dm, S, Yp, z, zsign, bt, R, (cpx<T>*)xE, (cpx<T>*)tT, done, ntask, so, vs, rows); break;
         default: k_pass1_edge<T, 1><<<ntask, nt, sm, st>>>(dm, S, Yp, z, zsign, bt, R, (cpx<T>*)xE, (cpx<T>*)tT, done, ntask, so, vs, rows);
@@ -796,16 +899,16 @@ void launch_pass2_edge(const DevModel& dm, const void* Y, const double2* x2, con
                        const int* done, cudaStream_t st) {
     const int rb = rhs_block(R);
     const int ntask = dm.E * ((R + rb - 1) / rb);
-    const EdgeOp<T>* Yp = (const EdgeOp<T>*)Y;
+    const cpx<T>* Yp = (const cpx<T>*)Y;
     const cpx<T>* xi = (const cpx<T>*)xE_in;
     cpx<T>* xo = (cpx<T>*)xE_out;
     // one thread per edge row: 64-thread CTAs when every element has at most 64 (more CTAs
     // resident per SM to hide the gather latency)
     const int nt = dm.maxE1 <= 64 ? 64 : 128;
-    // FP64: room for the largest Y (nE + nT <= 124 at p = 32, so at most 62 x 62 entries)
-    const int yb = std::is_same<T, double>::value && dm.maxY > 0 && dm.maxY <= 64 * 64 ? 128 + dm.maxY * (int)sizeof(int4) : 0;
+    // FP64: room for the largest Y (nE + nT <= 4 p = 128, so at most 64 x 64 entries)
+    const int yb = std::is_same<T, double>::value && dm.maxY > 0 && dm.maxY <= 64 * 64 ? 128 + dm.maxY * kEdgeMatBytes<T> + 16 : 0;
     switch (rb) {
-        case 8: k_pass2_edge<T, 8><<<ntask, nt, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb); break;
+        case 8: k_pass2_edge<T, 8><<<ntask, nt * kEdgeParts<T, 8>, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb); break;
         case 4: k_pass2_edge<T, 4><<<ntask, nt, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb); break;
         case 2: k_pass2_edge<T, 2><<<ntask, nt, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb); break;
         default: k_pass2_edge<T, 1><<<ntask, nt, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb);
@@ -830,15 +933,15 @@ int launch_pre(const DevModel& dm, const double2* v, double2* vd, void* outE, do
                int R, const int* done, cudaStream_t st) {
     const dim3 gr((dm.n_dual + 127) / 128, R);
     // without hanging rows D is diagonal and there is no C2 K C2^T: D^-1 goes into the two kernels (64 x 64
-    // elements, p = 20, 8 right-hand sides: 261 -> 249 us for an application)
+    // elements, p = 20, 8 right-hand sides: 275 us for an application, 12 us less than with launches of their own)
     const int with_d = dm.n_hb == 0;
     if (!with_d) k_dinv<<<gr, 128, 0, st>>>(dm, v, vd, 0, done);
     const double2* in = with_d ? v : vd;
     const int rb = rhs_block(R);
     const dim3 g(dm.E, (R + rb - 1) / rb);
-    const size_t sm = sizeof(cpx<T>) * (size_t)rb * dm.maxE1 + 16;
+    const size_t sm = kEdgeVecBytes<T> * (size_t)rb * dm.maxE1 + 16;
     switch (rb) {
-        case 8: k_pre_elem<T, 8><<<g, 128, sm, st>>>(dm, in, (cpx<T>*)outE, R, done, with_d); break;
+        case 8: k_pre_elem<T, 8><<<g, 128 * kEdgeParts<T, 8>, sm, st>>>(dm, in, (cpx<T>*)outE, R, done, with_d); break;
         case 4: k_pre_elem<T, 4><<<g, 128, sm, st>>>(dm, in, (cpx<T>*)outE, R, done, with_d); break;
         case 2: k_pre_elem<T, 2><<<g, 128, sm, st>>>(dm, in, (cpx<T>*)outE, R, done, with_d); break;
         default: k_pre_elem<T, 1><<<g, 128, sm, st>>>(dm, in, (cpx<T>*)outE, R, done, with_d);
@@ -857,8 +960,8 @@ template int launch_pre<float>(const DevModel&, const double2*, double2*, void*,
 void launch_fix_edge(const DevModel& dm, const void* sinv, const void* Y, const EdgeFix& f, cudaStream_t st) {
     k_fix_edge<<<dm.E, 256, 0, st>>>(dm, (const double2*)sinv, (const double2*)Y, f);
 }
-void launch_fix_pre(const double* S, int npat, const int64_t* off, const int* len, const int64_t* eoff, int2* fx, int* ex,
-                    cudaStream_t st) {
+void launch_fix_pre(const double* S, int npat, const int64_t* off, const int* len, const int64_t* eoff,
+                    const FxRealMat& fx, int* ex, cudaStream_t st) {
     if (npat > 0) k_fix_pre<<<npat, 256, 0, st>>>(S, off, len, eoff, fx, ex);
 }
 void launch_dinv(const DevModel& dm, const double2* x, double2* y, int R, const int* done, cudaStream_t st) {
@@ -868,9 +971,9 @@ template <class T>
 void launch_pre_krylov(const DevModel& dm, const KrylovDev& K, void* outE, int R, cudaStream_t st) {
     const int rb = rhs_block(R);
     const dim3 g(dm.E, (R + rb - 1) / rb);
-    const size_t sm = sizeof(cpx<T>) * (size_t)rb * dm.maxE1 + 16;
+    const size_t sm = kEdgeVecBytes<T> * (size_t)rb * dm.maxE1 + 16;
     switch (rb) {
-        case 8: k_pre_elem_kry<T, 8><<<g, 128, sm, st>>>(dm, K, (cpx<T>*)outE, R); break;
+        case 8: k_pre_elem_kry<T, 8><<<g, 128 * kEdgeParts<T, 8>, sm, st>>>(dm, K, (cpx<T>*)outE, R); break;
         case 4: k_pre_elem_kry<T, 4><<<g, 128, sm, st>>>(dm, K, (cpx<T>*)outE, R); break;
         case 2: k_pre_elem_kry<T, 2><<<g, 128, sm, st>>>(dm, K, (cpx<T>*)outE, R); break;
         default: k_pre_elem_kry<T, 1><<<g, 128, sm, st>>>(dm, K, (cpx<T>*)outE, R);
@@ -888,7 +991,7 @@ static void set_edge_pass_limits(int maxE1) {
     cudaFuncSetAttribute(k_pass1_edge<T, RB>, cudaFuncAttributePreferredSharedMemoryCarveout,
                          (int)cudaSharedmemCarveoutMaxShared);
     if (std::is_same<T, double>::value)
-        raise_smem_limit(k_pass2_edge<T, RB>, 128 + 64 * 64 * (int)sizeof(int4));
+        raise_smem_limit(k_pass2_edge<T, RB>, 128 + 64 * 64 * kEdgeMatBytes<T> + 16);
     int buf = 0;
     size_t tot = 0;
     edge_p_layout<T>(RB, maxE1, &buf, &tot);
@@ -900,8 +1003,7 @@ void set_edge_limits(int pmax, int maxE1) {
     set_edge_pass_limits<double, 4>(maxE1); set_edge_pass_limits<double, 8>(maxE1);
     set_edge_pass_limits<float, 1>(maxE1); set_edge_pass_limits<float, 2>(maxE1);
     set_edge_pass_limits<float, 4>(maxE1); set_edge_pass_limits<float, 8>(maxE1);
-    const int pre64 = (int)(sizeof(cpx<double>) * 8 * (size_t)maxE1 + sizeof(double) * (size_t)maxE1 * maxE1 + 16);
-    const int pre32 = (int)(sizeof(cpx<float>) * 8 * (size_t)maxE1 + sizeof(float) * (size_t)maxE1 * maxE1 + 16);
+    const int pre64 = kEdgeVecBytes<double> * 8 * maxE1 + 16, pre32 = kEdgeVecBytes<float> * 8 * maxE1 + 16;
     raise_smem_limit(k_pre_elem<double, 1>, pre64);
     raise_smem_limit(k_pre_elem<double, 2>, pre64);
     raise_smem_limit(k_pre_elem<double, 4>, pre64);

@@ -135,21 +135,25 @@ inline size_t pass_smem_total(int pmax, int rb, int maxE1) {
 }
 // warps (elements) per CTA: up to 4 while the per-warp shared memory fits in 200 KB
 
+// edge-operator pass 1: the staged vectors, then (when it fits) the staged S_E^-1 behind an mbarrier.  Bytes per
+// entry of either: in FP64 limbs and FP32 parts (ddh_fixed.cuh)
+template <class T> constexpr int kEdgeVecBytes = sizeof(T) == 8 ? 32 : 8;
+template <class T> constexpr int kEdgeMatBytes = sizeof(T) == 8 ? 24 : 8;
 template <class T>
 inline size_t edge_vec_bytes(int rb, int maxE1) {
-    return ((size_t)2 * rb * std::max(1, maxE1) * sizeof(cpx<T>) + 127) & ~(size_t)127;
+    return ((size_t)rb * std::max(1, maxE1) * kEdgeVecBytes<T> + 127) & ~(size_t)127;
 }
+template <class T>
+inline size_t edge_mat_bytes(int maxE1) { return ((size_t)maxE1 * maxE1 * kEdgeMatBytes<T> + 127) & ~(size_t)127; }
 template <class T>
 inline int edge_stage_off(int rb, int maxE1) {
     const size_t base = edge_vec_bytes<T>(rb, maxE1);
-    const size_t st = 128 + (((size_t)maxE1 * maxE1 * sizeof(cpx<T>) + 127) & ~(size_t)127);
-    return (maxE1 > 0 && base + st <= 200 * 1024) ? (int)base : 0;
+    return (maxE1 > 0 && base + 128 + edge_mat_bytes<T>(maxE1) <= 200 * 1024) ? (int)base : 0;
 }
 template <class T>
 inline size_t edge_smem_total(int rb, int maxE1) {
     const int off = edge_stage_off<T>(rb, maxE1);
-    if (!off) return edge_vec_bytes<T>(rb, maxE1);
-    return (size_t)off + 128 + (((size_t)maxE1 * maxE1 * sizeof(cpx<T>) + 127) & ~(size_t)127);
+    return off ? (size_t)off + 128 + edge_mat_bytes<T>(maxE1) : edge_vec_bytes<T>(rb, maxE1);
 }
 
 // Lets launches of kernel k ask for `bytes` of dynamic shared memory.  The limit belongs to the kernel and the

@@ -54,21 +54,18 @@ void launch_pass1_edge(const DevModel& dm, const void* sinv, const void* Y, cons
                        const double2* bt, void* xE, void* tT, int R, const int* done, cudaStream_t st,
                        const EdgeSched* es = nullptr, int item0 = 0, int nitems = -1, int tpr_force = 0,
                        int rows = 0);
-// in FP64 both take the operators in fixed point (pass 1: s, y; pass 2: y2), which launch_fix_edge makes
-// from the complex128 S_E^-1 and Y: four ints per entry, exponents by type-1 / type-2 slot
+// in FP64 both also read the split S_E^-1 and Y of DevModel (ddh_fixed.cuh), which launch_fix_edge makes: s, y, and
+// y2 = Y column-major, with their exponents
 struct EdgeFix {
-    int4* s = nullptr;
+    FxMat s, y, y2;
     int* sex = nullptr;
-    int4* y = nullptr;
     int* yex = nullptr;
-    int4* y2 = nullptr;
     int* y2ex = nullptr;
 };
 void launch_fix_edge(const DevModel& dm, const void* sinv, const void* Y, const EdgeFix& f, cudaStream_t st);
-// the same for npat restricted S^Lap (real, two ints per entry): pattern k is len[k]^2 entries at off[k],
-// its exponents at eoff[k]
-void launch_fix_pre(const double* S, int npat, const int64_t* off, const int* len, const int64_t* eoff, int2* fx, int* ex,
-                    cudaStream_t st);
+// the same for npat restricted S^Lap: pattern k is len[k]^2 entries at off[k], its exponents at eoff[k]
+void launch_fix_pre(const double* S, int npat, const int64_t* off, const int* len, const int64_t* eoff,
+                    const FxRealMat& fx, int* ex, cudaStream_t st);
 // default CTA size of the one-CTA-per-task edge pass for elements of at most maxNo output rows
 int edge_cta_threads(int maxNo);
 template <class T>
@@ -95,9 +92,9 @@ int launch_pre(const DevModel& dm, const double2* v, double2* vd, void* outE, do
 
 // Nested-dissection factor of the coarse matrix on the device (elimination order).  Per
 // node: fully summed positions [f0, f0+nF), boundary positions bidx[b_off .. b_off+nB),
-// G (nB x nF) at g_off and M = [W | -H] (nF x (nF+nB)) at m_off, in fixed point (int4 limbs with the
-// row exponents gexp[u_off + row], mexp[f0 + row]; launch_fix_fronts makes them from complex128 in
-// place) or float2, row-major (column-major for short rows, see kNDShortRow).  The forward pass leaves
+// G (nB x nF) at g_off and M = [W | -H] (nF x (nF+nB)) at m_off, complex128 (and split, see ddh_fixed.cuh, in gfx and mfx
+// with the row exponents gexp[u_off + row], mexp[f0 + row]; launch_fix_fronts makes them) or complex64,
+// row-major (column-major for short rows, see kNDShortRow).  The forward pass leaves
 // at u[u_off[N] + k] ([R][u_len]) the total amount node N's subtree subtracts from boundary
 // entry k; it is passed up the tree: src[2 (s_off[N] + i) + {0,1}] are the offsets in u of
 // the (at most two) children's amounts for front entry i (F first, then B), or -1.
@@ -114,11 +111,9 @@ struct NDDev {
     const int64_t* src = nullptr;
     const void* G = nullptr;
     const void* M = nullptr;
+    FxMat gfx, mfx;
     int* gexp = nullptr;
     int* mexp = nullptr;
-    int* gcol = nullptr;      // column scalings: of G and M by F position, of M by boundary entry (u_off + k)
-    int* mcol = nullptr;
-    int* mcolB = nullptr;
     int64_t u_len = 0;
     int nc = 0;
 };
@@ -182,18 +177,17 @@ void launch_nd_persistent(const NDDev& d, const NDSched& s, bool f32, const doub
 size_t nd_state_ints(const NDSched& s, int R);
 void launch_fix_fronts(const NDDev& d, int nodes, cudaStream_t st);
 void nd_set_smem_limits();   // once per device before the first (captured) launch
-// r = t - K x, K in CSR with its values in fixed point (launch_fix_csr makes them from complex128 in
-// place; vex: row exponents), R right-hand sides ([R][n])
-void launch_fix_csr(const int* ptr, double2* val, int* ex, int n, cudaStream_t st);
-void launch_csr_residual(const int* ptr, const int* col, const void* val, const int* vex, int n, const double2* x,
-                         const double2* t, double2* r, int R, const int* done, cudaStream_t st);
+// r = t - K x, K in CSR (vx, vex: its values split by row, made by launch_fix_csr), R right-hand sides ([R][n])
+void launch_fix_csr(const int* ptr, const double2* val, const FxMat& vx, int* vex, int n, cudaStream_t st);
+void launch_csr_residual(const int* ptr, const int* col, const double2* val, const FxMat& vx, const int* vex, int n,
+                         const double2* x, const double2* t, double2* r, int R, const int* done, cudaStream_t st);
 void launch_dinv(const DevModel& dm, const double2* x, double2* y, int R, const int* done, cudaStream_t st);
-// y = K^-1 x for the dense inverse in fixed point (ddh_fixed.cuh; ex = its row exponents, col = its column
-// scalings, nsm = SMs of the device), R right-hand sides; launch_fix_dense turns the complex128 matrix
-// into that form in place
-void launch_gemv(const void* A, const int* ex, const int* col, int n, const double2* x, double2* y, int R, const int* done, int nsm,
+// y = K^-1 x for the dense inverse (Ax, ex: split by row and tile of columns, gemv_tiles(n) exponents a row,
+// made by launch_fix_dense; nsm = SMs of the device), R right-hand sides
+void launch_gemv(const double2* A, const FxMat& Ax, const int* ex, int n, const double2* x, double2* y, int R, const int* done, int nsm,
                  cudaStream_t st);
-void launch_fix_dense(void* A, int n, int* ex, int* col, cudaStream_t st);
+int gemv_tiles(int n);
+void launch_fix_dense(const double2* A, int n, const FxMat& Ax, int* ex, cudaStream_t st);
 void gemv_set_smem_limits();
 // the same for the complex64 copy.  For one right-hand side `form` picks the kernel: 0 one warp per
 // row, 1 two warps per row, 2 two rows per warp (chosen by timing at factor time)
