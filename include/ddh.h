@@ -171,9 +171,8 @@ typedef struct {
                               coarse solve, 8 sum_fronts nF (nF + 2 nB): forward G y_F and backward
                               [W | -H] [y_F; x_B] (reported also when the dense K^-1 is in use) */
     int32_t coarse_form;   /* form in use: DDH_COARSE_DENSE, DDH_COARSE_ND or DDH_COARSE_ND_LEVELS */
-    int32_t coarse_subtrees; /* DDH_COARSE_ND_LEVELS: subtrees (of the deepest cut offered to the tuner)
-                                whose levels can run as one launch per direction (0: the tree has too
-                                few nodes; every level is its own launch) */
+    int32_t coarse_subtrees; /* DDH_COARSE_ND_LEVELS: subtrees whose levels run as one launch per direction
+                                (0: every level is its own launch) */
 } ddh_info;
 
 typedef struct {

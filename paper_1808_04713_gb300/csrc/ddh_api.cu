@@ -95,9 +95,7 @@ struct ddh_ctx {
     NDDev nd64, nd32;
     const int4* nd_items = nullptr;
     void* nd_u = nullptr;                          // forward updates [R][u_len] (work buffer)
-    std::vector<NDBottom> nd_bottom;               // cut levels below which a CTA per subtree runs the tree
-    struct BottomPick { int at = -1, rb_fwd = 0, rb_bwd = 0; };
-    std::map<int, BottomPick> nd_pick;             // per R: the tuned cut (index, -1 none) and RHS blocks
+    NDBottom nd_bottom;                            // levels that a CTA per subtree runs (nsub = 0: none)
     std::vector<int> nd_fwd_off, nd_fwd_n, nd_fwd_rows;   // per level: first item, items, staged rows
     std::vector<int> nd_bwd_off, nd_bwd_n, nd_bwd_rows;
     std::map<int, std::vector<int>> nd_rb;         // per R: tuned RHS block of each level (fwd, then bwd)
@@ -230,8 +228,7 @@ static void free_model(ddh_ctx* ctx) {
     ctx->nd32 = NDDev();
     ctx->nd_items = nullptr;
     ctx->nd_u = nullptr;
-    ctx->nd_bottom.clear();
-    ctx->nd_pick.clear();
+    ctx->nd_bottom = NDBottom();
     ctx->nd_fwd_off.clear(); ctx->nd_fwd_n.clear(); ctx->nd_fwd_rows.clear();
     ctx->nd_bwd_off.clear(); ctx->nd_bwd_n.clear(); ctx->nd_bwd_rows.clear();
     ctx->nd_sched = NDSched();
@@ -779,21 +776,28 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         }
         for (int lv = 0; lv < L; ++lv)
             if (ctx->nd_bwd_rows[lv] > 12800) return fail(ctx, DDH_ERR_INVALID_ARG, "coarse front too large for shared memory");
-        // bottom launches: cut at the first level with at least 12, 40 or 120 nodes (the tuner picks one);
-        // a CTA walks the levels of the subtree below each node of that level
+        // bottom launches: a CTA walks the levels of the subtree below each node of a cut level.  The sums of a
+        // front's rows are dealt to lanes differently there than in the level launches, so the cut follows from
+        // the tree alone, neither from timings nor from the number of right-hand sides: the first level with at
+        // least 12, else 40, else 120 nodes whose subtrees stage at most 160 entries at a time (longer fronts
+        // keep a warp too long) and hold at most twice their mean of matrix entries.  One coarse solve, 1 / 8
+        // right-hand sides, by subtrees (0: none): 16 x 16 elements, l = 5 (99 entries at 16 subtrees) 0: 98 /
+        // 135 us, 64: 93 / 119, 16: 88 / 98; 32 x 32, l = 5 (199 at 16) 0: 142 / 229, 128: 125 / 215, 64: 123 /
+        // 190, 16: 177 / 200; 64 x 64, l = 5 (199 at 64, 399 at 16) 0: 279 / 715, 128: 232 / 533, 64: 297 / 517,
+        // 16: 800 / 785; disk refined twice (uneven) 0: 118 / 162, 52: 128 / 184.
         {
             std::vector<int> count(L, 0);
             for (const auto& N : m.cnode) count[N.depth]++;
-            for (const int least : {120, 40, 12}) {
+            for (const int least : {12, 40, 120}) {
                 NDBottom b;
                 for (b.cut = 1; b.cut < L && count[b.cut] < least; ++b.cut) {}
-                if (b.cut >= L || (!ctx->nd_bottom.empty() && ctx->nd_bottom.back().cut == b.cut)) continue;
+                if (b.cut >= L) break;
                 b.nlev = L - b.cut;
                 for (int lv = b.cut; lv < L; ++lv) {
                     b.fwd_rows = std::max(b.fwd_rows, ctx->nd_fwd_rows[lv]);
                     b.bwd_rows = std::max(b.bwd_rows, ctx->nd_bwd_rows[lv]);
                 }
-                if (!nd_bottom_block(b.fwd_rows, 1) || !nd_bottom_block(b.bwd_rows, 1)) continue;
+                if (std::max(b.fwd_rows, b.bwd_rows) > 160) continue;
                 // ancestors at the cut (node ids are postorder: a parent's id is the larger)
                 std::vector<int> sub(nn, -1);
                 for (int id = nn - 1; id >= 0; --id) {
@@ -801,6 +805,12 @@ static ddh_status upload_model(ddh_ctx* ctx) {
                     if (N.depth == b.cut) sub[id] = b.nsub++;
                     else if (N.depth > b.cut) sub[id] = sub[N.parent];
                 }
+                std::vector<double> held(b.nsub, 0.0);
+                for (int id = 0; id < nn; ++id)
+                    if (sub[id] >= 0) held[sub[id]] += m.cnode[id].nF * (m.cnode[id].nF + 2.0 * m.cnode[id].B.size());
+                double sum = 0, most = 0;
+                for (double h : held) { sum += h; most = std::max(most, h); }
+                if (most * b.nsub > 2 * sum) continue;
                 // backward rows per level and subtree: 16 by 2 slices while that still gives every warp an
                 // item, else 4 by 8
                 std::vector<int> brows((size_t)b.nsub * b.nlev, 0);
@@ -831,7 +841,8 @@ static ddh_status upload_model(ddh_ctx* ctx) {
                 if ((st = upload(ctx, ba, &b.bitems))) return st;
                 if ((st = upload(ctx, fp, &b.fptr))) return st;
                 if ((st = upload(ctx, bp, &b.bptr))) return st;
-                ctx->nd_bottom.push_back(b);
+                ctx->nd_bottom = b;
+                break;
             }
         }
         // one-launch schedule: forward items deepest level first, then backward items root
@@ -1044,11 +1055,10 @@ static ddh_status nd_tune(ddh_ctx* ctx, const Work& w, int R) {
     CK(cudaMemsetAsync(y, 0, sizeof(double2) * (size_t)R * nc, s));
     CK(cudaMemsetAsync(u, 0, sizeof(double2) * (size_t)R * ctx->nd64.u_len, s));
     std::vector<int> best(2 * (size_t)L, 0);
-    std::vector<float> cost(2 * (size_t)L, 0.f);
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    // fastest right-hand-side block of one launch, and its time
+    // fastest right-hand-side block of one launch
     auto pick_rb = [&](int rb_max, int& pick, const std::function<void(int)>& run) {
         float tbest = 1e30f;
         for (int rb = rb_max; rb >= 1; rb >>= 1) {
@@ -1061,44 +1071,29 @@ static ddh_status nd_tune(ddh_ctx* ctx, const Work& w, int R) {
             cudaEventElapsedTime(&ms, e0, e1);
             if (ms < 0.97f * tbest) { tbest = ms; pick = rb; }
         }
-        return tbest;
     };
+    const NDBottom& bot = ctx->nd_bottom;
+    const int cut = bot.nsub > 0 ? bot.cut : L;
     for (int dir = 0; dir < 2; ++dir)
-        for (int lv = dir ? 0 : 1; lv < L; ++lv) {
+        for (int lv = dir ? 0 : 1; lv < cut; ++lv) {
             const int n = dir ? ctx->nd_bwd_n[lv] : ctx->nd_fwd_n[lv];
             const int rows = dir ? ctx->nd_bwd_rows[lv] : ctx->nd_fwd_rows[lv];
             if (!n) continue;
-            cost[(size_t)dir * L + lv] = pick_rb(nd_rhs_block(rows, R), best[(size_t)dir * L + lv], [&](int rb) {
+            pick_rb(nd_rhs_block(rows, R), best[(size_t)dir * L + lv], [&](int rb) {
                 if (dir) launch_nd_backward(ctx->nd64, false, ctx->nd_items + ctx->nd_bwd_off[lv], n, rows, lv == 0, w.t, u,
                                             y, w.x2, R, nullptr, s, rb);
                 else launch_nd_forward(ctx->nd64, false, ctx->nd_items + ctx->nd_fwd_off[lv], n, rows, w.t, y, u, R,
                                        nullptr, s, rb);
             });
         }
-    // the bottom launches against the level launches that they replace
-    ddh_ctx::BottomPick bot;
-    float gain = 0.f;
-    for (size_t c = 0; c < ctx->nd_bottom.size(); ++c) {
-        const NDBottom& b = ctx->nd_bottom[c];
-        ddh_ctx::BottomPick p;
-        p.at = (int)c;
-        float ms = pick_rb(nd_bottom_block(b.fwd_rows, R), p.rb_fwd, [&](int rb) {
-            launch_nd_bottom(true, ctx->nd64, false, b, w.t, y, w.x2, u, R, nullptr, s, rb);
+    for (int dir = 0; dir < 2 && cut < L; ++dir) {
+        int rb_best = 0;
+        pick_rb(nd_bottom_block(dir ? bot.bwd_rows : bot.fwd_rows, R), rb_best, [&](int rb) {
+            launch_nd_bottom(dir == 0, ctx->nd64, false, bot, w.t, y, w.x2, u, R, nullptr, s, rb);
         });
-        ms += pick_rb(nd_bottom_block(b.bwd_rows, R), p.rb_bwd, [&](int rb) {
-            launch_nd_bottom(false, ctx->nd64, false, b, w.t, y, w.x2, u, R, nullptr, s, rb);
-        });
-        float levels = 0.f;
-        for (int lv = b.cut; lv < L; ++lv) levels += cost[lv] + cost[(size_t)L + lv];
-        if (levels - ms > gain) { gain = levels - ms; bot = p; }
+        for (int lv = cut; lv < L; ++lv) best[(size_t)dir * L + lv] = rb_best;
     }
-    if (bot.at >= 0)
-        for (int lv = ctx->nd_bottom[bot.at].cut; lv < L; ++lv) {
-            best[lv] = bot.rb_fwd;
-            best[(size_t)L + lv] = bot.rb_bwd;
-        }
     CK(cudaGetLastError());
-    ctx->nd_pick[R] = bot;
     ctx->nd_rb[R] = best;
     ctx->nd_chains[R] = 1;
     float tbest = 1e30f;
@@ -1452,11 +1447,10 @@ static void nd_level_chain(ddh_ctx* ctx, const NDDev& D, bool f32nd, const doubl
     const int L = (int)ctx->nd_fwd_rows.size();
     const auto tuned = ctx->nd_rb.find(R);
     const std::vector<int>* rbs = tuned != ctx->nd_rb.end() ? &tuned->second : nullptr;
-    const auto pk = ctx->nd_pick.find(R);
-    const NDBottom* bot = pk != ctx->nd_pick.end() && pk->second.at >= 0 ? &ctx->nd_bottom[pk->second.at] : nullptr;
+    const NDBottom* bot = ctx->nd_bottom.nsub > 0 ? &ctx->nd_bottom : nullptr;
     const int cut = bot ? bot->cut : L;
     if (bot) {
-        launch_nd_bottom(true, D, f32nd, *bot, t, y, x2, u, R, done, s, pk->second.rb_fwd);
+        launch_nd_bottom(true, D, f32nd, *bot, t, y, x2, u, R, done, s, rbs ? (*rbs)[cut] : 0);
         ctx->launches++;
     }
     // every level launch after the first of the chain is a programmatic dependent of the one
@@ -1479,7 +1473,7 @@ static void nd_level_chain(ddh_ctx* ctx, const NDDev& D, bool f32nd, const doubl
         ctx->launches++;
     }
     if (bot) {
-        launch_nd_bottom(false, D, f32nd, *bot, t, y, x2, u, R, done, s, pk->second.rb_bwd);
+        launch_nd_bottom(false, D, f32nd, *bot, t, y, x2, u, R, done, s, rbs ? (*rbs)[L + cut] : 0);
         ctx->launches++;
     }
 }
@@ -2488,7 +2482,7 @@ ddh_status ddh_get_info(const ddh_ctx* ctx, ddh_info* out) {
     for (const auto& N : m.cnode) fl += 8.0 * N.nF * ((double)N.nF + 2.0 * (double)N.B.size());
     out->coarse_nd_flops = fl;
     out->coarse_form = m.dense_coarse ? DDH_COARSE_DENSE : (ctx->nd_levels ? DDH_COARSE_ND_LEVELS : DDH_COARSE_ND);
-    out->coarse_subtrees = m.dense_coarse || ctx->nd_bottom.empty() ? 0 : ctx->nd_bottom[0].nsub;
+    out->coarse_subtrees = m.dense_coarse ? 0 : ctx->nd_bottom.nsub;
     return DDH_OK;
 }
 
