@@ -44,15 +44,11 @@ UNIT = "solves/s"
 WORKLOAD = "random_eps_64"
 TOL = 1e-10
 CPU_SAMPLE_BLOCK = 16           # the oracle times the 16 x 16-element corner of the workload
-# The FP64-accurate dense products run in fixed point on the integer pipe: 2.3 complex multiply-adds (twelve
-# 32 x 32 + 64 bit multiply-adds each, timed) per SM and clock x 8 FLOP x 152 SMs x 2.07 GHz.  The FP64 pipe
-# (2 FMA per SM and clock) would give 1.25 TFLOP/s.
-FIXED_PEAK_TFLOPS = 5.8
+# The FP64-accurate dense products run on the integer pipe: 26 multiply-adds 32 x 32 + 64 bits (timed) per SM and
+# clock, twelve per complex multiply-add of 8 FLOP, 152 SMs, 2.07 GHz.  The FP64 pipe (2 FMA per SM and
+# clock) would give 1.25 TFLOP/s.
+FIXED_PEAK_TFLOPS = 5.45
 FP32_PEAK_TFLOPS = 70.0         # FP32 SIMT FMA throughput timed on this GPU
-# DRAM bytes of one coarse solve of the headline workload (8 RHS in two chains of 4) from an ncu capture
-# with one launch per tree level (cold cache per launch; profiles/nd_coarse_random_eps_64.md); the lower
-# levels have since become one launch per direction, which reads the same factor
-ND_TRAFFIC_BYTES_2CHAINS = 290.1e6
 
 
 def _dist():
@@ -205,8 +201,8 @@ def roofline(comp_ms, info, R: int, p: int, fp64_elements: bool, coarse_name: st
     achieved = fl / t / 1e12
     return {"kernel": names[dom], "bound": "alu", "achieved": round(achieved, 4), "peak": peak, "unit": "TFLOP/s",
             "frac": round(achieved / peak, 4), "traffic": None, "flops_per_launch": fl,
-            "peak_source": ("fixed point 5.8 TFLOP/s: 152 SMs x 2.3 complex multiply-adds/clk (timed) x 8 FLOP "
-                            "x 2.07 GHz; the FP64 pipe's peak is 1.25") if fp64 else "FP32 SIMT 70 TFLOP/s timed on this GPU",
+            "peak_source": ("integer pipe 5.45 TFLOP/s: 152 SMs x 26 multiply-adds/clk (timed) / 12 x 8 FLOP x 2.07 GHz; "
+                            "the FP64 pipe's peak is 1.25") if fp64 else "FP32 SIMT 70 TFLOP/s timed on this GPU",
             "component_ms": {k: round(float(v), 5) for k, v in zip(COMPONENTS, comp_ms)}}
 
 
@@ -512,12 +508,8 @@ def run_ours(args):
     e2e_value = aggregate_rate(ws, len(e2e_t), R, e2e_total)
     e2e_same = bool(torch.equal(uh, u.cpu()))     # repeated solves are bit-identical
     comp = s.profile_op(R, ddh.PREC_MIXED_FP32, reps=10)
-    roof = roofline(comp, info, R, 20, False, "coarse solve (nested dissection, FP64: k_nd_forward/backward levels)")
+    roof = roofline(comp, info, R, 20, False, "coarse solve (nested dissection: k_nd_bottom, k_nd_forward/backward)")
     tuning = s.get_tuning(R, ddh.PREC_MIXED_FP32)
-    if tuning.get("nd_chains") == 2 and "nested dissection" in roof["kernel"]:
-        roof["traffic"] = ND_TRAFFIC_BYTES_2CHAINS
-        roof["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the 52 level launches of one "
-                                  "coarse solve (two chains of 4 RHS), cold cache per launch")
     clocks = clk.summary()
     s.close()
     del u, b
@@ -528,7 +520,7 @@ def run_ours(args):
         _, sp_, bp, up, plain = _form(WORKLOAD, ddh.PREC_FP64, local, stream, flush, 1, max(3, min(args.steps, 10)))
         compp = sp_.profile_op(R, ddh.PREC_FP64, reps=10)
         plain["roofline"] = roofline(compp, sp_.info(), R, 20, True,
-                                     "coarse solve (nested dissection, FP64: k_nd_forward/backward levels)")
+                                     "coarse solve (nested dissection: k_nd_bottom, k_nd_forward/backward)")
         sp_.close()
         del bp, up
         extras["plain_fp64"] = plain
@@ -545,7 +537,7 @@ def run_ours(args):
         _, s2, b2, u2, c2 = _form("plane_16x16", ddh.PREC_FP64, local, stream, flush, 3, max(3, args.steps))
         i2 = s2.info()
         comp2 = s2.profile_op(1, ddh.PREC_FP64, reps=20)
-        c2["roofline"] = roofline(comp2, i2, 1, 16, True, "coarse solve (dense K^-1 GEMV, fixed point)")
+        c2["roofline"] = roofline(comp2, i2, 1, 16, True, "coarse solve (dense K^-1: k_gemv_fx)")
         # the same coarse solve measured against the nested-dissection factor's work (the
         # method's own coarse cost): what the dense GEMV delivers per unit of necessary work
         c2["roofline"]["coarse_frac_of_nd_work"] = round(i2.coarse_nd_flops / (comp2[2] * 1e-3) / 1e12
