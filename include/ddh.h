@@ -114,7 +114,9 @@ typedef struct {
     int32_t coarse_form;   /* coarse solve K x2 = t (ddh_coarse_form): DDH_COARSE_AUTO (default) applies
                               a dense K^-1 built from the factor when n_coarse <= 2048 and the
                               per-level nested-dissection solve otherwise; DDH_COARSE_DENSE forces
-                              the dense K^-1 (n_coarse <= 16384, else DDH_ERR_INVALID_ARG);
+                              the dense K^-1, whose columns cost n_coarse host solves (worth it up
+                              to about 4000 unknowns where a hundred or more solves with one
+                              right-hand side follow a factorisation) (n_coarse <= 16384, else DDH_ERR_INVALID_ARG);
                               DDH_COARSE_ND and DDH_COARSE_ND_LEVELS force the nested-dissection
                               solve at any size, in one launch or one launch per tree level */
     int32_t robin_modified;/* 1: the Robin-modified local problems of Sec. 2.3.4.  Elements get

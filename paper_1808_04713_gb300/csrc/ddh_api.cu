@@ -88,7 +88,6 @@ struct ddh_ctx {
     float2* Kinv32 = nullptr;
     FxMat Kinv_fx;                                 // the same split (ddh_fixed.cuh), with its exponents
     int* Kinv_ex = nullptr;
-    int gemv_form = 1;                             // single-RHS complex64 GEMV kernel (timed at upload)
     int nsm = 0;                                   // SMs of the device
     // nested-dissection factor: complex128 matrices, their complex64 copy (nd32.G/M null
     // unless mixed precision with coarse_fp32), and per tree level the work items
@@ -653,33 +652,6 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         CK(cudaDeviceGetAttribute(&ctx->nsm, cudaDevAttrMultiProcessorCount, ctx->device));
         launch_fix_dense(ctx->Kinv, nc, ctx->Kinv_fx, ctx->Kinv_ex, ctx->stream);
         gemv_set_smem_limits();
-        // autotune: time the single-RHS GEMV forms on the complex64 K^-1 and keep the fastest
-        if (want32) {
-            double2 *xs = nullptr, *ys = nullptr;
-            if (cudaMalloc(&xs, sizeof(double2) * nc) == cudaSuccess && cudaMalloc(&ys, sizeof(double2) * nc) == cudaSuccess) {
-                cudaMemsetAsync(xs, 0, sizeof(double2) * nc, ctx->stream);
-                cudaEvent_t e0, e1;
-                cudaEventCreate(&e0);
-                cudaEventCreate(&e1);
-                float best = 1e30f;
-                for (int f = 0; f < 3; ++f) {
-                    launch_gemv32(ctx->Kinv32, nc, xs, ys, 1, nullptr, ctx->stream, f);
-                    cudaEventRecord(e0, ctx->stream);
-                    for (int rep = 0; rep < 5; ++rep) launch_gemv32(ctx->Kinv32, nc, xs, ys, 1, nullptr, ctx->stream, f);
-                    cudaEventRecord(e1, ctx->stream);
-                    cudaEventSynchronize(e1);
-                    float ms = 0;
-                    cudaEventElapsedTime(&ms, e0, e1);
-                    if (ms < best) { best = ms; ctx->gemv_form = f; }
-                }
-                cudaEventDestroy(e0);
-                cudaEventDestroy(e1);
-            }
-            cudaStreamSynchronize(ctx->stream);
-            if (xs) cudaFree(xs);
-            if (ys) cudaFree(ys);
-            cudaGetLastError();
-        }
     } else {
         const int nn = (int)m.cnode.size();
         std::vector<int> f0(nn), nF(nn), nB(nn), bidx;
@@ -1402,7 +1374,7 @@ static void coarse_solve_once(ddh_ctx* ctx, const double2* t, double2* x2, doubl
     cudaStream_t s = ctx->stream;
     const bool f32 = ctx->coarse32;
     if (ctx->Kinv) {
-        if (f32) launch_gemv32(ctx->Kinv32, nc, t, x2, R, done, s, ctx->gemv_form);
+        if (f32) launch_gemv32(ctx->Kinv32, nc, t, x2, R, done, s);
         else launch_gemv(ctx->Kinv, ctx->Kinv_fx, ctx->Kinv_ex, nc, t, x2, R, done, ctx->nsm, s);
         ctx->launches++;
         return;

@@ -45,19 +45,18 @@ __global__ void k_fix_fronts(NDDev d) {
 }
 
 // ------------------------------------------------------------------ dense K^-1
-// y = A x for a dense row-major complex matrix (n_out x n_in) and R right-hand sides, one
-// warp per output row; the row is read once and applied to up to 8 RHS per pass (vectors and
-// accumulation FP64; the matrix is the complex64 K^-1 of the mixed-precision inner solves).
-// mode 0: y = A x ; mode 1: y -= A x ; mode 2: y = c - A x (c given)
-template <class M, int RB>
-__global__ void k_gemv(const M* __restrict__ A, int n_out, int n_in, const double2* __restrict__ x,
-                       double2* __restrict__ y, const double2* __restrict__ c, int mode,
-                       int64_t xs, int64_t ys, int r0, const int* __restrict__ done) {
+// y = K^-1 x for the complex64 copy (the mixed-precision inner solves with coarse_fp32) and RB right-hand sides,
+// one warp per row; vectors and accumulation FP64, which bounds it.  n = 1921, one right-hand side: 57 us; two
+// warps per row or two rows per warp measured the same within 3 %.
+template <int RB>
+__global__ void k_gemv(const float2* __restrict__ A, int n, const double2* __restrict__ x, double2* __restrict__ y, int r0,
+                       const int* __restrict__ done) {
     if (done && *done) return;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (warp >= n_out) return;
-    const M* a = A + (int64_t)warp * n_in;
+    if (warp >= n) return;
+    const float2* a = A + (int64_t)warp * n;
+    const double2* xr = x + (int64_t)r0 * n;
     double sx[RB], sy[RB];
 #pragma unroll
     for (int q = 0; q < RB; ++q) { sx[q] = 0; sy[q] = 0; }
@@ -65,10 +64,9 @@ __global__ void k_gemv(const M* __restrict__ A, int n_out, int n_in, const doubl
     if (RB == 1) {
         // one right-hand side: four loads in flight per lane, two accumulator chains
         double tx = 0, ty = 0;
-        for (; j + 96 < n_in; j += 128) {
-            const M a0 = a[j], a1 = a[j + 32], a2 = a[j + 64], a3 = a[j + 96];
-            const double2 x0 = x[r0 * xs + j], x1 = x[r0 * xs + j + 32];
-            const double2 x2 = x[r0 * xs + j + 64], x3 = x[r0 * xs + j + 96];
+        for (; j + 96 < n; j += 128) {
+            const float2 a0 = a[j], a1 = a[j + 32], a2 = a[j + 64], a3 = a[j + 96];
+            const double2 x0 = xr[j], x1 = xr[j + 32], x2 = xr[j + 64], x3 = xr[j + 96];
             sx[0] = fma((double)a0.x, x0.x, fma(-(double)a0.y, x0.y, sx[0]));
             sy[0] = fma((double)a0.x, x0.y, fma((double)a0.y, x0.x, sy[0]));
             tx = fma((double)a1.x, x1.x, fma(-(double)a1.y, x1.y, tx));
@@ -81,12 +79,12 @@ __global__ void k_gemv(const M* __restrict__ A, int n_out, int n_in, const doubl
         sx[0] += tx;
         sy[0] += ty;
     }
-    for (; j < n_in; j += 32) {
-        const M av = a[j];
+    for (; j < n; j += 32) {
+        const float2 av = a[j];
         const double ax = (double)av.x, ay = (double)av.y;
 #pragma unroll
         for (int q = 0; q < RB; ++q) {
-            const double2 xv = x[(r0 + q) * xs + j];
+            const double2 xv = xr[(int64_t)q * n + j];
             sx[q] = fma(ax, xv.x, fma(-ay, xv.y, sx[q]));
             sy[q] = fma(ax, xv.y, fma(ay, xv.x, sy[q]));
         }
@@ -102,91 +100,7 @@ __global__ void k_gemv(const M* __restrict__ A, int n_out, int n_in, const doubl
         double vx = 0, vy = 0;
 #pragma unroll
         for (int q = 0; q < RB; ++q) if (q == lane) { vx = sx[q]; vy = sy[q]; }
-        double2* yr = y + (r0 + lane) * ys;
-        if (mode == 0) yr[warp] = make_double2(vx, vy);
-        else if (mode == 1) { yr[warp].x -= vx; yr[warp].y -= vy; }
-        else { const double2 cv = c[(r0 + lane) * ys + warp]; yr[warp] = make_double2(cv.x - vx, cv.y - vy); }
-    }
-}
-
-// y = A x for one right-hand side: two warps per row (interleaved 32-column blocks), so that
-// twice as many warps per SM keep loads in flight for the FP64 pipe; 4 rows per 256 threads
-template <class M>
-__global__ void __launch_bounds__(256) k_gemv1(const M* __restrict__ A, int n_out, int n_in,
-                                               const double2* __restrict__ x, double2* __restrict__ y,
-                                               const double2* __restrict__ c, int mode, const int* __restrict__ done) {
-    if (done && *done) return;
-    __shared__ double2 red[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = blockIdx.x * 4 + (warp >> 1), h = warp & 1;
-    double sx = 0, sy = 0, tx = 0, ty = 0;
-    if (row < n_out) {
-        const M* a = A + (int64_t)row * n_in;
-        int j = h * 32 + lane;
-        for (; j + 64 < n_in; j += 128) {
-            const M a0 = a[j], a1 = a[j + 64];
-            const double2 x0 = x[j], x1 = x[j + 64];
-            sx = fma((double)a0.x, x0.x, fma(-(double)a0.y, x0.y, sx));
-            sy = fma((double)a0.x, x0.y, fma((double)a0.y, x0.x, sy));
-            tx = fma((double)a1.x, x1.x, fma(-(double)a1.y, x1.y, tx));
-            ty = fma((double)a1.x, x1.y, fma((double)a1.y, x1.x, ty));
-        }
-        if (j < n_in) {
-            const M a0 = a[j];
-            const double2 x0 = x[j];
-            sx = fma((double)a0.x, x0.x, fma(-(double)a0.y, x0.y, sx));
-            sy = fma((double)a0.x, x0.y, fma((double)a0.y, x0.x, sy));
-        }
-    }
-    sx += tx; sy += ty;
-    for (int o = 16; o > 0; o >>= 1) {
-        sx += __shfl_xor_sync(0xffffffffu, sx, o);
-        sy += __shfl_xor_sync(0xffffffffu, sy, o);
-    }
-    if (lane == 0) red[warp] = make_double2(sx, sy);
-    __syncthreads();
-    if (h == 0 && lane == 0 && row < n_out) {
-        const double vx = red[warp].x + red[warp + 1].x, vy = red[warp].y + red[warp + 1].y;
-        if (mode == 0) y[row] = make_double2(vx, vy);
-        else if (mode == 1) { y[row].x -= vx; y[row].y -= vy; }
-        else { const double2 cv = c[row]; y[row] = make_double2(cv.x - vx, cv.y - vy); }
-    }
-}
-
-// y = A x for one right-hand side, two rows per warp: each x entry loaded feeds both rows
-// (8 FP64 FMAs per three 16-byte loads instead of four per two)
-template <class M>
-__global__ void __launch_bounds__(128) k_gemv2r(const M* __restrict__ A, int n_out, int n_in,
-                                                const double2* __restrict__ x, double2* __restrict__ y,
-                                                const double2* __restrict__ c, int mode, const int* __restrict__ done) {
-    if (done && *done) return;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    const int row = 2 * warp;
-    if (row >= n_out) return;
-    const bool two = row + 1 < n_out;
-    const M* a0 = A + (int64_t)row * n_in;
-    const M* a1 = two ? a0 + n_in : a0;
-    double s0x = 0, s0y = 0, s1x = 0, s1y = 0;
-    for (int j = lane; j < n_in; j += 32) {
-        const double2 xv = x[j];
-        const M u = a0[j], v = a1[j];
-        s0x = fma((double)u.x, xv.x, fma(-(double)u.y, xv.y, s0x));
-        s0y = fma((double)u.x, xv.y, fma((double)u.y, xv.x, s0y));
-        s1x = fma((double)v.x, xv.x, fma(-(double)v.y, xv.y, s1x));
-        s1y = fma((double)v.x, xv.y, fma((double)v.y, xv.x, s1y));
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        s0x += __shfl_xor_sync(0xffffffffu, s0x, o);
-        s0y += __shfl_xor_sync(0xffffffffu, s0y, o);
-        s1x += __shfl_xor_sync(0xffffffffu, s1x, o);
-        s1y += __shfl_xor_sync(0xffffffffu, s1y, o);
-    }
-    if (lane < (two ? 2 : 1)) {
-        const int rr = row + lane;
-        const double vx = lane ? s1x : s0x, vy = lane ? s1y : s0y;
-        if (mode == 0) y[rr] = make_double2(vx, vy);
-        else if (mode == 1) { y[rr].x -= vx; y[rr].y -= vy; }
-        else { const double2 cv = c[rr]; y[rr] = make_double2(cv.x - vx, cv.y - vy); }
+        y[(int64_t)(r0 + lane) * n + warp] = make_double2(vx, vy);
     }
 }
 
@@ -1158,16 +1072,13 @@ void launch_fix_dense(const double2* A, int n, const FxMat& Ax, int* ex, cudaStr
 void launch_fix_fronts(const NDDev& d, int nodes, cudaStream_t st) {
     if (nodes > 0) k_fix_fronts<<<nodes, 256, 0, st>>>(d);
 }
-void launch_gemv32(const void* A, int n, const double2* x, double2* y, int R, const int* done, cudaStream_t st, int form) {
-    const float2* a = (const float2*)A;
-    if (R == 1 && form == 1) { k_gemv1<float2><<<(n + 3) / 4, 256, 0, st>>>(a, n, n, x, y, nullptr, 0, done); return; }
-    if (R == 1 && form == 2) { k_gemv2r<float2><<<(n + 7) / 8, 128, 0, st>>>(a, n, n, x, y, nullptr, 0, done); return; }
+void launch_gemv32(const float2* a, int n, const double2* x, double2* y, int R, const int* done, cudaStream_t st) {
     const dim3 g((n + 3) / 4);
     // right-hand sides in chunks of 8, 4, 2, 1: every FMA issued does useful work
     for (int r0 = 0; r0 < R;) {
         const int left = R - r0;
         const int rb = left >= 8 ? 8 : (left >= 4 ? 4 : (left >= 2 ? 2 : 1));
-#define DDH_GEMV(RBV) k_gemv<float2, RBV><<<g, 128, 0, st>>>(a, n, n, x, y, nullptr, 0, n, n, r0, done);
+#define DDH_GEMV(RBV) k_gemv<RBV><<<g, 128, 0, st>>>(a, n, x, y, r0, done);
         switch (rb) { case 8: DDH_GEMV(8) break; case 4: DDH_GEMV(4) break; case 2: DDH_GEMV(2) break; default: DDH_GEMV(1) }
 #undef DDH_GEMV
         r0 += rb;

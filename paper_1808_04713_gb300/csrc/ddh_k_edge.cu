@@ -22,7 +22,7 @@ namespace ddh {
 // slot), i.e. per output row of pass 1.  Pass 2, which sums over the columns, reads a copy of Y that is
 // column-major, so that a warp's load is contiguous over the rows, with an exponent per row (y2_ex, by type-1
 // slot).  In FP64 a staged vector is its limbs and its FP32 parts.  64 x 64 elements, p = 20, 8 right-hand
-// sides, pass 2: 0.15 ms, 0.41 ms in FP64.
+// sides, pass 2: 0.15 ms, 0.30 ms in FP64.
 template <class T> struct EdgeVec {
     cpx<T>* v;
     __device__ __forceinline__ EdgeVec(void* p, int) : v(reinterpret_cast<cpx<T>*>(p)) {}
@@ -593,7 +593,7 @@ __global__ void k_jump_gather(DevModel dm, const cpx<T>* __restrict__ xE, const 
 // ------------------------------------------------------------------ preconditioner
 // y = D^-1 x, D = C1_E C1_E^T + C2 C2^T: 1/2 on conforming rows, dense blocks on hanging edges;
 // in the Poisson mode D = C1 W C1^T (diagonal, one weight per row)
-__global__ void k_dinv(DevModel dm, const double2* __restrict__ x, double2* __restrict__ y, int lumped,
+__global__ void k_dinv(DevModel dm, const double2* __restrict__ x, double2* __restrict__ y,
                        const int* __restrict__ done) {
     if (done && *done) return;
     const int row = blockIdx.x * blockDim.x + threadIdx.x;
@@ -621,7 +621,6 @@ __global__ void k_dinv(DevModel dm, const double2* __restrict__ x, double2* __re
         sy += Di[j] * v.y;
     }
     y[ro + row] = make_double2(sx, sy);
-    (void)lumped;
 }
 
 // out_E = S^Lap[E1][E1] (C1^T v) per element (stiffness Schur complement, shared per degree);
@@ -935,7 +934,7 @@ int launch_pre(const DevModel& dm, const double2* v, double2* vd, void* outE, do
     // without hanging rows D is diagonal and there is no C2 K C2^T: D^-1 goes into the two kernels (64 x 64
     // elements, p = 20, 8 right-hand sides: 275 us for an application, 12 us less than with launches of their own)
     const int with_d = dm.n_hb == 0;
-    if (!with_d) k_dinv<<<gr, 128, 0, st>>>(dm, v, vd, 0, done);
+    if (!with_d) k_dinv<<<gr, 128, 0, st>>>(dm, v, vd, done);
     const double2* in = with_d ? v : vd;
     const int rb = rhs_block(R);
     const dim3 g(dm.E, (R + rb - 1) / rb);
@@ -947,7 +946,7 @@ int launch_pre(const DevModel& dm, const double2* v, double2* vd, void* outE, do
         default: k_pre_elem<T, 1><<<g, 128, sm, st>>>(dm, in, (cpx<T>*)outE, R, done, with_d);
     }
     k_pre_rows<T><<<gr, 128, 0, st>>>(dm, (const cpx<T>*)outE, in, with_d ? z : m, with_d, done);
-    if (!with_d) k_dinv<<<gr, 128, 0, st>>>(dm, m, z, 0, done);
+    if (!with_d) k_dinv<<<gr, 128, 0, st>>>(dm, m, z, done);
     return with_d ? 2 : 4;
 }
 
@@ -965,7 +964,7 @@ void launch_fix_pre(const double* S, int npat, const int64_t* off, const int* le
     if (npat > 0) k_fix_pre<<<npat, 256, 0, st>>>(S, off, len, eoff, fx, ex);
 }
 void launch_dinv(const DevModel& dm, const double2* x, double2* y, int R, const int* done, cudaStream_t st) {
-    k_dinv<<<dim3((dm.n_dual + 127) / 128, R), 128, 0, st>>>(dm, x, y, 1, done);
+    k_dinv<<<dim3((dm.n_dual + 127) / 128, R), 128, 0, st>>>(dm, x, y, done);
 }
 template <class T>
 void launch_pre_krylov(const DevModel& dm, const KrylovDev& K, void* outE, int R, cudaStream_t st) {

@@ -189,10 +189,8 @@ void launch_gemv(const double2* A, const FxMat& Ax, const int* ex, int n, const 
 int gemv_tiles(int n);
 void launch_fix_dense(const double2* A, int n, const FxMat& Ax, int* ex, cudaStream_t st);
 void gemv_set_smem_limits();
-// the same for the complex64 copy.  For one right-hand side `form` picks the kernel: 0 one warp per
-// row, 1 two warps per row, 2 two rows per warp (chosen by timing at factor time)
-void launch_gemv32(const void* A, int n, const double2* x, double2* y, int R, const int* done, cudaStream_t st,
-                   int form = 1);
+// the same for the complex64 copy
+void launch_gemv32(const float2* A, int n, const double2* x, double2* y, int R, const int* done, cudaStream_t st);
 // Lifting of point-source Dirichlet data (tilde basis, boundary slots only; `out` zeroed by the
 // caller): per degree table t, tr_nq[t] Gauss-Legendre nodes tr_x[tr_xoff[t] ..] and the weights
 // tr_Q[tr_off[t] ..] ((p - 1) x nq, bubble m = 2..p by node); src [2R] source centres
