@@ -291,6 +291,7 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         d.maxE1 = std::max(d.maxE1, m.el[e].nE1);
         d.maxNo = std::max(d.maxNo, m.el[e].nE1 + m.el[e].nT);
         d.maxY = std::max(d.maxY, m.el[e].nE1 * m.el[e].nT);
+        d.maxT = std::max(d.maxT, m.el[e].nT);
     }
     if ((st = upload(ctx, p, &d.p))) return st;
     if ((st = upload(ctx, off, &d.off))) return st;
@@ -752,11 +753,12 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         // front's rows are dealt to lanes differently there than in the level launches, so the cut follows from
         // the tree alone, neither from timings nor from the number of right-hand sides: the first level with at
         // least 12, else 40, else 120 nodes whose subtrees stage at most 160 entries at a time (longer fronts
-        // keep a warp too long) and hold at most twice their mean of matrix entries.  One coarse solve, 1 / 8
-        // right-hand sides, by subtrees (0: none): 16 x 16 elements, l = 5 (99 entries at 16 subtrees) 0: 98 /
+        // keep a warp too long) and hold at most twice their mean of matrix entries, at a level that is at least
+        // half full (else few CTAs walk a local refinement).  One coarse solve, 1 / 8 right-hand sides, by
+        // subtrees (0: none): 16 x 16 elements, l = 5 (99 entries at 16 subtrees) 0: 98 /
         // 135 us, 64: 93 / 119, 16: 88 / 98; 32 x 32, l = 5 (199 at 16) 0: 142 / 229, 128: 125 / 215, 64: 123 /
         // 190, 16: 177 / 200; 64 x 64, l = 5 (199 at 64, 399 at 16) 0: 279 / 715, 128: 232 / 533, 64: 297 / 517,
-        // 16: 800 / 785; disk refined twice (uneven) 0: 118 / 162, 52: 128 / 184.
+        // 16: 800 / 785; disk refined twice 0: 118 / 162, 52 (of 256): 128 / 184.
         {
             std::vector<int> count(L, 0);
             for (const auto& N : m.cnode) count[N.depth]++;
@@ -782,7 +784,7 @@ static ddh_status upload_model(ddh_ctx* ctx) {
                     if (sub[id] >= 0) held[sub[id]] += m.cnode[id].nF * (m.cnode[id].nF + 2.0 * m.cnode[id].B.size());
                 double sum = 0, most = 0;
                 for (double h : held) { sum += h; most = std::max(most, h); }
-                if (most * b.nsub > 2 * sum) continue;
+                if (most * b.nsub > 2 * sum || 2 * (int64_t)b.nsub < (1ll << std::min(b.cut, 40))) continue;
                 // backward rows per level and subtree: 16 by 2 slices while that still gives every warp an
                 // item, else 4 by 8
                 std::vector<int> brows((size_t)b.nsub * b.nlev, 0);
