@@ -31,6 +31,7 @@ struct DevModel {
     int E = 0, l = 0, pmax = 0;
     int maxE1 = 0;                      // largest number of type-1 edge slots of an element
     int maxY = 0;                       // largest nE1 nT of an element
+    int maxT = 0;                       // largest nT
     int maxNo = 0;                      // largest nE1 + nT of an element (edge-pass output rows)
     int* err = nullptr;                 // device error word (0 = ok), read by the host after solves
     int64_t n_local = 0;

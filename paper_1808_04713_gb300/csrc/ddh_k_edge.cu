@@ -21,8 +21,9 @@ namespace ddh {
 // Y.  S_E^-1 has an exponent per row (DevModel::sinv_ex, by type-1 slot), Y one per column (y_ex, by type-2
 // slot), i.e. per output row of pass 1.  Pass 2, which sums over the columns, reads a copy of Y that is
 // column-major, so that a warp's load is contiguous over the rows, with an exponent per row (y2_ex, by type-1
-// slot).  In FP64 a staged vector is its limbs and its FP32 parts.  64 x 64 elements, p = 20, 8 right-hand
-// sides, pass 2: 0.15 ms, 0.30 ms in FP64.
+// slot).  In FP64 a staged vector is its limbs, its FP32 parts and, for results that are formed again in FP64,
+// its entries.  64 x 64 elements, p = 20, 8 right-hand
+// sides, pass 2: 0.13 ms, 0.30 ms in FP64.
 template <class T> struct EdgeVec {
     cpx<T>* v;
     __device__ __forceinline__ EdgeVec(void* p, int) : v(reinterpret_cast<cpx<T>*>(p)) {}
@@ -30,7 +31,9 @@ template <class T> struct EdgeVec {
 template <> struct EdgeVec<double> {
     int4* i;
     float4* f;
-    __device__ __forceinline__ EdgeVec(void* p, int n) : i(reinterpret_cast<int4*>(p)), f(reinterpret_cast<float4*>(i + n)) {}
+    double2* d;
+    __device__ __forceinline__ EdgeVec(void* p, int n)
+        : i(reinterpret_cast<int4*>(p)), f(reinterpret_cast<float4*>(i + n)), d(reinterpret_cast<double2*>(f + n)) {}
 };
 // In FP64 a thread takes at most four of the RB right-hand sides of a CTA (a sum is twelve registers), and a
 // CTA of eight has twice the threads.
@@ -87,6 +90,7 @@ __device__ __forceinline__ void edge_stage(const F& load, int n, int vs, int cnt
                     const FxVec w = fx_vec(v[k], ef);
                     sm.i[q * vs + lane + 32 * k] = w.i;
                     sm.f[q * vs + lane + 32 * k] = w.f;
+                    sm.d[q * vs + lane + 32 * k] = v[k];
                 }
             if (lane == 0) ex[q] = ef;
         }
@@ -157,19 +161,17 @@ __device__ __forceinline__ void edge_rows_f(const DevModel& dm, const cpx<T>* S,
 }
 
 // The same with the products of ddh_fixed.cuh.  Two or four threads per output row by the row count alone
-// (edge_tpr), so that the order of a row's terms does not depend on the launch form.  load: the staged
-// vectors' entries, for the results that are formed again in FP64.  Integer multiply-adds bound it (22 per SM
-// and clock, twelve a term): 64 x 64 elements, p = 20, 8 right-hand sides 0.50 ms, 1.09 ms in FP64; at two
+// (edge_tpr), so that the order of a row's terms does not depend on the launch form.  Integer multiply-adds bound it (22 per SM
+// and clock, twelve a term): 64 x 64 elements, p = 20, 8 right-hand sides 0.48 ms, 1.09 ms in FP64; at two
 // CTAs of ten warps per SM, 96 registers a thread.
 template <class T>
 __device__ __forceinline__ int edge_tpr(int rows, int other) {
     return std::is_same<T, double>::value ? (rows <= 64 ? 4 : 2) : other;
 }
-template <int RB, class F>
+template <int RB>
 __device__ __forceinline__ void edge_rows_fx(const DevModel& dm, const FxMat& S, const FxMat& Ye, const double2* S64,
                                              const double2* Y64, int nE, int nT,
-                                             const EdgeVec<double>& rE, const int* ex, const F& load, int vs, int cnt,
-                                             int tpr, int r0, int e1o, int to, cpx<double>* __restrict__ xE_out,
+                                             const EdgeVec<double>& rE, const int* ex, int vs, int cnt, int tpr, int r0, int e1o, int to, cpx<double>* __restrict__ xE_out,
                                              cpx<double>* __restrict__ tT_out, int o_lo, int o_hi, int tid, int nt, int q0) {
     for (int base = 0; base < (o_hi - o_lo) * tpr; base += nt) {
         const int slot = base + tid;
@@ -183,16 +185,22 @@ __device__ __forceinline__ void edge_rows_fx(const DevModel& dm, const FxMat& S,
         for (int i = 0; i < RB; ++i) fx_clear(s[i]);
         if (in) {
             // nE <= 124 terms: one chain; the next entry's load is issued ahead
-            int4 ni = make_int4(0, 0, 0, 0);
-            float2 nf = make_float2(0.f, 0.f);
-            if (part < nE) { ni = col0.i[part * ld]; nf = col0.f[part * ld]; }
-#pragma unroll 1
-            for (int j = part; j < nE; j += tpr) {
-                const FxEntry a = fx_entry(ni, nf);
-                if (j + tpr < nE) { ni = col0.i[(j + tpr) * ld]; nf = col0.f[(j + tpr) * ld]; }
+            auto run = [&](auto all) {
+                int4 ni = make_int4(0, 0, 0, 0);
+                float2 nf = make_float2(0.f, 0.f);
+                if (part < nE) { ni = col0.i[part * ld]; nf = col0.f[part * ld]; }
+#pragma unroll(RB <= 2 ? 4 : 1)
+                for (int j = part; j < nE; j += tpr) {
+                    const FxEntry a = fx_entry(ni, nf);
+                    if (j + tpr < nE) { ni = col0.i[(j + tpr) * ld]; nf = col0.f[(j + tpr) * ld]; }
 #pragma unroll
-                for (int q = 0; q < RB; ++q) fx_mac(s[q], a, rE.i[(q0 + q) * vs + j], rE.f[(q0 + q) * vs + j]);
-            }
+                    for (int q = 0; q < RB; ++q)
+                        if (decltype(all)::value || q0 + q < cnt) fx_mac(s[q], a, rE.i[(q0 + q) * vs + j], rE.f[(q0 + q) * vs + j]);
+                }
+            };
+            // a block that is not full skips what it has not (thirteen right-hand sides: three of sixteen)
+            if (RB < 4 || q0 + RB <= cnt) run(std::true_type());
+            else run(std::false_type());
         }
 #pragma unroll
         for (int q = 0; q < RB; ++q) {
@@ -216,11 +224,11 @@ __device__ __forceinline__ void edge_rows_fx(const DevModel& dm, const FxMat& S,
                 double2 d;
                 const double2* c64 = !in || o < nE ? S64 + (in ? o : 0) : Y64 + (o - nE);
                 const int4 *ci = col0.i, *xi = rE.i + (q0 + q) * vs;
-                const int qq = q0 + q;
-                const unsigned keep = fx_again(tpr, bad ? 1u << (part & 1) : 0, nE, ea, ex[qq], [=](int j) { return c64[j * ld]; },
+                const double2* xd = rE.d + (q0 + q) * vs;
+                const unsigned keep = fx_again(tpr, bad ? 1u << (part & 1) : 0, nE, ea, ex[q0 + q],
+                                               [=](int j) { return c64[j * ld]; },
                                                [=](int j) { const int4 u = ci[j * ld]; return make_int2(u.x, u.z); },
-                                               [=](int j) { return xi[j]; },
-                                               [=](int j) { const cpx<double> x = load(qq, j); return make_double2(x.x, x.y); }, d);
+                                               [=](int j) { return xi[j]; }, [=](int j) { return xd[j]; }, d);
                 if (bad && !(keep >> (part & 1) & 1)) v = part & 1 ? d.y : d.x;
             }
             if (mine) {
@@ -232,16 +240,16 @@ __device__ __forceinline__ void edge_rows_fx(const DevModel& dm, const FxMat& S,
     }
 }
 // S: S_E^-1, staged or not; in FP64 S, Ye point at the complex128 matrices and Sx at the split S_E^-1
-template <class T, int RB, class F>
+template <class T, int RB>
 __device__ __forceinline__ void edge_rows(const DevModel& dm, int e, const cpx<T>* S, const FxMat& Sx, const cpx<T>* Ye, int nE,
-                                          int nT, const EdgeVec<T>& rE, const int* ex, const F& load, int vs, int cnt, int tpr,
+                                          int nT, const EdgeVec<T>& rE, const int* ex, int vs, int cnt, int tpr,
                                           int r0, int e1o, int to, cpx<T>* __restrict__ xE_out,
                                           cpx<T>* __restrict__ tT_out, int o_lo, int o_hi) {
     if constexpr (std::is_same<T, double>::value) {
         constexpr int parts = kEdgeParts<T, RB>;
         const int nt = blockDim.x / parts, part = threadIdx.x / nt;
         edge_rows_fx<RB / parts>(dm, Sx, dm.y_fx.at(dm.pq_off[e]), reinterpret_cast<const double2*>(S),
-                                 reinterpret_cast<const double2*>(Ye), nE, nT, rE, ex, load, vs, cnt, tpr, r0, e1o, to, xE_out,
+                                 reinterpret_cast<const double2*>(Ye), nE, nT, rE, ex, vs, cnt, tpr, r0, e1o, to, xE_out,
                                  tT_out, o_lo, o_hi, threadIdx.x - part * nt, nt, part * (RB / parts));
     } else edge_rows_f<T, RB>(dm, S, Ye, nE, nT, rE.v, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
 }
@@ -270,8 +278,7 @@ __device__ __forceinline__ void edge_copy(uint64_t* bar, char* dst, const DevMod
     }
 }
 
-// entry i of r_E of right-hand side r0 + q.  (The staged vectors' loads capture by value: what they hold also stays
-// in registers where fx_again is called.)
+// entry i of r_E of right-hand side r0 + q
 template <class T>
 __device__ __forceinline__ auto pass1_load(const DevModel& dm, const double2* z, double zsign, const double2* bt, int r0,
                                            int e1o, int64_t off) {
@@ -331,7 +338,7 @@ __global__ void __launch_bounds__(kEdgeParts<T, RB> == 2 ? 640 : 256) k_pass1_ed
     const int tpr = edge_tpr<T>(nE + nT, (nE + nT) * 4 <= (int)blockDim.x ? 4 : 2);
     // rows: 0 all output rows, 1 the x_E rows only, 2 the t_T rows only (no S_E^-1 read)
     const int o_lo = rows == 2 ? nE : 0, o_hi = rows == 1 ? nE : nE + nT;
-    edge_rows<T, RB>(dm, e, S, Sx, Y + dm.pq_off[e], nE, nT, rE, ex, load, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
+    edge_rows<T, RB>(dm, e, S, Sx, Y + dm.pq_off[e], nE, nT, rE, ex, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, o_lo, o_hi);
 }
 
 // The same pass as one persistent launch over a degree-sorted work list.  Task t is (element
@@ -405,7 +412,7 @@ __global__ void __launch_bounds__(kEdgeParts<T, RB> == 2 ? 640 : 256) k_pass1_ed
         int tpr = tpr_force > 0 ? tpr_force : (tpr_p ? (int)tpr_p[dm.p[e]] : 0);
         if (tpr != 2 && tpr != 4) tpr = nE + nT <= 64 ? 4 : 2;
         tpr = edge_tpr<T>(nE + nT, tpr);
-        edge_rows<T, RB>(dm, e, S, Sx, Y + dm.pq_off[e], nE, nT, rE, ex, load, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, 0,
+        edge_rows<T, RB>(dm, e, S, Sx, Y + dm.pq_off[e], nE, nT, rE, ex, vs, cnt, tpr, r0, e1o, to, xE_out, tT_out, 0,
                          nE + nT);
         __syncthreads();
     }
@@ -422,10 +429,9 @@ template <class T, int RB>
 __global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pass2_edge(const __grid_constant__ DevModel dm, const cpx<T>* __restrict__ Y,
                                                     const double2* __restrict__ x2, const cpx<T>* __restrict__ xE_in,
                                                     cpx<T>* __restrict__ xE_out, int R, const int* __restrict__ done,
-                                                    int ntask, int y_bytes) {
+                                                    int ntask, int vs, int y_off, int y_staged) {
     if (done && *done) return;
     constexpr bool fx = std::is_same<T, double>::value;
-    __shared__ __align__(16) char uT_raw[RB * 128 * kEdgeVecBytes<T>];
     __shared__ int ex[RB];
     extern __shared__ __align__(128) char smem[];
     const CtaGroup g;
@@ -436,8 +442,9 @@ __global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pass2_edge(const __
     const int nE = dm.nE1[e], e1o = dm.e1_off[e], nT = dm.nT[e], to = dm.t_off[e];
     // FP64: the split Y comes into shared memory (in flight while u_T is gathered); a bulk copy starts at a
     // multiple of 16 bytes, so the fractions of an element at an odd offset are read where they lie
-    uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
-    const bool staged = y_bytes > 0 && nE > 0 && nT > 0;
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + y_off);
+    char* Y_s = smem + y_off + 128;
+    const bool staged = y_staged && nE > 0 && nT > 0;
     FxMat Yx = dm.y2_fx.at(dm.pq_off[e]);
     if constexpr (fx)
         if (staged) {
@@ -447,13 +454,13 @@ __global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pass2_edge(const __
                 asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 bulk_expect(bar, b0 + b1);
-                bulk_copy(bar, smem + 128, Yx.i, b0);
-                if (b1) bulk_copy(bar, smem + 128 + b0, Yx.f, b1);
+                bulk_copy(bar, Y_s, Yx.i, b0);
+                if (b1) bulk_copy(bar, Y_s + b0, Yx.f, b1);
             }
-            Yx.i = reinterpret_cast<int4*>(smem + 128);
-            if (b1) Yx.f = reinterpret_cast<float2*>(smem + 128 + b0);
+            Yx.i = reinterpret_cast<int4*>(Y_s);
+            if (b1) Yx.f = reinterpret_cast<float2*>(Y_s + b0);
         }
-    const EdgeVec<T> uT(uT_raw, RB * 128);
+    const EdgeVec<T> uT(smem, RB * vs);
     const auto load = [dp = &dm, x2, to, r0](int q, int i) {
         const int r = r0 + q;
         cpx<T> u = mk<T>(0, 0);
@@ -465,7 +472,7 @@ __global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pass2_edge(const __
         }
         return u;
     };
-    edge_stage<T, RB>(load, nT, 128, cnt, uT, ex);
+    edge_stage<T, RB>(load, nT, vs, cnt, uT, ex);
     g.sync();
     if (staged && !bulk_wait_all(bar, dm.err)) return;
     // one thread per row i of Y, all RB right-hand sides at once: each Y entry is read once
@@ -485,12 +492,12 @@ __global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pass2_edge(const __
             int4 ni = make_int4(0, 0, 0, 0);
             float2 nf = make_float2(0.f, 0.f);
             if (nT > 0) { ni = Yx.i[i]; nf = Yx.f[i]; }
-#pragma unroll 2
+#pragma unroll(RT <= 2 ? 4 : 2)
             for (int t = 0; t < nT; ++t) {
                 const FxEntry y = fx_entry(ni, nf);
                 if (t + 1 < nT) { ni = Yx.i[(t + 1) * nE + i]; nf = Yx.f[(t + 1) * nE + i]; }
 #pragma unroll
-                for (int q = 0; q < RT; ++q) fx_mac(s[q], y, uT.i[(q0 + q) * 128 + t], uT.f[(q0 + q) * 128 + t]);
+                for (int q = 0; q < RT; ++q) fx_mac(s[q], y, uT.i[(q0 + q) * vs + t], uT.f[(q0 + q) * vs + t]);
             }
 #pragma unroll
             for (int q = 0; q < RT; ++q) {
@@ -505,12 +512,11 @@ __global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pass2_edge(const __
                 }
                 if (bad) {
                     double2 d;
-                    const int4 *yi = Yx.i + i, *xi = uT.i + (q0 + q) * 128;
-                    const int qq = q0 + q;
-                    bad &= ~fx_again(1, bad, nT, ea, ex[qq], [=](int t) { return yd[t]; },
+                    const int4 *yi = Yx.i + i, *xi = uT.i + (q0 + q) * vs;
+                    const double2* xd = uT.d + (q0 + q) * vs;
+                    bad &= ~fx_again(1, bad, nT, ea, ex[q0 + q], [=](int t) { return yd[t]; },
                                      [=](int t) { const int4 u = yi[t * nE]; return make_int2(u.x, u.z); },
-                                     [=](int t) { return xi[t]; },
-                                     [=](int t) { const cpx<double> x = load(qq, t); return make_double2(x.x, x.y); }, d);
+                                     [=](int t) { return xi[t]; }, [=](int t) { return xd[t]; }, d);
                     if (bad & 1) a[q].x = d.x;
                     if (bad & 2) a[q].y = d.y;
                 }
@@ -522,7 +528,7 @@ __global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pass2_edge(const __
                 const cpx<T> y = yr[t];
 #pragma unroll
                 for (int q = 0; q < RT; ++q)
-                    if (q < cnt) fma_c(a[q], y, uT.v[q * 128 + t]);
+                    if (q < cnt) fma_c(a[q], y, uT.v[q * vs + t]);
             }
         }
 #pragma unroll
@@ -628,11 +634,10 @@ __global__ void k_dinv(DevModel dm, const double2* __restrict__ x, double2* __re
 // out_E = S x for the restricted stiffness Schur complement S (n_E x n_E, symmetric, read from
 // global memory column by column: coalesced across output rows, shared by the elements of a
 // degree pattern and L1/L2-resident); tpr adjacent threads share an output row.  FP64: the products of
-// ddh_fixed.cuh, exponents pre_ex by row; load gives the staged vectors' entries (an application as below
-// 0.28 ms, 0.52 ms in FP64).
-template <class T, int RB, class F>
+// ddh_fixed.cuh, exponents pre_ex by row (an application as below 0.28 ms, 0.52 ms in FP64).
+template <class T, int RB>
 __device__ __forceinline__ void pre_apply(const DevModel& dm, int e, int nE, int cnt, const EdgeVec<T>& in, const int* ex,
-                                          const F& load, cpx<T>* __restrict__ out, int64_t ostride,
+                                          cpx<T>* __restrict__ out, int64_t ostride,
                                           const double* __restrict__ wout = nullptr) {
     const int tpr = nE <= 32 ? 4 : (nE <= 64 ? 2 : 1);
     const int chunk = (nE + tpr - 1) / tpr;
@@ -649,18 +654,27 @@ __device__ __forceinline__ void pre_apply(const DevModel& dm, int e, int nE, int
             FxSum s[RT];
 #pragma unroll
             for (int k = 0; k < RT; ++k) fx_clear(s[k]);
-            // nE <= 124 terms: one chain; the next entry's load is issued ahead
-            int2 ni = make_int2(0, 0);
-            float nf = 0.f;
-            auto fetch = [&](int j) { ni = __ldg(Sx.i + j * nE + i); nf = __ldg(Sx.f + j * nE + i); };
-            if (part * chunk < j1) fetch(part * chunk);
-#pragma unroll 2
-            for (int j = part * chunk; j < j1; ++j) {
-                const FxReal a = fx_real(ni.x, ni.y, nf);
-                if (j + 1 < j1) fetch(j + 1);
+            // nE <= 124 terms: one chain, loads of the next entries ahead (few right-hand sides: eight, the
+            // latency bounds it; 16 x 16 elements, p = 16, one right-hand side)
+            constexpr int ahead = RT <= 2 ? 8 : 2;
+            int2 ni[ahead];
+            float nf[ahead];
+            auto fetch = [&](int k, int j) {
+                ni[k] = j < j1 ? __ldg(Sx.i + j * nE + i) : make_int2(0, 0);
+                nf[k] = j < j1 ? __ldg(Sx.f + j * nE + i) : 0.f;
+            };
+            const int j0 = part * chunk;
 #pragma unroll
-                for (int q = 0; q < RT; ++q) fx_mac(s[q], a, in.i[(q0 + q) * nE + j], in.f[(q0 + q) * nE + j]);
-            }
+            for (int k = 0; k < ahead; ++k) fetch(k, j0 + k);
+            for (int jb = j0; jb < j1; jb += ahead)
+#pragma unroll
+                for (int k = 0; k < ahead; ++k) {
+                    const int j = min(jb + k, nE - 1);     // past the end the entry of S is zero
+                    const FxReal a = fx_real(ni[k].x, ni[k].y, nf[k]);
+                    fetch(k, jb + k + ahead);
+#pragma unroll
+                    for (int q = 0; q < RT; ++q) fx_mac(s[q], a, in.i[(q0 + q) * nE + j], in.f[(q0 + q) * nE + j]);
+                }
 #pragma unroll
             for (int q = 0; q < RT; ++q) {
                 unsigned bad = 0;
@@ -681,10 +695,10 @@ __device__ __forceinline__ void pre_apply(const DevModel& dm, int e, int nE, int
                     const double* S64 = S + i;
                     const int2* Si = Sx.i + i;
                     const int4* xi = in.i + (q0 + q) * nE;
-                    const int qq = q0 + q;
-                    bad &= ~fx_again(tpr, bad, nE, ea, ex[qq], [=](int j) { return make_double2(S64[j * nE], 0.0); },
+                    const double2* xd = in.d + (q0 + q) * nE;
+                    bad &= ~fx_again(tpr, bad, nE, ea, ex[q0 + q], [=](int j) { return make_double2(S64[j * nE], 0.0); },
                                      [=](int j) { return make_int2(Si[j * nE].x, 0); }, [=](int j) { return xi[j]; },
-                                     [=](int j) { const cpx<double> x = load(qq, j); return make_double2(x.x, x.y); }, d);
+                                     [=](int j) { return xd[j]; }, d);
                     if (bad & 1) v.x = d.x;
                     if (bad & 2) v.y = d.y;
                 }
@@ -752,7 +766,7 @@ __global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pre_elem(const __gr
     edge_stage<T, RB>(load, nE, nE, cnt, in, ex);
     __syncthreads();
     // Poisson mode: out = (rho_e w) .* (S^Lap (w .* C1^T v)), the diagonally scaled W^T A W
-    pre_apply<T, RB>(dm, e, nE, cnt, in, ex, load, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot,
+    pre_apply<T, RB>(dm, e, nE, cnt, in, ex, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot,
                      dm.e1_wout ? dm.e1_wout + e1o : nullptr);
 }
 
@@ -784,7 +798,7 @@ __global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pre_elem_kry(const 
     };
     edge_stage<T, RB>(load, nE, nE, cnt, in, ex);
     __syncthreads();
-    pre_apply<T, RB>(dm, e, nE, cnt, in, ex, load, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot);
+    pre_apply<T, RB>(dm, e, nE, cnt, in, ex, outE + (int64_t)r0 * dm.nE1_tot + e1o, dm.nE1_tot);
 }
 
 // z = D^-1 (outE[c] - outE[f]) with D = 2 I, written to zw and to the Krylov store Zb[r][j]
@@ -905,12 +919,14 @@ void launch_pass2_edge(const DevModel& dm, const void* Y, const double2* x2, con
     // resident per SM to hide the gather latency)
     const int nt = dm.maxE1 <= 64 ? 64 : 128;
     // FP64: room for the largest Y (nE + nT <= 4 p = 128, so at most 64 x 64 entries)
-    const int yb = std::is_same<T, double>::value && dm.maxY > 0 && dm.maxY <= 64 * 64 ? 128 + dm.maxY * kEdgeMatBytes<T> + 16 : 0;
+    const int vs = std::max(1, dm.maxT), yo = (int)edge_vec_bytes<T>(rb, vs);
+    const int ys = std::is_same<T, double>::value && dm.maxY > 0 && dm.maxY <= 64 * 64;
+    const size_t sm = yo + (ys ? 128 + dm.maxY * kEdgeMatBytes<T> + 16 : 0);
     switch (rb) {
-        case 8: k_pass2_edge<T, 8><<<ntask, nt * kEdgeParts<T, 8>, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb); break;
-        case 4: k_pass2_edge<T, 4><<<ntask, nt, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb); break;
-        case 2: k_pass2_edge<T, 2><<<ntask, nt, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb); break;
-        default: k_pass2_edge<T, 1><<<ntask, nt, yb, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, yb);
+        case 8: k_pass2_edge<T, 8><<<ntask, nt * kEdgeParts<T, 8>, sm, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, vs, yo, ys); break;
+        case 4: k_pass2_edge<T, 4><<<ntask, nt, sm, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, vs, yo, ys); break;
+        case 2: k_pass2_edge<T, 2><<<ntask, nt, sm, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, vs, yo, ys); break;
+        default: k_pass2_edge<T, 1><<<ntask, nt, sm, st>>>(dm, Yp, x2, xi, xo, R, done, ntask, vs, yo, ys);
     }
 }
 template void launch_pass1_edge<double>(const DevModel&, const void*, const void*, const double2*, double, const double2*, void*, void*, int, const int*, cudaStream_t, const EdgeSched*, int, int, int, int);
@@ -990,7 +1006,7 @@ static void set_edge_pass_limits(int maxE1) {
     cudaFuncSetAttribute(k_pass1_edge<T, RB>, cudaFuncAttributePreferredSharedMemoryCarveout,
                          (int)cudaSharedmemCarveoutMaxShared);
     if (std::is_same<T, double>::value)
-        raise_smem_limit(k_pass2_edge<T, RB>, 128 + 64 * 64 * kEdgeMatBytes<T> + 16);
+        raise_smem_limit(k_pass2_edge<T, RB>, (int)edge_vec_bytes<T>(RB, 128) + 128 + 64 * 64 * kEdgeMatBytes<T> + 16);
     int buf = 0;
     size_t tot = 0;
     edge_p_layout<T>(RB, maxE1, &buf, &tot);

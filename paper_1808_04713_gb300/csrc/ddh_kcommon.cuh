@@ -136,8 +136,8 @@ inline size_t pass_smem_total(int pmax, int rb, int maxE1) {
 // warps (elements) per CTA: up to 4 while the per-warp shared memory fits in 200 KB
 
 // edge-operator pass 1: the staged vectors, then (when it fits) the staged S_E^-1 behind an mbarrier.  Bytes per
-// entry of either: in FP64 limbs and FP32 parts (ddh_fixed.cuh)
-template <class T> constexpr int kEdgeVecBytes = sizeof(T) == 8 ? 32 : 8;
+// entry of either: in FP64 limbs and FP32 parts (ddh_fixed.cuh), and a vector's FP64 entries
+template <class T> constexpr int kEdgeVecBytes = sizeof(T) == 8 ? 48 : 8;
 template <class T> constexpr int kEdgeMatBytes = sizeof(T) == 8 ? 24 : 8;
 template <class T>
 inline size_t edge_vec_bytes(int rb, int maxE1) {
