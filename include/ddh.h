@@ -415,8 +415,9 @@ ddh_status ddh_table_fdm(int32_t p, double* V_out, double* mu_out);
 /* Gauss-Legendre nodes/weights by the Golub-Welsch method (own eigensolver). */
 ddh_status ddh_table_gauss(int32_t m, double* x_out, double* w_out);
 /* The dot product of the FP64 kernels (csrc/ddh_fixed.cuh) on the host: out[2] = sum_j a_j x_j of n complex
- * numbers (interleaved), terms dealt to `lanes` lanes; fp64_out[2]: the component was formed in FP64. */
-ddh_status ddh_fixed_dot(int32_t n, int32_t lanes, const double* a, const double* x, double* out,
+ * numbers (interleaved), terms dealt to `lanes` lanes, a in the packed form of the dense K^-1 or not;
+ * fp64_out[2]: the component was formed in FP64. */
+ddh_status ddh_fixed_dot(int32_t n, int32_t lanes, int32_t packed, const double* a, const double* x, double* out,
                          int32_t* fp64_out);
 
 /* Host-only setup and factorisation (no device work) of a mesh, for checks of the host

@@ -86,7 +86,7 @@ struct ddh_ctx {
     int tc_maxT = 0;
     double2* Kinv = nullptr;                       // dense coarse inverse (elimination order)
     float2* Kinv32 = nullptr;
-    FxMat Kinv_fx;                                 // the same split (ddh_fixed.cuh), with its exponents
+    longlong2* Kinv_fx = nullptr;                  // the same packed (ddh_fixed.cuh), with its exponents
     int* Kinv_ex = nullptr;
     int nsm = 0;                                   // SMs of the device
     // nested-dissection factor: complex128 matrices, their complex64 copy (nd32.G/M null
@@ -649,7 +649,7 @@ static ddh_status upload_model(ddh_ctx* ctx) {
         if ((st = upload(ctx, conv32(Kn), &a32))) return st;
         ctx->Kinv32 = (float2*)a32;
         if ((st = model_alloc(ctx, sizeof(int) * (size_t)nc * gemv_tiles(nc), (void**)&ctx->Kinv_ex))) return st;
-        if ((st = alloc_split(ctx, (size_t)nc * nc, ctx->Kinv_fx))) return st;
+        if ((st = model_alloc(ctx, sizeof(longlong2) * (size_t)nc * nc, (void**)&ctx->Kinv_fx))) return st;
         CK(cudaDeviceGetAttribute(&ctx->nsm, cudaDevAttrMultiProcessorCount, ctx->device));
         launch_fix_dense(ctx->Kinv, nc, ctx->Kinv_fx, ctx->Kinv_ex, ctx->stream);
         gemv_set_smem_limits();
@@ -2864,7 +2864,8 @@ ddh_status ddh_table_gauss(int32_t m, double* x, double* w) {
     std::memcpy(w, ww.data(), sizeof(double) * m);
     return DDH_OK;
 }
-ddh_status ddh_fixed_dot(int32_t n, int32_t lanes, const double* a, const double* x, double* out, int32_t* fp64) {
+ddh_status ddh_fixed_dot(int32_t n, int32_t lanes, int32_t packed, const double* a, const double* x, double* out,
+                         int32_t* fp64) {
     if (n < 0 || lanes < 1 || !a || !x || !out || !fp64) return DDH_ERR_INVALID_ARG;
     if ((int64_t)lanes * ((n / lanes + 1) / kFxChain + 1) > kFxFlushes) return DDH_ERR_INVALID_ARG;
     auto at = [](const double* v, int j) { return make_double2(v[2 * j], v[2 * j + 1]); };
@@ -2887,7 +2888,8 @@ ddh_status ddh_fixed_dot(int32_t n, int32_t lanes, const double* a, const double
             const FxVec v = fx_vec(at(x, j), ex);
             int4 ai;
             float2 af;
-            fx_put(FxMat{&ai, &af}, 0, at(a, j), ea);
+            if (packed) fx_unpack(make_longlong2(fx_pack(a[2 * j], ea), fx_pack(a[2 * j + 1], ea)), ai, af);
+            else fx_put(FxMat{&ai, &af}, 0, at(a, j), ea);
             fx_mac(s, fx_entry(ai, af), v.i, v.f);
             if (++c == kFxChain) {
                 c = 0;
@@ -2897,6 +2899,7 @@ ddh_status ddh_fixed_dot(int32_t n, int32_t lanes, const double* a, const double
         flush();
     }
     const bool special = ea == 0x7ff || ex == 0x7ff;
+    const int bits = packed ? kFxSmallPacked : kFxSmall;
     FxWeight w = {0.f, 0.f};
     double sx = 0, sy = 0;
     for (int j = 0; j < n; ++j) {
@@ -2906,7 +2909,7 @@ ddh_status ddh_fixed_dot(int32_t n, int32_t lanes, const double* a, const double
         sy = std::fma(u.x, v.y, std::fma(u.y, v.x, sy));
     }
     for (int i = 0; i < 2; ++i) {
-        fp64[i] = !fx_value(h[i], l[i], ea, ex, out[i]) && (special || !fx_heavy(i ? w.y : w.x));
+        fp64[i] = !fx_value(h[i], l[i], ea, ex, out[i], bits) && (special || !fx_heavy(i ? w.y : w.x, bits));
         if (fp64[i]) out[i] = i ? sy : sx;
     }
     return DDH_OK;

@@ -270,13 +270,13 @@ bool coarse_factor(Model& m, const std::vector<int32_t>& kn_ptr, const std::vect
     // ---- dense inverse for small coarse problems (elimination order), refined like the solves
     // automatic form: K^-1 up to 2048 unknowns.  Its columns are n_c solves on the host, so the line is a trade of
     // factor time against the time of a solve.  One application in FP64, 1 / 8 right-hand sides, and the whole
-    // factorisation: n_c = 1921 dense 23 / 126 us, 0.14 s, nested dissection 82 / 89 us, 0.04 s; 2413: 37 / 165
-    // us, 0.15 s against 99 / 106 us, 0.05 s; 2961: 60 / 295 us, 0.21 s against 97 / 107 us, 0.05 s; 3888: 80 / 403
-    // us, 0.36 s against 111 / 117 us, 0.06 s; 5320: 143 / 762 us, 0.66 s against 110 / 130 us, 0.07 s.  From 2048
+    // factorisation: n_c = 1921 dense 25 / 138 us, 0.13 s, nested dissection 82 / 90 us, 0.04 s; 2413: 32 / 174
+    // us, 0.14 s against 98 / 105 us, 0.05 s; 2961: 59 / 301 us, 0.21 s against 98 / 109 us, 0.05 s; 3888: 78 / 429
+    // us, 0.35 s against 110 / 121 us, 0.06 s; 5320: 137 / 777 us, 0.66 s against 117 / 131 us, 0.07 s.  From 2048
     // on a solve with several right-hand sides is always faster by nested dissection; one with a single
-    // right-hand side loses 1.6 ms (n_c = 2413) or 1.3 ms (2961, 3888), which the factorisation gains back
+    // right-hand side loses 1.7 ms (n_c = 2413) or 1.3 ms (2961, 3888), which the factorisation gains back
     // unless 60 (2413) to 230 (3888) such solves follow it: coarse_form = DDH_COARSE_DENSE is for those.  The
-    // complex64 copy: dense 121 / 587 us at 1921 and 217 / 1080 us at 2961 against 139 / 154 and 161 / 175 us.
+    // complex64 copy: dense 126 / 586 us at 1921 and 222 / 1081 us at 2961 against 141 / 153 and 161 / 175 us.
     m.dense_coarse = m.coarse_form == 1 || (m.coarse_form == 0 && nc <= 2048);   // 2, 3: nested dissection
     m.Kinv.clear();
     if (m.dense_coarse) {

@@ -7,7 +7,7 @@
 // A number v with |v| < 2^e is held as X = v 2^(52 - e) = h 2^26 + l + f: -2^26 <= h < 2^26, 0 <= l < 2^26,
 // 0 <= f < 1.  The exponent e is shared: by one row of the matrix (fixed when the matrix is laid
 // out) and by one staged vector (its largest component, found while it is staged).  A matrix is kept in this
-// form (24 bytes an entry) beside its complex128 one.  Then
+// form (24 bytes an entry, or packed in 16) beside its complex128 one.  Then
 //   a x = ah xh 2^52 + (ah xl + al xh) 2^26 + [ (ah xf + af xh) 2^26 + al xl + af xf ] + (al xf + af xl, below
 //         2^-25 of the bracket's bound)
 // The first two kinds are summed in 64-bit integers, without error; the bracket in FP32.  The bracket is at most
@@ -184,6 +184,22 @@ DDH_FX void fx_put(const FxRealMat& m, int64_t k, double v, int ef) {
     m.i[k] = make_int2(a.h, a.l);
     m.f[k] = a.f;
 }
+// The same in 16 bytes, 11 bits of f left: for a matrix that is read faster than its products are formed.  A
+// sum comes out to 2^-64 (60 terms) to 2^-63 (255) of the scale, so P must reach 2^-kFxSmallPacked of it.
+DDH_FX long long fx_pack(double v, int ef) {
+    const FxNum a = fx_split(v, ef);
+    const long long f = (long long)(a.f * 0x1p-15f);       // f 2^11, rounded down
+    return v != 0.0 ? (((((long long)a.h << kFxLow) + a.l) << 11) + f) | 1 : 0;
+}
+DDH_FX void fx_unpack(const longlong2& p, int4& i, float2& f) {
+    const unsigned xl = (unsigned)p.x, xh = (unsigned)(p.x >> 32), yl = (unsigned)p.y, yh = (unsigned)(p.y >> 32);
+    constexpr unsigned mask = (1u << kFxLow) - 1;
+    i.x = (int)xh >> 5;
+    i.y = (int)(fx_funnel(xl, xh, 11) & mask);
+    i.z = (int)yh >> 5;
+    i.w = (int)(fx_funnel(yl, yh, 11) & mask);
+    f = make_float2((float)(int)(xl & 2047) * 0x1p15f, (float)(int)(yl & 2047) * 0x1p15f);
+}
 struct FxReal {
     int h, l;
     FxPair fh, fl, f;
@@ -257,16 +273,16 @@ DDH_FX void fx_flush(const FxSum& s, int c, long long& h, long long& l) {
     l += ((t & 255) << 28) + ((sl & ((1ll << kFxLow) - 1)) << 2) + (long long)rintf((c ? p + q : p - q) * 0x1p-24f);
     if (p != 0.f || q != 0.f || sl != 0) l += 1ll << 50;
 }
-// 2^-kFxSmall of the scale: results and weights below it
-constexpr int kFxSmall = 16;
+// 2^-kFxSmall of the scale: results and weights below it (of a packed matrix 2^-kFxSmallPacked)
+constexpr int kFxSmall = 16, kFxSmallPacked = 10;
 // The value of a sum on the scales of exponents ea (matrix row) and ex (vector).  False: it is small, or
 // not a number (fx_again decides what it is to be).
-DDH_FX bool fx_carry(long long& h, long long& l, int ea, int ex) {
+DDH_FX bool fx_carry(long long& h, long long& l, int ea, int ex, int bits) {
     const long long any = (l + (1ll << 49)) >> 50;
     l -= any << 50;
     h += l >> 36;
     l &= (1ll << 36) - 1;
-    constexpr long long small = 1ll << (2 * kFxBits - 60 - kFxSmall);             // the scale is 2^104, h counts 2^60
+    const long long small = 1ll << (2 * kFxBits - 60 - bits);                     // the scale is 2^104, h counts 2^60
     return ea != 0x7ff && ex != 0x7ff && (any == 0 || h >= small || h < -small);
 }
 DDH_FX double fx_pow2(int s) { return fx_double((unsigned long long)(1023 + s) << 52); }       // -1022 <= s <= 1023
@@ -276,8 +292,8 @@ DDH_FX double fx_ldexp(double d, int s) {
     return r ? d * fx_pow2(r > 1000 ? 1000 : (r < -1000 ? -1000 : r)) : d;
 }
 DDH_FX int fx_scale_exp(int ea, int ex) { return ea + ex - 2044 - 2 * kFxBits; }                // of a unit of the sum
-DDH_FX bool fx_value(long long h, long long l, int ea, int ex, double& v) {
-    const bool ok = fx_carry(h, l, ea, ex);
+DDH_FX bool fx_value(long long h, long long l, int ea, int ex, double& v, int bits = kFxSmall) {
+    const bool ok = fx_carry(h, l, ea, ex, bits);
     const unsigned long long m = (unsigned long long)(h ^ (h >> 63));
 #ifdef __CUDA_ARCH__
     int k = __clzll((long long)m) - 1;                     // headroom of h
@@ -290,7 +306,7 @@ DDH_FX bool fx_value(long long h, long long l, int ea, int ex, double& v) {
 }
 // the same as hi + lo, each of at most 53 bits
 DDH_FX bool fx_value2(long long h, long long l, int ea, int ex, double& hi, double& lo) {
-    const bool ok = fx_carry(h, l, ea, ex);
+    const bool ok = fx_carry(h, l, ea, ex, kFxSmall);
     hi = fx_ldexp((double)(h & ~2047ll), 60 + fx_scale_exp(ea, ex));
     lo = fx_ldexp((double)(((h & 2047) << 36) | l), 24 + fx_scale_exp(ea, ex));
     return ok;
@@ -304,7 +320,7 @@ DDH_FX void fx_weigh(FxWeight& w, int ah, int bh, const int4& x) {
     w.x += ax * xx + ay * xy;
     w.y += ax * xy + ay * xx;
 }
-DDH_FX bool fx_heavy(float w) { return w >= (float)(1ll << (2 * kFxLow - kFxSmall)); }        // the scale is 2^52
+DDH_FX bool fx_heavy(float w, int bits) { return w >= (float)(1ll << (2 * kFxLow - bits)); }  // the scale is 2^52
 
 #ifdef __CUDACC__
 // What is to become of the components that fx_value turned down, of one row and one vector, by the G lanes
@@ -313,7 +329,7 @@ DDH_FX bool fx_heavy(float w) { return w >= (float)(1ll << (2 * kFxLow - kFxSmal
 // are; d holds the FP64 sums for the others.
 template <class FA, class FH, class FI, class FX>
 __device__ __noinline__ unsigned fx_again(int G, unsigned bad, int n, int ea, int ex, const FA& a, const FH& ah, const FI& xi,
-                                          const FX& x, double2& d) {
+                                          const FX& x, double2& d, int bits = kFxSmall) {
     const int j0 = threadIdx.x & (G - 1);
     for (int o = G >> 1; o > 0; o >>= 1) bad |= __shfl_xor_sync(0xffffffffu, bad, o);
     FxWeight w = {0.f, 0.f};
@@ -327,7 +343,7 @@ __device__ __noinline__ unsigned fx_again(int G, unsigned bad, int n, int ea, in
         w.x += __shfl_xor_sync(0xffffffffu, w.x, o);
         w.y += __shfl_xor_sync(0xffffffffu, w.y, o);
     }
-    const unsigned keep = (fx_heavy(w.x) ? 1 : 0) | (fx_heavy(w.y) ? 2 : 0);
+    const unsigned keep = (fx_heavy(w.x, bits) ? 1 : 0) | (fx_heavy(w.y, bits) ? 2 : 0);
     const bool need = (bad & ~keep) != 0;
     if (G > 1 ? !__any_sync(0xffffffffu, need) : !need) return keep;
     double sx = 0, sy = 0;

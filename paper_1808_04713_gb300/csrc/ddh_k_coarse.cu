@@ -18,14 +18,20 @@ __device__ __forceinline__ void fix_row(const double2* a, const FxMat& d, int64_
     for (int j = lane; j < n; j += 32) fx_put(d, j * cs, a[j * cs], ef);
     if (lane == 0) *ex = ef;
 }
-// K^-1: one exponent per row and tile of kGemvTile columns
+// K^-1, packed: one exponent per row and tile of kGemvTile columns
 constexpr int kGemvThreads = 512, kGemvTile = 736;
-__global__ void k_fix_dense(const double2* __restrict__ A, int n, FxMat d, int* __restrict__ ex) {
-    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nt = (n + kGemvTile - 1) / kGemvTile;
+__global__ void k_fix_dense(const double2* __restrict__ A, int n, longlong2* __restrict__ d, int* __restrict__ ex) {
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int nt = (n + kGemvTile - 1) / kGemvTile;
     if (row >= n) return;
     for (int t = 0; t < nt; ++t) {
         const int64_t at = (int64_t)row * n + t * kGemvTile;
-        fix_row(A + at, d.at(at), 1, min(kGemvTile, n - t * kGemvTile), ex + (int64_t)row * nt + t);
+        const int w = min(kGemvTile, n - t * kGemvTile);
+        unsigned m = 0;
+        for (int j = lane; j < w; j += 32) m = max(m, fx_mag(A[at + j]));
+        const int ef = fx_exp(__reduce_max_sync(0xffffffffu, m));
+        for (int j = lane; j < w; j += 32) d[at + j] = make_longlong2(fx_pack(A[at + j].x, ef), fx_pack(A[at + j].y, ef));
+        if (lane == 0) ex[(int64_t)row * nt + t] = ef;
     }
 }
 // the two matrices of one nested-dissection front per CTA (layouts: NDDev)
@@ -184,10 +190,12 @@ __device__ __forceinline__ void group_sum_transpose(T (&v)[V]) {
 // y = K^-1 x with the products of ddh_fixed.cuh.  A CTA of 16 warps owns `rpc` rows (one CTA per SM), one warp
 // per row.  It stages x in shared memory as limbs, G tiles of kGemvTile columns at a time (each tile of a
 // row and of a vector has its own exponent, so a right-hand side's result does not depend on RB), and adds
-// the tiles up in FP64.  n = 1921: 23 us for one right-hand side (35 us in FP64; reading 24 n^2 bytes bounds it),
-// 126 us for eight; n = 2961: 60 and 295 us.
+// the tiles up in FP64.  K^-1 is packed: in the 24 bytes of the split form it does not stay in L2 between the
+// iterations of a solve (n = 1921, one right-hand side: 1.95 ms a solve instead of 1.77 ms).  n = 1921: 25 us for one
+// right-hand side (35 us in FP64), 138 us for eight; n = 2961: 59 and 301 us.
 template <int RB>
-__global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const double2* __restrict__ A, FxMat Ax, const int* __restrict__ aex, int n,
+__global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const double2* __restrict__ A, const longlong2* __restrict__ Ap,
+                                                         const int* __restrict__ aex, int n,
                                                          const double2* __restrict__ x, double2* __restrict__ y,
                                                          int r0, int nr, int rpc, const int* __restrict__ done) {
     if (done && *done) return;
@@ -250,21 +258,19 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const double2* __restr
 #pragma unroll
                 for (int i = 0; i < RB; ++i) fx_clear(s[i]);
                 constexpr int U = RB == 1 ? 6 : (RB == 2 ? 4 : 2);     // loads issued ahead of their use
-                int4 av[U];
-                float2 af[U];
-                const FxMat ax = Ax.at((int64_t)(row0 + k) * n + c0);
-                auto fetch = [&](int u, int j) {
-                    av[u] = j < w ? __ldg(ax.i + j) : make_int4(0, 0, 0, 0);
-                    af[u] = j < w ? __ldg(ax.f + j) : make_float2(0.f, 0.f);
-                };
+                longlong2 av[U];
+                const longlong2* ap = Ap + (int64_t)(row0 + k) * n + c0;
 #pragma unroll
-                for (int u = 0; u < U; ++u) fetch(u, lane + 32 * u);
+                for (int u = 0; u < U; ++u) av[u] = lane + 32 * u < w ? __ldg(ap + lane + 32 * u) : make_longlong2(0, 0);
                 for (int j = lane; j < w; j += 32 * U) {
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const FxEntry v = fx_entry(av[u], af[u]);
-                        const int jj = o + min(j + 32 * u, w - 1);
-                        fetch(u, j + 32 * (U + u));
+                        int4 ai;
+                        float2 af;
+                        fx_unpack(av[u], ai, af);
+                        const FxEntry v = fx_entry(ai, af);
+                        const int jj = o + min(j + 32 * u, w - 1), jn = j + 32 * (U + u);
+                        av[u] = jn < w ? __ldg(ap + jn) : make_longlong2(0, 0);
 #pragma unroll
                         for (int b = 0; b < RB; ++b) fx_mac(s[b], v, xs[b * stride + jj], xf[b * stride + jj]);
                     }
@@ -280,7 +286,7 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const double2* __restr
 #pragma unroll
                 for (int i = 0; i < 8; ++i) e = i == tl * RB + (q >> 1) ? ex[i] : e;
                 double v = 0;
-                const bool bad = (q >> 1) < nr && !fx_value(hs, ls, ea, e, v);
+                const bool bad = (q >> 1) < nr && !fx_value(hs, ls, ea, e, v, kFxSmallPacked);
                 if (__any_sync(0xffffffffu, bad)) {
 #pragma unroll 1
                     for (int b = 0; b < nr; ++b) {
@@ -291,10 +297,10 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv_fx(const double2* __restr
 #pragma unroll
                         for (int i = 0; i < 8; ++i) eb = i == tl * RB + b ? ex[i] : eb;
                         double2 r;
-                        const int4 *ai = ax.i, *xi = xs + b * stride + o;
+                        const int4* xi = xs + b * stride + o;
                         const unsigned keep = fx_again(32, this_b ? 1u << (q & 1) : 0, w, ea, eb, [=](int j) { return a[j]; },
-                                                       [=](int j) { const int4 u = ai[j]; return make_int2(u.x, u.z); },
-                                                       [=](int j) { return xi[j]; }, [=](int j) { return xq[j]; }, r);
+                                                       [=](int j) { const longlong2 u = ap[j]; return make_int2((int)(u.x >> 37), (int)(u.y >> 37)); },
+                                                       [=](int j) { return xi[j]; }, [=](int j) { return xq[j]; }, r, kFxSmallPacked);
                         if (this_b && !(keep >> (q & 1) & 1)) v = q & 1 ? r.y : r.x;
                     }
                 }
@@ -1066,8 +1072,8 @@ void launch_csr_residual(const int* ptr, const int* col, const double2* v, const
     else k_csr_residual<1><<<dim3(g, 1), 128, 0, st>>>(ptr, col, v, vx, vex, n, x, t, r, R, done);
 }
 int gemv_tiles(int n) { return (n + kGemvTile - 1) / kGemvTile; }
-void launch_fix_dense(const double2* A, int n, const FxMat& Ax, int* ex, cudaStream_t st) {
-    k_fix_dense<<<(n + 3) / 4, 128, 0, st>>>(A, n, Ax, ex);
+void launch_fix_dense(const double2* A, int n, longlong2* Ap, int* ex, cudaStream_t st) {
+    k_fix_dense<<<(n + 3) / 4, 128, 0, st>>>(A, n, Ap, ex);
 }
 void launch_fix_fronts(const NDDev& d, int nodes, cudaStream_t st) {
     if (nodes > 0) k_fix_fronts<<<nodes, 256, 0, st>>>(d);
@@ -1092,7 +1098,7 @@ void gemv_set_smem_limits() {
     raise_smem_limit(k_gemv_fx<2>, most);
     raise_smem_limit(k_gemv_fx<4>, most);
 }
-void launch_gemv(const double2* A, const FxMat& Ax, const int* ex, int n, const double2* x, double2* y, int R, const int* done, int nsm,
+void launch_gemv(const double2* A, const longlong2* Ap, const int* ex, int n, const double2* x, double2* y, int R, const int* done, int nsm,
                  cudaStream_t st) {
     const int rpc = gemv_rows(n, nsm);
     const int g = (n + rpc - 1) / rpc;
@@ -1100,7 +1106,7 @@ void launch_gemv(const double2* A, const FxMat& Ax, const int* ex, int n, const 
         const int left = std::min(R - r0, 4);                  // a sum is twelve registers
         const int rb = left >= 3 ? 4 : left;
         const size_t sm = (size_t)rb * ((8 / rb * kGemvTile + 1) * (sizeof(int4) + sizeof(float4)) + (size_t)rpc * 2 * sizeof(double));
-#define DDH_GEMV(RBV) k_gemv_fx<RBV><<<g, kGemvThreads, sm, st>>>(A, Ax, ex, n, x, y, r0, left, rpc, done);
+#define DDH_GEMV(RBV) k_gemv_fx<RBV><<<g, kGemvThreads, sm, st>>>(A, Ap, ex, n, x, y, r0, left, rpc, done);
         switch (rb) { case 4: DDH_GEMV(4) break; case 2: DDH_GEMV(2) break; default: DDH_GEMV(1) }
 #undef DDH_GEMV
         r0 += left;

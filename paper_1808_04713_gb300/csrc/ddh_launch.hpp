@@ -182,12 +182,12 @@ void launch_fix_csr(const int* ptr, const double2* val, const FxMat& vx, int* ve
 void launch_csr_residual(const int* ptr, const int* col, const double2* val, const FxMat& vx, const int* vex, int n,
                          const double2* x, const double2* t, double2* r, int R, const int* done, cudaStream_t st);
 void launch_dinv(const DevModel& dm, const double2* x, double2* y, int R, const int* done, cudaStream_t st);
-// y = K^-1 x for the dense inverse (Ax, ex: split by row and tile of columns, gemv_tiles(n) exponents a row,
+// y = K^-1 x for the dense inverse (Ap, ex: packed by row and tile of columns, gemv_tiles(n) exponents a row,
 // made by launch_fix_dense; nsm = SMs of the device), R right-hand sides
-void launch_gemv(const double2* A, const FxMat& Ax, const int* ex, int n, const double2* x, double2* y, int R, const int* done, int nsm,
+void launch_gemv(const double2* A, const longlong2* Ap, const int* ex, int n, const double2* x, double2* y, int R, const int* done, int nsm,
                  cudaStream_t st);
 int gemv_tiles(int n);
-void launch_fix_dense(const double2* A, int n, const FxMat& Ax, int* ex, cudaStream_t st);
+void launch_fix_dense(const double2* A, int n, longlong2* Ap, int* ex, cudaStream_t st);
 void gemv_set_smem_limits();
 // the same for the complex64 copy
 void launch_gemv32(const float2* A, int n, const double2* x, double2* y, int R, const int* done, cudaStream_t st);

@@ -88,7 +88,7 @@ _SIGS = {
     "ddh_table_affine": (C.c_int, [C.c_int32, C.c_double, C.c_double, C.c_void_p]),
     "ddh_table_fdm": (C.c_int, [C.c_int32, C.c_void_p, C.c_void_p]),
     "ddh_table_gauss": (C.c_int, [C.c_int32, C.c_void_p, C.c_void_p]),
-    "ddh_fixed_dot": (C.c_int, [C.c_int32, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
+    "ddh_fixed_dot": (C.c_int, [C.c_int32, C.c_int32, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
     "ddh_host_factor": (C.c_int, [C.c_int32, C.c_void_p, C.c_void_p, C.c_int32, C.c_double, C.c_void_p,
                                   C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p]),
 }
@@ -366,12 +366,12 @@ def table_gauss(m: int):
     return x, w
 
 
-def fixed_dot(a, x, lanes: int = 1):
+def fixed_dot(a, x, lanes: int = 1, packed: bool = False):
     """(sum_j a_j x_j as the FP64 kernels form it, (real, imaginary part formed in FP64))."""
     a = np.ascontiguousarray(a, dtype=np.complex128)
     x = np.ascontiguousarray(x, dtype=np.complex128)
     out, fp64 = np.zeros(2), np.zeros(2, np.int32)
-    st = load_library().ddh_fixed_dot(len(a), int(lanes), a.ctypes.data, x.ctypes.data, out.ctypes.data, fp64.ctypes.data)
+    st = load_library().ddh_fixed_dot(len(a), int(lanes), int(packed), a.ctypes.data, x.ctypes.data, out.ctypes.data, fp64.ctypes.data)
     if st:
         raise DDHError(st, "fixed_dot")
     return complex(out[0], out[1]), (bool(fp64[0]), bool(fp64[1]))

@@ -4,19 +4,25 @@ host against exact rational sums.
 Bound: per component, 2^-52 P with P = sum of the absolute products in it.  (FP64 itself is bounded by
 2 K 2^-53 P for K complex terms.  A component kept from the integer sum is rounded once, 2^-53 of at most
 P, and the FP32 part adds 2^-72 to 2^-69 of the scale where P is 2^-16 of it or more, 2^-53 P at the most;
-one formed in FP64 has random rounding errors, so it gets the FP64 bound.)"""
+one formed in FP64 has random rounding errors, so it gets the FP64 bound.  The packed form's entries are
+cut at 2^-64 of their scale, which makes 2^-64 to 2^-63 of the scale where P is 2^-10 of it or more, 2^-53 P,
+one standard deviation: 2^-51 P.)"""
 from fractions import Fraction
 
 import numpy as np
 import pytest
 
 
-@pytest.fixture(scope="module")
-def dot():
+@pytest.fixture(scope="module", params=[False, True], ids=["split", "packed"])
+def dot(request):
     from paper_1808_04713_gb300 import build as b
     b.build()
     from paper_1808_04713_gb300 import ddh
-    return ddh.fixed_dot
+
+    def f(a, x, lanes):
+        return ddh.fixed_dot(a, x, lanes, packed=request.param)
+    f.tol = 2 if request.param else 1
+    return f
 
 
 def _exact(a, x):
@@ -35,7 +41,7 @@ def _check(dot, a, x, lanes):
     y, fp64 = dot(a, x, lanes)
     ref, P = _exact(a, x)
     for c, got in enumerate((y.real, y.imag)):
-        tol = P[c] * Fraction(max(1, len(a)) if fp64[c] else 1, 2 ** 52)
+        tol = P[c] * Fraction(max(1, len(a)) if fp64[c] else dot.tol, 2 ** 52)
         assert abs(Fraction(got) - ref[c]) <= tol, (c, fp64, got, float(ref[c]), float(P[c]))
     return y, fp64
 
@@ -68,7 +74,8 @@ def test_graded_rows_and_vectors(dot, g, K, lanes):
     # two regions: nothing of the vector's large part meets the row's
     half = np.where(np.arange(K) < K // 2, 1.0, g)
     _, fp64 = _check(dot, a * half, x * half[::-1], lanes)
-    assert fp64 == (g < 1e-4, g < 1e-4)
+    if g < 1e-4:                         # P is at most K g of the scale (at 1e-4: between the two forms' limits)
+        assert fp64 == (True, True)
     # a small imaginary part of everything
     _check(dot, a.real * (1 + 0j), x.real + 1j * g * x.imag, lanes)
     _check(dot, a.real + 1j * g * a.imag, x, lanes)
