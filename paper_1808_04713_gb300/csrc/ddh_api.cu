@@ -79,6 +79,7 @@ struct ddh_ctx {
     std::map<int, std::vector<int>> edge_tpr_host;
     std::map<int, bool> edge_persist;              // per (precision, RHS block): persistent form timed faster
     std::map<int, int> edge_nt;                    // per (precision, RHS block): CTA size of the one-CTA form
+    std::map<int, bool> edge_staged;               // and whether it stages S_E^-1
     std::map<int, FdmCfg> fdm1, fdm2;              // per (precision, RHS block): shapes of the FDM passes
     const float* tc_W = nullptr;                   // [S_E^-1; Y^T] planes for the tensor-core pass 1
     const int64_t* tc_off = nullptr;
@@ -214,6 +215,7 @@ static void free_model(ddh_ctx* ctx) {
     ctx->edge_tpr_host.clear();
     ctx->edge_persist.clear();
     ctx->edge_nt.clear();
+    ctx->edge_staged.clear();
     ctx->fdm1.clear();
     ctx->fdm2.clear();
     ctx->tc_W = nullptr;
@@ -1157,17 +1159,27 @@ static ddh_status edge_tune(ddh_ctx* ctx, const Work& w, int R, bool fp64) {
         return st;
     }
     // then the whole pass in each launch form: the tuned persistent one over the sorted list, and
-    // one CTA per (element, RHS block) with 256 threads or with the size rule of the launcher
-    // (two threads per output row of the widest element); keep the fastest
+    // one CTA per (element, RHS block) with 256 threads or with the size rule of the launcher (two threads per
+    // output row of the widest element); keep the fastest.  In FP64 a CTA of eight right-hand sides has twice the
+    // threads at 96 registers, so smaller ones, which take the rows in several turns, put more CTAs on an SM;
+    // and without S_E^-1 in shared memory two fit where its copy leaves room for one.  No sum depends on either.
     es.tpr_p = dt;
+    struct Form { int threads; bool stage; };               // threads 0: persistent
+    std::vector<Form> forms = {{0, true}, {256, true}};
     const int nt_rule = edge_cta_threads(d.maxNo);
-    const int forms[3][2] = {{1, 0}, {0, 256}, {0, nt_rule}};     // {persistent, CTA threads}
-    float tm[3] = {1e30f, 1e30f, 1e30f};
-    for (int f = 0; f < 3; ++f) {
-        if (f == 2 && nt_rule == 256) continue;
+    if (nt_rule != 256) forms.push_back({nt_rule, true});
+    if (fp64) {
+        for (int nt : {160, 128, 96})
+            if (nt != nt_rule) forms.push_back({nt, true});
+        for (size_t f = 1, n = forms.size(); f < n; ++f) forms.push_back({forms[f].threads, false});
+    }
+    float persistent = 1e30f, best = 1e30f;
+    Form pick = forms[1];
+    for (const Form& f : forms) {
         EdgeSched one;
-        one.cta_threads = forms[f][1];
-        const EdgeSched* sp = forms[f][0] ? &es : &one;
+        one.cta_threads = f.threads;
+        one.stage = f.stage;
+        const EdgeSched* sp = f.threads ? &one : &es;
         auto run = [&] {
             if (fp64) launch_pass1_edge<double>(d, sinv, Y, w.vd, 1.0, nullptr, w.xE, w.tT, R, nullptr, s, sp);
             else launch_pass1_edge<float>(d, sinv, Y, w.vd, 1.0, nullptr, w.xE, w.tT, R, nullptr, s, sp);
@@ -1177,16 +1189,19 @@ static ddh_status edge_tune(ddh_ctx* ctx, const Work& w, int R, bool fp64) {
         for (int rep = 0; rep < 5; ++rep) run();
         cudaEventRecord(e1, s);
         cudaEventSynchronize(e1);
-        cudaEventElapsedTime(&tm[f], e0, e1);
+        float ms = 0;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (!f.threads) persistent = ms;
+        else if (ms < 0.99f * best) { best = ms; pick = f; }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     CK(cudaGetLastError());
     ctx->edge_tpr[key] = dt;
     ctx->edge_tpr_host[key] = host;
-    const int one_best = tm[2] < tm[1] ? 2 : 1;
-    ctx->edge_nt[key] = forms[one_best][1];
-    ctx->edge_persist[key] = ctx->opt.edge_launch == DDH_EDGE_LAUNCH_AUTO ? tm[0] < tm[one_best]
+    ctx->edge_nt[key] = pick.threads;
+    ctx->edge_staged[key] = pick.stage;
+    ctx->edge_persist[key] = ctx->opt.edge_launch == DDH_EDGE_LAUNCH_AUTO ? persistent < best
                                                                          : ctx->opt.edge_launch == DDH_EDGE_LAUNCH_PERSISTENT;
     return DDH_OK;
 }
@@ -1282,7 +1297,10 @@ static EdgeSched edge_sched(const ddh_ctx* ctx, bool fp64, int R) {
     EdgeSched es;
     const int key = edge_key(fp64, R);
     const auto nt = ctx->edge_nt.find(key);
-    if (nt != ctx->edge_nt.end()) es.cta_threads = nt->second;
+    if (nt != ctx->edge_nt.end()) {
+        es.cta_threads = nt->second;
+        es.stage = ctx->edge_staged.at(key);
+    }
     const auto pt = ctx->edge_persist.find(key);
     if (pt == ctx->edge_persist.end() || !pt->second) return es;   // one CTA per task
     es.items = ctx->edge_items;

@@ -8,8 +8,9 @@
 // 0 <= f < 1.  The exponent e is shared: by one row of the matrix (fixed when the matrix is laid
 // out) and by one staged vector (its largest component, found while it is staged).  A matrix is kept in this
 // form (24 bytes an entry, or packed in 16) beside its complex128 one.  Then
-//   a x = ah xh 2^52 + (ah xl + al xh) 2^26 + [ (ah xf + af xh) 2^26 + al xl + af xf ] + (al xf + af xl, below
-//         2^-25 of the bracket's bound)
+//   a x = ah xh 2^52 + (ah xl + al xh) 2^26 + [ (ah xf + af xh) 2^26 + al xl ] + (al xf + af xl + af xf)
+// and the last part is below 2^-25 of the bracket's bound (af xf is kept where ah = 0, so that nothing is left
+// of a product only where a factor is zero).
 // The first two kinds are summed in 64-bit integers, without error; the bracket in FP32.  The bracket is at most
 // 2^-51 of the scale 2^(ea + ex) of a row and a vector, whatever the size of the term itself, and FP32
 // rounds each of its additions, so a sum comes out to 2^-72 (30 terms) to 2^-69 (255) of the scale.
@@ -23,8 +24,7 @@
 // Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication by using fast routines
 // of matrix multiplication", 2012.)
 //
-// Everything here but the two bit helpers is plain C++: host code calls the same functions
-// (ddh_fixed_dot).
+// Everything here but fx_again compiles for the host as well, where ddh_fixed_dot calls it.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>

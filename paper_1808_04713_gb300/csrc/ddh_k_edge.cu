@@ -261,16 +261,16 @@ __device__ __forceinline__ void bulk_copy(uint64_t* bar, void* dst, const void* 
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
-// Staging of S_E^-1 by bulk copies: in FP64 its limbs, then its fractions
+// Staging of S_E^-1 by a bulk copy: in FP64 its limbs; the fractions are read where they lie, so that two CTAs fit
+// on an SM up to n_E = 72 (n_E = 64, 8 right-hand sides: 220 us, 366 us with both staged and one CTA)
 template <class T>
 __device__ __forceinline__ void edge_copy(uint64_t* bar, char* dst, const DevModel& dm, const cpx<T>* sinv, int e, int nE) {
     const size_t n = (size_t)nE * nE;
     const int64_t off = dm.sinv_off[e];
     if constexpr (std::is_same<T, double>::value) {
-        const uint32_t b0 = (uint32_t)(n * sizeof(int4)), b1 = (uint32_t)(n * sizeof(float2) + 15) & ~15u;
-        bulk_expect(bar, b0 + b1);
+        const uint32_t b0 = (uint32_t)(n * sizeof(int4));
+        bulk_expect(bar, b0);
         bulk_copy(bar, dst, dm.sinv_fx.i + off, b0);
-        bulk_copy(bar, dst + b0, dm.sinv_fx.f + off, b1);
     } else {
         const uint32_t b = (uint32_t)(n * sizeof(cpx<T>) + 15) & ~15u;
         bulk_expect(bar, b);
@@ -295,7 +295,7 @@ __device__ __forceinline__ auto pass1_load(const DevModel& dm, const double2* z,
 template <class T>
 __device__ __forceinline__ void edge_staged(char* sm, int nE, const cpx<T>*& S, FxMat& Sx) {
     if constexpr (std::is_same<T, double>::value)
-        Sx = {reinterpret_cast<int4*>(sm), reinterpret_cast<float2*>(sm + (size_t)nE * nE * sizeof(int4))};
+        Sx.i = reinterpret_cast<int4*>(sm);
     else S = reinterpret_cast<const cpx<T>*>(sm);
 }
 
@@ -634,7 +634,8 @@ __global__ void k_dinv(DevModel dm, const double2* __restrict__ x, double2* __re
 // out_E = S x for the restricted stiffness Schur complement S (n_E x n_E, symmetric, read from
 // global memory column by column: coalesced across output rows, shared by the elements of a
 // degree pattern and L1/L2-resident); tpr adjacent threads share an output row.  FP64: the products of
-// ddh_fixed.cuh, exponents pre_ex by row (an application as below 0.28 ms, 0.52 ms in FP64).
+// ddh_fixed.cuh, exponents pre_ex by row (an application as below 0.28 ms, 0.52 ms in FP64).  At
+// most 80 registers a thread: 24 warps per SM instead of 16 (230 -> 228 us here, 73.9 -> 67.7 us at 40 x 40, p = 12).
 template <class T, int RB>
 __device__ __forceinline__ void pre_apply(const DevModel& dm, int e, int nE, int cnt, const EdgeVec<T>& in, const int* ex,
                                           cpx<T>* __restrict__ out, int64_t ostride,
@@ -740,7 +741,7 @@ __global__ void k_fix_pre(const double* __restrict__ S, const int64_t* __restric
 }
 
 template <class T, int RB>
-__global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pre_elem(const __grid_constant__ DevModel dm, const double2* __restrict__ v, cpx<T>* __restrict__ outE,
+__global__ void __launch_bounds__(128 * kEdgeParts<T, RB>, std::is_same<T, double>::value && RB >= 4 ? 6 / kEdgeParts<T, RB> : 1) k_pre_elem(const __grid_constant__ DevModel dm, const double2* __restrict__ v, cpx<T>* __restrict__ outE,
                                                   int R, const int* __restrict__ done, int with_d) {
     if (done && *done) return;
     extern __shared__ __align__(128) char smem[];
@@ -773,7 +774,7 @@ __global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pre_elem(const __gr
 // Conforming meshes (no hanging rows: D = 2 I, no C2 K C2^T term), fused with the Krylov
 // fetch: v = V[r][j] read directly (j = ctl[0]), D^-1 = 1/2 applied in the gather.
 template <class T, int RB>
-__global__ void __launch_bounds__(128 * kEdgeParts<T, RB>) k_pre_elem_kry(const __grid_constant__ DevModel dm, const __grid_constant__ KrylovDev K, cpx<T>* __restrict__ outE, int R) {
+__global__ void __launch_bounds__(128 * kEdgeParts<T, RB>, std::is_same<T, double>::value && RB >= 4 ? 6 / kEdgeParts<T, RB> : 1) k_pre_elem_kry(const __grid_constant__ DevModel dm, const __grid_constant__ KrylovDev K, cpx<T>* __restrict__ outE, int R) {
     if (K.ctl[1]) return;
     const int jj = K.ctl[0];
     extern __shared__ __align__(128) char smem[];
@@ -892,9 +893,10 @@ void launch_pass1_edge(const DevModel& dm, const void* sinv, const void* Y, cons
         return;
     }
     // the t_T rows alone read no S_E^-1: no staging
-    const int so = rows == 2 ? 0 : edge_stage_off<T>(rb, dm.maxE1);
+    const bool stage = rows != 2 && !(es && !es->stage);
+    const int so = stage ? edge_stage_off<T>(rb, dm.maxE1) : 0;
     const int ntask = dm.E * ((R + rb - 1) / rb);
-    const size_t sm = rows == 2 ? edge_vec_bytes<T>(rb, dm.maxE1) : edge_smem_total<T>(rb, dm.maxE1);
+    const size_t sm = stage ? edge_smem_total<T>(rb, dm.maxE1) : edge_vec_bytes<T>(rb, dm.maxE1);
     const int vs = std::max(1, dm.maxE1);
     // CTA size: two threads per output row of the widest element when that is more than 64
     // rows (rounded up to whole warps), else 256; the CTA takes the rows in one pass and fewer

@@ -136,15 +136,17 @@ inline size_t pass_smem_total(int pmax, int rb, int maxE1) {
 // warps (elements) per CTA: up to 4 while the per-warp shared memory fits in 200 KB
 
 // edge-operator pass 1: the staged vectors, then (when it fits) the staged S_E^-1 behind an mbarrier.  Bytes per
-// entry of either: in FP64 limbs and FP32 parts (ddh_fixed.cuh), and a vector's FP64 entries
+// entry of a vector (in FP64 limbs, FP32 parts and the entry, ddh_fixed.cuh), of an operator (limbs and
+// fractions) and of the staged S_E^-1 (limbs)
 template <class T> constexpr int kEdgeVecBytes = sizeof(T) == 8 ? 48 : 8;
 template <class T> constexpr int kEdgeMatBytes = sizeof(T) == 8 ? 24 : 8;
+template <class T> constexpr int kEdgeStageBytes = sizeof(T) == 8 ? 16 : 8;
 template <class T>
 inline size_t edge_vec_bytes(int rb, int maxE1) {
     return ((size_t)rb * std::max(1, maxE1) * kEdgeVecBytes<T> + 127) & ~(size_t)127;
 }
 template <class T>
-inline size_t edge_mat_bytes(int maxE1) { return ((size_t)maxE1 * maxE1 * kEdgeMatBytes<T> + 127) & ~(size_t)127; }
+inline size_t edge_mat_bytes(int maxE1) { return ((size_t)maxE1 * maxE1 * kEdgeStageBytes<T> + 127) & ~(size_t)127; }
 template <class T>
 inline int edge_stage_off(int rb, int maxE1) {
     const size_t base = edge_vec_bytes<T>(rb, maxE1);

@@ -42,6 +42,7 @@ struct EdgeSched {
     const int* items = nullptr;
     const signed char* tpr_p = nullptr;
     int cta_threads = 0;        // one-CTA-per-task form: CTA size (0 = the size rule of the launcher)
+    bool stage = true;          // and S_E^-1 through shared memory, where it fits
 };
 // Krylov-loop passes with the explicit edge operators Y = [A11^-1 A_1T]_E (no FDM; pass 1
 // requires a load without interior components, pass 2 no recovery).  With es (and es->items)
