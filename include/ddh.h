@@ -271,7 +271,10 @@ ddh_status ddh_solve_dirichlet(ddh_ctx* ctx, const void* b_dev, const void* g_de
  * fast-diagonalisation solver (Sec. 2.2.1 fast solver; Sec. 2.3.3 block inversion), the
  * coarse matrix K = A22 - A12^T A11^-1 A12 and its nested-dissection factor, the preconditioner
  * pieces.  Returns DDH_WARN_NEAR_RESONANT when an element is within 1e-6 of a resonance of
- * A11 (the factorisation is still usable).  opt may be NULL (defaults). */
+ * A11 (the factorisation is still usable).  opt may be NULL (defaults).
+ * Device memory: the coarse factor takes 40 bytes per complex entry (32 as a dense K^-1), being kept also
+ * in the form that the FP64 products read; S_E^-1 and Y take 16, and 24 and 48 more from the first FP64
+ * application on (ddh_solve in FP64, ddh_apply_dual_operator). */
 ddh_status ddh_factor(ddh_ctx* ctx, const ddh_options* opt);
 
 ddh_status ddh_get_info(const ddh_ctx* ctx, ddh_info* out);
@@ -356,7 +359,8 @@ ddh_status ddh_primal_residual_noalloc(ddh_ctx* ctx, const void* b_dev, const vo
  *   *edge_persistent   launch form of the Krylov-loop pass 1 with explicit edge operators: 1 the
  *                      persistent form over the degree-sorted element list, 0 one CTA per
  *                      (element, RHS block), -1 not tuned (nested-dissection-only or FDM form);
- *   *edge_cta_threads  CTA size of the one-CTA-per-task form (0 when not tuned);
+ *   *edge_cta_threads  CTA size of the one-CTA-per-task form (0 when not tuned; in FP64 a CTA of eight
+ *                      right-hand sides has twice as many);
  *   tpr_by_degree[33]  threads sharing one output row in the persistent Krylov-loop pass 1 for
  *                      each element degree p (2 or 4; 0 where no element has degree p or the
  *                      pass has not been tuned for this R).  None of the shapes reported here
